@@ -71,7 +71,9 @@ typedef struct {
                                 * Brandes passes (bcpp_brandes, bcpp_brandes_batched, Brandes++ without
                                 * non-frontier nodes); Dijkstra_SK, Brandes_SK with Centrality and
                                 * bcpp_sssp use 32. */
-    int32_t ctas_per_sm;       /* resident source batches per SM: 0 = auto */
+    int32_t ctas_per_sm;       /* resident source batches per SM of the lockstep kernel: 0 = auto (the
+                                * level-mask kernel, which serves FP64 calls with weights up to 32, takes
+                                * its own launch shape whatever this and `cluster` say) */
     int32_t validate;          /* reserved: the CSR, S and the partition are always checked */
     int32_t host_buffers;      /* 1: array arguments are host pointers (copied in and out) */
     int32_t order_sources;     /* 1 (default): batch the targets in order of their breadth-first level

@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "csr.cuh"
+#include "levels.cuh"
 #include "lockstep.cuh"
 #include "partition.cuh"
 #include "prims.cuh"
@@ -557,6 +558,7 @@ int finish_status(bcpp_ctx* c, bcpp_stats* st) {
         st->ms_batch_backward = (float)(hp[1] * 1e-6);
     }
     if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
+    if (c->hflags[FLAG_TIMEOUT]) return BCPP_ETIMEOUT;
     if (c->hflags[FLAG_CAPACITY]) return BCPP_ECAPACITY;
     if (c->hflags[FLAG_SIGMA_OVF]) return BCPP_EOVERFLOW_SIGMA;
     return BCPP_OK;
@@ -607,6 +609,7 @@ int build_in_csr(bcpp_ctx* c, const bcpp_graph* g, InCsr& T) {
 struct OrderWs {
     int64_t ns = 0;
     int32_t n = 0, k = 0;
+    int32_t depth = 0;        // deepest level from the hub
     const int32_t* S = nullptr;
     const int32_t* part = nullptr;
     DBuf<int32_t> pos;        // [n] discovery position of every node
@@ -762,6 +765,7 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
     c->launches++;
     int32_t hmax = 0;
     CK_RC(to_host(c, &hmax, maxl.p, 1));
+    w.depth = hmax;
     const int32_t lmax = std::min(hmax, ORDER_MAX_LEVELS);
     std::vector<int32_t> hcnt((size_t)lmax + 1);
     CK_RC(to_host(c, hcnt.data(), cnt.p, (int64_t)lmax + 1));
@@ -826,6 +830,176 @@ int order_targets(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
     return order_emit(c, w, g->directed != 0);
 }
 
+// --------------------------------------------------------------------------- level-mask passes
+// Workspace and waves of a call that runs on the level-mask kernel (levels.cu): the batches in order,
+// as many per wave as the budget holds.
+struct LmWave {
+    int32_t i0, i1, tile0, ntiles, run0, nruns, natiles;
+};
+struct LmWs {
+    std::vector<LmWave> waves;
+    int lcap = 0;
+    bool narrow = true;
+    int32_t tpb = 0;           // uniform layout: tiles per batch
+    int64_t nodes = 0;         // global nodes
+    DBuf<uint32_t> lev, seen, ctl;
+    DBuf<char> sg;
+    DBuf<double> cc, dsum, bcs, bcc;
+    DBuf<int32_t> tile0, tile_item;
+    DBuf<LmRun> runs;
+};
+
+// Row state kept in flight at most: enough rows that a level's work hides its barrier and its last
+// tiles, small enough that a first call does not wait for the allocation.
+constexpr int64_t LM_WAVE_BYTES = 24ll << 30;
+
+int64_t free_bytes(bcpp_ctx* c) {
+    size_t fr = 0, tot = 0;
+    cudaMemGetInfo(&fr, &tot);
+    int64_t reusable = 0;
+    for (auto& b : c->pool)
+        if (!b.used) reusable += (int64_t)b.bytes;
+    return (int64_t)((double)((int64_t)fr + reusable) * 0.80);
+}
+
+// Calls the level-mask kernel serves: FP64 dependencies, batches of 32 sources, weights up to
+// LM_MAX_WEIGHT, 32-bit arc offsets.  (FP32 dependencies keep the lockstep kernel: their sums would be
+// taken in another order, and FP32 sums in another order differ in the 8th digit.)  A call whose
+// batches prove too deep, or whose path counts outgrow 32 bits, reruns with order_factor 64, which
+// the lockstep kernel serves.
+bool lm_serves(const bcpp_ctx* c, const bcpp_opts& o, int spl, int32_t n, int64_t arcs, uint64_t wmax) {
+    return o.precision != BCPP_FP32_DELTA && spl == 1 && c->order_factor < 64 && arcs < (1ll << 31) &&
+           n < (1 << 25) && wmax <= LM_MAX_WEIGHT;
+}
+
+// Levels to provide for: with unit weights on an undirected graph whose levels from the hub are known,
+// no node of the hub's component is further from another than twice the deepest level.
+int lm_levels(bool weighted, bool directed, const OrderWs* ord) {
+    if (weighted) return LM_MAX_LEVELS;
+    if (!ord) return 64;
+    return std::max(directed ? 64 : 24, 2 * std::min(ord->depth, LM_MAX_LEVELS) + 4);
+}
+
+// false: not enough memory for one batch (the caller takes the lockstep kernel).  sizes: node count of
+// an item's graph; one_graph: every batch is of the same graph.
+template <class F>
+int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_graph, F&& size_of, int64_t nodes,
+             int lcap, bool narrow, bool* fits) {
+    *fits = false;
+    const int nitems = (int)items.size();
+    if (nitems == 0 || lcap > LM_MAX_LEVELS) return BCPP_OK;
+    L.lcap = lcap;
+    L.narrow = narrow;
+    L.nodes = nodes;
+    const int64_t row_bytes = 32 * ((narrow ? 4 : 8) + 8) + 8 + 4 + 4ll * lcap;
+    const int64_t budget = free_bytes(c);
+    int64_t total = 0, largest = 0;
+    std::vector<int32_t> tile0;
+    if (!one_graph) tile0.resize((size_t)nitems + 1);
+    for (int i = 0; i < nitems; i++) {
+        const int64_t t = (size_of(items[i].g) + 31) / 32;
+        if (!one_graph) tile0[i] = (int32_t)total;
+        total += t;
+        largest = std::max(largest, t);
+        if (total >= (1ll << 31)) return BCPP_OK;
+    }
+    if (!one_graph) tile0[nitems] = (int32_t)total;
+    const int64_t tile_bytes = 32 * row_bytes;
+    const int64_t extra = total * 4 + (int64_t)nitems * 8 + 16 * nodes;
+    if (largest * tile_bytes + extra > budget) return BCPP_OK;
+    int64_t cap = std::max(largest, std::min(budget - extra, LM_WAVE_BYTES) / tile_bytes);
+    cap = std::min<int64_t>(cap, (1ll << 31) / 32 - 1);   // rows of a wave below 2^31
+    if (largest > cap) return BCPP_OK;
+    // waves of about equal size
+    const int64_t nwaves = (total + cap - 1) / cap;
+    const int64_t goal = std::min(cap, (total + nwaves - 1) / nwaves + largest);
+    std::vector<LmRun> runs;
+    int64_t most = 0;
+    int most_items = 0, tbase = 0;
+    for (int i = 0; i < nitems;) {
+        LmWave w{i, i, tbase, 0, (int32_t)runs.size(), 0, 0};
+        while (w.i1 < nitems) {
+            const int32_t t = (int32_t)((size_of(items[w.i1].g) + 31) / 32);
+            if (w.i1 > w.i0 && w.ntiles + t > goal) break;
+            if (w.nruns == 0 || runs.back().g != items[w.i1].g) {
+                runs.push_back(LmRun{items[w.i1].g, w.i1 - w.i0, 0, w.natiles});
+                w.nruns++;
+                w.natiles += t;
+            }
+            runs.back().count++;
+            w.ntiles += t;
+            w.i1++;
+        }
+        tbase += w.ntiles;
+        most = std::max<int64_t>(most, w.ntiles);
+        most_items = std::max(most_items, w.i1 - w.i0);
+        L.waves.push_back(w);
+        i = w.i1;
+    }
+    const int64_t rows = most * 32;
+    CK_ALLOC(L.lev.alloc(c, rows * lcap));
+    CK_ALLOC(L.seen.alloc(c, rows));
+    CK_ALLOC(L.sg.alloc(c, rows * 32 * (narrow ? 4 : 8)));
+    CK_ALLOC(L.cc.alloc(c, rows * 32));
+    CK_ALLOC(L.dsum.alloc(c, rows));
+    CK_ALLOC(L.ctl.alloc(c, lm_ctl_words(lcap, most_items)));
+    CK_ALLOC(L.bcs.alloc(c, nodes));
+    CK_ALLOC(L.bcc.alloc(c, nodes));
+    CK_ALLOC(L.runs.alloc(c, (int64_t)runs.size()));
+    CK_RC(to_dev(c, L.runs.p, runs.data(), (int64_t)runs.size()));
+    if (one_graph) {
+        L.tpb = (int32_t)largest;
+    } else {
+        CK_ALLOC(L.tile0.alloc(c, (int64_t)nitems + 1));
+        CK_ALLOC(L.tile_item.alloc(c, total));
+        CK_RC(to_dev(c, L.tile0.p, tile0.data(), (int64_t)nitems + 1));
+        lm_tile_items(L.tile0.p, nitems, (int32_t)total, L.tile_item.p, c->stream);
+        c->launches++;
+    }
+    *fits = true;
+    return BCPP_OK;
+}
+
+// All waves and the sum over sources (device work only): out = scale * sum.
+int lm_emit(bcpp_ctx* c, LmWs& L, const LsArena& A, const LsParams& P, const LsItem* items, uint64_t wmax,
+            double scale, double* out, Timer* tb) {
+    CK_CUDA(cudaMemsetAsync(L.bcs.p, 0, (size_t)L.nodes * sizeof(double), c->stream));
+    CK_CUDA(cudaMemsetAsync(L.bcc.p, 0, (size_t)L.nodes * sizeof(double), c->stream));
+    if (tb) tb->start();
+    for (const LmWave& w : L.waves) {
+        LmArgs a{};
+        a.rp = A.rp; a.col = A.col; a.w = A.w;
+        a.irp = A.irp; a.icol = A.icol; a.iw = A.iw;
+        a.node_off = A.node_off;
+        a.items = items + w.i0;
+        a.item_tile0 = L.tpb ? nullptr : L.tile0.p + w.i0;
+        a.tile_item = L.tile_item.p;
+        a.tile_base = L.tpb ? 0 : w.tile0;
+        a.item_base = w.i0;
+        a.tpb = L.tpb;
+        a.nitems = w.i1 - w.i0;
+        a.ntiles = w.ntiles;
+        a.srcs = P.srcs;
+        a.in_s = P.in_s;
+        a.lev = L.lev.p; a.seen = L.seen.p; a.sg = L.sg.p; a.cc = L.cc.p; a.dsum = L.dsum.p;
+        a.rows = (int64_t)w.ntiles * 32;
+        a.lcap = L.lcap;
+        a.wmax = (int32_t)wmax;
+        a.ctl = L.ctl.p;
+        a.flags = P.flags;
+        a.phase_ns = P.phase_ns;
+        CK_CUDA(cudaMemsetAsync(L.ctl.p, 0, (size_t)lm_ctl_words(L.lcap, a.nitems) * sizeof(uint32_t), c->stream));
+        CK_CUDA(lm_launch(a, L.narrow, c->num_sms, c->stream));
+        lm_accumulate(a, L.runs.p + w.run0, w.nruns, w.natiles, L.bcs.p, L.bcc.p, c->stream);
+        c->launches += 2;
+    }
+    if (tb) tb->stop();
+    combine_launch(L.bcs.p, L.bcc.p, 1, L.nodes, L.nodes, scale, out, c->stream);
+    c->launches++;
+    CK_CUDA(cudaGetLastError());
+    return BCPP_OK;
+}
+
 // --------------------------------------------------------------------------- plain Brandes
 // A plain-Brandes evaluation in two parts: plain_prepare takes every host decision (input
 // checks, sizes, batches, workspace) and plain_emit queues the device work only, so that the
@@ -849,6 +1023,8 @@ struct PlainRun {
     DBuf<LsItem> items;
     DBuf<int64_t> node_off;
     SlotWs ws;
+    LmWs lm;
+    bool levels = false;           // on the level-mask kernel
     int nitems = 0, slots = 0, spl = 1, cl = 1, nb = 2;
     LsArena A{};
     LsParams P{};
@@ -927,8 +1103,11 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     shard_sources(o, r.ns, s0, s1);
     r.spl = choose_spl(c, s1 - s0, o);
     std::vector<LsItem> hitems = make_items(0, s0, s1, 32 * r.spl);
+    if (lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1))
+        CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
+                       lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
     r.cl = r.spl == 1 ? choose_cluster(c, (int)hitems.size(), o) : 1;
-    if (r.spl == 1) {
+    if (r.spl == 1 && !r.levels) {
         const int b = balanced_width(s1 - s0, slot_capacity(c, o, r.cl), 32);
         if (b < 32) hitems = make_items(0, s0, s1, b);
     }
@@ -940,10 +1119,12 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     const int64_t hoff[2] = {0, n};
     CK_RC(to_dev(c, r.node_off.p, hoff, 2));
     r.nb = g->w ? (int)r.wmax + 1 : 2;
-    const int ef = entry_factor(c, g->w != nullptr, r.spl);
-    r.slots = choose_slots(c, r.nitems, o.ctas_per_sm, slot_bytes(n, r.nb, fp32, ef, r.spl), (int64_t)n * 24, r.cl);
-    CK_RC(alloc_slots(c, r.ws, r.slots, n, r.nb, fp32, n, r.spl, ef, false));
-    r.ws.narrow = use_narrow(c, g->w != nullptr);
+    if (!r.levels) {
+        const int ef = entry_factor(c, g->w != nullptr, r.spl);
+        r.slots = choose_slots(c, r.nitems, o.ctas_per_sm, slot_bytes(n, r.nb, fp32, ef, r.spl), (int64_t)n * 24, r.cl);
+        CK_RC(alloc_slots(c, r.ws, r.slots, n, r.nb, fp32, n, r.spl, ef, false));
+        r.ws.narrow = use_narrow(c, g->w != nullptr);
+    }
     LsArena& A = r.A;
     A.rp = g->row_ptr; A.col = g->col; A.w = (const int32_t*)g->w; A.mu = nullptr;
     if (g->directed) {
@@ -980,6 +1161,8 @@ int plain_emit(bcpp_ctx* c, PlainRun& r, Timer* tb) {
     }
     if (g->directed) CK_RC(in_csr_emit(c, g, r.T));
     if (r.ordered) CK_RC(order_emit(c, r.ord, g->directed != 0));
+    const bool halve = !g->directed && r.o.halve_undirected != 0;
+    if (r.levels) return lm_emit(c, r.lm, r.A, r.P, r.items.p, g->w ? r.wmax : 1, halve ? 0.5 : 1.0, r.bc_out, tb);
     CK_RC(init_slots(c, r.ws));
     if (tb) tb->start();
     ls_launch(r.o.precision == BCPP_FP32_DELTA, !g->directed, r.A, r.P, r.ws.W, r.items.p, r.nitems, r.slots,
@@ -987,7 +1170,6 @@ int plain_emit(bcpp_ctx* c, PlainRun& r, Timer* tb) {
     c->launches++;
     if (tb) tb->stop();
     CK_CUDA(cudaGetLastError());
-    const bool halve = !g->directed && r.o.halve_undirected != 0;
     combine_launch(r.ws.W.bc_sum, r.ws.W.bc_cmp, r.slots, n, n, halve ? 0.5 : 1.0, r.bc_out, c->stream);
     c->launches++;
     CK_CUDA(cudaGetLastError());
@@ -1834,7 +2016,7 @@ int brandes_pp_all_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* part, in
         ms_ce += L.tce->resolve();
         calls += L.calls;
     }
-    if (merged[FLAG_INVALID] | merged[FLAG_CAPACITY] | merged[FLAG_SIGMA_OVF] | merged[FLAG_DEPTH]) {
+    if (merged[FLAG_INVALID] | merged[FLAG_CAPACITY] | merged[FLAG_SIGMA_OVF] | merged[FLAG_DEPTH] | merged[FLAG_TIMEOUT]) {
         CK_RC(sync_flags(c));
         for (int f = 0; f < FLAG_COUNT; f++) merged[f] |= c->hflags[f];
         CK_CUDA(cudaMemcpyAsync(c->flags, merged, sizeof(merged), cudaMemcpyHostToDevice, c->stream));
@@ -1910,13 +2092,11 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
     iota(srcs.p, maxn, c->stream);
     c->launches++;
     const int nb = g->w ? (int)wmax + 1 : 2;
-    const int slots =
-        choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxn, nb, fp32, entry_factor(c, g->w != nullptr, spl), spl),
-                     (int64_t)n * 24);
-    SlotWs ws;
-    CK_RC(alloc_slots(c, ws, slots, maxn, nb, fp32, n, spl, entry_factor(c, g->w != nullptr, spl), false));
-    ws.narrow = use_narrow(c, g->w != nullptr);
-    CK_RC(init_slots(c, ws));
+    bool levels = false;
+    LmWs lm;
+    if (lm_serves(c, o, spl, (int32_t)maxn, g->num_arcs, g->w ? wmax : 1))
+        CK_RC(lm_alloc(c, lm, hitems, false, [&](int32_t gi) { return off[gi + 1] - off[gi]; }, n,
+                       lm_levels(g->w != nullptr, false, nullptr), true, &levels));
     LsArena A{};
     A.rp = g->row_ptr; A.col = lcol.p; A.w = (const int32_t*)g->w;
     A.irp = g->row_ptr; A.icol = lcol.p; A.iw = (const int32_t*)g->w;
@@ -1925,9 +2105,26 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
     P.mode = LS_BRANDES;
     P.nb = nb;
     P.srcs = srcs.p;
-    P.item_counter = ws.counter.p;
     P.flags = c->flags;
     P.phase_ns = c->phase;
+    if (levels) {
+        CK_RC(lm_emit(c, lm, A, P, items.p, g->w ? wmax : 1, o.halve_undirected ? 0.5 : 1.0, bc_out, &tb));
+        int rc = finish_status(c, st);
+        tt.stop();
+        if (st) {
+            st->ms_brandes_sk = tb.acc;
+            st->ms_total = tt.acc;
+        }
+        return rc;
+    }
+    const int slots =
+        choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxn, nb, fp32, entry_factor(c, g->w != nullptr, spl), spl),
+                     (int64_t)n * 24);
+    SlotWs ws;
+    CK_RC(alloc_slots(c, ws, slots, maxn, nb, fp32, n, spl, entry_factor(c, g->w != nullptr, spl), false));
+    ws.narrow = use_narrow(c, g->w != nullptr);
+    CK_RC(init_slots(c, ws));
+    P.item_counter = ws.counter.p;
     tb.start();
     ls_launch(fp32, true, A, P, ws.W, items.p, nitems, slots, c->stream, spl, 1, ws.narrow);
     c->launches++;

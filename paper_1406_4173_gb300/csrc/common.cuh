@@ -18,6 +18,7 @@ enum : int {
     FLAG_INVALID = 2,       // input validation failed
     FLAG_INVALID_WHY = 3,   // first reason code of an invalid input
     FLAG_DEPTH = 4,         // a one-byte distance or 32-bit path count would overflow (rerun with wide rows)
+    FLAG_TIMEOUT = 5,       // a grid barrier gave up waiting
     FLAG_COUNT = 8
 };
 

@@ -1,0 +1,617 @@
+// Level-mask passes of plain Brandes (Eq. 2 / Eq. 5-7) for many batches of 32 sources at once.
+//
+// Layout.  A row is one (batch, node) pair; its 32 positions are the batch's sources.  Instead of a
+// distance per source, a row has one 32-bit mask per distance level: bit s of lev[D][row] says that
+// source s reaches the node at distance D.  One 4-byte gather then answers for 32 sources what a
+// distance row answers with 32 to 128 bytes.
+//
+// Forward, level D (pull): every row that some source has not reached gathers lev[D - w] of its
+// in-neighbours; the sources found there and not seen before are the row's new mask, and their path
+// counts are the sums over exactly the arcs whose gathered mask has the source's bit.  No tentative
+// distances, no buckets, no settle lists, no atomics on global memory.
+// Backward, level D from the deepest: a row with a mask at D gathers lev[D + w] of its
+// out-neighbours; c(s,u) = (I + delta) / sigma is summed over the arcs whose mask has the bit.  A
+// pair whose c is zero (no target behind it) is taken out of the mask, so nobody adds it.
+//
+// Work split.  The whole GPU takes one level of all batches of a wave at a time (a cooperative launch
+// with a grid barrier per level); warps take tiles of 32 rows in order, so that the SMs sweep one or
+// two batches at a time, whose count rows (n * 128 bytes) stay in L2.  In a tile, arcs are spread
+// over lanes (a lane per arc: heads and masks), the few arcs with a bit in common are compacted
+// in shared memory, and then (row, source) pairs are spread over lanes: a lane sums the counts (or
+// dependencies) of its pair over the row's compacted arcs.  So neither low degrees nor rows with
+// few active sources leave lanes idle, and the FP64 adds of the backward pass, which GB300 issues at
+// 2 lanes per SM and cycle, are done for packed pairs only.
+//
+// Measured against the lockstep kernel (whole call, FP64): Chung-Lu n = 50,000, every node a target
+// 251 -> 125 ms; n = 1,000,000, 4,096 targets 709 -> 156 ms; directed, n = 100,000, weights 1 to 16,
+// 2,000 targets 141 -> 39 ms; 4,096 random graphs 427 -> 185 ms; n = 2,000, every node 1.76 -> 1.30 ms.
+// Bound by the latency of its gathers (a profile at n = 10,000: instructions issued on 27% of the
+// cycles, FP64 pipe busy 30%) and, in the backward pass, by FP64 adds.
+#include <algorithm>
+
+#include "levels.cuh"
+
+namespace bcpp {
+namespace {
+
+constexpr int LM_THREADS = 256;
+constexpr int LM_WARPS = LM_THREADS / 32;
+// resident blocks per SM (48 registers): 40 warps.  4 blocks 127 / 164 / 38 / 189 ms on the four large
+// workloads above, 5: 122 / 148 / 37 / 181, 6 (spills): 124 / 148 / 47 / 183
+#ifndef BCPP_LM_MINB
+#define BCPP_LM_MINB 5
+#endif
+#ifndef BCPP_LM_PU
+#define BCPP_LM_PU 4           // values a pair's sum has in flight
+#endif
+#ifndef BCPP_LM_BU
+#define BCPP_LM_BU 4           // the same for a row of many arcs (8: no faster)
+#endif
+constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of larger degree go one by one)
+constexpr int CTL_BAR = 0, CTL_GEN = 1, CTL_ABORT = 2, CTL_LVL = 8;
+constexpr unsigned LVL_ANY = 1u, LVL_ERR = 2u;
+constexpr unsigned LM_SPIN_MAX = 1u << 28;   // polls of the grid barrier before it gives up
+
+// 1/x for small path counts, correctly rounded by the compiler
+constexpr int RCP_N = 1024;
+struct RcpTable {
+    double v[RCP_N];
+    constexpr RcpTable() : v() {
+        for (int i = 1; i < RCP_N; i++) v[i] = 1.0 / i;
+    }
+};
+__device__ const RcpTable c_rcp{};
+
+__device__ __forceinline__ double recip_of(uint64_t s) {
+    if (s < (uint64_t)RCP_N) return __ldg(&c_rcp.v[(int)s]);
+    // single-precision seed and one Newton-Raphson step (relative error below 1.5e-14)
+    const double x = (double)s;
+    const double r = (double)__frcp_rn((float)x);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
+struct WarpSm {
+    uint2 list[LM_CAP];        // arcs with a bit in common: head row, mask
+    uint32_t nm[32];           // masks found, by candidate
+    uint32_t rowm[32];         // masks found, by row of the tile
+    double ds[32];             // dependencies, by row of the tile
+    int seg[33];               // first list entry of each candidate
+    int idx[32];               // compaction scratch
+    int pad;
+};
+
+// Barrier over all blocks of the cooperative launch.  false: gave up (never with co-resident blocks).
+__device__ bool grid_barrier(uint32_t* ctl, uint32_t* flags) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        volatile uint32_t* gen = ctl + CTL_GEN;
+        volatile uint32_t* ab = ctl + CTL_ABORT;
+        const uint32_t g = *gen;
+        __threadfence();
+        if (atomicAdd(ctl + CTL_BAR, 1u) == gridDim.x - 1) {
+            ctl[CTL_BAR] = 0u;
+            __threadfence();
+            atomicAdd(ctl + CTL_GEN, 1u);
+        } else {
+            unsigned polls = 0;
+            while (*gen == g && *ab == 0u) {
+                __nanosleep(20);
+                if (++polls == LM_SPIN_MAX) {
+                    atomicOr(&flags[FLAG_TIMEOUT], 1u);
+                    atomicExch(ctl + CTL_ABORT, 1u);
+                }
+            }
+        }
+        s_ok = *ab == 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// position of the n-th set bit (from 0) of x; n < popc(x)
+__device__ __forceinline__ int nth_bit(uint32_t x, int n) {
+    int pos = 0;
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) {
+        const int c = __popc(x & ((1u << h) - 1u));
+        const bool up = n >= c;
+        n -= up ? c : 0;
+        pos += up ? h : 0;
+        x = up ? x >> h : x;
+    }
+    return pos;
+}
+
+// Every (lane, bit) of the lanes' masks, 32 at a time in order: f(ok, k, s, first) for source s of
+// lane k's mask; `first` has a bit for every lane of the chunk that starts a new k.
+template <class F>
+__device__ __forceinline__ void for_pairs(uint32_t mask, int lane, int* idx, F&& f) {
+    const unsigned le = 0xffffffffu >> (31 - lane);
+    const unsigned nb = __ballot_sync(FULL, mask != 0u);
+    if (nb == 0u) return;
+    if (mask) idx[__popc(nb & (le >> 1))] = lane;
+    const int cnt = __popc(mask);
+    const int incl = warp_incl_scan(cnt, lane);
+    const int total = __shfl_sync(FULL, incl, 31);
+    const int st = incl - cnt;
+    __syncwarp();
+    int kb = -1;
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        const unsigned at = (unsigned)(st - p0);
+        const unsigned first = __reduce_or_sync(FULL, mask != 0u && at < 32u ? 1u << at : 0u);
+        const int k = idx[kb + __popc(first & le)];
+        kb += __popc(first);
+        const uint32_t mk = __shfl_sync(FULL, mask, k);
+        const int n = p0 + lane - __shfl_sync(FULL, st, k);
+        const bool ok = p0 + lane < total;
+        f(ok, k, ok ? nth_bit(mk, n) : 0, first);
+    }
+    __syncwarp();
+}
+
+// The tile's sums over its candidates' arcs.  FWD: in-arcs, masks at D - w, counts; else out-arcs,
+// masks at D + w, dependencies.  need / a0 / deg: this lane's row (need = 0: none).  Found masks go to
+// sm.rowm by row (zeroed by the caller).
+//   pair_done(ok, r, s, acc, first): the sum of source s of the tile's row r (packed pairs)
+//   row_done(r, mask, acc): the same for all 32 sources of one row, lane = source
+template <bool FWD, bool WEIGHTED, typename V, typename ACC, class PD, class RD>
+__device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane, uint32_t need, int64_t a0, int deg,
+                                          int D, int bd, int64_t rb, const int32_t* __restrict__ col,
+                                          const int32_t* __restrict__ wt, const V* vals, PD&& pair_done,
+                                          RD&& row_done) {
+    const unsigned le = 0xffffffffu >> (31 - lane), lt = le >> 1;
+    const bool cand = need != 0u && deg > 0;
+    const unsigned cm = __ballot_sync(FULL, cand);
+    if (cm == 0u) return;
+    // candidates to the front lanes
+    const int K = __popc(cm);
+    if (cand) sm.idx[__popc(cm & lt)] = lane;
+    __syncwarp();
+    const int crow = lane < K ? sm.idx[lane] : 0;
+    __syncwarp();
+    const uint32_t cneed = __shfl_sync(FULL, need, crow);
+    const uint32_t ca0 = __shfl_sync(FULL, (uint32_t)a0, crow);   // fewer than 2^31 arcs
+    const int cd = __shfl_sync(FULL, deg, crow);
+    const int cdeg = lane < K ? cd : 0;
+    const int pre = warp_incl_scan(cdeg, lane);
+    const uint32_t* L1 = A.lev + (int64_t)(FWD ? D - 1 : D + 1) * A.rows + rb;   // unit weights
+    auto gather = [&](int32_t v, int32_t w) -> uint32_t {
+        if constexpr (!WEIGHTED) return L1[v];
+        const int d2 = FWD ? D - w : D + w;
+        return (FWD ? d2 >= 0 : d2 <= bd) ? A.lev[(int64_t)d2 * A.rows + rb + v] : 0u;
+    };
+    int k0 = 0;
+    while (k0 < K) {
+        const int base = __shfl_sync(FULL, pre - cdeg, k0);
+        const unsigned fit = __ballot_sync(FULL, lane >= k0 && lane < K && pre - base <= LM_CAP);
+        if (fit == 0u) {
+            // one row of many arcs: lane = source
+            const uint32_t nd = __shfl_sync(FULL, cneed, k0);
+            const uint32_t b0 = __shfl_sync(FULL, ca0, k0);
+            const int dg = __shfl_sync(FULL, cdeg, k0);
+            const int r = __shfl_sync(FULL, crow, k0);
+            ACC acc = (ACC)0;
+            uint32_t found = 0u;
+            for (int c0 = 0; c0 < dg; c0 += 32) {
+                int32_t v = 0;
+                uint32_t m = 0u;
+                if (c0 + lane < dg) {
+                    v = __ldg(col + b0 + c0 + lane);
+                    m = gather(v, WEIGHTED ? __ldg(wt + b0 + c0 + lane) : 1) & nd;
+                }
+                found |= m;
+                unsigned tb = __ballot_sync(FULL, m != 0u);
+                while (tb) {
+                    V t[BCPP_LM_BU];
+#pragma unroll
+                    for (int q = 0; q < BCPP_LM_BU; q++) {
+                        const int j = tb ? __ffs(tb) - 1 : 0;
+                        const bool on = tb != 0u;
+                        tb &= tb - 1u;
+                        const int32_t vq = __shfl_sync(FULL, v, j);
+                        const uint32_t mq = __shfl_sync(FULL, m, j);
+                        t[q] = (V)0;
+                        if (on && (mq >> lane) & 1u) t[q] = vals[(rb + vq) * 32 + lane];
+                    }
+#pragma unroll
+                    for (int q = 0; q < BCPP_LM_BU; q++) acc += t[q];
+                }
+            }
+            found = __reduce_or_sync(FULL, found);
+            if (found) {
+                if (lane == 0) sm.rowm[r] = found;
+                row_done(r, found, acc);
+            }
+            k0++;
+            continue;
+        }
+        const int k1 = k0 + __popc(fit);
+        const int T = __shfl_sync(FULL, pre, k1 - 1) - base;
+        const bool inr = lane >= k0 && lane < k1;
+        const int st = pre - cdeg - base;
+        sm.nm[lane] = 0u;
+        __syncwarp();
+        int pos = 0, kb = k0 - 1;
+        for (int i0 = 0; i0 < T; i0 += 32) {
+            const unsigned at = (unsigned)(st - i0);
+            const unsigned first = __reduce_or_sync(FULL, inr && at < 32u ? 1u << at : 0u);
+            const int k = kb + __popc(first & le);
+            kb += __popc(first);
+            const uint32_t off = __shfl_sync(FULL, ca0 - (uint32_t)st, k);
+            const uint32_t nd = __shfl_sync(FULL, cneed, k);
+            int32_t v = 0;
+            uint32_t m = 0u;
+            const int i = i0 + lane;
+            if (i < T) {
+                v = __ldg(col + off + i);
+                m = gather(v, WEIGHTED ? __ldg(wt + off + i) : 1) & nd;
+            }
+            const unsigned tb = __ballot_sync(FULL, m != 0u);
+            const int p = pos + __popc(tb & lt);
+            if (m) {
+                sm.list[p] = make_uint2((uint32_t)v, m);
+                atomicOr(&sm.nm[k], m);
+            }
+            if ((first >> lane) & 1u) sm.seg[k] = p;
+            pos += __popc(tb);
+        }
+        if (lane == 0) sm.seg[k1] = pos;
+        __syncwarp();
+        const uint32_t nm = inr ? sm.nm[lane] : 0u;
+        if (nm) sm.rowm[crow] = nm;
+        if (pos > 0) {
+            for_pairs(nm, lane, sm.idx, [&](bool ok, int k, int s, unsigned first) {
+                const int e1 = ok ? sm.seg[k + 1] : 0;
+                int e = ok ? sm.seg[k] : 0;
+                const int r = __shfl_sync(FULL, crow, k);
+                const V* vs = vals + rb * 32 + s;
+                ACC acc = (ACC)0;
+                while (e < e1) {
+                    V t[BCPP_LM_PU];
+#pragma unroll
+                    for (int q = 0; q < BCPP_LM_PU; q++) {
+                        t[q] = (V)0;
+                        if (e + q < e1) {
+                            const uint2 x = sm.list[e + q];
+                            if ((x.y >> s) & 1u) t[q] = vs[(int64_t)x.x * 32];
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < BCPP_LM_PU; q++) acc += t[q];
+                    e += BCPP_LM_PU;
+                }
+                pair_done(ok, r, s, acc, first);
+            });
+        }
+        __syncwarp();
+        k0 = k1;
+    }
+}
+
+template <typename SG, bool WEIGHTED>
+__global__ void __launch_bounds__(LM_THREADS, BCPP_LM_MINB) lm_kernel(const LmArgs A) {
+    __shared__ WarpSm s_warp[LM_WARPS];
+    const int lane = threadIdx.x & 31;
+    WarpSm& sm = s_warp[threadIdx.x >> 5];
+    const int wid = blockIdx.x * LM_WARPS + (threadIdx.x >> 5);
+    const int nw = gridDim.x * LM_WARPS;
+    SG* sg = static_cast<SG*>(A.sg);
+    double* cc = A.cc;
+    uint32_t* lvl = A.ctl + CTL_LVL;
+    uint32_t* bdepth = lvl + A.lcap + 1;
+    const int wmax = WEIGHTED ? A.wmax : 1;
+    unsigned long long t0 = 0, t1 = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+
+    struct Tile {
+        LsItem I;
+        int32_t n, u;
+        int64_t base, rb;
+        int it;
+    };
+    auto tile_of = [&](int t) {
+        Tile x;
+        int tile0;
+        if (A.item_tile0) {
+            x.it = __ldg(A.tile_item + t + A.tile_base) - A.item_base;
+            tile0 = __ldg(A.item_tile0 + x.it) - A.tile_base;
+        } else {
+            x.it = t / A.tpb;
+            tile0 = x.it * A.tpb;
+        }
+        const int4 q = __ldg(reinterpret_cast<const int4*>(A.items) + x.it);
+        x.I.g = q.x; x.I.src_off = q.y; x.I.nsrc = q.z; x.I.aux = q.w;
+        x.base = __ldg(A.node_off + x.I.g);
+        x.n = (int32_t)(__ldg(A.node_off + x.I.g + 1) - x.base);
+        x.u = (t - tile0) * 32 + lane;
+        x.rb = (int64_t)tile0 * 32;
+        return x;
+    };
+
+    // Tiles go out in order: the first of every warp by its index, the others from one counter per
+    // pass and level, a few at a time (a fixed assignment of all of them left warps waiting for the
+    // rows of high degree: 245 -> 164 ms on 1,000,000 nodes and 4,096 sources).
+    uint32_t* work = bdepth + A.nitems;
+    const int grab = max(1, min(8, A.ntiles / (16 * nw)));
+    auto for_tiles = [&](uint32_t* ctr, auto&& f) {
+        const bool more = A.ntiles > nw;
+        int mine = 0;
+        if (more && lane == 0) mine = nw + (int)atomicAdd(ctr, (uint32_t)grab);
+        if (wid < A.ntiles) f(wid);
+        if (!more) return;
+        for (;;) {
+            const int t0 = __shfl_sync(FULL, mine, 0);
+            if (t0 >= A.ntiles) break;
+            if (lane == 0) mine = nw + (int)atomicAdd(ctr, (uint32_t)grab);   // the next ones, while these run
+            const int t1 = min(t0 + grab, A.ntiles);
+            for (int t = t0; t < t1; t++) f(t);
+        }
+    };
+
+    // level 0: each batch's sources
+    for (int t = wid; t < A.ntiles; t += nw) {
+        const Tile x = tile_of(t);
+        const int64_t row = (int64_t)t * 32 + lane;
+        const int32_t src = lane < x.I.nsrc ? __ldg(A.srcs + x.I.src_off + lane) : -1;
+        const int local = src - (x.u - lane);
+        sm.rowm[lane] = 0u;
+        __syncwarp();
+        if (src >= 0 && local >= 0 && local < 32) {
+            atomicOr(&sm.rowm[local], 1u << lane);
+            sg[(x.rb + src) * 32 + lane] = (SG)1;
+        }
+        __syncwarp();
+        const uint32_t m = sm.rowm[lane];
+        A.lev[row] = m;
+        A.seen[row] = m;
+        A.dsum[row] = 0.0;
+        __syncwarp();
+    }
+    if (!grid_barrier(A.ctl, A.flags)) return;
+
+    // ------------------------------------------------------------------ forward
+    int depth = 0;
+    for (int D = 1;; D++) {
+        if (D >= A.lcap) {
+            // a later level than the masks provide for (or the last one, unseen): the call reruns
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                atomicOr(&A.flags[FLAG_DEPTH], 1u);
+                atomicOr(&A.flags[FLAG_CAPACITY], 1u);
+            }
+            return;
+        }
+        bool any = false, ovf = false;
+        for_tiles(work + D, [&](int t) {
+            const Tile x = tile_of(t);
+            // finished batches: nothing new within the largest weight.  (A cached load: the values of
+            // earlier levels decide, and this SM's own store below shows up in it.)
+            const int bd = (int)bdepth[x.it];
+            if (bd + wmax < D) return;
+            const int64_t row = (int64_t)t * 32 + lane;
+            const uint32_t full = x.I.nsrc >= 32 ? 0xffffffffu : (1u << x.I.nsrc) - 1u;
+            uint32_t seen = 0u, need = 0u;
+            int64_t a0 = 0;
+            int deg = 0;
+            if (x.u < x.n) {
+                seen = A.seen[row];
+                need = full & ~seen;
+                if (need) {
+                    const int64_t* rp = A.irp + x.base + x.u;
+                    a0 = __ldg(rp);
+                    deg = (int)(__ldg(rp + 1) - a0);
+                }
+            }
+            sm.rowm[lane] = 0u;
+            __syncwarp();
+            SG* srow = sg + (int64_t)t * 1024;
+            tile_sums<true, WEIGHTED, SG, uint64_t>(
+                A, sm, lane, need, a0, deg, D, 0, x.rb, A.icol, A.iw, sg,
+                [&](bool ok, int r, int s, uint64_t acc, unsigned) {
+                    if (ok) srow[r * 32 + s] = (SG)acc;
+                    if constexpr (sizeof(SG) == 4) ovf |= ok && (acc >> 32) != 0;
+                },
+                [&](int r, uint32_t mask, uint64_t acc) {
+                    if ((mask >> lane) & 1u) srow[r * 32 + lane] = (SG)acc;
+                    if constexpr (sizeof(SG) == 4) ovf |= ((mask >> lane) & 1u) && (acc >> 32) != 0;
+                });
+            __syncwarp();
+            const uint32_t got = sm.rowm[lane];
+            A.lev[(int64_t)D * A.rows + row] = got;
+            if (got) A.seen[row] = seen | got;
+            if (__any_sync(FULL, got != 0u)) {
+                any = true;
+                if (lane == 0 && bd != D) bdepth[x.it] = (uint32_t)D;
+            }
+            __syncwarp();
+        });
+        if (__any_sync(FULL, ovf)) {
+            if (lane == 0) atomicOr(lvl + D, LVL_ERR | LVL_ANY);
+        } else if (any && lane == 0 && (__ldcg(lvl + D) & LVL_ANY) == 0u) {
+            atomicOr(lvl + D, LVL_ANY);
+        }
+        if (!grid_barrier(A.ctl, A.flags)) return;
+        // every block reads the same word: nobody writes level D's status any more
+        const uint32_t w = __ldcg(lvl + D);
+        if (w & LVL_ERR) {
+            // a path count past 32 bits: the call reruns with 64-bit rows
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                atomicOr(&A.flags[FLAG_DEPTH], 1u);
+                atomicOr(&A.flags[FLAG_CAPACITY], 1u);
+            }
+            return;
+        }
+        if (w & LVL_ANY) depth = D;
+        if (D - depth >= wmax) break;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+
+    // ------------------------------------------------------------------ backward
+    // (level 0 is the sources themselves: nothing is credited to them and nobody reads their c)
+    for (int D = depth; D >= 1; D--) {
+        for_tiles(work + A.lcap + D, [&](int t) {
+            const int64_t row = (int64_t)t * 32 + lane;
+            const Tile x = tile_of(t);
+            const int bd = (int)bdepth[x.it];
+            if (D > bd) return;
+            uint32_t* lrow = A.lev + (int64_t)D * A.rows + row;
+            const uint32_t need = *lrow;
+            if (!__any_sync(FULL, need != 0u)) return;
+            int64_t a0 = 0;
+            int deg = 0;
+            bool tgt = false;
+            if (need) {
+                if (D < bd) {
+                    const int64_t* rp = A.rp + x.base + x.u;
+                    a0 = __ldg(rp);
+                    deg = (int)(__ldg(rp + 1) - a0);
+                }
+                tgt = A.in_s ? __ldg(A.in_s + x.base + x.u) != 0 : true;
+            }
+            const unsigned tm = __ballot_sync(FULL, tgt);
+            sm.rowm[lane] = 0u;
+            sm.ds[lane] = 0.0;
+            __syncwarp();
+            const SG* srow = sg + (int64_t)t * 1024;
+            double* crow = cc + (int64_t)t * 1024;
+            tile_sums<false, WEIGHTED, double, double>(
+                A, sm, lane, need, a0, deg, D, bd, x.rb, A.col, A.w, cc,
+                [&](bool ok, int r, int s, double acc, unsigned first) {
+                    double delta = 0.0;
+                    if (ok) {
+                        const SG sv = srow[r * 32 + s];
+                        delta = (double)sv * acc;
+                        crow[r * 32 + s] = (tm >> r) & 1u ? acc + recip_of(sv) : acc;
+                    }
+                    // sum of each row's run of lanes, then one lane per row adds it
+                    const unsigned up = lane < 31 ? first >> (lane + 1) : 0u;
+                    const int end = up ? lane + __ffs(up) : 32;   // first lane of the next row
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const bool in = lane + o < end;
+                        if (!__any_sync(FULL, in)) break;
+                        const double y = __shfl_down_sync(FULL, delta, o);
+                        if (in) delta += y;
+                    }
+                    if (ok && (lane == 0 || (first >> lane) & 1u)) sm.ds[r] += delta;
+                    __syncwarp();
+                },
+                [&](int r, uint32_t mask, double acc) {
+                    double delta = 0.0;
+                    if ((mask >> lane) & 1u) {
+                        const SG sv = srow[r * 32 + lane];
+                        delta = (double)sv * acc;
+                        crow[r * 32 + lane] = (tm >> r) & 1u ? acc + recip_of(sv) : acc;
+                    }
+                    delta = warp_sum(delta);
+                    if (lane == 0) sm.ds[r] += delta;
+                    __syncwarp();
+                });
+            __syncwarp();
+            const uint32_t inner = sm.rowm[lane];
+            const uint32_t leaf = tgt ? need & ~inner : 0u;   // no successor: c = 1 / sigma
+            for_pairs(leaf, lane, sm.idx, [&](bool ok, int r, int s, unsigned) {
+                if (ok) crow[r * 32 + s] = recip_of(srow[r * 32 + s]);
+            });
+            if ((inner | leaf) != need) *lrow = inner | leaf;
+            const double ds = sm.ds[lane];
+            if (ds != 0.0) A.dsum[row] += ds;
+            __syncwarp();
+        });
+        if (D > 1 && !grid_barrier(A.ctl, A.flags)) return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) {
+        unsigned long long t2;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t2));
+        atomicAdd(&A.phase_ns[0], (t1 - t0) * (unsigned long long)A.nitems);
+        atomicAdd(&A.phase_ns[1], (t2 - t1) * (unsigned long long)A.nitems);
+    }
+}
+
+__global__ void lm_accumulate_kernel(const LmArgs A, const LmRun* __restrict__ runs, int nruns, int natiles, double* bcs,
+                                     double* bcc) {
+    const int lane = threadIdx.x & 31;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < natiles; q += nw) {
+        int lo = 0, hi = nruns - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (runs[mid].atile0 <= q) lo = mid;
+            else hi = mid - 1;
+        }
+        const LmRun r = runs[lo];
+        const int64_t base = A.node_off[r.g];
+        const int32_t n = (int32_t)(A.node_off[r.g + 1] - base);
+        const int tpb = (n + 31) >> 5;
+        const int tile0 = A.item_tile0 ? A.item_tile0[r.first] - A.tile_base : r.first * A.tpb;
+        const int u = (q - r.atile0) * 32 + lane;
+        if (u >= n) continue;
+        const double* x = A.dsum + ((int64_t)tile0 * 32 + u);
+        const int64_t step = (int64_t)(A.item_tile0 ? tpb : A.tpb) * 32;
+        double s = bcs[base + u], c = bcc[base + u];
+        int b = 0;
+        for (; b + 8 <= r.count; b += 8) {
+            double y[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) y[i] = x[(b + i) * step];
+#pragma unroll
+            for (int i = 0; i < 8; i++) neumaier_add(s, c, y[i]);
+        }
+        for (; b < r.count; b++) neumaier_add(s, c, x[b * step]);
+        bcs[base + u] = s;
+        bcc[base + u] = c;
+    }
+}
+
+__global__ void lm_tile_items_kernel(const int32_t* __restrict__ item_tile0, int nitems, int32_t ntiles,
+                                     int32_t* tile_item) {
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x) {
+        int lo = 0, hi = nitems - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (item_tile0[mid] <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        tile_item[t] = lo;
+    }
+}
+
+template <typename SG, bool WEIGHTED>
+cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
+    int per_sm = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, WEIGHTED>, LM_THREADS, 0);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorLaunchOutOfResources;
+    const int blocks = std::min(per_sm * num_sms, std::max(1, (A.ntiles + LM_WARPS - 1) / LM_WARPS));
+    LmArgs a = A;
+    void* args[] = {&a};
+    return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, WEIGHTED>, dim3(blocks), dim3(LM_THREADS), args, 0,
+                                       st);
+}
+
+}  // namespace
+
+int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + nitems + 2 * (int64_t)lcap; }
+
+cudaError_t lm_launch(const LmArgs& A, bool narrow, int num_sms, cudaStream_t st) {
+    if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;
+    const bool weighted = A.w != nullptr;
+    if (narrow) return weighted ? lm_go<uint32_t, true>(A, num_sms, st) : lm_go<uint32_t, false>(A, num_sms, st);
+    return weighted ? lm_go<uint64_t, true>(A, num_sms, st) : lm_go<uint64_t, false>(A, num_sms, st);
+}
+
+void lm_accumulate(const LmArgs& A, const LmRun* runs, int nruns, int natiles, double* bcs, double* bcc,
+                   cudaStream_t st) {
+    if (nruns <= 0 || natiles <= 0) return;
+    const int blocks = std::min((natiles + 3) / 4, 152 * 16);
+    lm_accumulate_kernel<<<blocks, 128, 0, st>>>(A, runs, nruns, natiles, bcs, bcc);
+}
+
+void lm_tile_items(const int32_t* item_tile0, int nitems, int32_t ntiles, int32_t* tile_item, cudaStream_t st) {
+    if (nitems <= 0 || ntiles <= 0) return;
+    lm_tile_items_kernel<<<std::min((ntiles + 255) / 256, 152 * 16), 256, 0, st>>>(item_tile0, nitems, ntiles,
+                                                                                  tile_item);
+}
+
+}  // namespace bcpp

@@ -1,0 +1,89 @@
+"""GPU parity of the level-mask kernel (plain Brandes and batched graphs in FP64) at the sizes where
+its tiling can go wrong, against the CPU oracle: node counts around a tile of 32 rows, source counts
+around a batch of 32, degrees around the 256-arc round of a tile, unreachable nodes, depths and path
+counts past what it serves (the call then reruns on the lockstep kernel), weights around its limit.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1406_4173_gb300 import gen
+
+pytestmark = pytest.mark.gpu
+
+FP64_TOL = 1e-12       # the FP64 bar of the other parity tests
+
+
+@pytest.fixture(scope="module")
+def bc():
+    import torch
+    import paper_1406_4173_gb300 as m
+    from paper_1406_4173_gb300 import _build
+    _build.build()
+    torch.cuda.set_device(0)
+    return m
+
+
+def rel_err(x, ref):
+    x = np.asarray(x, np.float64)
+    ref = np.asarray(ref, np.float64)
+    return float(np.max(np.abs(x - ref) / np.maximum(np.abs(ref), 1.0))) if x.size else 0.0
+
+
+def union(*graphs):
+    """Disjoint union of edge lists (unreachable pairs)."""
+    off, src, dst = 0, [], []
+    for g in graphs:
+        src.append(g.src + off)
+        dst.append(g.dst + off)
+        off += g.n
+    return gen.EdgeList(n=off, src=np.concatenate(src).astype(np.int32), dst=np.concatenate(dst).astype(np.int32))
+
+
+def wheel_of(deg, extra, seed):
+    """One hub of the given degree over a sparse random graph of its neighbours."""
+    g = gen.erdos_renyi(deg, min(1.0, extra / deg), seed=seed)
+    src = np.concatenate([np.zeros(deg, np.int32), g.src + 1]).astype(np.int32)
+    dst = np.concatenate([np.arange(1, deg + 1, dtype=np.int32), g.dst + 1]).astype(np.int32)
+    return gen.EdgeList(n=deg + 1, src=src, dst=dst)
+
+
+CASES = {
+    **{f"n{n}": (gen.erdos_renyi(n, min(1.0, 3.5 / n), seed=n), None) for n in (2, 3, 31, 32, 33, 63, 64, 65, 97)},
+    **{f"S{k}": (gen.planted_partition(300, 5, 0.06, 0.004, seed=4), k) for k in (2, 31, 32, 33, 64, 65)},
+    **{f"deg{d}": (wheel_of(d, 2.0, seed=d), None) for d in (255, 256, 257, 300, 513)},
+    "star": (gen.star(700), None),
+    "complete": (gen.complete(90), None),
+    "islands": (union(gen.path(40), gen.complete(9), gen.star(33), gen.cycle(50)), None),
+    "path-deep": (gen.path(400), None),
+    "grid-counts": (gen.grid(34, 34), 70),
+    "w-limit": (gen.planted_partition(400, 4, 0.03, 0.004, seed=5, wmax=32), None),
+    "w-past-limit": (gen.planted_partition(400, 4, 0.03, 0.004, seed=6, wmax=33), None),
+    "w-deep": (gen.with_weights(gen.grid(20, 20), 32, seed=7), None),
+    "directed-w": (gen.chung_lu_communities(500, [125] * 4, 2.3, 5.0, 0.85, seed=8, directed=True, wmax=9), None),
+    "directed": (gen.chung_lu_communities(500, [125] * 4, 2.3, 5.0, 0.85, seed=9, directed=True), 77),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_levels_match_oracle(bc, name):
+    g, k = CASES[name]
+    S = None if k is None else gen.sample_targets(g.n, k, seed=3)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    assert rel_err(bc.brandes(G, S).cpu().numpy(), ref) <= FP64_TOL
+    # the same batches in another order of the sources, and as two shards
+    assert rel_err(bc.brandes(G, S, order_sources=False).cpu().numpy(), ref) <= FP64_TOL
+    parts = [bc.brandes(G, S, shard=(r, 2)).cpu().numpy() for r in range(2)]
+    assert rel_err(parts[0] + parts[1], ref) <= FP64_TOL
+
+
+def test_levels_batched(bc):
+    gs = [gen.erdos_renyi(n, min(1.0, 4.0 / n), seed=n) for n in (1, 2, 31, 32, 33, 64, 65, 130, 257)]
+    gs += [gen.path(300), gen.star(290)]
+    arena = bc.build_arena(gs)
+    got = bc.brandes_batched(arena).cpu().numpy()
+    for i, g in enumerate(gs):
+        ref, _ = oracle.brandes(g, None)
+        x = got[arena.node_ptr_host[i]:arena.node_ptr_host[i + 1]]
+        assert rel_err(x, ref) <= FP64_TOL, i
