@@ -970,7 +970,10 @@ int lm_emit(bcpp_ctx* c, LmWs& L, const LsArena& A, const LsParams& P, const LsI
         LmArgs a{};
         a.rp = A.rp; a.col = A.col; a.w = A.w;
         a.irp = A.irp; a.icol = A.icol; a.iw = A.iw;
+        a.imu = A.imu;
+        a.mud = static_cast<const double*>(A.mud);
         a.node_off = A.node_off;
+        a.bc_map = P.bc_map;
         a.items = items + w.i0;
         a.item_tile0 = L.tpb ? nullptr : L.tile0.p + w.i0;
         a.tile_item = L.tile_item.p;
@@ -1468,6 +1471,8 @@ struct PpRun {
     SlotWs ws;
     bool unit = true, mult = false;
     bool rows_by_item = false;   // Brandes_SK in one dynamic pass with a row set per batch
+    bool levels = false;         // Brandes_SK on the level-mask kernel
+    LmWs lm;
     int nb = 2, spl = 1, nitems = 0, cl = 1, slots = 1;
     std::vector<CentralityUnit> hunits;
     DBuf<uint8_t> sk_in_s;
@@ -1480,6 +1485,86 @@ struct PpRun {
     DBuf<LsItem> items;
     LsArena A{};
 };
+
+// Workspace of Brandes_SK on the level-mask kernel followed by Centrality: every batch of a chunk has its
+// rows (distances, counts, dependencies, which Centrality reads) and its partial sums; as many
+// batches per chunk as memory allows (all of them, unless opts.pp_chunks asks for chunks of the
+// lockstep kernel's size).  r.levels stays false when not even one batch fits.
+int pp_levels_alloc(bcpp_ctx* c, PpRun& r, int nitems, int lcap) {
+    if (lcap > LM_MAX_LEVELS) return BCPP_OK;
+    const int64_t n = r.g.n, cap_n = ((int64_t)r.K.N + 31) / 32 * 32;
+    const int64_t each = cap_n * (32 * (4 + 8 + 8) + 8 + 4 + 4ll * lcap) + n * 16;
+    int64_t chunk = std::min<int64_t>(nitems, free_bytes(c) / each);
+    chunk = std::min<int64_t>(chunk, ((1ll << 31) - 1) / cap_n);
+    if (r.o.pp_chunks) chunk = std::min<int64_t>(chunk, slot_capacity(c, r.o, choose_cluster(c, nitems, r.o)));
+    if (chunk < 1) return BCPP_OK;
+    chunk = div_up(nitems, div_up(nitems, chunk));   // equal chunks
+    const int64_t rows = chunk * cap_n;
+    CK_ALLOC(r.ws.d.alloc(c, rows * 32));
+    CK_ALLOC(r.ws.sg.alloc(c, rows * 32));
+    CK_ALLOC(r.ws.dl.alloc(c, rows * 32 * 8));
+    CK_ALLOC(r.ws.bcs.alloc(c, chunk * n));
+    CK_ALLOC(r.ws.bcc.alloc(c, chunk * n));
+    CK_ALLOC(r.lm.lev.alloc(c, rows * lcap));
+    CK_ALLOC(r.lm.seen.alloc(c, rows));
+    CK_ALLOC(r.lm.dsum.alloc(c, rows));
+    CK_ALLOC(r.lm.ctl.alloc(c, lm_ctl_words(lcap, (int)chunk)));
+    r.lm.lcap = lcap;
+    r.lm.narrow = false;
+    r.lm.tpb = (int32_t)(cap_n / 32);
+    r.ws.sum_slots = (int)chunk;
+    r.slots = (int)chunk;
+    LsSlots& W = r.ws.W;
+    W.d = r.ws.d.p; W.sg = r.ws.sg.p; W.dl = r.ws.dl.p; W.cap_n = cap_n;
+    W.bc_sum = r.ws.bcs.p; W.bc_cmp = r.ws.bcc.p; W.cap_bc = n;
+    r.levels = true;
+    return BCPP_OK;
+}
+
+// Device work of the same: per chunk Brandes_SK, its partial sums, Centrality.
+int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
+    const LsSlots& W = r.ws.W;
+    Skeleton& K = r.K;
+    const SkTables T = K.tables();
+    CK_CUDA(cudaMemsetAsync(W.bc_sum, 0, (size_t)r.slots * W.cap_bc * sizeof(double), c->stream));
+    CK_CUDA(cudaMemsetAsync(W.bc_cmp, 0, (size_t)r.slots * W.cap_bc * sizeof(double), c->stream));
+    for (int c0 = 0; c0 < r.nitems; c0 += r.slots) {
+        const int cn = std::min(r.slots, r.nitems - c0);
+        LmArgs a{};
+        a.rp = r.A.rp; a.col = r.A.col; a.w = r.A.w;
+        a.mud = static_cast<const double*>(r.A.mud);
+        a.irp = r.A.irp; a.icol = r.A.icol; a.iw = r.A.iw; a.imu = r.A.imu;
+        a.node_off = r.A.node_off;
+        a.items = r.items.p + c0;
+        a.tpb = r.lm.tpb;
+        a.nitems = cn;
+        a.ntiles = cn * r.lm.tpb;
+        a.srcs = r.tsk.p;
+        a.in_s = r.sk_in_s.p;
+        a.bc_map = K.sknode.p;
+        a.lev = r.lm.lev.p; a.seen = r.lm.seen.p; a.sg = W.sg; a.cc = static_cast<double*>(W.dl);
+        a.dsum = r.lm.dsum.p; a.drow = W.d;
+        a.rows = (int64_t)a.ntiles * 32;
+        a.lcap = r.lm.lcap;
+        a.wmax = (int32_t)K.wmax_sk;
+        a.ctl = r.lm.ctl.p;
+        a.flags = c->flags;
+        a.phase_ns = c->phase;
+        if (tbr) tbr->start();
+        CK_CUDA(cudaMemsetAsync(a.ctl, 0, (size_t)lm_ctl_words(a.lcap, cn) * sizeof(uint32_t), c->stream));
+        CK_CUDA(lm_launch(a, false, c->num_sms, c->stream));
+        lm_scatter(a, K.N, W.bc_sum, W.bc_cmp, W.cap_bc, c->stream);
+        c->launches += 2;
+        if (tbr) tbr->stop();
+        if (tce) tce->start();
+        centrality_launch(false, K.tdmax <= CT_H16_MAX, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, K.skbase.p,
+                          W.d, W.sg, W.dl, W.cap_n, W.bc_sum, W.bc_cmp, W.cap_bc, c->flags, c->stream);
+        c->launches++;
+        if (tce) tce->stop();
+        CK_CUDA(cudaGetLastError());
+    }
+    return BCPP_OK;
+}
 
 int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin, const int32_t* Ssing,
                int32_t nsing, const int32_t* Ssrc, int32_t nsrc, const uint8_t* dflag, const int32_t* part, int32_t k,
@@ -1522,18 +1607,27 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
     // without non-frontier nodes Brandes_SK runs alone and may use 64-source batches
     r.spl = r.hunits.empty() ? choose_spl(c, s1 - s0, o) : 1;
     std::vector<LsItem> hitems = make_items(0, s0, s1, 32 * r.spl);
+    if (N > 0 && !hitems.empty() && lm_serves(c, o, r.spl, N, K.arcs, K.wmax_sk)) {
+        // skeleton distances are the distances in G
+        const int lcap = lm_levels(g->w != nullptr, g->directed != 0, o.order_sources && ns > 2 * LS_LANES ? &r.ord : nullptr);
+        if (r.hunits.empty())
+            CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return N; }, n, lcap, r.unit, &r.levels));
+        else
+            CK_RC(pp_levels_alloc(c, r, (int)hitems.size(), lcap));
+    }
     r.cl = (!hitems.empty() && r.spl == 1) ? choose_cluster(c, (int)hitems.size(), o) : 1;
-    if (r.spl == 1 && r.hunits.empty()) {
+    if (r.spl == 1 && r.hunits.empty() && !r.levels) {
         // without a Centrality step (whose cost grows with the batch count, not their width)
         const int b = balanced_width(s1 - s0, slot_capacity(c, o, r.cl), 32);
         if (b < 32) hitems = make_items(0, s0, s1, b);
     }
     r.nitems = (int)hitems.size();
     const int ef = entry_factor(c, !r.unit, r.spl);
+    if (!r.levels)
     r.slots = r.nitems > 0 ? choose_slots(c, r.nitems, o.ctas_per_sm,
                                           slot_bytes(std::max(N, 1), r.nb, fp32, ef, r.spl), (int64_t)n * 24, r.cl)
                            : 1;
-    if (!r.hunits.empty() && r.nitems > r.slots) {
+    if (!r.levels && !r.hunits.empty() && r.nitems > r.slots) {
         // More batches than slots.  When memory allows, every batch gets its own set of distance,
         // count and dependency rows (what the Centrality step reads) and its own partial sums, so
         // Brandes_SK schedules all batches dynamically over the slots in one launch and one
@@ -1557,8 +1651,9 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
         }
     }
     // partial sums live in the lockstep slots (or per batch); combine at the end
-    CK_RC(alloc_slots(c, r.ws, r.slots, std::max(N, 1), r.nb, fp32, n, r.spl, ef, false,
-                      r.rows_by_item ? r.nitems : 0, r.rows_by_item ? r.nitems : 0));
+    if (!r.levels)
+        CK_RC(alloc_slots(c, r.ws, r.slots, std::max(N, 1), r.nb, fp32, n, r.spl, ef, false,
+                          r.rows_by_item ? r.nitems : 0, r.rows_by_item ? r.nitems : 0));
     r.ws.narrow = r.hunits.empty() && use_narrow(c, !r.unit);   // Centrality reads int32 rows
     if (r.nitems > 0) {
         CK_ALLOC(r.sk_in_s.alloc(c, N));
@@ -1605,7 +1700,7 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
     const bool fp32 = r.o.precision == BCPP_FP32_DELTA;
     Skeleton& K = r.K;
     const int32_t N = K.N;
-    CK_RC(init_slots(c, r.ws));
+    if (!r.levels) CK_RC(init_slots(c, r.ws));
     if (r.nitems > 0) {
         sk_gather_flags(N, K.sknode.p, r.dflag, r.sk_in_s.p, c->stream);
         c->launches++;
@@ -1619,7 +1714,19 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             c->launches += 2;
         }
         const SkTables T = K.tables();
-        if (r.hunits.empty()) {
+        if (r.levels && r.hunits.empty()) {
+            // no non-frontier nodes: Brandes_SK alone
+            LsParams P{};
+            P.srcs = r.tsk.p;
+            P.in_s = r.sk_in_s.p;
+            P.bc_map = K.sknode.p;
+            P.flags = c->flags;
+            P.phase_ns = c->phase;
+            return lm_emit(c, r.lm, r.A, P, r.items.p, K.wmax_sk, r.scale, r.bc_out, tbr);
+        }
+        if (r.levels) {
+            CK_RC(pp_levels_emit(c, r, tbr, tce));
+        } else if (r.hunits.empty()) {
             // no non-frontier nodes: Brandes_SK alone, batches scheduled dynamically
             LsParams P{};
             P.mode = LS_BRANDES;
@@ -1637,7 +1744,7 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tbr) tbr->stop();
             CK_CUDA(cudaGetLastError());
         }
-        if (!r.hunits.empty() && r.rows_by_item) {
+        if (!r.levels && !r.hunits.empty() && r.rows_by_item) {
             // all batches in one dynamic Brandes_SK launch, each into its own rows, then one
             // Centrality launch over all batches (row set and partial sums of batch i: index i)
             LsParams P{};
@@ -1664,7 +1771,7 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tce) tce->stop();
             CK_CUDA(cudaGetLastError());
         }
-        for (int c0 = 0; c0 < r.nitems && !r.hunits.empty() && !r.rows_by_item; c0 += r.slots) {
+        for (int c0 = 0; c0 < r.nitems && !r.levels && !r.hunits.empty() && !r.rows_by_item; c0 += r.slots) {
             const int cn = std::min(r.slots, r.nitems - c0);
             LsParams P{};
             P.mode = LS_SKEL;

@@ -1,4 +1,4 @@
-// Level-mask passes of plain Brandes (Eq. 2 / Eq. 5-7) for many batches of 32 sources at once.
+// Level-mask passes of plain Brandes (Eq. 2 / Eq. 5-7) and Brandes_SK (Eq. 11 / Eq. 12) for many batches of 32 sources at once.
 //
 // Layout.  A row is one (batch, node) pair; its 32 positions are the batch's sources.  Instead of a
 // distance per source, a row has one 32-bit mask per distance level: bit s of lev[D][row] says that
@@ -25,6 +25,9 @@
 // Measured against the lockstep kernel (whole call, FP64): Chung-Lu n = 50,000, every node a target
 // 251 -> 125 ms; n = 1,000,000, 4,096 targets 709 -> 156 ms; directed, n = 100,000, weights 1 to 16,
 // 2,000 targets 141 -> 39 ms; 4,096 random graphs 427 -> 185 ms; n = 2,000, every node 1.76 -> 1.30 ms.
+// Brandes_SK (Eq. 11 / Eq. 12: weights, multiplicities, 64-bit counts, and the distance rows that the
+// Centrality step reads) 51 -> 4.5 ms at n = 100,000 and 512 targets, 695 -> 144 ms at n = 1,000,000 and
+// 2,048 targets.
 // Bound by the latency of its gathers (a profile at n = 10,000: instructions issued on 27% of the
 // cycles, FP64 pipe busy 30%) and, in the backward pass, by FP64 adds.
 #include <algorithm>
@@ -40,6 +43,9 @@ constexpr int LM_WARPS = LM_THREADS / 32;
 // workloads above, 5: 122 / 148 / 37 / 181, 6 (spills): 124 / 148 / 47 / 183
 #ifndef BCPP_LM_MINB
 #define BCPP_LM_MINB 5
+#endif
+#ifndef BCPP_LM_MINB64
+#define BCPP_LM_MINB64 4        // with 64-bit path counts
 #endif
 #ifndef BCPP_LM_PU
 #define BCPP_LM_PU 4           // values a pair's sum has in flight
@@ -70,14 +76,15 @@ __device__ __forceinline__ double recip_of(uint64_t s) {
     return fma(r, fma(-x, r, 1.0), r);
 }
 
+template <bool MULT>
 struct WarpSm {
     uint2 list[LM_CAP];        // arcs with a bit in common: head row, mask
+    uint64_t mult[MULT ? LM_CAP : 1];   // their multiplicities (uint64 forward, double backward)
     uint32_t nm[32];           // masks found, by candidate
     uint32_t rowm[32];         // masks found, by row of the tile
     double ds[32];             // dependencies, by row of the tile
     int seg[33];               // first list entry of each candidate
     int idx[32];               // compaction scratch
-    int pad;
 };
 
 // Barrier over all blocks of the cooperative launch.  false: gave up (never with co-resident blocks).
@@ -156,10 +163,11 @@ __device__ __forceinline__ void for_pairs(uint32_t mask, int lane, int* idx, F&&
 // sm.rowm by row (zeroed by the caller).
 //   pair_done(ok, r, s, acc, first): the sum of source s of the tile's row r (packed pairs)
 //   row_done(r, mask, acc): the same for all 32 sources of one row, lane = source
-template <bool FWD, bool WEIGHTED, typename V, typename ACC, class PD, class RD>
-__device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane, uint32_t need, int64_t a0, int deg,
+//   ovf: a 64-bit count wrapped
+template <bool FWD, bool WEIGHTED, bool MULT, typename V, typename ACC, class PD, class RD>
+__device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int lane, uint32_t need, int64_t a0, int deg,
                                           int D, int bd, int64_t rb, const int32_t* __restrict__ col,
-                                          const int32_t* __restrict__ wt, const V* vals, PD&& pair_done,
+                                          const int32_t* __restrict__ wt, const V* vals, bool& ovf, PD&& pair_done,
                                           RD&& row_done) {
     const unsigned le = 0xffffffffu >> (31 - lane), lt = le >> 1;
     const bool cand = need != 0u && deg > 0;
@@ -182,6 +190,17 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane,
         const int d2 = FWD ? D - w : D + w;
         return (FWD ? d2 >= 0 : d2 <= bd) ? A.lev[(int64_t)d2 * A.rows + rb + v] : 0u;
     };
+    // multiplicity of arc a, as 64 bits
+    auto mult_of = [&](uint32_t a) -> uint64_t {
+        if constexpr (!MULT) return 0;
+        else return FWD ? __ldg(A.imu + a) : (uint64_t)__double_as_longlong(__ldg(A.mud + a));
+    };
+    // acc += mult * t
+    auto add = [&](ACC& acc, V t, uint64_t mu) {
+        if constexpr (sizeof(V) == 4) acc += t;   // fewer than 2^31 counts below 2^32
+        else if constexpr (!FWD) acc = MULT ? fma(__longlong_as_double((long long)mu), t, acc) : acc + t;
+        else acc = MULT ? madd_ck(acc, t, mu, ovf) : add_ck(acc, t, ovf);
+    };
     int k0 = 0;
     while (k0 < K) {
         const int base = __shfl_sync(FULL, pre - cdeg, k0);
@@ -197,14 +216,17 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane,
             for (int c0 = 0; c0 < dg; c0 += 32) {
                 int32_t v = 0;
                 uint32_t m = 0u;
+                uint64_t mu = 0;
                 if (c0 + lane < dg) {
                     v = __ldg(col + b0 + c0 + lane);
                     m = gather(v, WEIGHTED ? __ldg(wt + b0 + c0 + lane) : 1) & nd;
+                    if (MULT && m) mu = mult_of(b0 + c0 + lane);
                 }
                 found |= m;
                 unsigned tb = __ballot_sync(FULL, m != 0u);
                 while (tb) {
                     V t[BCPP_LM_BU];
+                    uint64_t muq[BCPP_LM_BU];
 #pragma unroll
                     for (int q = 0; q < BCPP_LM_BU; q++) {
                         const int j = tb ? __ffs(tb) - 1 : 0;
@@ -212,11 +234,12 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane,
                         tb &= tb - 1u;
                         const int32_t vq = __shfl_sync(FULL, v, j);
                         const uint32_t mq = __shfl_sync(FULL, m, j);
+                        muq[q] = MULT ? shfl_u64(mu, j) : 0;
                         t[q] = (V)0;
                         if (on && (mq >> lane) & 1u) t[q] = vals[(rb + vq) * 32 + lane];
                     }
 #pragma unroll
-                    for (int q = 0; q < BCPP_LM_BU; q++) acc += t[q];
+                    for (int q = 0; q < BCPP_LM_BU; q++) add(acc, t[q], muq[q]);
                 }
             }
             found = __reduce_or_sync(FULL, found);
@@ -252,6 +275,7 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane,
             const int p = pos + __popc(tb & lt);
             if (m) {
                 sm.list[p] = make_uint2((uint32_t)v, m);
+                if constexpr (MULT) sm.mult[p] = mult_of(off + i);
                 atomicOr(&sm.nm[k], m);
             }
             if ((first >> lane) & 1u) sm.seg[k] = p;
@@ -279,7 +303,7 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane,
                         }
                     }
 #pragma unroll
-                    for (int q = 0; q < BCPP_LM_PU; q++) acc += t[q];
+                    for (int q = 0; q < BCPP_LM_PU; q++) add(acc, t[q], MULT ? sm.mult[min(e + q, e1 - 1)] : 0);
                     e += BCPP_LM_PU;
                 }
                 pair_done(ok, r, s, acc, first);
@@ -290,11 +314,11 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm& sm, int lane,
     }
 }
 
-template <typename SG, bool WEIGHTED>
-__global__ void __launch_bounds__(LM_THREADS, BCPP_LM_MINB) lm_kernel(const LmArgs A) {
-    __shared__ WarpSm s_warp[LM_WARPS];
+template <typename SG, bool WEIGHTED, bool MULT>
+__global__ void __launch_bounds__(LM_THREADS, sizeof(SG) == 4 ? BCPP_LM_MINB : BCPP_LM_MINB64) lm_kernel(const LmArgs A) {
+    __shared__ WarpSm<MULT> s_warp[LM_WARPS];
     const int lane = threadIdx.x & 31;
-    WarpSm& sm = s_warp[threadIdx.x >> 5];
+    WarpSm<MULT>& sm = s_warp[threadIdx.x >> 5];
     const int wid = blockIdx.x * LM_WARPS + (threadIdx.x >> 5);
     const int nw = gridDim.x * LM_WARPS;
     SG* sg = static_cast<SG*>(A.sg);
@@ -357,10 +381,19 @@ __global__ void __launch_bounds__(LM_THREADS, BCPP_LM_MINB) lm_kernel(const LmAr
         const int32_t src = lane < x.I.nsrc ? __ldg(A.srcs + x.I.src_off + lane) : -1;
         const int local = src - (x.u - lane);
         sm.rowm[lane] = 0u;
+        if (sizeof(SG) == 8 && A.drow) {
+            int4* dr = reinterpret_cast<int4*>(A.drow + (int64_t)t * 1024);
+            double2* cr = reinterpret_cast<double2*>(cc + (int64_t)t * 1024);
+#pragma unroll 4
+            for (int i = lane; i < 256; i += 32) dr[i] = make_int4(DINF, DINF, DINF, DINF);
+#pragma unroll 4
+            for (int i = lane; i < 512; i += 32) cr[i] = make_double2(0.0, 0.0);
+        }
         __syncwarp();
         if (src >= 0 && local >= 0 && local < 32) {
             atomicOr(&sm.rowm[local], 1u << lane);
             sg[(x.rb + src) * 32 + lane] = (SG)1;
+            if (sizeof(SG) == 8 && A.drow) A.drow[(x.rb + src) * 32 + lane] = 0;
         }
         __syncwarp();
         const uint32_t m = sm.rowm[lane];
@@ -382,7 +415,7 @@ __global__ void __launch_bounds__(LM_THREADS, BCPP_LM_MINB) lm_kernel(const LmAr
             }
             return;
         }
-        bool any = false, ovf = false;
+        bool any = false, wide = false, ovf = false;
         for_tiles(work + D, [&](int t) {
             const Tile x = tile_of(t);
             // finished batches: nothing new within the largest weight.  (A cached load: the values of
@@ -406,16 +439,18 @@ __global__ void __launch_bounds__(LM_THREADS, BCPP_LM_MINB) lm_kernel(const LmAr
             sm.rowm[lane] = 0u;
             __syncwarp();
             SG* srow = sg + (int64_t)t * 1024;
-            tile_sums<true, WEIGHTED, SG, uint64_t>(
-                A, sm, lane, need, a0, deg, D, 0, x.rb, A.icol, A.iw, sg,
-                [&](bool ok, int r, int s, uint64_t acc, unsigned) {
-                    if (ok) srow[r * 32 + s] = (SG)acc;
-                    if constexpr (sizeof(SG) == 4) ovf |= ok && (acc >> 32) != 0;
-                },
-                [&](int r, uint32_t mask, uint64_t acc) {
-                    if ((mask >> lane) & 1u) srow[r * 32 + lane] = (SG)acc;
-                    if constexpr (sizeof(SG) == 4) ovf |= ((mask >> lane) & 1u) && (acc >> 32) != 0;
-                });
+            int32_t* drow = sizeof(SG) == 8 && A.drow ? A.drow + (int64_t)t * 1024 : nullptr;
+            auto settle = [&](bool ok, int r, int s, uint64_t acc) {
+                if (ok) {
+                    srow[r * 32 + s] = (SG)acc;
+                    if (drow) drow[r * 32 + s] = D;
+                    if constexpr (sizeof(SG) == 4) wide |= (acc >> 32) != 0;
+                }
+            };
+            tile_sums<true, WEIGHTED, MULT, SG, uint64_t>(
+                A, sm, lane, need, a0, deg, D, 0, x.rb, A.icol, A.iw, sg, ovf,
+                [&](bool ok, int r, int s, uint64_t acc, unsigned) { settle(ok, r, s, acc); },
+                [&](int r, uint32_t mask, uint64_t acc) { settle((mask >> lane) & 1u, r, lane, acc); });
             __syncwarp();
             const uint32_t got = sm.rowm[lane];
             A.lev[(int64_t)D * A.rows + row] = got;
@@ -426,7 +461,8 @@ __global__ void __launch_bounds__(LM_THREADS, BCPP_LM_MINB) lm_kernel(const LmAr
             }
             __syncwarp();
         });
-        if (__any_sync(FULL, ovf)) {
+        if (sizeof(SG) == 8 && __any_sync(FULL, ovf) && lane == 0) atomicOr(&A.flags[FLAG_SIGMA_OVF], 1u);
+        if (__any_sync(FULL, wide)) {
             if (lane == 0) atomicOr(lvl + D, LVL_ERR | LVL_ANY);
         } else if (any && lane == 0 && (__ldcg(lvl + D) & LVL_ANY) == 0u) {
             atomicOr(lvl + D, LVL_ANY);
@@ -475,8 +511,9 @@ __global__ void __launch_bounds__(LM_THREADS, BCPP_LM_MINB) lm_kernel(const LmAr
             __syncwarp();
             const SG* srow = sg + (int64_t)t * 1024;
             double* crow = cc + (int64_t)t * 1024;
-            tile_sums<false, WEIGHTED, double, double>(
-                A, sm, lane, need, a0, deg, D, bd, x.rb, A.col, A.w, cc,
+            bool no_ovf = false;
+            tile_sums<false, WEIGHTED, MULT, double, double>(
+                A, sm, lane, need, a0, deg, D, bd, x.rb, A.col, A.w, cc, no_ovf,
                 [&](bool ok, int r, int s, double acc, unsigned first) {
                     double delta = 0.0;
                     if (ok) {
@@ -549,7 +586,8 @@ __global__ void lm_accumulate_kernel(const LmArgs A, const LmRun* __restrict__ r
         if (u >= n) continue;
         const double* x = A.dsum + ((int64_t)tile0 * 32 + u);
         const int64_t step = (int64_t)(A.item_tile0 ? tpb : A.tpb) * 32;
-        double s = bcs[base + u], c = bcc[base + u];
+        const int64_t ix = A.bc_map ? (int64_t)A.bc_map[base + u] : base + u;
+        double s = bcs[ix], c = bcc[ix];
         int b = 0;
         for (; b + 8 <= r.count; b += 8) {
             double y[8];
@@ -559,8 +597,22 @@ __global__ void lm_accumulate_kernel(const LmArgs A, const LmRun* __restrict__ r
             for (int i = 0; i < 8; i++) neumaier_add(s, c, y[i]);
         }
         for (; b < r.count; b++) neumaier_add(s, c, x[b * step]);
-        bcs[base + u] = s;
-        bcc[base + u] = c;
+        bcs[ix] = s;
+        bcc[ix] = c;
+    }
+}
+
+__global__ void lm_scatter_kernel(const LmArgs A, int32_t n, double* bc_sum, double* bc_cmp, int64_t cap_bc) {
+    const int64_t stride = (int64_t)A.tpb * 32;
+    const int i = blockIdx.y;
+    for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
+        const double x = A.dsum[i * stride + u];
+        if (x == 0.0) continue;
+        const int64_t ix = (int64_t)i * cap_bc + A.bc_map[u];
+        double s = bc_sum[ix], c = bc_cmp[ix];
+        neumaier_add(s, c, x);
+        bc_sum[ix] = s;
+        bc_cmp[ix] = c;
     }
 }
 
@@ -577,16 +629,16 @@ __global__ void lm_tile_items_kernel(const int32_t* __restrict__ item_tile0, int
     }
 }
 
-template <typename SG, bool WEIGHTED>
+template <typename SG, bool WEIGHTED, bool MULT = false>
 cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, WEIGHTED>, LM_THREADS, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, WEIGHTED, MULT>, LM_THREADS, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
     const int blocks = std::min(per_sm * num_sms, std::max(1, (A.ntiles + LM_WARPS - 1) / LM_WARPS));
     LmArgs a = A;
     void* args[] = {&a};
-    return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, WEIGHTED>, dim3(blocks), dim3(LM_THREADS), args, 0,
+    return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, WEIGHTED, MULT>, dim3(blocks), dim3(LM_THREADS), args, 0,
                                        st);
 }
 
@@ -598,6 +650,7 @@ cudaError_t lm_launch(const LmArgs& A, bool narrow, int num_sms, cudaStream_t st
     if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;
     const bool weighted = A.w != nullptr;
     if (narrow) return weighted ? lm_go<uint32_t, true>(A, num_sms, st) : lm_go<uint32_t, false>(A, num_sms, st);
+    if (A.mud) return weighted ? lm_go<uint64_t, true, true>(A, num_sms, st) : cudaErrorInvalidValue;
     return weighted ? lm_go<uint64_t, true>(A, num_sms, st) : lm_go<uint64_t, false>(A, num_sms, st);
 }
 
@@ -606,6 +659,18 @@ void lm_accumulate(const LmArgs& A, const LmRun* runs, int nruns, int natiles, d
     if (nruns <= 0 || natiles <= 0) return;
     const int blocks = std::min((natiles + 3) / 4, 152 * 16);
     lm_accumulate_kernel<<<blocks, 128, 0, st>>>(A, runs, nruns, natiles, bcs, bcc);
+}
+
+void lm_scatter(const LmArgs& A, int32_t n, double* bc_sum, double* bc_cmp, int64_t cap_bc, cudaStream_t st) {
+    if (n <= 0) return;
+    // at most 65,535 batches per launch (grid.y)
+    for (int i0 = 0; i0 < A.nitems; i0 += 65535) {
+        LmArgs a = A;
+        a.dsum = A.dsum + (int64_t)i0 * A.tpb * 32;
+        const dim3 grid((unsigned)std::min((n + 255) / 256, 1024), (unsigned)std::min(A.nitems - i0, 65535));
+        lm_scatter_kernel<<<grid, 256, 0, st>>>(a, n, bc_sum + (int64_t)i0 * cap_bc, bc_cmp + (int64_t)i0 * cap_bc,
+                                                cap_bc);
+    }
 }
 
 void lm_tile_items(const int32_t* item_tile0, int nitems, int32_t ntiles, int32_t* tile_item, cudaStream_t st) {

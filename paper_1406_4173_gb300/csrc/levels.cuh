@@ -19,9 +19,11 @@ struct LmArgs {
     const int64_t* rp;          // out-arcs
     const int32_t* col;
     const int32_t* w;           // nullptr = unit weights
+    const double* mud;          // multiplicities as doubles; nullptr = 1
     const int64_t* irp;         // in-arcs
     const int32_t* icol;
     const int32_t* iw;
+    const uint64_t* imu;
     const int64_t* node_off;    // graph g: nodes [node_off[g], node_off[g + 1])
     const LsItem* items;        // the wave's batches
     const int32_t* item_tile0;  // first tile of each batch plus tile_base; nullptr: uniform, batch i at i * tpb
@@ -35,7 +37,10 @@ struct LmArgs {
     uint32_t* seen;             // [rows]: sources that reached it so far
     void* sg;                   // [rows][32] path counts (32- or 64-bit)
     double* cc;                 // [rows][32] (I + delta) / sigma
+    int32_t* drow;              // [rows][32] distances (DINF = unreached), or nullptr; with it cc is zero
+                                // wherever it is not written
     double* dsum;               // [rows] dependencies summed over the batch's sources
+    const int32_t* bc_map;      // global node -> index of the sums over sources (nullptr = same)
     int64_t rows;               // 32 ntiles
     int32_t lcap;               // levels provided for
     int32_t wmax;
@@ -58,6 +63,9 @@ struct LmRun {
 // bcs / bcc (Neumaier sum and compensation per global node) += dsum over the runs' batches
 void lm_accumulate(const LmArgs& A, const LmRun* runs, int nruns, int natiles, double* bcs, double* bcc,
                    cudaStream_t st);
+
+// Partial sums of batch i at i * cap_bc (single graph, uniform layout): bc_sum / bc_cmp [bc_map[u]] += dsum
+void lm_scatter(const LmArgs& A, int32_t n, double* bc_sum, double* bc_cmp, int64_t cap_bc, cudaStream_t st);
 
 // tile_item[t] = batch of tile t, for all batches
 void lm_tile_items(const int32_t* item_tile0, int nitems, int32_t ntiles, int32_t* tile_item, cudaStream_t st);

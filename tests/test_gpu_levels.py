@@ -87,3 +87,26 @@ def test_levels_batched(bc):
         ref, _ = oracle.brandes(g, None)
         x = got[arena.node_ptr_host[i]:arena.node_ptr_host[i + 1]]
         assert rel_err(x, ref) <= FP64_TOL, i
+
+
+# Brandes_SK on the level-mask kernel: 64-bit counts, multiplicities, distance rows for the Centrality
+# step; skeleton rows below and above the 256-arc round, batches of 1 to 65 sources, chunks of batches
+PP_CASES = {
+    "planted": (gen.planted_partition(600, 6, 0.05, 0.004, seed=21), 65),
+    "planted-w": (gen.planted_partition(500, 5, 0.05, 0.004, seed=22, wmax=9), 33),
+    "dense-cliques": (gen.planted_partition(800, 2, 0.02, 0.006, seed=23), 32),
+    "directed-w": (gen.chung_lu_communities(500, [125] * 4, 2.3, 6.0, 0.85, seed=24, directed=True, wmax=7), 64),
+    "w-past-limit": (gen.planted_partition(400, 4, 0.05, 0.004, seed=25, wmax=40), 40),
+    "all-targets": (gen.planted_partition(300, 5, 0.06, 0.004, seed=26), None),
+}
+
+
+@pytest.mark.parametrize("name", list(PP_CASES))
+def test_levels_skeleton_matches_oracle(bc, name):
+    g, k = PP_CASES[name]
+    S = None if k is None else gen.sample_targets(g.n, k, seed=3)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    for kw in ({}, {"pp_chunks": 1}, {"order_sources": False}):
+        got = bc.brandes_pp(G, S, g.part, **kw).cpu().numpy()
+        assert rel_err(got, ref) <= FP64_TOL, kw
