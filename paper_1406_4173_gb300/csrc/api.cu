@@ -2294,6 +2294,49 @@ int partition_lp_dev(bcpp_ctx* c, const bcpp_graph* g, int32_t max_rounds, int32
 }
 
 // --------------------------------------------------------------------------- inspection
+// Distances and counts on the level-mask kernel: forward passes with distance rows, turned around into
+// the caller's [source][node] arrays.  *done stays false when not even one batch fits into memory.
+int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem* items, int nitems,
+                const int32_t* src, uint64_t wmax, int32_t* dist_out, uint64_t* sigma_out, bool* done) {
+    const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr);
+    const int64_t tpb = ((int64_t)g->n + 31) / 32, cap_n = tpb * 32;
+    const int64_t each = cap_n * (32 * (4 + 8) + 8 + 4 + 4ll * lcap);
+    int64_t chunk = std::min<int64_t>(nitems, std::min(free_bytes(c), std::max(LM_WAVE_BYTES, each)) / each);
+    chunk = std::min<int64_t>(chunk, ((1ll << 31) - 1) / cap_n);
+    if (chunk < 1) return BCPP_OK;
+    const int64_t rows = chunk * cap_n;
+    DBuf<int32_t> d(c, rows * 32);
+    DBuf<uint64_t> sg(c, rows * 32);
+    DBuf<uint32_t> lev(c, rows * lcap), seen(c, rows), ctl(c, lm_ctl_words(lcap, (int)chunk));
+    DBuf<double> dsum(c, rows);
+    CK_ALLOC(d); CK_ALLOC(sg); CK_ALLOC(lev); CK_ALLOC(seen); CK_ALLOC(ctl); CK_ALLOC(dsum);
+    for (int c0 = 0; c0 < nitems; c0 += (int)chunk) {
+        const int cn = (int)std::min<int64_t>(chunk, nitems - c0);
+        LmArgs a{};
+        a.rp = A.rp; a.col = A.col; a.w = A.w;
+        a.irp = A.irp; a.icol = A.icol; a.iw = A.iw;
+        a.node_off = A.node_off;
+        a.items = items + c0;
+        a.tpb = (int32_t)tpb;
+        a.nitems = cn;
+        a.ntiles = (int32_t)(cn * tpb);
+        a.srcs = src;
+        a.lev = lev.p; a.seen = seen.p; a.sg = sg.p; a.dsum = dsum.p; a.drow = d.p;
+        a.rows = (int64_t)a.ntiles * 32;
+        a.lcap = lcap;
+        a.wmax = (int32_t)wmax;
+        a.ctl = ctl.p;
+        a.flags = c->flags;
+        CK_CUDA(cudaMemsetAsync(ctl.p, 0, (size_t)lm_ctl_words(lcap, cn) * sizeof(uint32_t), c->stream));
+        CK_CUDA(lm_launch(a, false, c->num_sms, c->stream));
+        lm_paths_out(a, g->n, dist_out, sigma_out, c->stream);
+        c->launches += 2;
+    }
+    CK_CUDA(cudaGetLastError());
+    *done = true;
+    return BCPP_OK;
+}
+
 int sssp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* src, int32_t nsrc, int32_t* dist_out,
              uint64_t* sigma_out, const bcpp_opts& o) {
     CK_RC(check_graph_struct(g));
@@ -2321,13 +2364,6 @@ int sssp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* src, int32_t nsrc,
     CK_RC(to_dev(c, items.p, hitems.data(), nitems));
     const int64_t hoff[2] = {0, n};
     CK_RC(to_dev(c, node_off.p, hoff, 2));
-    // a batch holds each source at most once: split repeated sources across batches is not
-    // needed because LS_SSSP lanes are independent rows (a repeat only repeats the row)
-    const int nb = g->w ? (int)wmax + 1 : 2;
-    const int ef = entry_factor(c, g->w != nullptr, 1);
-    const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(n, nb, false, ef), 0);
-    SlotWs ws;
-    CK_RC(alloc_slots(c, ws, slots, n, nb, false, 0, 1, ef));
     LsArena A{};
     A.rp = g->row_ptr; A.col = g->col; A.w = (const int32_t*)g->w;
     if (g->directed) {
@@ -2336,6 +2372,18 @@ int sssp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* src, int32_t nsrc,
         A.irp = g->row_ptr; A.icol = g->col; A.iw = (const int32_t*)g->w;
     }
     A.node_off = node_off.p;
+    if (lm_serves(c, o, 1, n, g->num_arcs, g->w ? wmax : 1)) {
+        bool done = false;
+        CK_RC(sssp_levels(c, g, A, items.p, nitems, src, wmax, dist_out, sigma_out, &done));
+        if (done) return finish_status(c, nullptr);
+    }
+    // a batch holds each source at most once: split repeated sources across batches is not
+    // needed because LS_SSSP lanes are independent rows (a repeat only repeats the row)
+    const int nb = g->w ? (int)wmax + 1 : 2;
+    const int ef = entry_factor(c, g->w != nullptr, 1);
+    const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(n, nb, false, ef), 0);
+    SlotWs ws;
+    CK_RC(alloc_slots(c, ws, slots, n, nb, false, 0, 1, ef));
     LsParams P{};
     P.mode = LS_SSSP;
     P.nb = nb;

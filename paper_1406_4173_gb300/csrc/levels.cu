@@ -386,8 +386,9 @@ __global__ void __launch_bounds__(LM_THREADS, sizeof(SG) == 4 ? BCPP_LM_MINB : B
             double2* cr = reinterpret_cast<double2*>(cc + (int64_t)t * 1024);
 #pragma unroll 4
             for (int i = lane; i < 256; i += 32) dr[i] = make_int4(DINF, DINF, DINF, DINF);
+            if (cc)
 #pragma unroll 4
-            for (int i = lane; i < 512; i += 32) cr[i] = make_double2(0.0, 0.0);
+                for (int i = lane; i < 512; i += 32) cr[i] = make_double2(0.0, 0.0);
         }
         __syncwarp();
         if (src >= 0 && local >= 0 && local < 32) {
@@ -483,6 +484,7 @@ __global__ void __launch_bounds__(LM_THREADS, sizeof(SG) == 4 ? BCPP_LM_MINB : B
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
 
+    if (!cc) return;
     // ------------------------------------------------------------------ backward
     // (level 0 is the sources themselves: nothing is credited to them and nobody reads their c)
     for (int D = depth; D >= 1; D--) {
@@ -616,6 +618,34 @@ __global__ void lm_scatter_kernel(const LmArgs A, int32_t n, double* bc_sum, dou
     }
 }
 
+// A block turns tiles of 32 rows x 32 sources around in shared memory (both sides coalesced).
+__global__ void lm_paths_out_kernel(const LmArgs A, int32_t n, int32_t* dist, uint64_t* sigma) {
+    __shared__ int32_t s_d[32][33];
+    __shared__ uint64_t s_s[32][33];
+    const int x = threadIdx.x & 31, y0 = threadIdx.x >> 5;
+    const uint64_t* sg = static_cast<const uint64_t*>(A.sg);
+    for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
+        const int it = t / A.tpb;
+        const LsItem I = A.items[it];
+        const int u0 = (t - it * A.tpb) * 32;
+        for (int y = y0; y < 32; y += LM_WARPS) {
+            const int64_t o = ((int64_t)t * 32 + y) * 32 + x;
+            const int32_t d = A.drow[o];
+            s_d[y][x] = d;
+            s_s[y][x] = d == DINF ? 0ull : sg[o];
+        }
+        __syncthreads();
+        for (int y = y0; y < I.nsrc; y += LM_WARPS) {
+            if (u0 + x < n) {
+                const int64_t o = (int64_t)(I.src_off + y) * n + u0 + x;
+                dist[o] = s_d[x][y];
+                sigma[o] = s_s[x][y];
+            }
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void lm_tile_items_kernel(const int32_t* __restrict__ item_tile0, int nitems, int32_t ntiles,
                                      int32_t* tile_item) {
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x) {
@@ -671,6 +701,11 @@ void lm_scatter(const LmArgs& A, int32_t n, double* bc_sum, double* bc_cmp, int6
         lm_scatter_kernel<<<grid, 256, 0, st>>>(a, n, bc_sum + (int64_t)i0 * cap_bc, bc_cmp + (int64_t)i0 * cap_bc,
                                                 cap_bc);
     }
+}
+
+void lm_paths_out(const LmArgs& A, int32_t n, int32_t* dist, uint64_t* sigma, cudaStream_t st) {
+    if (n > 0 && A.ntiles > 0)
+        lm_paths_out_kernel<<<std::min(A.ntiles, 152 * 16), LM_THREADS, 0, st>>>(A, n, dist, sigma);
 }
 
 void lm_tile_items(const int32_t* item_tile0, int nitems, int32_t ntiles, int32_t* tile_item, cudaStream_t st) {

@@ -36,7 +36,7 @@ struct LmArgs {
     uint32_t* lev;              // [lcap][rows]: sources that reach the row's node at that distance
     uint32_t* seen;             // [rows]: sources that reached it so far
     void* sg;                   // [rows][32] path counts (32- or 64-bit)
-    double* cc;                 // [rows][32] (I + delta) / sigma
+    double* cc;                 // [rows][32] (I + delta) / sigma; nullptr: forward pass only
     int32_t* drow;              // [rows][32] distances (DINF = unreached), or nullptr; with it cc is zero
                                 // wherever it is not written
     double* dsum;               // [rows] dependencies summed over the batch's sources
@@ -66,6 +66,10 @@ void lm_accumulate(const LmArgs& A, const LmRun* runs, int nruns, int natiles, d
 
 // Partial sums of batch i at i * cap_bc (single graph, uniform layout): bc_sum / bc_cmp [bc_map[u]] += dsum
 void lm_scatter(const LmArgs& A, int32_t n, double* bc_sum, double* bc_cmp, int64_t cap_bc, cudaStream_t st);
+
+// Distances and counts of a forward-only wave with distance rows (single graph, uniform layout):
+// dist / sigma [source position][n], DINF and 0 where unreached
+void lm_paths_out(const LmArgs& A, int32_t n, int32_t* dist, uint64_t* sigma, cudaStream_t st);
 
 // tile_item[t] = batch of tile t, for all batches
 void lm_tile_items(const int32_t* item_tile0, int nitems, int32_t ntiles, int32_t* tile_item, cudaStream_t st);

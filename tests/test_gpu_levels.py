@@ -110,3 +110,17 @@ def test_levels_skeleton_matches_oracle(bc, name):
     for kw in ({}, {"pp_chunks": 1}, {"order_sources": False}):
         got = bc.brandes_pp(G, S, g.part, **kw).cpu().numpy()
         assert rel_err(got, ref) <= FP64_TOL, kw
+
+
+@pytest.mark.parametrize("name", ["n33", "n65", "S33", "star", "islands", "path-deep", "grid-counts", "w-limit",
+                                  "w-past-limit", "w-deep", "directed-w", "directed"])
+def test_levels_paths_match_oracle(bc, name):
+    """Distances and counts, bit for bit; 33 sources, one of them twice."""
+    g, _ = CASES[name]
+    src = np.concatenate([np.arange(0, g.n, max(1, g.n // 32))[:32], [0]]).astype(np.int32)
+    d, s = bc.sssp(bc.graph_from_edgelist(g), src)
+    d, s = d.cpu().numpy(), s.cpu().numpy().view(np.uint64)
+    for i, v in enumerate(src):
+        rd, rs, _ = oracle.sssp(g, int(v))
+        assert np.array_equal(d[i], rd), i
+        assert np.array_equal(s[i], rs), i
