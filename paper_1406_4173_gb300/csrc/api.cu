@@ -227,18 +227,6 @@ __global__ void group_by_part_kernel(const int32_t* part, int32_t n, int32_t k, 
     }
 }
 
-// largest finite value of a distance table (DINF = unreachable) into *out
-__global__ void table_max_kernel(const int32_t* t, int64_t n, unsigned* out) {
-    unsigned m = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = t[i];
-        if (v != DINF && (unsigned)v > m) m = (unsigned)v;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(FULL, m, o));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
 __global__ void accumulate_kernel(const double* x, int32_t n, double* sum, double* comp) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         double s = sum[i], c = comp[i];
@@ -1201,7 +1189,6 @@ struct Skeleton {
     int64_t arcs = 0, edges = 0, table_entries = 0;
     int32_t lcs = 0, k_nonempty = 0;
     uint64_t wmax_sk = 1, mmax_sk = 1;
-    uint32_t tdmax = 0;   // largest finite distance in the entry and exit tables
     DBuf<int32_t> partp, pstart, nf, loc, skid, sknode, skbase;
     DBuf<uint8_t> fr;
     DBuf<uint32_t> pnodes;
@@ -1407,24 +1394,6 @@ int build_sk(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS_eff,
             if (c->hflags[FLAG_CAPACITY]) return BCPP_ECAPACITY;
         }
     }
-    // the largest finite table distance (the Centrality step takes a 16-bit path when it is small)
-    if (reuse) {
-        K.tdmax = reuse->tdmax;
-    } else if (K.table_entries > 0) {
-        DBuf<unsigned> tm(c, 1);
-        CK_ALLOC(tm);
-        CK_CUDA(cudaMemsetAsync(tm.p, 0, sizeof(unsigned), c->stream));
-        const unsigned blocks = (unsigned)std::min<int64_t>((K.table_entries + 255) / 256, 152 * 8);
-        table_max_kernel<<<blocks, 256, 0, c->stream>>>(K.td.p, K.table_entries, tm.p);
-        c->launches++;
-        if (K.tdr.p) {
-            table_max_kernel<<<blocks, 256, 0, c->stream>>>(K.tdr.p, K.table_entries, tm.p);
-            c->launches++;
-        }
-        unsigned h = 0;
-        CK_RC(to_host(c, &h, tm.p, 1));
-        K.tdmax = h;
-    }
     // skeleton arcs: R with <w,1>, X_i with <d_i, sigma_i>
     {
         const SkTables T = K.tables();
@@ -1475,6 +1444,14 @@ struct PpRun {
     LmWs lm;
     int nb = 2, spl = 1, nitems = 0, cl = 1, slots = 1;
     std::vector<CentralityUnit> hunits;
+    struct Lists {           // Centrality: frontiers of each non-frontier node (entries, exits)
+        DBuf<int64_t> rp;
+        DBuf<int2> ft;
+        DBuf<uint64_t> mu;
+        CentralityLists view() const { return CentralityLists{rp.p, ft.p, mu.p}; }
+    } entry, exit;
+    CentralityLists entries() const { return entry.view(); }
+    CentralityLists exits() const { return exit.rp.p ? exit.view() : entry.view(); }
     DBuf<uint8_t> sk_in_s;
     DBuf<int64_t> irp, icnt, itmp;
     DBuf<int32_t> icol, iw;
@@ -1485,6 +1462,26 @@ struct PpRun {
     DBuf<LsItem> items;
     LsArena A{};
 };
+
+// Centrality's frontier lists of the non-frontier nodes, from the entry or exit tables.
+int centrality_lists(bcpp_ctx* c, PpRun& r, int32_t interior, bool exits, PpRun::Lists& L) {
+    const SkTables T = r.K.tables();
+    const int nunits = (int)r.hunits.size();
+    DBuf<int64_t> cnt(c, (int64_t)interior + 1), tmp(c, scan_tmp_elems((int64_t)interior + 1));
+    CK_ALLOC(cnt); CK_ALLOC(tmp);
+    CK_ALLOC(L.rp.alloc(c, (int64_t)interior + 1));
+    CK_CUDA(cudaMemsetAsync(cnt.p + interior, 0, sizeof(int64_t), c->stream));
+    ct_count(r.units.p, nunits, T, exits, cnt.p, c->stream);
+    exclusive_scan<int64_t>(cnt.p, L.rp.p, (int64_t)interior + 1, nullptr, tmp.p, c->stream, c->launches);
+    int64_t total = 0;
+    CK_RC(to_host(c, &total, L.rp.p + interior, 1));
+    CK_ALLOC(L.ft.alloc(c, total));
+    CK_ALLOC(L.mu.alloc(c, total));
+    ct_fill(r.units.p, nunits, T, exits, r.K.skbase.p, L.rp.p, L.ft.p, L.mu.p, c->stream);
+    c->launches += 2;
+    CK_CUDA(cudaGetLastError());
+    return BCPP_OK;
+}
 
 // Workspace of Brandes_SK on the level-mask kernel followed by Centrality: every batch of a chunk has its
 // rows (distances, counts, dependencies, which Centrality reads) and its partial sums; as many
@@ -1557,8 +1554,8 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         c->launches += 2;
         if (tbr) tbr->stop();
         if (tce) tce->start();
-        centrality_launch(false, K.tdmax <= CT_H16_MAX, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, K.skbase.p,
-                          W.d, W.sg, W.dl, W.cap_n, W.bc_sum, W.bc_cmp, W.cap_bc, c->flags, c->stream);
+        centrality_launch(false, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, r.entries(), r.exits(), W.d, W.sg,
+                          W.dl, W.cap_n, W.bc_sum, W.bc_cmp, W.cap_bc, c->flags, c->stream);
         c->launches++;
         if (tce) tce->stop();
         CK_CUDA(cudaGetLastError());
@@ -1599,10 +1596,14 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
     int64_t s0, s1;
     shard_sources(o, r.nt, s0, s1);
     // Centrality work units: chunks of 64 non-frontier nodes of parts with frontiers
+    int32_t interior = 0;
     for (int32_t i = 0; i < K.kp; i++) {
         const int32_t sz = K.h_pstart[i + 1] - K.h_pstart[i];
         if (K.h_nf[i] < 1 || sz <= K.h_nf[i]) continue;
-        for (int32_t v0 = K.h_nf[i]; v0 < sz; v0 += 64) r.hunits.push_back({i, v0, std::min(sz, v0 + 64), 0});
+        for (int32_t v0 = K.h_nf[i]; v0 < sz; v0 += 64) {
+            r.hunits.push_back({i, v0, std::min(sz, v0 + 64), interior});
+            interior += std::min(sz, v0 + 64) - v0;
+        }
     }
     // without non-frontier nodes Brandes_SK runs alone and may use 64-source batches
     r.spl = r.hunits.empty() ? choose_spl(c, s1 - s0, o) : 1;
@@ -1686,6 +1687,10 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
         A.node_off = r.node_off.p;
         CK_ALLOC(r.units.alloc(c, (int64_t)r.hunits.size()));
         CK_RC(to_dev(c, r.units.p, r.hunits.data(), (int64_t)r.hunits.size()));
+        if (!r.hunits.empty()) {
+            CK_RC(centrality_lists(c, r, interior, false, r.entry));
+            if (g->directed) CK_RC(centrality_lists(c, r, interior, true, r.exit));
+        }
         CK_ALLOC(r.items.alloc(c, r.nitems));
         CK_RC(to_dev(c, r.items.p, hitems.data(), r.nitems));
     }
@@ -1763,9 +1768,8 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tbr) tbr->stop();
             CK_CUDA(cudaGetLastError());
             if (tce) tce->start();
-            centrality_launch(fp32, K.tdmax <= CT_H16_MAX, r.units.p, (int)r.hunits.size(), r.nitems, T, K.pnodes.p,
-                              K.skbase.p, r.ws.W.d,
-                              r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
+            centrality_launch(fp32, r.units.p, (int)r.hunits.size(), r.nitems, T, K.pnodes.p, r.entries(), r.exits(),
+                              r.ws.W.d, r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
                               c->flags, c->stream);
             c->launches++;
             if (tce) tce->stop();
@@ -1788,9 +1792,8 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tbr) tbr->stop();
             CK_CUDA(cudaGetLastError());
             if (tce) tce->start();
-            centrality_launch(fp32, K.tdmax <= CT_H16_MAX, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p,
-                              K.skbase.p, r.ws.W.d,
-                              r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
+            centrality_launch(fp32, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, r.entries(), r.exits(),
+                              r.ws.W.d, r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
                               c->flags, c->stream);
             c->launches++;
             if (tce) tce->stop();

@@ -51,14 +51,24 @@ void sk_gather_flags(int32_t N, const int32_t* sknode, const uint8_t* in_s, uint
 // out[j] = skeleton id of target S[j], or -1 when it is no skeleton node (isolated)
 void sk_target_ids(const int32_t* S, int32_t nS, const int32_t* skid, int32_t* out, cudaStream_t st);
 
-// Centrality (Eq. 13) for the slots of one Brandes_SK chunk.
+// Centrality (Eq. 13), see centrality.cu.  A unit is up to 64 non-frontier nodes of a part (locals
+// [v0, v1)); pad is the index of its first node among all of them.
 struct CentralityUnit { int32_t part; int32_t v0; int32_t v1; int32_t pad; };
-// h16: every finite table distance is at most CT_H16_MAX (the 16-bit distance path may run)
-constexpr uint32_t CT_H16_MAX = 1023;
-void centrality_launch(bool fp32_delta, bool h16, const CentralityUnit* units, int nunits, int nslots, SkTables T,
-                       const uint32_t* pnodes, const int32_t* skbase, const int32_t* d, const uint64_t* sg,
-                       const void* dl, int64_t cap_n, double* bc_sum, double* bc_cmp, int64_t cap_bc,
-                       uint32_t* flags, cudaStream_t st);
+// per non-frontier node the frontiers with a non-zero path count: skeleton row and distance, and the count
+struct CentralityLists {
+    const int64_t* rp;       // [nodes + 1]
+    const int2* ft;
+    const uint64_t* mu;
+};
+// list lengths, and the lists at rp, from the entry tables (exits: from the exit tables)
+void ct_count(const CentralityUnit* units, int nunits, SkTables T, bool exits, int64_t* cnt, cudaStream_t st);
+void ct_fill(const CentralityUnit* units, int nunits, SkTables T, bool exits, const int32_t* skbase, const int64_t* rp,
+             int2* ft, uint64_t* mu, cudaStream_t st);
+// all units for the slots of one Brandes_SK chunk; E, X: entry and exit lists (undirected: the same)
+void centrality_launch(bool fp32_delta, const CentralityUnit* units, int nunits, int nslots, SkTables T,
+                       const uint32_t* pnodes, CentralityLists E, CentralityLists X, const int32_t* d,
+                       const uint64_t* sg, const void* dl, int64_t cap_n, double* bc_sum, double* bc_cmp,
+                       int64_t cap_bc, uint32_t* flags, cudaStream_t st);
 
 // bc_out[v] = scale * sum over slots of (bc_sum + bc_cmp), Neumaier over slots
 void combine_launch(const double* bc_sum, const double* bc_cmp, int nslots, int64_t cap_bc, int64_t n, double scale,

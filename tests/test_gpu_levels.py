@@ -124,3 +124,29 @@ def test_levels_paths_match_oracle(bc, name):
         rd, rs, _ = oracle.sssp(g, int(v))
         assert np.array_equal(d[i], rd), i
         assert np.array_equal(s[i], rs), i
+
+
+def spoked(k, wmax=None):
+    """Part 0: a hub and its k neighbours, each tied to one node of a ring (part 1): the hub is a
+    non-frontier node with k frontiers that all reach it directly."""
+    i = np.arange(1, k + 1)
+    src = np.concatenate([np.zeros(k, np.int64), i, i + k])
+    dst = np.concatenate([i, i + k, np.roll(i + k, -1)])
+    lo, hi = np.minimum(src, dst), np.maximum(src, dst)
+    g = gen.EdgeList(n=2 * k + 1, src=lo.astype(np.int32), dst=hi.astype(np.int32),
+                     part=(np.arange(2 * k + 1) > k).astype(np.int32))
+    return g if wmax is None else gen.with_weights(g, wmax, seed=k)
+
+
+@pytest.mark.parametrize("k", [3, 31, 32, 33, 127, 128, 129, 300])
+@pytest.mark.parametrize("wmax", [None, 5])
+def test_centrality_list_lengths(bc, k, wmax):
+    """Centrality's frontier lists around its chunk of 32 and its stage of 128 entries."""
+    g = spoked(k, wmax)
+    S = np.arange(k + 1, 2 * k + 1, max(1, k // 40), dtype=np.int32)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    got = bc.brandes_pp(G, S, g.part).cpu().numpy()
+    assert rel_err(got, ref) <= FP64_TOL
+    f32 = bc.brandes_pp(G, S, g.part, precision="fp32").cpu().numpy()
+    assert rel_err(f32, ref) <= 2e-6   # the FP32 bar of the other parity tests on small graphs
