@@ -23,13 +23,13 @@
 // 2 lanes per SM and cycle, are done for packed pairs only.
 //
 // Measured against the lockstep kernel (whole call, FP64): Chung-Lu n = 50,000, every node a target
-// 251 -> 125 ms; n = 1,000,000, 4,096 targets 709 -> 156 ms; directed, n = 100,000, weights 1 to 16,
-// 2,000 targets 141 -> 39 ms; 4,096 random graphs 427 -> 185 ms; n = 2,000, every node 1.76 -> 1.30 ms.
+// 251 -> 120 ms; n = 1,000,000, 4,096 targets 709 -> 140 ms; directed, n = 100,000, weights 1 to 16,
+// 2,000 targets 141 -> 39 ms; 4,096 random graphs 427 -> 176 ms; n = 2,000, every node 1.76 -> 1.25 ms.
 // Brandes_SK (Eq. 11 / Eq. 12: weights, multiplicities, 64-bit counts, and the distance rows that the
-// Centrality step reads) 51 -> 4.5 ms at n = 100,000 and 512 targets, 695 -> 144 ms at n = 1,000,000 and
+// Centrality step reads) 51 -> 4.4 ms at n = 100,000 and 512 targets, 695 -> 135 ms at n = 1,000,000 and
 // 2,048 targets.
 // Bound by the latency of its gathers (a profile at n = 10,000: instructions issued on 27% of the
-// cycles, FP64 pipe busy 30%) and, in the backward pass, by FP64 adds.
+// cycles, FP64 pipe busy 33%) and, in the backward pass, by FP64 adds (pipe busy 63% of it).
 #include <algorithm>
 
 #include "levels.cuh"
@@ -39,20 +39,17 @@ namespace {
 
 constexpr int LM_THREADS = 256;
 constexpr int LM_WARPS = LM_THREADS / 32;
-// resident blocks per SM (48 registers): 40 warps.  4 blocks 127 / 164 / 38 / 189 ms on the four large
-// workloads above, 5: 122 / 148 / 37 / 181, 6 (spills): 124 / 148 / 47 / 183
-#ifndef BCPP_LM_MINB
-#define BCPP_LM_MINB 5
-#endif
-#ifndef BCPP_LM_MINB64
-#define BCPP_LM_MINB64 4        // with 64-bit path counts
-#endif
-#ifndef BCPP_LM_PU
-#define BCPP_LM_PU 4           // values a pair's sum has in flight
-#endif
-#ifndef BCPP_LM_BU
-#define BCPP_LM_BU 4           // the same for a row of many arcs (8: no faster)
-#endif
+// Resident blocks per SM: 5 (48 registers, 40 warps) with 32-bit counts, 4 with 64-bit counts.  The two large
+// Chung-Lu and the batched workload below on 4 blocks: 126 / 151 / 184 ms, on 5: 119 / 136 / 174, on 6
+// (spills): 128 / 152 / 183.
+constexpr int lm_min_blocks(bool narrow) { return narrow ? 5 : 4; }
+// Values in flight per pair (unit weights: 2 131 / 166 / 195 ms, 3 119 / 137 / 173, 4 121 / 140 / 174 on the
+// three workloads above) and chunks of 32 arcs whose gathers overlap (1 127 / 154 / 181, 2 125 / 144 / 178;
+// with weights, Brandes_SK at n = 1,000,000: 1 148 ms, 2 139, 3 135).
+template <bool WEIGHTED>
+constexpr int LM_PAIRS = WEIGHTED ? 4 : 3;
+template <bool WEIGHTED>
+constexpr int LM_GATHERS = WEIGHTED ? 3 : 2;
 constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of larger degree go one by one)
 constexpr int CTL_BAR = 0, CTL_GEN = 1, CTL_ABORT = 2, CTL_LVL = 8;
 constexpr unsigned LVL_ANY = 1u, LVL_ERR = 2u;
@@ -80,10 +77,10 @@ template <bool MULT>
 struct WarpSm {
     uint2 list[LM_CAP];        // arcs with a bit in common: head row, mask
     uint64_t mult[MULT ? LM_CAP : 1];   // their multiplicities (uint64 forward, double backward)
+    int seg[33];               // first list entry of each candidate
     uint32_t nm[32];           // masks found, by candidate
     uint32_t rowm[32];         // masks found, by row of the tile
     double ds[32];             // dependencies, by row of the tile
-    int seg[33];               // first list entry of each candidate
     int idx[32];               // compaction scratch
 };
 
@@ -131,9 +128,22 @@ __device__ __forceinline__ int nth_bit(uint32_t x, int n) {
     return pos;
 }
 
-// Every (lane, bit) of the lanes' masks, 32 at a time in order: f(ok, k, s, first) for source s of
-// lane k's mask; `first` has a bit for every lane of the chunk that starts a new k.
-template <class F>
+// 32 x 32 bit transpose: bit s of lane j's x becomes bit j of lane s's result
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane) {
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) {
+        // bits whose index has the h bit clear
+        const uint32_t lowm = h == 16 ? 0x0000ffffu : h == 8 ? 0x00ff00ffu : h == 4 ? 0x0f0f0f0fu
+                                                  : h == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(FULL, x, h);
+        x = lane & h ? (x & ~lowm) | ((y >> h) & lowm) : (x & lowm) | ((y << h) & ~lowm);
+    }
+    return x;
+}
+
+// Every (lane, bit) of the lanes' masks, in order, U chunks of 32 at a time: f(ok[], k[], s[], first[]) for
+// source s of lane k's mask; `first` has a bit for every lane of the chunk that starts a new k.
+template <int U, class F>
 __device__ __forceinline__ void for_pairs(uint32_t mask, int lane, int* idx, F&& f) {
     const unsigned le = 0xffffffffu >> (31 - lane);
     const unsigned nb = __ballot_sync(FULL, mask != 0u);
@@ -145,15 +155,22 @@ __device__ __forceinline__ void for_pairs(uint32_t mask, int lane, int* idx, F&&
     const int st = incl - cnt;
     __syncwarp();
     int kb = -1;
-    for (int p0 = 0; p0 < total; p0 += 32) {
-        const unsigned at = (unsigned)(st - p0);
-        const unsigned first = __reduce_or_sync(FULL, mask != 0u && at < 32u ? 1u << at : 0u);
-        const int k = idx[kb + __popc(first & le)];
-        kb += __popc(first);
-        const uint32_t mk = __shfl_sync(FULL, mask, k);
-        const int n = p0 + lane - __shfl_sync(FULL, st, k);
-        const bool ok = p0 + lane < total;
-        f(ok, k, ok ? nth_bit(mk, n) : 0, first);
+    for (int p0 = 0; p0 < total; p0 += 32 * U) {
+        unsigned first[U];
+        int k[U], s[U];
+        bool ok[U];
+#pragma unroll
+        for (int g = 0; g < U; g++) {
+            const unsigned at = (unsigned)(st - p0 - 32 * g);
+            first[g] = __reduce_or_sync(FULL, mask != 0u && at < 32u ? 1u << at : 0u);
+            k[g] = idx[kb + __popc(first[g] & le)];
+            kb += __popc(first[g]);
+            const uint32_t mk = __shfl_sync(FULL, mask, k[g]);
+            const int n = p0 + 32 * g + lane - __shfl_sync(FULL, st, k[g]);
+            ok[g] = p0 + 32 * g + lane < total;
+            s[g] = ok[g] ? nth_bit(mk, n) : 0;
+        }
+        f(ok, k, s, first);
     }
     __syncwarp();
 }
@@ -169,16 +186,35 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                                           int D, int bd, int64_t rb, const int32_t* __restrict__ col,
                                           const int32_t* __restrict__ wt, const V* vals, bool& ovf, PD&& pair_done,
                                           RD&& row_done) {
+    constexpr int PU = LM_PAIRS<WEIGHTED>, GU = LM_GATHERS<WEIGHTED>;
+    // A row of many arcs: with unit weights many of a chunk's arcs have a bit in common, and each source takes
+    // its own of them; with weights few have, and the warp takes them one after the other.
+    constexpr int BU = WEIGHTED ? 4 : 2;
     const unsigned le = 0xffffffffu >> (31 - lane), lt = le >> 1;
     const bool cand = need != 0u && deg > 0;
     const unsigned cm = __ballot_sync(FULL, cand);
     if (cm == 0u) return;
-    // candidates to the front lanes
+    // candidates to the front lanes; with unit weights (many pairs per visit) by degree, so that
+    // neighbouring pairs have sums of similar length (n = 50,000: 125 -> 121 ms; with weights the sort
+    // costs more than it gives)
     const int K = __popc(cm);
-    if (cand) sm.idx[__popc(cm & lt)] = lane;
-    __syncwarp();
-    const int crow = lane < K ? sm.idx[lane] : 0;
-    __syncwarp();
+    int crow;
+    if constexpr (WEIGHTED) {
+        if (cand) sm.idx[__popc(cm & lt)] = lane;
+        __syncwarp();
+        crow = lane < K ? sm.idx[lane] : 0;
+        __syncwarp();
+    } else {
+        uint32_t key = cand ? ((uint32_t)min(deg, 1 << 26) << 5) | (uint32_t)lane : 0xffffffffu;
+#pragma unroll
+        for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                const uint32_t y = __shfl_xor_sync(FULL, key, j);
+                key = ((lane & j) == 0) == ((lane & k) == 0) ? min(key, y) : max(key, y);
+            }
+        crow = lane < K ? (int)(key & 31u) : 0;
+    }
     const uint32_t cneed = __shfl_sync(FULL, need, crow);
     const uint32_t ca0 = __shfl_sync(FULL, (uint32_t)a0, crow);   // fewer than 2^31 arcs
     const int cd = __shfl_sync(FULL, deg, crow);
@@ -223,23 +259,24 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                     if (MULT && m) mu = mult_of(b0 + c0 + lane);
                 }
                 found |= m;
-                unsigned tb = __ballot_sync(FULL, m != 0u);
-                while (tb) {
-                    V t[BCPP_LM_BU];
-                    uint64_t muq[BCPP_LM_BU];
+                uint32_t own = WEIGHTED ? __ballot_sync(FULL, m != 0u) : transpose_bits(m, lane);
+                while (__any_sync(FULL, own != 0u)) {
+                    V t[BU];
+                    uint64_t muq[BU];
 #pragma unroll
-                    for (int q = 0; q < BCPP_LM_BU; q++) {
-                        const int j = tb ? __ffs(tb) - 1 : 0;
-                        const bool on = tb != 0u;
-                        tb &= tb - 1u;
+                    for (int q = 0; q < BU; q++) {
+                        const int j = own ? __ffs(own) - 1 : 0;
                         const int32_t vq = __shfl_sync(FULL, v, j);
-                        const uint32_t mq = __shfl_sync(FULL, m, j);
                         muq[q] = MULT ? shfl_u64(mu, j) : 0;
-                        t[q] = (V)0;
-                        if (on && (mq >> lane) & 1u) t[q] = vals[(rb + vq) * 32 + lane];
+                        uint32_t mq = 0xffffffffu;
+                        if constexpr (WEIGHTED) mq = __shfl_sync(FULL, m, j);
+                        const bool on = own != 0u && (mq >> lane) & 1u;
+                        t[q] = on ? vals[(rb + vq) * 32 + lane] : (V)0;
+                        own &= own - 1u;
                     }
 #pragma unroll
-                    for (int q = 0; q < BCPP_LM_BU; q++) add(acc, t[q], muq[q]);
+                    for (int q = 0; q < BU; q++)
+                        if (q == 0 || FWD || __any_sync(FULL, t[q] != (V)0)) add(acc, t[q], muq[q]);
                 }
             }
             found = __reduce_or_sync(FULL, found);
@@ -257,65 +294,79 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
         sm.nm[lane] = 0u;
         __syncwarp();
         int pos = 0, kb = k0 - 1;
-        for (int i0 = 0; i0 < T; i0 += 32) {
-            const unsigned at = (unsigned)(st - i0);
-            const unsigned first = __reduce_or_sync(FULL, inr && at < 32u ? 1u << at : 0u);
-            const int k = kb + __popc(first & le);
-            kb += __popc(first);
-            const uint32_t off = __shfl_sync(FULL, ca0 - (uint32_t)st, k);
-            const uint32_t nd = __shfl_sync(FULL, cneed, k);
-            int32_t v = 0;
-            uint32_t m = 0u;
-            const int i = i0 + lane;
-            if (i < T) {
-                v = __ldg(col + off + i);
-                m = gather(v, WEIGHTED ? __ldg(wt + off + i) : 1) & nd;
+        for (int i0 = 0; i0 < T; i0 += 32 * GU) {
+            unsigned first[GU];
+            int k[GU];
+            uint32_t a[GU], m[GU];
+            int32_t v[GU], w[GU];
+#pragma unroll
+            for (int g = 0; g < GU; g++) {
+                const unsigned at = (unsigned)(st - i0 - 32 * g);
+                first[g] = __reduce_or_sync(FULL, inr && at < 32u ? 1u << at : 0u);
+                k[g] = kb + __popc(first[g] & le);
+                kb += __popc(first[g]);
+                a[g] = __shfl_sync(FULL, ca0 - (uint32_t)st, k[g]) + (uint32_t)(i0 + 32 * g + lane);
+                m[g] = __shfl_sync(FULL, cneed, k[g]);
+                v[g] = 0;
+                w[g] = 1;
+                if (i0 + 32 * g + lane < T) {
+                    v[g] = __ldg(col + a[g]);
+                    if (WEIGHTED) w[g] = __ldg(wt + a[g]);
+                } else {
+                    m[g] = 0u;
+                }
             }
-            const unsigned tb = __ballot_sync(FULL, m != 0u);
-            const int p = pos + __popc(tb & lt);
-            if (m) {
-                sm.list[p] = make_uint2((uint32_t)v, m);
-                if constexpr (MULT) sm.mult[p] = mult_of(off + i);
-                atomicOr(&sm.nm[k], m);
+#pragma unroll
+            for (int g = 0; g < GU; g++)
+                if (m[g]) m[g] &= gather(v[g], w[g]);
+#pragma unroll
+            for (int g = 0; g < GU; g++) {
+                const unsigned tb = __ballot_sync(FULL, m[g] != 0u);
+                const int p = pos + __popc(tb & lt);
+                if (m[g]) {
+                    sm.list[p] = make_uint2((uint32_t)v[g], m[g]);
+                    if constexpr (MULT) sm.mult[p] = mult_of(a[g]);
+                    atomicOr(&sm.nm[k[g]], m[g]);
+                }
+                if ((first[g] >> lane) & 1u) sm.seg[k[g]] = p;
+                pos += __popc(tb);
             }
-            if ((first >> lane) & 1u) sm.seg[k] = p;
-            pos += __popc(tb);
         }
         if (lane == 0) sm.seg[k1] = pos;
         __syncwarp();
         const uint32_t nm = inr ? sm.nm[lane] : 0u;
         if (nm) sm.rowm[crow] = nm;
-        if (pos > 0) {
-            for_pairs(nm, lane, sm.idx, [&](bool ok, int k, int s, unsigned first) {
-                const int e1 = ok ? sm.seg[k + 1] : 0;
-                int e = ok ? sm.seg[k] : 0;
-                const int r = __shfl_sync(FULL, crow, k);
-                const V* vs = vals + rb * 32 + s;
-                ACC acc = (ACC)0;
-                while (e < e1) {
-                    V t[BCPP_LM_PU];
+        for_pairs<1>(nm, lane, sm.idx, [&](const bool* ok, const int* k, const int* s, const unsigned* first) {
+            // the row's listed arcs, in step for all its sources (their values share cache lines)
+            const int e1 = ok[0] ? sm.seg[k[0] + 1] : 0;
+            int e = ok[0] ? sm.seg[k[0]] : 0;
+            const int r = __shfl_sync(FULL, crow, k[0]);
+            const V* vs = vals + rb * 32 + s[0];
+            ACC acc = (ACC)0;
+            while (e < e1) {
+                V t[PU];
 #pragma unroll
-                    for (int q = 0; q < BCPP_LM_PU; q++) {
-                        t[q] = (V)0;
-                        if (e + q < e1) {
-                            const uint2 x = sm.list[e + q];
-                            if ((x.y >> s) & 1u) t[q] = vs[(int64_t)x.x * 32];
-                        }
+                for (int q = 0; q < PU; q++) {
+                    t[q] = (V)0;
+                    if (e + q < e1) {
+                        const uint2 x = sm.list[e + q];
+                        if ((x.y >> s[0]) & 1u) t[q] = vs[(int64_t)x.x * 32];
                     }
-#pragma unroll
-                    for (int q = 0; q < BCPP_LM_PU; q++) add(acc, t[q], MULT ? sm.mult[min(e + q, e1 - 1)] : 0);
-                    e += BCPP_LM_PU;
                 }
-                pair_done(ok, r, s, acc, first);
-            });
-        }
+#pragma unroll
+                for (int q = 0; q < PU; q++)
+                    add(acc, t[q], MULT ? sm.mult[min(e + q, e1 - 1)] : 0);
+                e += PU;
+            }
+            pair_done(ok[0], r, s[0], acc, first[0]);
+        });
         __syncwarp();
         k0 = k1;
     }
 }
 
 template <typename SG, bool WEIGHTED, bool MULT>
-__global__ void __launch_bounds__(LM_THREADS, sizeof(SG) == 4 ? BCPP_LM_MINB : BCPP_LM_MINB64) lm_kernel(const LmArgs A) {
+__global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm_kernel(const LmArgs A) {
     __shared__ WarpSm<MULT> s_warp[LM_WARPS];
     const int lane = threadIdx.x & 31;
     WarpSm<MULT>& sm = s_warp[threadIdx.x >> 5];
@@ -550,8 +601,13 @@ __global__ void __launch_bounds__(LM_THREADS, sizeof(SG) == 4 ? BCPP_LM_MINB : B
             __syncwarp();
             const uint32_t inner = sm.rowm[lane];
             const uint32_t leaf = tgt ? need & ~inner : 0u;   // no successor: c = 1 / sigma
-            for_pairs(leaf, lane, sm.idx, [&](bool ok, int r, int s, unsigned) {
-                if (ok) crow[r * 32 + s] = recip_of(srow[r * 32 + s]);
+            for_pairs<2>(leaf, lane, sm.idx, [&](const bool* ok, const int* r, const int* s, const unsigned*) {
+                SG v[2];
+#pragma unroll
+                for (int g = 0; g < 2; g++) v[g] = ok[g] ? srow[r[g] * 32 + s[g]] : (SG)1;
+#pragma unroll
+                for (int g = 0; g < 2; g++)
+                    if (ok[g]) crow[r[g] * 32 + s[g]] = recip_of(v[g]);
             });
             if ((inner | leaf) != need) *lrow = inner | leaf;
             const double ds = sm.ds[lane];
