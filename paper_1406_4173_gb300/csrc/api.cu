@@ -2468,6 +2468,30 @@ int csr_build_dev(bcpp_ctx* c, int32_t n, int64_t m, const int32_t* eu, const in
     if (ew && !w_out && m > 0) return BCPP_EINVAL;
     CK_RC(reset_flags(c));
     const int64_t na = directed ? m : 2 * m;
+    if (m > 0 && n > 0) {
+        DBuf<uint32_t> counts(c, (int64_t)n + 1), place(c, na), longest(c, 2);   // longest row, long rows
+        DBuf<int64_t> stmp(c, scan_tmp_elems((int64_t)n + 1));
+        CK_ALLOC(counts); CK_ALLOC(place); CK_ALLOC(longest); CK_ALLOC(stmp);
+        CK_CUDA(cudaMemsetAsync(counts.p, 0, ((size_t)n + 1) * sizeof(uint32_t), c->stream));
+        CK_CUDA(cudaMemsetAsync(longest.p, 0, 2 * sizeof(uint32_t), c->stream));
+        csr_count(n, m, eu, ev, ew, directed, counts.p, place.p, longest.p, c->flags, c->stream);
+        c->launches += 2;
+        uint32_t hl = 0;
+        CK_CUDA(cudaMemcpyAsync(&hl, longest.p, sizeof(hl), cudaMemcpyDeviceToHost, c->stream));
+        CK_RC(sync_flags(c));
+        if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
+        if (hl <= CSR_LONG_ROW) {
+            exclusive_scan<uint32_t>(counts.p, rp, (int64_t)n + 1, nullptr, stmp.p, c->stream, c->launches);
+            csr_scatter(m, eu, ev, ew, directed, rp, place.p, col, ew ? w_out : nullptr, c->stream);
+            // (the counts are no longer needed: the list of long rows takes their place)
+            CK_CUDA(csr_sort_rows(n, hl, rp, col, ew ? w_out : nullptr, reinterpret_cast<int32_t*>(counts.p),
+                                  longest.p + 1, c->flags, c->stream));
+            c->launches += 3;
+            CK_CUDA(cudaGetLastError());
+            *num_arcs_out = na;
+            return finish_status(c, nullptr);
+        }
+    }
     DBuf<uint64_t> keys(c, na), kb(c, na);
     DBuf<uint32_t> vals(c, na), vb(c, na);
     DBuf<int64_t> hist(c, radix_hist_elems(na)), tmp(c, scan_tmp_elems(radix_hist_elems(na)));

@@ -4,7 +4,18 @@
 
 namespace bcpp {
 
-// keys[i] = tail * n + head, vals[i] = weight (2 arcs per undirected edge); flags input errors
+// Build by counting: arcs per tail (counts zeroed before), every arc's place in its row, the longest row; flags
+// input errors.  place: one word per arc (undirected: 2i is u -> v, 2i + 1 is v -> u).
+void csr_count(int32_t n, int64_t m, const int32_t* eu, const int32_t* ev, const uint32_t* ew, int directed,
+               uint32_t* counts, uint32_t* place, uint32_t* longest, uint32_t* flags, cudaStream_t st);
+void csr_scatter(int64_t m, const int32_t* eu, const int32_t* ev, const uint32_t* ew, int directed, const int64_t* rp,
+                 const uint32_t* place, int32_t* col, uint32_t* w, cudaStream_t st);
+// sort every row (of at most CSR_LONG_ROW arcs) and flag repeated arcs; longrows: n words, nlong: one zeroed word
+constexpr uint32_t CSR_LONG_ROW = 16384;
+cudaError_t csr_sort_rows(int32_t n, uint32_t longest, const int64_t* rp, int32_t* col, uint32_t* w, int32_t* longrows,
+                          uint32_t* nlong, uint32_t* flags, cudaStream_t st);
+
+// Build by one sort of all arcs (rows longer than CSR_LONG_ROW): keys[i] = tail * n + head, vals[i] = weight (2 arcs per undirected edge); flags input errors
 void csr_expand(int32_t n, int64_t m, const int32_t* eu, const int32_t* ev, const uint32_t* ew, int directed,
                 uint64_t* keys, uint32_t* vals, uint32_t* flags, cudaStream_t st);
 // from sorted keys: col, weights, row_ptr; flags repeated arcs
