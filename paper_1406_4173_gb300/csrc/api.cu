@@ -868,18 +868,19 @@ int lm_levels(bool weighted, bool directed, const OrderWs* ord) {
     return std::max(directed ? 64 : 24, 2 * std::min(ord->depth, LM_MAX_LEVELS) + 4);
 }
 
-// false: not enough memory for one batch (the caller takes the lockstep kernel).  sizes: node count of
+// *fits = false: not enough memory for one batch (the caller takes the lockstep kernel).  forward: no backward
+// pass, no sums over sources.  sizes: node count of
 // an item's graph; one_graph: every batch is of the same graph.
 template <class F>
 int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_graph, F&& size_of, int64_t nodes,
-             int lcap, bool narrow, bool* fits) {
+             int lcap, bool narrow, bool* fits, bool forward = false) {
     *fits = false;
     const int nitems = (int)items.size();
     if (nitems == 0 || lcap > LM_MAX_LEVELS) return BCPP_OK;
     L.lcap = lcap;
     L.narrow = narrow;
     L.nodes = nodes;
-    const int64_t row_bytes = 32 * ((narrow ? 4 : 8) + 8) + 8 + 4 + 4ll * lcap;
+    const int64_t row_bytes = 32 * ((narrow ? 4 : 8) + (forward ? 0 : 8)) + 8 + 4 + 4ll * lcap;
     const int64_t budget = free_bytes(c);
     int64_t total = 0, largest = 0;
     std::vector<int32_t> tile0;
@@ -928,13 +929,15 @@ int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_gr
     CK_ALLOC(L.lev.alloc(c, rows * lcap));
     CK_ALLOC(L.seen.alloc(c, rows));
     CK_ALLOC(L.sg.alloc(c, rows * 32 * (narrow ? 4 : 8)));
-    CK_ALLOC(L.cc.alloc(c, rows * 32));
     CK_ALLOC(L.dsum.alloc(c, rows));
     CK_ALLOC(L.ctl.alloc(c, lm_ctl_words(lcap, most_items)));
-    CK_ALLOC(L.bcs.alloc(c, nodes));
-    CK_ALLOC(L.bcc.alloc(c, nodes));
-    CK_ALLOC(L.runs.alloc(c, (int64_t)runs.size()));
-    CK_RC(to_dev(c, L.runs.p, runs.data(), (int64_t)runs.size()));
+    if (!forward) {
+        CK_ALLOC(L.cc.alloc(c, rows * 32));
+        CK_ALLOC(L.bcs.alloc(c, nodes));
+        CK_ALLOC(L.bcc.alloc(c, nodes));
+        CK_ALLOC(L.runs.alloc(c, (int64_t)runs.size()));
+        CK_RC(to_dev(c, L.runs.p, runs.data(), (int64_t)runs.size()));
+    }
     if (one_graph) {
         L.tpb = (int32_t)largest;
     } else {
@@ -948,6 +951,37 @@ int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_gr
     return BCPP_OK;
 }
 
+// The arguments of one wave.
+LmArgs lm_wave_args(const LmWs& L, const LmWave& w, const LsArena& A, const LsParams& P, const LsItem* items,
+                    uint64_t wmax) {
+    LmArgs a{};
+    a.rp = A.rp; a.col = A.col; a.w = A.w;
+    a.irp = A.irp; a.icol = A.icol; a.iw = A.iw;
+    a.imu = A.imu;
+    a.mud = static_cast<const double*>(A.mud);
+    a.node_off = A.node_off;
+    a.nfront = P.nfront; a.toff = P.toff; a.td = P.td; a.ts = P.ts;
+    a.bc_map = P.bc_map;
+    a.items = items + w.i0;
+    a.item_tile0 = L.tpb ? nullptr : L.tile0.p + w.i0;
+    a.tile_item = L.tile_item.p;
+    a.tile_base = L.tpb ? 0 : w.tile0;
+    a.item_base = w.i0;
+    a.tpb = L.tpb;
+    a.nitems = w.i1 - w.i0;
+    a.ntiles = w.ntiles;
+    a.srcs = P.srcs;
+    a.in_s = P.in_s;
+    a.lev = L.lev.p; a.seen = L.seen.p; a.sg = L.sg.p; a.cc = L.cc.p; a.dsum = L.dsum.p;
+    a.rows = (int64_t)w.ntiles * 32;
+    a.lcap = L.lcap;
+    a.wmax = (int32_t)wmax;
+    a.ctl = L.ctl.p;
+    a.flags = P.flags;
+    a.phase_ns = P.phase_ns;
+    return a;
+}
+
 // All waves and the sum over sources (device work only): out = scale * sum.
 int lm_emit(bcpp_ctx* c, LmWs& L, const LsArena& A, const LsParams& P, const LsItem* items, uint64_t wmax,
             double scale, double* out, Timer* tb) {
@@ -955,30 +989,7 @@ int lm_emit(bcpp_ctx* c, LmWs& L, const LsArena& A, const LsParams& P, const LsI
     CK_CUDA(cudaMemsetAsync(L.bcc.p, 0, (size_t)L.nodes * sizeof(double), c->stream));
     if (tb) tb->start();
     for (const LmWave& w : L.waves) {
-        LmArgs a{};
-        a.rp = A.rp; a.col = A.col; a.w = A.w;
-        a.irp = A.irp; a.icol = A.icol; a.iw = A.iw;
-        a.imu = A.imu;
-        a.mud = static_cast<const double*>(A.mud);
-        a.node_off = A.node_off;
-        a.bc_map = P.bc_map;
-        a.items = items + w.i0;
-        a.item_tile0 = L.tpb ? nullptr : L.tile0.p + w.i0;
-        a.tile_item = L.tile_item.p;
-        a.tile_base = L.tpb ? 0 : w.tile0;
-        a.item_base = w.i0;
-        a.tpb = L.tpb;
-        a.nitems = w.i1 - w.i0;
-        a.ntiles = w.ntiles;
-        a.srcs = P.srcs;
-        a.in_s = P.in_s;
-        a.lev = L.lev.p; a.seen = L.seen.p; a.sg = L.sg.p; a.cc = L.cc.p; a.dsum = L.dsum.p;
-        a.rows = (int64_t)w.ntiles * 32;
-        a.lcap = L.lcap;
-        a.wmax = (int32_t)wmax;
-        a.ctl = L.ctl.p;
-        a.flags = P.flags;
-        a.phase_ns = P.phase_ns;
+        const LmArgs a = lm_wave_args(L, w, A, P, items, wmax);
         CK_CUDA(cudaMemsetAsync(L.ctl.p, 0, (size_t)lm_ctl_words(L.lcap, a.nitems) * sizeof(uint32_t), c->stream));
         CK_CUDA(lm_launch(a, L.narrow, c->num_sms, c->stream));
         lm_accumulate(a, L.runs.p + w.run0, w.nruns, w.natiles, L.bcs.p, L.bcc.p, c->stream);
@@ -1232,6 +1243,35 @@ int build_local_csr(bcpp_ctx* c, const Skeleton& K, const int64_t* rp, const int
     return BCPP_OK;
 }
 
+// Dijkstra_SK on the level-mask kernel.  *done stays false when the batches do not fit into memory or prove
+// too deep for it (or a count outgrows 32 bits): the lockstep kernel then fills the tables.
+int tables_levels(bcpp_ctx* c, const LsArena& A, const LsParams& P, const std::vector<LsItem>& hitems,
+                  const LsItem* items, const std::vector<int32_t>& pstart, uint64_t wmax, int64_t entries, bool* done) {
+    LmWs L;
+    bool fits = false;
+    CK_RC(lm_alloc(c, L, hitems, false, [&](int32_t i) { return (int64_t)(pstart[i + 1] - pstart[i]); }, 0,
+                   lm_levels(A.w != nullptr, true, nullptr), true, &fits, true));
+    if (!fits) return BCPP_OK;
+    fill_i32(P.td, DINF, entries, c->stream);
+    CK_CUDA(cudaMemsetAsync(P.ts, 0, (size_t)entries * sizeof(uint64_t), c->stream));
+    c->launches++;
+    for (const LmWave& w : L.waves) {
+        const LmArgs a = lm_wave_args(L, w, A, P, items, wmax);
+        CK_CUDA(cudaMemsetAsync(L.ctl.p, 0, (size_t)lm_ctl_words(L.lcap, a.nitems) * sizeof(uint32_t), c->stream));
+        CK_CUDA(lm_tables_launch(a, c->num_sms, c->stream));
+        c->launches++;
+    }
+    CK_RC(sync_flags(c));
+    if (c->hflags[FLAG_TIMEOUT]) return BCPP_ETIMEOUT;
+    if (c->hflags[FLAG_CAPACITY]) {
+        CK_CUDA(cudaMemsetAsync(c->flags + FLAG_CAPACITY, 0, sizeof(uint32_t), c->stream));
+        CK_CUDA(cudaMemsetAsync(c->flags + FLAG_DEPTH, 0, sizeof(uint32_t), c->stream));
+        return BCPP_OK;
+    }
+    *done = true;
+    return BCPP_OK;
+}
+
 // reuse (may be null): a skeleton of the same graph built for `part` without singletons.  Every
 // part that keeps its nodes under P' keeps its frontiers, its local order and so its Dijkstra_SK
 // tables, so they are read from `reuse` instead of being recomputed (Alg. 3 builds the
@@ -1357,12 +1397,7 @@ int build_sk(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS_eff,
         iota(srcs.p, maxnf, c->stream);
         c->launches++;
         const int nb = g->w ? (int)wmax + 1 : 2;
-        // parts are small: provide the worst case (one entry per node and frontier source)
-        const int ef = entry_factor(c, true, 1);
-        const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxpart_tab, nb, false, ef), 0);
         for (int dir = 0; dir < (g->directed ? 2 : 1); dir++) {
-            SlotWs ws;
-            CK_RC(alloc_slots(c, ws, slots, maxpart_tab, nb, false, 0, 1, ef));
             LsArena A{};
             if (dir == 0) {
                 A.rp = lrp.p; A.col = lcol.p; A.w = g->w ? lw.p : nullptr;
@@ -1382,8 +1417,17 @@ int build_sk(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS_eff,
             P.toff = K.toff.p;
             P.td = dir == 0 ? K.td.p : K.tdr.p;
             P.ts = dir == 0 ? K.ts.p : K.tsr.p;
-            P.item_counter = ws.counter.p;
             P.flags = c->flags;
+            bool done = false;
+            if (lm_serves(c, bcpp_opts{}, 1, maxpart_tab, g->num_arcs, g->w ? wmax : 1))
+                CK_RC(tables_levels(c, A, P, hitems, items.p, K.h_pstart, g->w ? wmax : 1, tofs, &done));
+            if (done) continue;
+            // parts are small: provide the worst case (one entry per node and frontier source)
+            const int ef = entry_factor(c, true, 1);
+            const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxpart_tab, nb, false, ef), 0);
+            SlotWs ws;
+            CK_RC(alloc_slots(c, ws, slots, maxpart_tab, nb, false, 0, 1, ef));
+            P.item_counter = ws.counter.p;
             ls_launch(false, !g->directed, A, P, ws.W, items.p, nitems, slots, c->stream);
             c->launches++;
             CK_CUDA(cudaGetLastError());

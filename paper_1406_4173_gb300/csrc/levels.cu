@@ -181,10 +181,13 @@ __device__ __forceinline__ void for_pairs(uint32_t mask, int lane, int* idx, F&&
 //   pair_done(ok, r, s, acc, first): the sum of source s of the tile's row r (packed pairs)
 //   row_done(r, mask, acc): the same for all 32 sources of one row, lane = source
 //   ovf: a 64-bit count wrapped
-template <bool FWD, bool WEIGHTED, bool MULT, typename V, typename ACC, class PD, class RD>
+// TABLE (Dijkstra_SK): a frontier other than the source (nodes below nf, distance above 0) takes part in the
+// distances but not in the counts, so its arcs add to the found masks only.
+template <bool FWD, bool WEIGHTED, bool MULT, bool TABLE, typename V, typename ACC, class PD, class RD>
 __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int lane, uint32_t need, int64_t a0, int deg,
                                           int D, int bd, int64_t rb, const int32_t* __restrict__ col,
-                                          const int32_t* __restrict__ wt, const V* vals, bool& ovf, PD&& pair_done,
+                                          const int32_t* __restrict__ wt, const V* vals, int32_t nf, bool& ovf,
+                                          PD&& pair_done,
                                           RD&& row_done) {
     constexpr int PU = LM_PAIRS<WEIGHTED>, GU = LM_GATHERS<WEIGHTED>;
     // A row of many arcs: with unit weights many of a chunk's arcs have a bit in common, and each source takes
@@ -237,6 +240,7 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
         else if constexpr (!FWD) acc = MULT ? fma(__longlong_as_double((long long)mu), t, acc) : acc + t;
         else acc = MULT ? madd_ck(acc, t, mu, ovf) : add_ck(acc, t, ovf);
     };
+    auto counts = [&](int32_t v, int32_t w) { return !TABLE || v >= nf || D == w; };
     int k0 = 0;
     while (k0 < K) {
         const int base = __shfl_sync(FULL, pre - cdeg, k0);
@@ -255,10 +259,12 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                 uint64_t mu = 0;
                 if (c0 + lane < dg) {
                     v = __ldg(col + b0 + c0 + lane);
-                    m = gather(v, WEIGHTED ? __ldg(wt + b0 + c0 + lane) : 1) & nd;
+                    const int32_t w = WEIGHTED ? __ldg(wt + b0 + c0 + lane) : 1;
+                    m = gather(v, w) & nd;
+                    found |= m;
+                    if (!counts(v, w)) m = 0u;
                     if (MULT && m) mu = mult_of(b0 + c0 + lane);
                 }
-                found |= m;
                 uint32_t own = WEIGHTED ? __ballot_sync(FULL, m != 0u) : transpose_bits(m, lane);
                 while (__any_sync(FULL, own != 0u)) {
                     V t[BU];
@@ -318,7 +324,13 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
             }
 #pragma unroll
             for (int g = 0; g < GU; g++)
-                if (m[g]) m[g] &= gather(v[g], w[g]);
+                if (m[g]) {
+                    m[g] &= gather(v[g], w[g]);
+                    if (TABLE && m[g] && !counts(v[g], w[g])) {
+                        atomicOr(&sm.nm[k[g]], m[g]);
+                        m[g] = 0u;
+                    }
+                }
 #pragma unroll
             for (int g = 0; g < GU; g++) {
                 const unsigned tb = __ballot_sync(FULL, m[g] != 0u);
@@ -365,7 +377,7 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
     }
 }
 
-template <typename SG, bool WEIGHTED, bool MULT>
+template <typename SG, bool WEIGHTED, bool MULT, bool TABLE>
 __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm_kernel(const LmArgs A) {
     __shared__ WarpSm<MULT> s_warp[LM_WARPS];
     const int lane = threadIdx.x & 31;
@@ -446,6 +458,11 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
             atomicOr(&sm.rowm[local], 1u << lane);
             sg[(x.rb + src) * 32 + lane] = (SG)1;
             if (sizeof(SG) == 8 && A.drow) A.drow[(x.rb + src) * 32 + lane] = 0;
+            if constexpr (TABLE) {
+                const int64_t o = __ldg(A.toff + x.I.g) + (int64_t)src * __ldg(A.nfront + x.I.g) + x.I.aux + lane;
+                A.td[o] = 0;
+                A.ts[o] = 1ull;
+            }
         }
         __syncwarp();
         const uint32_t m = sm.rowm[lane];
@@ -492,15 +509,21 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
             __syncwarp();
             SG* srow = sg + (int64_t)t * 1024;
             int32_t* drow = sizeof(SG) == 8 && A.drow ? A.drow + (int64_t)t * 1024 : nullptr;
+            const int32_t nf = TABLE ? __ldg(A.nfront + x.I.g) : 0;
+            const int64_t tab = TABLE ? __ldg(A.toff + x.I.g) + (int64_t)(x.u - lane) * nf + x.I.aux : 0;
             auto settle = [&](bool ok, int r, int s, uint64_t acc) {
                 if (ok) {
                     srow[r * 32 + s] = (SG)acc;
+                    if constexpr (TABLE) {
+                        A.td[tab + (int64_t)r * nf + s] = D;
+                        A.ts[tab + (int64_t)r * nf + s] = acc;
+                    }
                     if (drow) drow[r * 32 + s] = D;
                     if constexpr (sizeof(SG) == 4) wide |= (acc >> 32) != 0;
                 }
             };
-            tile_sums<true, WEIGHTED, MULT, SG, uint64_t>(
-                A, sm, lane, need, a0, deg, D, 0, x.rb, A.icol, A.iw, sg, ovf,
+            tile_sums<true, WEIGHTED, MULT, TABLE, SG, uint64_t>(
+                A, sm, lane, need, a0, deg, D, 0, x.rb, A.icol, A.iw, sg, nf, ovf,
                 [&](bool ok, int r, int s, uint64_t acc, unsigned) { settle(ok, r, s, acc); },
                 [&](int r, uint32_t mask, uint64_t acc) { settle((mask >> lane) & 1u, r, lane, acc); });
             __syncwarp();
@@ -535,7 +558,7 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
 
-    if (!cc) return;
+    if (TABLE || !cc) return;
     // ------------------------------------------------------------------ backward
     // (level 0 is the sources themselves: nothing is credited to them and nobody reads their c)
     for (int D = depth; D >= 1; D--) {
@@ -565,8 +588,8 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
             const SG* srow = sg + (int64_t)t * 1024;
             double* crow = cc + (int64_t)t * 1024;
             bool no_ovf = false;
-            tile_sums<false, WEIGHTED, MULT, double, double>(
-                A, sm, lane, need, a0, deg, D, bd, x.rb, A.col, A.w, cc, no_ovf,
+            tile_sums<false, WEIGHTED, MULT, false, double, double>(
+                A, sm, lane, need, a0, deg, D, bd, x.rb, A.col, A.w, cc, 0, no_ovf,
                 [&](bool ok, int r, int s, double acc, unsigned first) {
                     double delta = 0.0;
                     if (ok) {
@@ -715,16 +738,16 @@ __global__ void lm_tile_items_kernel(const int32_t* __restrict__ item_tile0, int
     }
 }
 
-template <typename SG, bool WEIGHTED, bool MULT = false>
+template <typename SG, bool WEIGHTED, bool MULT = false, bool TABLE = false>
 cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, WEIGHTED, MULT>, LM_THREADS, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, WEIGHTED, MULT, TABLE>, LM_THREADS, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
     const int blocks = std::min(per_sm * num_sms, std::max(1, (A.ntiles + LM_WARPS - 1) / LM_WARPS));
     LmArgs a = A;
     void* args[] = {&a};
-    return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, WEIGHTED, MULT>, dim3(blocks), dim3(LM_THREADS), args, 0,
+    return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, WEIGHTED, MULT, TABLE>, dim3(blocks), dim3(LM_THREADS), args, 0,
                                        st);
 }
 
@@ -738,6 +761,11 @@ cudaError_t lm_launch(const LmArgs& A, bool narrow, int num_sms, cudaStream_t st
     if (narrow) return weighted ? lm_go<uint32_t, true>(A, num_sms, st) : lm_go<uint32_t, false>(A, num_sms, st);
     if (A.mud) return weighted ? lm_go<uint64_t, true, true>(A, num_sms, st) : cudaErrorInvalidValue;
     return weighted ? lm_go<uint64_t, true>(A, num_sms, st) : lm_go<uint64_t, false>(A, num_sms, st);
+}
+
+cudaError_t lm_tables_launch(const LmArgs& A, int num_sms, cudaStream_t st) {
+    if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;
+    return A.w ? lm_go<uint32_t, true, false, true>(A, num_sms, st) : lm_go<uint32_t, false, false, true>(A, num_sms, st);
 }
 
 void lm_accumulate(const LmArgs& A, const LmRun* runs, int nruns, int natiles, double* bcs, double* bcc,

@@ -40,6 +40,10 @@ struct LmArgs {
     int32_t* drow;              // [rows][32] distances (DINF = unreached), or nullptr; with it cc is zero
                                 // wherever it is not written
     double* dsum;               // [rows] dependencies summed over the batch's sources
+    const int32_t* nfront;      // Dijkstra_SK tables: frontiers of each graph (its first nodes); nullptr: no tables
+    const int64_t* toff;        // table offset of each graph
+    int32_t* td;                // d_i[v][f], filled with DINF before
+    uint64_t* ts;               // sigma_i[v][f], zeroed before
     const int32_t* bc_map;      // global node -> index of the sums over sources (nullptr = same)
     int64_t rows;               // 32 ntiles
     int32_t lcap;               // levels provided for
@@ -54,6 +58,10 @@ int64_t lm_ctl_words(int lcap, int nitems);
 // Forward and backward pass of every batch of the wave; one cooperative launch.  narrow: 32-bit path
 // counts (a count of 2^32 or more aborts like a late level).
 cudaError_t lm_launch(const LmArgs& A, bool narrow, int num_sms, cudaStream_t st);
+
+// Dijkstra_SK (Eq. 10): forward pass of every batch (sources: frontiers aux .. aux + nsrc - 1 of graph g, cc =
+// nullptr) into the tables; 32-bit path counts as with narrow.
+cudaError_t lm_tables_launch(const LmArgs& A, int num_sms, cudaStream_t st);
 
 // A run of consecutive batches of one graph in a wave: dsum of its batches is summed per node.
 struct LmRun {

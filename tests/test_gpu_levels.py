@@ -126,6 +126,30 @@ def test_levels_paths_match_oracle(bc, name):
         assert np.array_equal(s[i], rs), i
 
 
+TABLE_CASES = {
+    "planted": (gen.planted_partition(400, 4, 0.05, 0.006, seed=31), 20),
+    "planted-w": (gen.planted_partition(400, 4, 0.05, 0.006, seed=32, wmax=9), 33),
+    "one-big-part": (gen.planted_partition(700, 2, 0.03, 0.004, seed=33), 10),
+    "directed-w": (gen.chung_lu_communities(300, [75] * 4, 2.3, 6.0, 0.85, seed=34, directed=True, wmax=7), 15),
+    "deep-part": (gen.path(300), 5),          # a part deeper than the kernel serves: the lockstep tables
+}
+
+
+@pytest.mark.parametrize("name", list(TABLE_CASES))
+def test_tables_give_the_oracle_skeleton(bc, name):
+    """Dijkstra_SK on the level-mask kernel (frontier parents excluded from the counts): the skeleton's arcs,
+    weights and multiplicities, exactly."""
+    g, k = TABLE_CASES[name]
+    part = g.part if g.part is not None else (np.arange(g.n) * 2 // g.n).astype(np.int32)
+    S = gen.sample_targets(g.n, k, seed=4)
+    nodes, (u, v, w, mu) = bc.skeleton(bc.graph_from_edgelist(g), S, part)
+    rn, (ru, rv, rw, rmu), _ = oracle.skeleton(g, S, part)
+    o, ro = np.lexsort((v, u)), np.lexsort((rv, ru))
+    assert np.array_equal(np.sort(nodes), np.sort(rn))
+    for x, rx in ((u, ru), (v, rv), (w, rw), (mu, rmu)):
+        assert np.array_equal(np.asarray(x)[o].astype(np.uint64), np.asarray(rx)[ro].astype(np.uint64))
+
+
 def spoked(k, wmax=None):
     """Part 0: a hub and its k neighbours, each tied to one node of a ring (part 1): the hub is a
     non-frontier node with k frontiers that all reach it directly."""
