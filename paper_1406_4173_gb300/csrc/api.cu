@@ -12,6 +12,7 @@
 #include "csr.cuh"
 #include "levels.cuh"
 #include "lockstep.cuh"
+#include "order.cuh"
 #include "partition.cuh"
 #include "prims.cuh"
 #include "skeleton.cuh"
@@ -591,59 +592,29 @@ int build_in_csr(bcpp_ctx* c, const bcpp_graph* g, InCsr& T) {
 // each other, so the nodes of the graph see few distinct distances per batch and a batch
 // settles fewer (node, step) entries.  Only the batching order changes, not the result.
 //
-// The positions depend on the graph only: order_prepare computes them (a single-source run
-// of the lockstep kernel for the levels, then one small sort per level; the level sizes are
-// read by the host), and order_emit sorts S by them (device work only, capturable).
+// The positions depend on the graph only: order_prepare computes them, and order_emit orders S by them
+// (device work only, capturable).  Unit weights: one launch gives the nodes in discovery order (order.cu), and
+// S is picked out of it.  Integer weights (levels of weighted distance): a single-source run of the lockstep
+// kernel, then one small sort per level (the level sizes are read by the host), and a sort of S.
 struct OrderWs {
     int64_t ns = 0;
     int32_t n = 0, k = 0;
     int32_t depth = 0;        // deepest level from the hub
     const int32_t* S = nullptr;
     const int32_t* part = nullptr;
-    DBuf<int32_t> pos;        // [n] discovery position of every node
+    DBuf<int32_t> queue;      // unit weights: [n] nodes in discovery order
+    DBuf<uint8_t> mem;        // [n] membership in S
+    DBuf<int32_t> flag;       // [n] the same in queue order
+    DBuf<int64_t> place;      // its prefix sums
+    DBuf<int32_t> pos;        // integer weights: [n] discovery position of every node
     DBuf<uint64_t> keys, kb;
     DBuf<uint32_t> vals, vb;
     DBuf<int64_t> hist, tmp;
     DBuf<int32_t> out;        // the ordered targets
 };
 
-constexpr int ORDER_MAX_LEVELS = 4096;   // deeper graphs keep plain level order past this level
-
 __global__ void hub_src_kernel(const unsigned long long* best, int32_t* src) {
     src[0] = (int32_t)(0xffffffffu - (uint32_t)(best[0] & 0xffffffffull));
-}
-// Breadth-first levels from one source over unit-weight arcs, as the lockstep kernel's LS_SSSP
-// mode would give them (DINF = unreached), but with the whole GPU on each level: warp w looks
-// at nodes [32w, 32w + 32) and scans the arcs of those at level L with all its lanes;
-// unreached heads get L + 1 (concurrent writers all write L + 1).  more[L] = some head was
-// reached; a level whose predecessor reached nothing returns at once.
-__global__ void bfs_seed_kernel(int32_t* level, const int32_t* src, int32_t* more, int32_t nmore) {
-    level[src[0]] = 0;
-    for (int i = 0; i < nmore; i++) more[i] = 0;
-}
-__global__ void bfs_level_kernel(const int64_t* __restrict__ rp, const int32_t* __restrict__ col, int32_t n,
-                                 int32_t* level, int32_t L, int32_t* more) {
-    if (L > 0 && more[L - 1] == 0) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    bool found = false;
-    for (int64_t b0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; b0 < n; b0 += nw * 32) {
-        const int64_t v = b0 + lane;
-        unsigned m = __ballot_sync(FULL, v < n && level[v] == L);
-        while (m) {
-            const int64_t u = b0 + (__ffs(m) - 1);
-            m &= m - 1;
-            const int64_t a1 = rp[u + 1];
-            for (int64_t a = rp[u] + lane; a < a1; a += 32) {
-                const int32_t w = col[a];
-                if (level[w] == DINF) {
-                    level[w] = L + 1;
-                    found = true;
-                }
-            }
-        }
-    }
-    if (__any_sync(FULL, found) && lane == 0) more[L] = 1;
 }
 // level histogram (levels >= cap counted at cap) and the deepest level
 __global__ void level_hist_kernel(const int32_t* level, int32_t n, int32_t cap, int32_t* cnt, int32_t* maxl) {
@@ -687,6 +658,33 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
                   uint64_t wmax, const int32_t* S, int64_t ns, const int32_t* part, int32_t k, OrderWs& w) {
     const int32_t n = g->n;
     w.ns = ns; w.n = n; w.k = k; w.S = S; w.part = part;
+    // buffers of the per-call ordering of S
+    const bool all = ns == n;   // S = V: the order of all nodes
+    CK_ALLOC(w.out.alloc(c, ns));
+    if (g->w || !all || part) {
+        CK_ALLOC(w.vals.alloc(c, ns));
+    }
+    if (g->w || part) {
+        CK_ALLOC(w.keys.alloc(c, ns)); CK_ALLOC(w.kb.alloc(c, ns));
+        CK_ALLOC(w.vb.alloc(c, ns));
+        CK_ALLOC(w.hist.alloc(c, radix_hist_elems(ns)));
+        CK_ALLOC(w.tmp.alloc(c, scan_tmp_elems(std::max<int64_t>(radix_hist_elems(ns), n))));
+    } else if (!all) {
+        CK_ALLOC(w.tmp.alloc(c, scan_tmp_elems(n)));
+    }
+    if (!g->w) {
+        DBuf<int32_t> par(c, n), depth(c, 1);
+        DBuf<uint32_t> ctl(c, order_ctl_words(c->num_sms));
+        CK_ALLOC(par); CK_ALLOC(depth); CK_ALLOC(ctl);
+        if (!all || part) CK_ALLOC(w.queue.alloc(c, n));
+        if (!all) {
+            CK_ALLOC(w.mem.alloc(c, n)); CK_ALLOC(w.flag.alloc(c, n)); CK_ALLOC(w.place.alloc(c, n));
+        }
+        CK_CUDA(order_bfs_launch(n, g->row_ptr, g->col, par.p, all && !part ? w.out.p : w.queue.p, ctl.p, depth.p,
+                                 c->flags, c->num_sms, c->stream));
+        c->launches++;
+        return to_host(c, &w.depth, depth.p, 1);
+    }
     // levels from the hub (the node of largest degree)
     DBuf<unsigned long long> best(c, 1);
     DBuf<int32_t> level(c, n), src(c, 1), cnt(c, ORDER_MAX_LEVELS + 1), maxl(c, 1);
@@ -704,30 +702,9 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
     hub_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, c->stream>>>(g->row_ptr, n, best.p);
     hub_src_kernel<<<1, 1, 0, c->stream>>>(best.p, src.p);
     c->launches += 2;
-    // Unit weights: level-synchronous breadth-first search over the whole GPU, 8 levels per
-    // host check; a graph deeper than BFS_LEVELS levels falls back to the lockstep kernel.
-    constexpr int32_t BFS_LEVELS = 256;
-    bool have_levels = false;
-    if (!g->w) {
-        DBuf<int32_t> more(c, BFS_LEVELS);
-        CK_ALLOC(more);
-        fill_i32(level.p, DINF, n, c->stream);
-        bfs_seed_kernel<<<1, 1, 0, c->stream>>>(level.p, src.p, more.p, BFS_LEVELS);
-        c->launches += 2;
-        const unsigned bblk = (unsigned)std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)c->num_sms * 8);
-        for (int32_t L0 = 0; L0 < BFS_LEVELS && !have_levels; L0 += 8) {
-            for (int32_t L = L0; L < L0 + 8; L++) {
-                bfs_level_kernel<<<bblk, 256, 0, c->stream>>>(g->row_ptr, g->col, n, level.p, L, more.p);
-                c->launches++;
-            }
-            int32_t last = 1;
-            CK_RC(to_host(c, &last, more.p + L0 + 7, 1));
-            have_levels = last == 0;
-        }
-    }
-    if (!have_levels) {
-        // levels (or weighted distances) from the lockstep kernel: one source, one 4-CTA cluster
-        const int nb = g->w ? (int)wmax + 1 : 2;
+    {
+        // weighted distances from the lockstep kernel: one source, one 4-CTA cluster
+        const int nb = (int)wmax + 1;
         SlotWs ws;
         CK_RC(alloc_slots(c, ws, 1, n, nb, false, 0, 1, entry_factor(c, g->w != nullptr, 1)));
         LsArena A{};
@@ -784,12 +761,6 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
         beg += cntL;
     }
     CK_CUDA(cudaGetLastError());
-    // buffers of the per-call sort of S
-    CK_ALLOC(w.keys.alloc(c, ns)); CK_ALLOC(w.kb.alloc(c, ns));
-    CK_ALLOC(w.vals.alloc(c, ns)); CK_ALLOC(w.vb.alloc(c, ns));
-    CK_ALLOC(w.hist.alloc(c, radix_hist_elems(ns)));
-    CK_ALLOC(w.tmp.alloc(c, scan_tmp_elems(radix_hist_elems(ns))));
-    CK_ALLOC(w.out.alloc(c, ns));
     CK_CUDA(cudaStreamSynchronize(c->stream));   // the local buffers above go back to the pool
     return BCPP_OK;
 }
@@ -797,10 +768,22 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
 int order_emit(bcpp_ctx* c, OrderWs& w, bool) {
     const int64_t ns = w.ns;
     const unsigned blocks = (unsigned)std::min<int64_t>((ns + 255) / 256, 8192);
-    level_keys_kernel<<<blocks, 256, 0, c->stream>>>(w.S, ns, w.pos.p, w.keys.p, w.vals.p);
-    radix_sort_pairs(w.keys.p, w.vals.p, w.kb.p, w.vb.p, ns, bits_for((uint64_t)std::max(w.n, 1)), w.hist.p, w.tmp.p,
-                     c->stream, c->launches);
-    c->launches++;
+    if (w.pos.p) {
+        level_keys_kernel<<<blocks, 256, 0, c->stream>>>(w.S, ns, w.pos.p, w.keys.p, w.vals.p);
+        radix_sort_pairs(w.keys.p, w.vals.p, w.kb.p, w.vb.p, ns, bits_for((uint64_t)std::max(w.n, 1)), w.hist.p, w.tmp.p,
+                         c->stream, c->launches);
+        c->launches++;
+    } else if (w.mem.p) {
+        CK_CUDA(cudaMemsetAsync(w.mem.p, 0, (size_t)w.n, c->stream));
+        order_member(w.S, ns, w.queue.p, w.n, w.mem.p, w.flag.p, c->stream);
+        exclusive_scan<int32_t>(w.flag.p, w.place.p, w.n, nullptr, w.tmp.p, c->stream, c->launches);
+        order_compact(w.queue.p, w.flag.p, w.place.p, w.n, w.vals.p, c->stream);
+        c->launches += 3;
+    } else if (w.part) {
+        CK_CUDA(cudaMemcpyAsync(w.vals.p, w.queue.p, ns * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream));
+    } else {
+        return BCPP_OK;   // S = V: order_prepare wrote the order itself
+    }
     if (w.part) {
         part_keys_kernel<<<blocks, 256, 0, c->stream>>>(w.vals.p, ns, w.part, w.keys.p);
         radix_sort_pairs(w.keys.p, w.vals.p, w.kb.p, w.vb.p, ns, bits_for((uint64_t)w.k), w.hist.p, w.tmp.p,

@@ -32,6 +32,7 @@
 // cycles, FP64 pipe busy 33%) and, in the backward pass, by FP64 adds (pipe busy 63% of it).
 #include <algorithm>
 
+#include "gridbar.cuh"
 #include "levels.cuh"
 
 namespace bcpp {
@@ -51,9 +52,8 @@ constexpr int LM_PAIRS = WEIGHTED ? 4 : 3;
 template <bool WEIGHTED>
 constexpr int LM_GATHERS = WEIGHTED ? 3 : 2;
 constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of larger degree go one by one)
-constexpr int CTL_BAR = 0, CTL_GEN = 1, CTL_ABORT = 2, CTL_LVL = 8;
+constexpr int CTL_LVL = CTL_WORDS;
 constexpr unsigned LVL_ANY = 1u, LVL_ERR = 2u;
-constexpr unsigned LM_SPIN_MAX = 1u << 28;   // polls of the grid barrier before it gives up
 
 // 1/x for small path counts, correctly rounded by the compiler
 constexpr int RCP_N = 1024;
@@ -83,36 +83,6 @@ struct WarpSm {
     double ds[32];             // dependencies, by row of the tile
     int idx[32];               // compaction scratch
 };
-
-// Barrier over all blocks of the cooperative launch.  false: gave up (never with co-resident blocks).
-__device__ bool grid_barrier(uint32_t* ctl, uint32_t* flags) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile uint32_t* gen = ctl + CTL_GEN;
-        volatile uint32_t* ab = ctl + CTL_ABORT;
-        const uint32_t g = *gen;
-        __threadfence();
-        if (atomicAdd(ctl + CTL_BAR, 1u) == gridDim.x - 1) {
-            ctl[CTL_BAR] = 0u;
-            __threadfence();
-            atomicAdd(ctl + CTL_GEN, 1u);
-        } else {
-            unsigned polls = 0;
-            while (*gen == g && *ab == 0u) {
-                __nanosleep(20);
-                if (++polls == LM_SPIN_MAX) {
-                    atomicOr(&flags[FLAG_TIMEOUT], 1u);
-                    atomicExch(ctl + CTL_ABORT, 1u);
-                }
-            }
-        }
-        s_ok = *ab == 0u;
-        __threadfence();
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
 
 // position of the n-th set bit (from 0) of x; n < popc(x)
 __device__ __forceinline__ int nth_bit(uint32_t x, int n) {
