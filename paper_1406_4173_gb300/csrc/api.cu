@@ -811,11 +811,12 @@ struct LmWs {
     std::vector<LmWave> waves;
     int lcap = 0;
     bool narrow = true;
+    bool fp32 = false;         // FP32 dependencies
     int32_t tpb = 0;           // uniform layout: tiles per batch
     int64_t nodes = 0;         // global nodes
     DBuf<uint32_t> lev, seen, ctl;
-    DBuf<char> sg;
-    DBuf<double> cc, dsum, bcs, bcc;
+    DBuf<char> sg, cc;
+    DBuf<double> dsum, bcs, bcc;
     DBuf<int32_t> tile0, tile_item;
     DBuf<LmRun> runs;
 };
@@ -833,13 +834,14 @@ int64_t free_bytes(bcpp_ctx* c) {
     return (int64_t)((double)((int64_t)fr + reusable) * 0.80);
 }
 
-// Calls the level-mask kernel serves: FP64 dependencies, batches of 32 sources, weights up to
-// LM_MAX_WEIGHT, 32-bit arc offsets.  (FP32 dependencies keep the lockstep kernel: their sums would be
-// taken in another order, and FP32 sums in another order differ in the 8th digit.)  A call whose
-// batches prove too deep, or whose path counts outgrow 32 bits, reruns with order_factor 64, which
-// the lockstep kernel serves.
-bool lm_serves(const bcpp_ctx* c, const bcpp_opts& o, int spl, int32_t n, int64_t arcs, uint64_t wmax) {
-    return o.precision != BCPP_FP32_DELTA && spl == 1 && c->order_factor < 64 && arcs < (1ll << 31) &&
+// Calls the level-mask kernel serves: batches of 32 sources, weights up to LM_MAX_WEIGHT, 32-bit arc offsets, FP64
+// dependencies, or FP32 ones on unit weights without a skeleton (fp32_too; there it adds in the lockstep
+// kernel's order, since FP32 sums in another order differ in the 8th digit).  A call whose batches prove too
+// deep, or whose path counts outgrow 32 bits, reruns with order_factor 64, which the lockstep kernel
+// serves.
+bool lm_serves(const bcpp_ctx* c, const bcpp_opts& o, int spl, int32_t n, int64_t arcs, uint64_t wmax,
+               bool fp32_too = false) {
+    return (o.precision != BCPP_FP32_DELTA || (fp32_too && wmax == 1)) && spl == 1 && c->order_factor < 64 && arcs < (1ll << 31) &&
            n < (1 << 25) && wmax <= LM_MAX_WEIGHT;
 }
 
@@ -863,7 +865,7 @@ int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_gr
     L.lcap = lcap;
     L.narrow = narrow;
     L.nodes = nodes;
-    const int64_t row_bytes = 32 * ((narrow ? 4 : 8) + (forward ? 0 : 8)) + 8 + 4 + 4ll * lcap;
+    const int64_t row_bytes = 32 * ((narrow ? 4 : 8) + (forward ? 0 : L.fp32 ? 4 : 8)) + 8 + 4 + 4ll * lcap;
     const int64_t budget = free_bytes(c);
     int64_t total = 0, largest = 0;
     std::vector<int32_t> tile0;
@@ -915,7 +917,7 @@ int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_gr
     CK_ALLOC(L.dsum.alloc(c, rows));
     CK_ALLOC(L.ctl.alloc(c, lm_ctl_words(lcap, most_items)));
     if (!forward) {
-        CK_ALLOC(L.cc.alloc(c, rows * 32));
+        CK_ALLOC(L.cc.alloc(c, rows * 32 * (L.fp32 ? 4 : 8)));
         CK_ALLOC(L.bcs.alloc(c, nodes));
         CK_ALLOC(L.bcc.alloc(c, nodes));
         CK_ALLOC(L.runs.alloc(c, (int64_t)runs.size()));
@@ -974,7 +976,7 @@ int lm_emit(bcpp_ctx* c, LmWs& L, const LsArena& A, const LsParams& P, const LsI
     for (const LmWave& w : L.waves) {
         const LmArgs a = lm_wave_args(L, w, A, P, items, wmax);
         CK_CUDA(cudaMemsetAsync(L.ctl.p, 0, (size_t)lm_ctl_words(L.lcap, a.nitems) * sizeof(uint32_t), c->stream));
-        CK_CUDA(lm_launch(a, L.narrow, c->num_sms, c->stream));
+        CK_CUDA(lm_launch(a, L.narrow, L.fp32, c->num_sms, c->stream));
         lm_accumulate(a, L.runs.p + w.run0, w.nruns, w.natiles, L.bcs.p, L.bcc.p, c->stream);
         c->launches += 2;
     }
@@ -1088,14 +1090,15 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     shard_sources(o, r.ns, s0, s1);
     r.spl = choose_spl(c, s1 - s0, o);
     std::vector<LsItem> hitems = make_items(0, s0, s1, 32 * r.spl);
-    if (lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1))
+    r.cl = r.spl == 1 ? choose_cluster(c, (int)hitems.size(), o) : 1;
+    const int width = r.spl == 1 ? balanced_width(s1 - s0, slot_capacity(c, o, r.cl), 32) : 32;
+    // (FP32 dependencies: the batches of the lockstep kernel, whose order of additions depends on them)
+    if (fp32 && width < 32) hitems = make_items(0, s0, s1, width);
+    r.lm.fp32 = fp32;
+    if (lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
                        lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
-    r.cl = r.spl == 1 ? choose_cluster(c, (int)hitems.size(), o) : 1;
-    if (r.spl == 1 && !r.levels) {
-        const int b = balanced_width(s1 - s0, slot_capacity(c, o, r.cl), 32);
-        if (b < 32) hitems = make_items(0, s0, s1, b);
-    }
+    if (!r.levels && width < 32) hitems = make_items(0, s0, s1, width);
     r.nitems = (int)hitems.size();
     if (r.nitems <= 0) return BCPP_OK;
     CK_ALLOC(r.items.alloc(c, r.nitems));
@@ -1566,7 +1569,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         a.srcs = r.tsk.p;
         a.in_s = r.sk_in_s.p;
         a.bc_map = K.sknode.p;
-        a.lev = r.lm.lev.p; a.seen = r.lm.seen.p; a.sg = W.sg; a.cc = static_cast<double*>(W.dl);
+        a.lev = r.lm.lev.p; a.seen = r.lm.seen.p; a.sg = W.sg; a.cc = W.dl;
         a.dsum = r.lm.dsum.p; a.drow = W.d;
         a.rows = (int64_t)a.ntiles * 32;
         a.lcap = r.lm.lcap;
@@ -1576,7 +1579,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         a.phase_ns = c->phase;
         if (tbr) tbr->start();
         CK_CUDA(cudaMemsetAsync(a.ctl, 0, (size_t)lm_ctl_words(a.lcap, cn) * sizeof(uint32_t), c->stream));
-        CK_CUDA(lm_launch(a, false, c->num_sms, c->stream));
+        CK_CUDA(lm_launch(a, false, false, c->num_sms, c->stream));
         lm_scatter(a, K.N, W.bc_sum, W.bc_cmp, W.cap_bc, c->stream);
         c->launches += 2;
         if (tbr) tbr->stop();
@@ -2231,7 +2234,8 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
     const int nb = g->w ? (int)wmax + 1 : 2;
     bool levels = false;
     LmWs lm;
-    if (lm_serves(c, o, spl, (int32_t)maxn, g->num_arcs, g->w ? wmax : 1))
+    lm.fp32 = fp32;
+    if (lm_serves(c, o, spl, (int32_t)maxn, g->num_arcs, g->w ? wmax : 1, !g->w))
         CK_RC(lm_alloc(c, lm, hitems, false, [&](int32_t gi) { return off[gi + 1] - off[gi]; }, n,
                        lm_levels(g->w != nullptr, false, nullptr), true, &levels));
     LsArena A{};
@@ -2358,7 +2362,7 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
         a.ctl = ctl.p;
         a.flags = c->flags;
         CK_CUDA(cudaMemsetAsync(ctl.p, 0, (size_t)lm_ctl_words(lcap, cn) * sizeof(uint32_t), c->stream));
-        CK_CUDA(lm_launch(a, false, c->num_sms, c->stream));
+        CK_CUDA(lm_launch(a, false, false, c->num_sms, c->stream));
         lm_paths_out(a, g->n, dist_out, sigma_out, c->stream);
         c->launches += 2;
     }

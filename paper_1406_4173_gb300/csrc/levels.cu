@@ -31,6 +31,7 @@
 // Bound by the latency of its gathers (a profile at n = 10,000: instructions issued on 27% of the
 // cycles, FP64 pipe busy 33%) and, in the backward pass, by FP64 adds (pipe busy 63% of it).
 #include <algorithm>
+#include <type_traits>
 
 #include "gridbar.cuh"
 #include "levels.cuh"
@@ -73,7 +74,45 @@ __device__ __forceinline__ double recip_of(uint64_t s) {
     return fma(r, fma(-x, r, 1.0), r);
 }
 
-template <bool MULT>
+template <typename DT>
+__device__ __forceinline__ DT recip_as(uint64_t s) {
+    if constexpr (sizeof(DT) == 4) return 1.0f / (float)s;
+    else return recip_of(s);
+}
+
+// FP32 sums are taken in the lockstep kernel's order, so that both give the same bits: with a sources at the
+// row's distance and K = 32 / (a rounded up to a power of two), arc j of the row goes to partial sum j mod K, in
+// order, and the partial sums are added pairwise (neighbours first).  Terms come as (arc, value); eight
+// partial sums are held at a time.
+struct TreeSum {
+    float (*p)[32];   // [8][lane], in shared memory: few terms, and a register array would cost eight selects each
+    int lane;
+    float a, b;
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int z = 0; z < 8; z++) p[z][lane] = 0.0f;
+    }
+    __device__ __forceinline__ void add(int arc, int K, int part, float t) {
+        const int z = arc & (K - 1);
+        if (t != 0.0f && (z >> 3) == part) p[z & 7][lane] += t;
+    }
+    // after the terms of partial sums 8 part .. 8 part + 7
+    __device__ __forceinline__ void close(int part) {
+        const float t = ((p[0][lane] + p[1][lane]) + (p[2][lane] + p[3][lane])) +
+                        ((p[4][lane] + p[5][lane]) + (p[6][lane] + p[7][lane]));
+        if (part == 0) a = t;
+        else if (part == 1) a = a + t;
+        else if (part == 2) b = t;
+        else b = b + t;
+    }
+    __device__ __forceinline__ float total(int K) const { return K > 16 ? a + b : a; }
+};
+__device__ __forceinline__ int partial_sums(uint32_t at_distance) {
+    const int a = __popc(at_distance);
+    return 32 >> (a <= 1 ? 0 : 32 - __clz(a - 1));
+}
+
+template <bool MULT, bool TREE = false>
 struct WarpSm {
     uint2 list[LM_CAP];        // arcs with a bit in common: head row, mask
     uint64_t mult[MULT ? LM_CAP : 1];   // their multiplicities (uint64 forward, double backward)
@@ -82,6 +121,7 @@ struct WarpSm {
     uint32_t rowm[32];         // masks found, by row of the tile
     double ds[32];             // dependencies, by row of the tile
     int idx[32];               // compaction scratch
+    float part[TREE ? 8 : 1][32];   // TreeSum
 };
 
 // position of the n-th set bit (from 0) of x; n < popc(x)
@@ -153,12 +193,13 @@ __device__ __forceinline__ void for_pairs(uint32_t mask, int lane, int* idx, F&&
 //   ovf: a 64-bit count wrapped
 // TABLE (Dijkstra_SK): a frontier other than the source (nodes below nf, distance above 0) takes part in the
 // distances but not in the counts, so its arcs add to the found masks only.
-template <bool FWD, bool WEIGHTED, bool MULT, bool TABLE, typename V, typename ACC, class PD, class RD>
-__device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int lane, uint32_t need, int64_t a0, int deg,
+template <bool FWD, bool WEIGHTED, bool MULT, bool TABLE, typename V, typename ACC, class SM, class PD, class RD>
+__device__ __forceinline__ void tile_sums(const LmArgs& A, SM& sm, int lane, uint32_t need, int64_t a0, int deg,
                                           int D, int bd, int64_t rb, const int32_t* __restrict__ col,
                                           const int32_t* __restrict__ wt, const V* vals, int32_t nf, bool& ovf,
                                           PD&& pair_done,
                                           RD&& row_done) {
+    constexpr bool TREE = std::is_same<V, float>::value;
     constexpr int PU = LM_PAIRS<WEIGHTED>, GU = LM_GATHERS<WEIGHTED>;
     // A row of many arcs: with unit weights many of a chunk's arcs have a bit in common, and each source takes
     // its own of them; with weights few have, and the warp takes them one after the other.
@@ -223,6 +264,10 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
             const int r = __shfl_sync(FULL, crow, k0);
             ACC acc = (ACC)0;
             uint32_t found = 0u;
+            TreeSum tree{sm.part, lane, 0.0f, 0.0f};
+            const int parts = TREE ? partial_sums(nd) : 1;
+            for (int part = 0; part < (TREE ? (parts + 7) / 8 : 1); part++) {
+            if (TREE && parts > 1) tree.clear();
             for (int c0 = 0; c0 < dg; c0 += 32) {
                 int32_t v = 0;
                 uint32_t m = 0u;
@@ -239,9 +284,11 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                 while (__any_sync(FULL, own != 0u)) {
                     V t[BU];
                     uint64_t muq[BU];
+                    int jq[BU];
 #pragma unroll
                     for (int q = 0; q < BU; q++) {
                         const int j = own ? __ffs(own) - 1 : 0;
+                        jq[q] = j;
                         const int32_t vq = __shfl_sync(FULL, v, j);
                         muq[q] = MULT ? shfl_u64(mu, j) : 0;
                         uint32_t mq = 0xffffffffu;
@@ -252,9 +299,13 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                     }
 #pragma unroll
                     for (int q = 0; q < BU; q++)
-                        if (q == 0 || FWD || __any_sync(FULL, t[q] != (V)0)) add(acc, t[q], muq[q]);
+                        if (TREE && parts > 1) tree.add(jq[q], parts, part, t[q]);
+                        else if (q == 0 || FWD || __any_sync(FULL, t[q] != (V)0)) add(acc, t[q], muq[q]);
                 }
             }
+            if (TREE && parts > 1) tree.close(part);
+            }
+            if (TREE && parts > 1) acc = tree.total(parts);
             found = __reduce_or_sync(FULL, found);
             if (found) {
                 if (lane == 0) sm.rowm[r] = found;
@@ -274,7 +325,7 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
             unsigned first[GU];
             int k[GU];
             uint32_t a[GU], m[GU];
-            int32_t v[GU], w[GU];
+            int32_t v[GU], w[GU], stk[GU];
 #pragma unroll
             for (int g = 0; g < GU; g++) {
                 const unsigned at = (unsigned)(st - i0 - 32 * g);
@@ -283,6 +334,7 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                 kb += __popc(first[g]);
                 a[g] = __shfl_sync(FULL, ca0 - (uint32_t)st, k[g]) + (uint32_t)(i0 + 32 * g + lane);
                 m[g] = __shfl_sync(FULL, cneed, k[g]);
+                stk[g] = TREE ? __shfl_sync(FULL, st, k[g]) : 0;
                 v[g] = 0;
                 w[g] = 1;
                 if (i0 + 32 * g + lane < T) {
@@ -306,7 +358,9 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                 const unsigned tb = __ballot_sync(FULL, m[g] != 0u);
                 const int p = pos + __popc(tb & lt);
                 if (m[g]) {
-                    sm.list[p] = make_uint2((uint32_t)v[g], m[g]);
+                    // (FP32: the arc's place in its row, mod 32, above the head's 25 bits)
+                    const uint32_t at = TREE ? (uint32_t)(i0 + 32 * g + lane - stk[g]) << 27 : 0u;
+                    sm.list[p] = make_uint2((uint32_t)v[g] | at, m[g]);
                     if constexpr (MULT) sm.mult[p] = mult_of(a[g]);
                     atomicOr(&sm.nm[k[g]], m[g]);
                 }
@@ -325,6 +379,28 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
             const int r = __shfl_sync(FULL, crow, k[0]);
             const V* vs = vals + rb * 32 + s[0];
             ACC acc = (ACC)0;
+            if constexpr (TREE) {
+                const int parts = partial_sums(__shfl_sync(FULL, cneed, k[0]));
+                TreeSum tree{sm.part, lane, 0.0f, 0.0f};
+                for (int part = 0; parts > 1 && part < (parts + 7) / 8; part++) {
+                    tree.clear();
+                    for (int i = e; i < e1; i += PU) {
+                        V t[PU];
+                        uint2 x[PU];
+#pragma unroll
+                        for (int q = 0; q < PU; q++) {
+                            t[q] = (V)0;
+                            x[q] = i + q < e1 ? sm.list[i + q] : make_uint2(0u, 0u);
+                            if ((x[q].y >> s[0]) & 1u) t[q] = vs[(int64_t)(x[q].x & 0x1ffffffu) * 32];
+                        }
+#pragma unroll
+                        for (int q = 0; q < PU; q++) tree.add((int)(x[q].x >> 27), parts, part, t[q]);
+                    }
+                    tree.close(part);
+                }
+                if (parts > 1) acc = tree.total(parts);   // (one partial sum: in order, below)
+                if (parts > 1) e = e1;
+            }
             while (e < e1) {
                 V t[PU];
 #pragma unroll
@@ -332,7 +408,7 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
                     t[q] = (V)0;
                     if (e + q < e1) {
                         const uint2 x = sm.list[e + q];
-                        if ((x.y >> s[0]) & 1u) t[q] = vs[(int64_t)x.x * 32];
+                        if ((x.y >> s[0]) & 1u) t[q] = vs[(int64_t)(TREE ? x.x & 0x1ffffffu : x.x) * 32];
                     }
                 }
 #pragma unroll
@@ -347,15 +423,16 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, WarpSm<MULT>& sm, int
     }
 }
 
-template <typename SG, bool WEIGHTED, bool MULT, bool TABLE>
+template <typename SG, typename DT, bool WEIGHTED, bool MULT, bool TABLE>
 __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm_kernel(const LmArgs A) {
-    __shared__ WarpSm<MULT> s_warp[LM_WARPS];
+    using Sm = WarpSm<MULT, std::is_same<DT, float>::value>;
+    __shared__ Sm s_warp[LM_WARPS];
     const int lane = threadIdx.x & 31;
-    WarpSm<MULT>& sm = s_warp[threadIdx.x >> 5];
+    Sm& sm = s_warp[threadIdx.x >> 5];
     const int wid = blockIdx.x * LM_WARPS + (threadIdx.x >> 5);
     const int nw = gridDim.x * LM_WARPS;
     SG* sg = static_cast<SG*>(A.sg);
-    double* cc = A.cc;
+    DT* cc = static_cast<DT*>(A.cc);
     uint32_t* lvl = A.ctl + CTL_LVL;
     uint32_t* bdepth = lvl + A.lcap + 1;
     const int wmax = WEIGHTED ? A.wmax : 1;
@@ -416,7 +493,7 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
         sm.rowm[lane] = 0u;
         if (sizeof(SG) == 8 && A.drow) {
             int4* dr = reinterpret_cast<int4*>(A.drow + (int64_t)t * 1024);
-            double2* cr = reinterpret_cast<double2*>(cc + (int64_t)t * 1024);
+            double2* cr = reinterpret_cast<double2*>(cc + (int64_t)t * 1024);   // (64-bit counts come with FP64 only)
 #pragma unroll 4
             for (int i = lane; i < 256; i += 32) dr[i] = make_int4(DINF, DINF, DINF, DINF);
             if (cc)
@@ -556,16 +633,16 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
             sm.ds[lane] = 0.0;
             __syncwarp();
             const SG* srow = sg + (int64_t)t * 1024;
-            double* crow = cc + (int64_t)t * 1024;
+            DT* crow = cc + (int64_t)t * 1024;
             bool no_ovf = false;
-            tile_sums<false, WEIGHTED, MULT, false, double, double>(
+            tile_sums<false, WEIGHTED, MULT, false, DT, DT>(
                 A, sm, lane, need, a0, deg, D, bd, x.rb, A.col, A.w, cc, 0, no_ovf,
-                [&](bool ok, int r, int s, double acc, unsigned first) {
+                [&](bool ok, int r, int s, DT acc, unsigned first) {
                     double delta = 0.0;
                     if (ok) {
                         const SG sv = srow[r * 32 + s];
-                        delta = (double)sv * acc;
-                        crow[r * 32 + s] = (tm >> r) & 1u ? acc + recip_of(sv) : acc;
+                        delta = (double)((DT)sv * acc);
+                        crow[r * 32 + s] = (tm >> r) & 1u ? acc + recip_as<DT>(sv) : acc;
                     }
                     // sum of each row's run of lanes, then one lane per row adds it
                     const unsigned up = lane < 31 ? first >> (lane + 1) : 0u;
@@ -580,12 +657,12 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
                     if (ok && (lane == 0 || (first >> lane) & 1u)) sm.ds[r] += delta;
                     __syncwarp();
                 },
-                [&](int r, uint32_t mask, double acc) {
+                [&](int r, uint32_t mask, DT acc) {
                     double delta = 0.0;
                     if ((mask >> lane) & 1u) {
                         const SG sv = srow[r * 32 + lane];
-                        delta = (double)sv * acc;
-                        crow[r * 32 + lane] = (tm >> r) & 1u ? acc + recip_of(sv) : acc;
+                        delta = (double)((DT)sv * acc);
+                        crow[r * 32 + lane] = (tm >> r) & 1u ? acc + recip_as<DT>(sv) : acc;
                     }
                     delta = warp_sum(delta);
                     if (lane == 0) sm.ds[r] += delta;
@@ -600,7 +677,7 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
                 for (int g = 0; g < 2; g++) v[g] = ok[g] ? srow[r[g] * 32 + s[g]] : (SG)1;
 #pragma unroll
                 for (int g = 0; g < 2; g++)
-                    if (ok[g]) crow[r[g] * 32 + s[g]] = recip_of(v[g]);
+                    if (ok[g]) crow[r[g] * 32 + s[g]] = recip_as<DT>(v[g]);
             });
             if ((inner | leaf) != need) *lrow = inner | leaf;
             const double ds = sm.ds[lane];
@@ -708,16 +785,16 @@ __global__ void lm_tile_items_kernel(const int32_t* __restrict__ item_tile0, int
     }
 }
 
-template <typename SG, bool WEIGHTED, bool MULT = false, bool TABLE = false>
+template <typename SG, bool WEIGHTED, bool MULT = false, bool TABLE = false, typename DT = double>
 cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, WEIGHTED, MULT, TABLE>, LM_THREADS, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, DT, WEIGHTED, MULT, TABLE>, LM_THREADS, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
     const int blocks = std::min(per_sm * num_sms, std::max(1, (A.ntiles + LM_WARPS - 1) / LM_WARPS));
     LmArgs a = A;
     void* args[] = {&a};
-    return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, WEIGHTED, MULT, TABLE>, dim3(blocks), dim3(LM_THREADS), args, 0,
+    return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, DT, WEIGHTED, MULT, TABLE>, dim3(blocks), dim3(LM_THREADS), args, 0,
                                        st);
 }
 
@@ -725,9 +802,13 @@ cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
 
 int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + nitems + 2 * (int64_t)lcap; }
 
-cudaError_t lm_launch(const LmArgs& A, bool narrow, int num_sms, cudaStream_t st) {
+cudaError_t lm_launch(const LmArgs& A, bool narrow, bool fp32, int num_sms, cudaStream_t st) {
     if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;
     const bool weighted = A.w != nullptr;
+    if (fp32) {
+        if (!narrow || weighted || A.mud) return cudaErrorInvalidValue;
+        return lm_go<uint32_t, false, false, false, float>(A, num_sms, st);
+    }
     if (narrow) return weighted ? lm_go<uint32_t, true>(A, num_sms, st) : lm_go<uint32_t, false>(A, num_sms, st);
     if (A.mud) return weighted ? lm_go<uint64_t, true, true>(A, num_sms, st) : cudaErrorInvalidValue;
     return weighted ? lm_go<uint64_t, true>(A, num_sms, st) : lm_go<uint64_t, false>(A, num_sms, st);

@@ -36,7 +36,7 @@ struct LmArgs {
     uint32_t* lev;              // [lcap][rows]: sources that reach the row's node at that distance
     uint32_t* seen;             // [rows]: sources that reached it so far
     void* sg;                   // [rows][32] path counts (32- or 64-bit)
-    double* cc;                 // [rows][32] (I + delta) / sigma; nullptr: forward pass only
+    void* cc;                   // [rows][32] (I + delta) / sigma, double or float; nullptr: forward pass only
     int32_t* drow;              // [rows][32] distances (DINF = unreached), or nullptr; with it cc is zero
                                 // wherever it is not written
     double* dsum;               // [rows] dependencies summed over the batch's sources
@@ -56,8 +56,8 @@ struct LmArgs {
 int64_t lm_ctl_words(int lcap, int nitems);
 
 // Forward and backward pass of every batch of the wave; one cooperative launch.  narrow: 32-bit path
-// counts (a count of 2^32 or more aborts like a late level).
-cudaError_t lm_launch(const LmArgs& A, bool narrow, int num_sms, cudaStream_t st);
+// counts (a count of 2^32 or more aborts like a late level).  fp32: FP32 dependencies (unit weights, narrow).
+cudaError_t lm_launch(const LmArgs& A, bool narrow, bool fp32, int num_sms, cudaStream_t st);
 
 // Dijkstra_SK (Eq. 10): forward pass of every batch (sources: frontiers aux .. aux + nsrc - 1 of graph g, cc =
 // nullptr) into the tables; 32-bit path counts as with narrow.
