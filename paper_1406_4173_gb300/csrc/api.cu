@@ -812,6 +812,7 @@ struct LmWs {
     int lcap = 0;
     bool narrow = true;
     bool fp32 = false;         // FP32 dependencies
+    double mean_degree = 16;   // arcs per node
     int32_t tpb = 0;           // uniform layout: tiles per batch
     int64_t nodes = 0;         // global nodes
     DBuf<uint32_t> lev, seen, ctl;
@@ -961,6 +962,7 @@ LmArgs lm_wave_args(const LmWs& L, const LmWave& w, const LsArena& A, const LsPa
     a.rows = (int64_t)w.ntiles * 32;
     a.lcap = L.lcap;
     a.wmax = (int32_t)wmax;
+    a.mean_degree = L.mean_degree;
     a.ctl = L.ctl.p;
     a.flags = P.flags;
     a.phase_ns = P.phase_ns;
@@ -1095,6 +1097,7 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     // (FP32 dependencies: the batches of the lockstep kernel, whose order of additions depends on them)
     if (fp32 && width < 32) hitems = make_items(0, s0, s1, width);
     r.lm.fp32 = fp32;
+    r.lm.mean_degree = (double)g->num_arcs / n;
     if (lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
                        lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
@@ -1574,6 +1577,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         a.rows = (int64_t)a.ntiles * 32;
         a.lcap = r.lm.lcap;
         a.wmax = (int32_t)K.wmax_sk;
+        a.mean_degree = r.lm.mean_degree;
         a.ctl = r.lm.ctl.p;
         a.flags = c->flags;
         a.phase_ns = c->phase;
@@ -1639,6 +1643,7 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
     r.spl = r.hunits.empty() ? choose_spl(c, s1 - s0, o) : 1;
     std::vector<LsItem> hitems = make_items(0, s0, s1, 32 * r.spl);
     if (N > 0 && !hitems.empty() && lm_serves(c, o, r.spl, N, K.arcs, K.wmax_sk)) {
+        r.lm.mean_degree = (double)K.arcs / N;
         // skeleton distances are the distances in G
         const int lcap = lm_levels(g->w != nullptr, g->directed != 0, o.order_sources && ns > 2 * LS_LANES ? &r.ord : nullptr);
         if (r.hunits.empty())
@@ -2235,6 +2240,7 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
     bool levels = false;
     LmWs lm;
     lm.fp32 = fp32;
+    lm.mean_degree = (double)g->num_arcs / n;
     if (lm_serves(c, o, spl, (int32_t)maxn, g->num_arcs, g->w ? wmax : 1, !g->w))
         CK_RC(lm_alloc(c, lm, hitems, false, [&](int32_t gi) { return off[gi + 1] - off[gi]; }, n,
                        lm_levels(g->w != nullptr, false, nullptr), true, &levels));
@@ -2359,6 +2365,7 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
         a.rows = (int64_t)a.ntiles * 32;
         a.lcap = lcap;
         a.wmax = (int32_t)wmax;
+        a.mean_degree = (double)g->num_arcs / g->n;
         a.ctl = ctl.p;
         a.flags = c->flags;
         CK_CUDA(cudaMemsetAsync(ctl.p, 0, (size_t)lm_ctl_words(lcap, cn) * sizeof(uint32_t), c->stream));

@@ -52,8 +52,13 @@ template <bool WEIGHTED>
 constexpr int LM_PAIRS = WEIGHTED ? 4 : 3;
 template <bool WEIGHTED>
 constexpr int LM_GATHERS = WEIGHTED ? 3 : 2;
+constexpr int LM_MAX_SUB = 3;      // units of 4 rows at least
 constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of larger degree go one by one)
 constexpr int CTL_LVL = CTL_WORDS;
+// Words between two batches' depths: a 128-byte line each, since every SM stores to them once per level (side by
+// side, stores of 152 SMs to a few lines held up everyone's loads: n = 10,000, every node a target 7.4 -> 6.3 ms,
+// Brandes++ at n = 100,000 8.6 -> 7.8 ms).
+constexpr int DEPTH_STRIDE = 32;
 constexpr unsigned LVL_ANY = 1u, LVL_ERR = 2u;
 
 // 1/x for small path counts, correctly rounded by the compiler
@@ -424,7 +429,8 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, SM& sm, int lane, uin
 }
 
 template <typename SG, typename DT, bool WEIGHTED, bool MULT, bool TABLE>
-__global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm_kernel(const LmArgs A) {
+__global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4))
+lm_kernel(const LmArgs A, const int sub_log) {
     using Sm = WarpSm<MULT, std::is_same<DT, float>::value>;
     __shared__ Sm s_warp[LM_WARPS];
     const int lane = threadIdx.x & 31;
@@ -464,22 +470,25 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
         return x;
     };
 
-    // Tiles go out in order: the first of every warp by its index, the others from one counter per
+    // With few tiles per warp a unit is a part of a tile (32 >> sub_log rows), so that a level's last and
+    // fullest tiles do not leave the other warps waiting (see lm_go for the rule).
+    // Units go out in order: the first of every warp by its index, the others from one counter per
     // pass and level, a few at a time (a fixed assignment of all of them left warps waiting for the
     // rows of high degree: 245 -> 164 ms on 1,000,000 nodes and 4,096 sources).
-    uint32_t* work = bdepth + A.nitems;
-    const int grab = max(1, min(8, A.ntiles / (16 * nw)));
-    auto for_tiles = [&](uint32_t* ctr, auto&& f) {
-        const bool more = A.ntiles > nw;
+    uint32_t* work = bdepth + (int64_t)A.nitems * DEPTH_STRIDE;
+    const int nunits = A.ntiles << sub_log;
+    const int grab = max(1, min(8, nunits / (16 * nw)));
+    auto for_units = [&](uint32_t* ctr, auto&& f) {
+        const bool more = nunits > nw;
         int mine = 0;
         if (more && lane == 0) mine = nw + (int)atomicAdd(ctr, (uint32_t)grab);
-        if (wid < A.ntiles) f(wid);
+        if (wid < nunits) f(wid);
         if (!more) return;
         for (;;) {
             const int t0 = __shfl_sync(FULL, mine, 0);
-            if (t0 >= A.ntiles) break;
+            if (t0 >= nunits) break;
             if (lane == 0) mine = nw + (int)atomicAdd(ctr, (uint32_t)grab);   // the next ones, while these run
-            const int t1 = min(t0 + grab, A.ntiles);
+            const int t1 = min(t0 + grab, nunits);
             for (int t = t0; t < t1; t++) f(t);
         }
     };
@@ -532,18 +541,20 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
             return;
         }
         bool any = false, wide = false, ovf = false;
-        for_tiles(work + D, [&](int t) {
+        for_units(work + D, [&](int unit) {
+            const int t = unit >> sub_log;
+            const bool mine = lane >> (5 - sub_log) == (unit & ((1 << sub_log) - 1));
             const Tile x = tile_of(t);
             // finished batches: nothing new within the largest weight.  (A cached load: the values of
             // earlier levels decide, and this SM's own store below shows up in it.)
-            const int bd = (int)bdepth[x.it];
+            const int bd = (int)bdepth[x.it * DEPTH_STRIDE];
             if (bd + wmax < D) return;
             const int64_t row = (int64_t)t * 32 + lane;
             const uint32_t full = x.I.nsrc >= 32 ? 0xffffffffu : (1u << x.I.nsrc) - 1u;
             uint32_t seen = 0u, need = 0u;
             int64_t a0 = 0;
             int deg = 0;
-            if (x.u < x.n) {
+            if (mine && x.u < x.n) {
                 seen = A.seen[row];
                 need = full & ~seen;
                 if (need) {
@@ -575,11 +586,11 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
                 [&](int r, uint32_t mask, uint64_t acc) { settle((mask >> lane) & 1u, r, lane, acc); });
             __syncwarp();
             const uint32_t got = sm.rowm[lane];
-            A.lev[(int64_t)D * A.rows + row] = got;
+            if (mine) A.lev[(int64_t)D * A.rows + row] = got;
             if (got) A.seen[row] = seen | got;
             if (__any_sync(FULL, got != 0u)) {
                 any = true;
-                if (lane == 0 && bd != D) bdepth[x.it] = (uint32_t)D;
+                if (lane == 0 && bd != D) bdepth[x.it * DEPTH_STRIDE] = (uint32_t)D;
             }
             __syncwarp();
         });
@@ -609,13 +620,15 @@ __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4)) lm
     // ------------------------------------------------------------------ backward
     // (level 0 is the sources themselves: nothing is credited to them and nobody reads their c)
     for (int D = depth; D >= 1; D--) {
-        for_tiles(work + A.lcap + D, [&](int t) {
+        for_units(work + A.lcap + D, [&](int unit) {
+            const int t = unit >> sub_log;
+            const bool mine = lane >> (5 - sub_log) == (unit & ((1 << sub_log) - 1));
             const int64_t row = (int64_t)t * 32 + lane;
             const Tile x = tile_of(t);
-            const int bd = (int)bdepth[x.it];
+            const int bd = (int)bdepth[x.it * DEPTH_STRIDE];
             if (D > bd) return;
             uint32_t* lrow = A.lev + (int64_t)D * A.rows + row;
-            const uint32_t need = *lrow;
+            const uint32_t need = mine ? *lrow : 0u;
             if (!__any_sync(FULL, need != 0u)) return;
             int64_t a0 = 0;
             int deg = 0;
@@ -791,16 +804,25 @@ cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lm_kernel<SG, DT, WEIGHTED, MULT, TABLE>, LM_THREADS, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorLaunchOutOfResources;
-    const int blocks = std::min(per_sm * num_sms, std::max(1, (A.ntiles + LM_WARPS - 1) / LM_WARPS));
+    // Parts of tiles until there are enough units: up to two per warp where rows are long (30 arcs on average:
+    // 1.74 ms on whole tiles, 1.07 on halves, 0.93 on quarters, 0.87 on eighths), none where whole tiles nearly
+    // fill the GPU and rows are short (6 arcs, 0.65 tiles per warp: 0.49 ms on whole tiles, 0.56 on halves, whose
+    // units have to be fetched).
+    const double warps = (double)per_sm * num_sms * LM_WARPS;
+    const double goal = warps * std::min(2.0, std::max(0.5, A.mean_degree / 16.0));
+    int sub_log = 0;
+    while (sub_log < LM_MAX_SUB && (double)((int64_t)A.ntiles << sub_log) < goal) sub_log++;
+    const int64_t units = (int64_t)A.ntiles << sub_log;
+    const int blocks = (int)std::min<int64_t>((int64_t)per_sm * num_sms, std::max<int64_t>(1, (units + LM_WARPS - 1) / LM_WARPS));
     LmArgs a = A;
-    void* args[] = {&a};
+    void* args[] = {&a, &sub_log};
     return cudaLaunchCooperativeKernel((const void*)lm_kernel<SG, DT, WEIGHTED, MULT, TABLE>, dim3(blocks), dim3(LM_THREADS), args, 0,
                                        st);
 }
 
 }  // namespace
 
-int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + nitems + 2 * (int64_t)lcap; }
+int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + (int64_t)nitems * DEPTH_STRIDE + 2 * (int64_t)lcap; }
 
 cudaError_t lm_launch(const LmArgs& A, bool narrow, bool fp32, int num_sms, cudaStream_t st) {
     if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;

@@ -48,6 +48,7 @@ struct LmArgs {
     int64_t rows;               // 32 ntiles
     int32_t lcap;               // levels provided for
     int32_t wmax;
+    double mean_degree;         // arcs per node
     uint32_t* ctl;              // lm_ctl_words() zeroed words: barrier, level status, depth of each batch
     uint32_t* flags;
     unsigned long long* phase_ns;
