@@ -155,7 +155,8 @@ def alu_peak_ops(num_sms, sm_mhz):
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("lockstep.cu", "lockstep.cuh", "lockstep_kernel.cuh", "common.cuh"):
+    for f in ("lockstep.cu", "lockstep.cuh", "lockstep_kernel.cuh", "common.cuh", "gridbar.cuh", "levels.cu",
+              "levels.cuh", "centrality.cu"):
         with open(os.path.join(ROOT, "paper_1406_4173_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -196,11 +197,35 @@ def model_bytes_per_source_skeleton(N, A, D, B=32, delta_bytes=8, weighted=True,
     return model_bytes_per_source(N, A, D, B, delta_bytes) + extra
 
 
+def model_bytes_per_source_levels(n, A, D, B=32, sigma_bytes=4, delta_bytes=8, weighted=False, mult=False):
+    """Bytes of one source on the level-mask kernel that its method cannot do without: heads (with weights
+    and multiplicities) and 4-byte source masks of every arc and 8-byte row pointers once per pass, shared by
+    the B sources; per tight arc the parent's count (forward) and the successor's dependency (backward);
+    per node the count written and read back, the dependency written, and its mask and its batch sum, shared."""
+    arc = (4 + 4 + (4 if weighted else 0)) / B
+    fwd = A * (arc + (8 / B if mult else 0)) + D * sigma_bytes + n * ((8 + 4) / B + sigma_bytes)
+    bwd = A * (arc + (8 / B if mult else 0)) + D * delta_bytes + n * ((8 + 4 + 8) / B + sigma_bytes + delta_bytes)
+    return fwd + bwd
+
+
 def centrality_ops_per_source(interior_entries):
     """Algorithmic integer operations of the Centrality step per source: for every (frontier,
     non-frontier node) table entry, one add and one compare in the forward min-plus and one
     add and one compare in the backward tight-exit test."""
     return 4.0 * interior_entries
+
+
+def centrality_bytes_per_source(frontiers, interior_nodes, delta_bytes=8):
+    """Bytes of the Centrality step that one source cannot do without: the distance, count and dependency
+    of every frontier of a part with non-frontier nodes read once, one result per non-frontier node."""
+    return frontiers * (4 + 8 + delta_bytes) + interior_nodes * 8
+
+
+def kernel_name(precision, weights_above_one, skeleton=False):
+    """The shortest-path kernel that a call takes (FP64: level masks; FP32 dependencies: level masks on
+    unit weights without a skeleton, else lockstep)."""
+    levels = precision == "fp64" or not (weights_above_one or skeleton)
+    return "lm_kernel" if levels else "ls_kernel"
 
 
 def dist_env():
@@ -552,7 +577,8 @@ def _skeleton_model(bc, g, G, S, part, ctx):
     sample = np.searchsorted(nodes, np.asarray(S)[np.linspace(0, len(S) - 1, 32).astype(int)]).astype(np.int32)
     D = _tight_arcs(bc, Gsk, sample, ctx)
     return {"N": N, "arcs": arcs, "D": D, "weighted": bool(aw.size and aw.max() > 1),
-            "mult": bool(amu.size and amu.max() > 1), "interior_entries": interior}
+            "mult": bool(amu.size and amu.max() > 1), "interior_entries": interior,
+            "frontiers": int(F[V > F].sum()), "interior_nodes": int((V - F)[F > 0].sum())}
 
 
 def _roof(bound, achieved, peak, unit, kernel, traffic, **extra):
@@ -682,39 +708,45 @@ def _run_single(args, bc, g, S, ctx, flush, dev, ws, rank, pool):
                                  "candidates_ms": {f"batch{b}_cluster{c}": t for (b, c), t in times.items()}}
 
     # rooflines of the three kernels of the step, per launch of this rank's shard of the sources
-    hbm, sm_mhz, peak_kind = measured_peaks()
+    hbm, _, peak_kind = measured_peaks()
     peak_src = ("MEASURED_PEAKS.json hbm_gbs (measured)" if peak_kind == "measured" else "fallback 6.8 TB/s")
     delta_bytes = 4 if prec == "fp32" else 8
     rooflines = {}
     if not args.no_roofline_model:
         D_avg = _tight_arcs(bc, G, np.linspace(0, n - 1, 32).astype(np.int32), ctx)
-        by_plain = model_bytes_per_source(n, A, D_avg, 32, delta_bytes) * my_ns
+        plain_kernel = kernel_name(prec, g.w is not None)
+        if plain_kernel == "lm_kernel":
+            by_plain = model_bytes_per_source_levels(n, A, D_avg, 32, 4, delta_bytes, g.w is not None) * my_ns
+        else:
+            by_plain = model_bytes_per_source(n, A, D_avg, 32, delta_bytes) * my_ns
         rooflines["plain"] = _roof(
-            "hbm", by_plain / (ls_ms / 1e3) / 1e9, hbm, "GB/s", "ls_kernel (plain Brandes, forward + backward)",
-            profiled_traffic("ls_kernel", args.workload), peak_source=peak_src,
+            "hbm", by_plain / (ls_ms / 1e3) / 1e9, hbm, "GB/s",
+            f"{plain_kernel} (plain Brandes, forward + backward)",
+            profiled_traffic(plain_kernel, args.workload), peak_source=peak_src,
             algorithmic_bytes_per_launch=by_plain, avg_launch_ms=ls_ms, tight_arcs_per_source=D_avg,
             sources_per_launch=my_ns)
         skm = _skeleton_model(bc, g, G, S_order, np.asarray(g.part), ctx)
         if sk_ms > 0:
-            by_sk = model_bytes_per_source_skeleton(skm["N"], skm["arcs"], skm["D"], 32, delta_bytes,
-                                                    skm["weighted"], skm["mult"]) * my_ns
+            sk_kernel = kernel_name(prec, True, skeleton=True)
+            if sk_kernel == "lm_kernel":
+                by_sk = model_bytes_per_source_levels(skm["N"], skm["arcs"], skm["D"], 32, 8, delta_bytes,
+                                                      skm["weighted"], skm["mult"]) * my_ns
+            else:
+                by_sk = model_bytes_per_source_skeleton(skm["N"], skm["arcs"], skm["D"], 32, delta_bytes,
+                                                        skm["weighted"], skm["mult"]) * my_ns
             rooflines["brandes_sk"] = _roof(
                 "hbm", by_sk / (sk_ms / 1e3) / 1e9, hbm, "GB/s",
-                "ls_kernel (Brandes_SK on the weighted skeleton, forward + backward, all chunks)",
-                profiled_traffic("ls_kernel_skel", args.workload), peak_source=peak_src,
+                f"{sk_kernel} (Brandes_SK on the weighted skeleton, forward + backward, all chunks)",
+                profiled_traffic(f"{sk_kernel}_skel", args.workload), peak_source=peak_src,
                 algorithmic_bytes_per_launch=by_sk, avg_ms=sk_ms, skeleton_nodes=skm["N"],
                 skeleton_arcs=skm["arcs"], tight_arcs_per_source=skm["D"], sources_per_launch=my_ns)
         if ce_ms > 0:
-            props = torch.cuda.get_device_properties(dev)
-            peak_ops = alu_peak_ops(props.multi_processor_count, sm_mhz)
-            ops = centrality_ops_per_source(skm["interior_entries"]) * my_ns
+            by_ce = centrality_bytes_per_source(skm["frontiers"], skm["interior_nodes"], delta_bytes) * my_ns
             rooflines["centrality"] = _roof(
-                "alu", ops / (ce_ms / 1e3) / 1e12, peak_ops / 1e12, "Tops/s",
-                "centrality_tiled_kernel (Eq. 13, forward min-plus + backward tight exits)", None,
-                peak_source=f"{props.multi_processor_count} SMs x 4 schedulers x 32 lanes x {sm_mhz:.0f} MHz "
-                            "(32-bit integer lane operations)",
-                algorithmic_ops_per_launch=ops, avg_ms=ce_ms, interior_table_entries=skm["interior_entries"],
-                sources_per_launch=my_ns)
+                "hbm", by_ce / (ce_ms / 1e3) / 1e9, hbm, "GB/s",
+                "centrality_kernel (Eq. 13 over the frontiers with a non-zero path count)", None,
+                peak_source=peak_src, algorithmic_bytes_per_launch=by_ce, avg_ms=ce_ms, frontiers=skm["frontiers"],
+                interior_nodes=skm["interior_nodes"], sources_per_launch=my_ns)
     times = {"plain": ls_ms, "brandes_sk": sk_ms, "centrality": ce_ms}
     dominant = max((k for k in rooflines), key=lambda k: times[k], default=None)
     roofline = dict(rooflines[dominant], dominant_of=sorted(rooflines)) if dominant else None
@@ -826,7 +858,7 @@ def _run_batched(args, bc, graphs, ctx, flush, dev, ws, rank):
     ref64, got32 = (a, b) if prec == "fp64" else (b, a)
     fp32 = {"ms": so["ms_total"] if prec == "fp64" else ms, "fp64_ms": ms if prec == "fp64" else so["ms_total"],
             "max_rel_err_fp32_vs_gpu_fp64": _rel(got32, ref64)}
-    # roofline of the batched lockstep launch: per graph, |V_g| sources of the per-source model
+    # roofline of the batched launch: per graph, |V_g| sources of the per-source model
     # bytes, with the tight-arc count D_g from the measured tight fraction of sampled graphs
     # (their distances from 4 sources each, on the GPU)
     rng = np.random.default_rng(0)
@@ -838,12 +870,13 @@ def _run_batched(args, bc, graphs, ctx, flush, dev, ws, rank):
         fracs.append(D / max(1, Gs.num_arcs))
     tight_frac = float(np.mean(fracs))
     delta_bytes = 4 if prec == "fp32" else 8
-    bytes_launch = float(sum(g.n * model_bytes_per_source(g.n, 2 * g.m, tight_frac * 2 * g.m, 32, delta_bytes)
+    bytes_launch = float(sum(g.n * model_bytes_per_source_levels(g.n, 2 * g.m, tight_frac * 2 * g.m, 32, 4, delta_bytes)
                              for g in mine))
     hbm, _, peak_kind = measured_peaks()
     ls_ms = statistics.mean(st["ms_brandes_sk"] for st in logs)
     achieved = bytes_launch / (ls_ms / 1e3) / 1e9
-    roofline = _roof("hbm", achieved, hbm, "GB/s", "ls_kernel (batched plain Brandes, forward + backward)", None,
+    roofline = _roof("hbm", achieved, hbm, "GB/s",
+                     f"{kernel_name(prec, False)} (batched plain Brandes, forward + backward)", None,
                      peak_source="MEASURED_PEAKS.json hbm_gbs (measured)" if peak_kind == "measured"
                      else "fallback 6.8 TB/s", algorithmic_bytes_per_launch=bytes_launch, avg_launch_ms=ls_ms,
                      tight_arc_fraction=tight_frac)

@@ -45,7 +45,7 @@ extern "C" {
 #define BCPP_EINVAL 1            /* malformed graph, targets, partition or options */
 #define BCPP_ENOMEM 2            /* device or host allocation failed */
 #define BCPP_ECUDA 3             /* a CUDA runtime call failed */
-#define BCPP_ETIMEOUT 4          /* reserved: a bounded device wait expired */
+#define BCPP_ETIMEOUT 4          /* a bounded device wait (grid barrier) expired */
 #define BCPP_EOVERFLOW_SIGMA 5   /* results written, but some path count exceeded 2^64 */
 #define BCPP_ECAPACITY 6         /* a per-batch device list outgrew its bound (see bcpp_strerror) */
 
