@@ -174,3 +174,22 @@ def test_centrality_list_lengths(bc, k, wmax):
     assert rel_err(got, ref) <= FP64_TOL
     f32 = bc.brandes_pp(G, S, g.part, precision="fp32").cpu().numpy()
     assert rel_err(f32, ref) <= 2e-6   # the FP32 bar of the other parity tests on small graphs
+
+
+@pytest.mark.parametrize("deg", [257, 383, 384, 385, 512, 1025])
+@pytest.mark.parametrize("wmax", [None, 9])
+def test_long_rows(bc, deg, wmax):
+    """Rows of more than 256 arcs around the 128 arcs that are looked at together."""
+    g = wheel_of(deg, 2.0, seed=deg)
+    g = g if wmax is None else gen.with_weights(g, wmax, seed=deg)
+    S = gen.sample_targets(g.n, 40, seed=3)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    assert rel_err(bc.brandes(G, S).cpu().numpy(), ref) <= FP64_TOL
+    f32 = bc.brandes(G, S, precision="fp32").cpu().numpy()
+    assert rel_err(f32, ref) <= 2e-6   # the FP32 bar of the other parity tests on small graphs
+    d, s = bc.sssp(G, S[:3])
+    for i, v in enumerate(S[:3]):
+        rd, rs, _ = oracle.sssp(g, int(v))
+        assert np.array_equal(d[i].cpu().numpy(), rd)
+        assert np.array_equal(s[i].cpu().numpy().view(np.uint64), rs)
