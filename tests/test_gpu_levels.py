@@ -193,3 +193,17 @@ def test_long_rows(bc, deg, wmax):
         rd, rs, _ = oracle.sssp(g, int(v))
         assert np.array_equal(d[i].cpu().numpy(), rd)
         assert np.array_equal(s[i].cpu().numpy().view(np.uint64), rs)
+
+
+@pytest.mark.parametrize("k", [1, 227, 228, 255, 256, 257])
+def test_source_order_small_levels(bc, k):
+    """Levels around the 256 nodes and 2,048 arcs that one block takes alone: a hub, k children with eight
+    leaves each, and a chain (every node a target, so a node missing from the order shows)."""
+    i = np.arange(1, k + 1)
+    leaves = k + 1 + np.arange(8 * k)
+    tail = np.concatenate([[0], 9 * k + 1 + np.arange(40)])
+    src = np.concatenate([np.zeros(k, np.int64), np.repeat(i, 8), tail[:-1]])
+    dst = np.concatenate([i, leaves, tail[1:]])
+    g = gen.EdgeList(n=9 * k + 41, src=src.astype(np.int32), dst=dst.astype(np.int32))
+    ref, _ = oracle.brandes(g, None)
+    assert rel_err(bc.brandes(bc.graph_from_edgelist(g), None).cpu().numpy(), ref) <= FP64_TOL
