@@ -810,6 +810,7 @@ struct LmWave {
 struct LmWs {
     std::vector<LmWave> waves;
     int lcap = 0;
+    bool probe = true;         // no bound on the levels
     bool narrow = true;
     bool fp32 = false;         // FP32 dependencies
     double mean_degree = 16;   // arcs per node
@@ -853,6 +854,9 @@ int lm_levels(bool weighted, bool directed, const OrderWs* ord) {
     if (!ord) return 64;
     return std::max(directed ? 64 : 24, 2 * std::min(ord->depth, LM_MAX_LEVELS) + 4);
 }
+
+// ... and then the masks are known to be enough.
+bool lm_bounded(bool weighted, bool directed, const OrderWs* ord) { return !weighted && !directed && ord; }
 
 // *fits = false: not enough memory for one batch (the caller takes the lockstep kernel).  forward: no backward
 // pass, no sums over sources.  sizes: node count of
@@ -961,6 +965,7 @@ LmArgs lm_wave_args(const LmWs& L, const LmWave& w, const LsArena& A, const LsPa
     a.lev = L.lev.p; a.seen = L.seen.p; a.sg = L.sg.p; a.cc = L.cc.p; a.dsum = L.dsum.p;
     a.rows = (int64_t)w.ntiles * 32;
     a.lcap = L.lcap;
+    a.probe = L.probe;
     a.wmax = (int32_t)wmax;
     a.mean_degree = L.mean_degree;
     a.ctl = L.ctl.p;
@@ -1098,6 +1103,7 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     if (fp32 && width < 32) hitems = make_items(0, s0, s1, width);
     r.lm.fp32 = fp32;
     r.lm.mean_degree = (double)g->num_arcs / n;
+    r.lm.probe = !lm_bounded(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr);
     if (lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
                        lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
@@ -1576,6 +1582,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         a.dsum = r.lm.dsum.p; a.drow = W.d;
         a.rows = (int64_t)a.ntiles * 32;
         a.lcap = r.lm.lcap;
+        a.probe = r.lm.probe;
         a.wmax = (int32_t)K.wmax_sk;
         a.mean_degree = r.lm.mean_degree;
         a.ctl = r.lm.ctl.p;
@@ -1645,7 +1652,9 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
     if (N > 0 && !hitems.empty() && lm_serves(c, o, r.spl, N, K.arcs, K.wmax_sk)) {
         r.lm.mean_degree = (double)K.arcs / N;
         // skeleton distances are the distances in G
-        const int lcap = lm_levels(g->w != nullptr, g->directed != 0, o.order_sources && ns > 2 * LS_LANES ? &r.ord : nullptr);
+        const OrderWs* ord = o.order_sources && ns > 2 * LS_LANES ? &r.ord : nullptr;
+        const int lcap = lm_levels(g->w != nullptr, g->directed != 0, ord);
+        r.lm.probe = !lm_bounded(g->w != nullptr, g->directed != 0, ord);
         if (r.hunits.empty())
             CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return N; }, n, lcap, r.unit, &r.levels));
         else
@@ -2364,6 +2373,7 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
         a.lev = lev.p; a.seen = seen.p; a.sg = sg.p; a.dsum = dsum.p; a.drow = d.p;
         a.rows = (int64_t)a.ntiles * 32;
         a.lcap = lcap;
+        a.probe = true;
         a.wmax = (int32_t)wmax;
         a.mean_degree = (double)g->num_arcs / g->n;
         a.ctl = ctl.p;

@@ -445,6 +445,38 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, SM& sm, int lane, uin
     }
 }
 
+// Pairs reached by level D and by D / 2, and rows, of a sample of the unfinished batches' rows.  (Its own function:
+// inlined, it cost the kernel's loops registers, n = 10,000: 6.1 -> 6.9 ms.)
+__device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int D, int wmax, const uint32_t* bdepth,
+                                          const int32_t* tile_item, int32_t item_base, int32_t tpb, uint32_t* probe) {
+    const int64_t nt = (int64_t)gridDim.x * LM_THREADS, step = max((int64_t)1, rows / nt);
+    uint32_t b1 = 0, b2 = 0, all = 0;
+    for (int64_t row = ((int64_t)blockIdx.x * LM_THREADS + threadIdx.x) * step; row < rows; row += nt * step) {
+        const int32_t t = (int32_t)(row >> 5);
+        const int it = tile_item ? __ldg(tile_item + t) - item_base : t / tpb;
+        if ((int)bdepth[it * DEPTH_STRIDE] + wmax < D) continue;   // (a batch that is done has no masks there)
+        all++;
+        for (int l = 0; l <= D; l++) {
+            const uint32_t c = __popc(__ldcg(lev + (int64_t)l * rows + row));
+            b2 += c;
+            if (l <= D / 2) b1 += c;
+        }
+    }
+    b1 = __reduce_add_sync(FULL, b1);
+    b2 = __reduce_add_sync(FULL, b2);
+    all = __reduce_add_sync(FULL, all);
+    if ((threadIdx.x & 31) == 0 && all) {
+        atomicAdd(probe, b1);
+        atomicAdd(probe + 1, b2);
+        atomicAdd(probe + 2, all);
+    }
+}
+// D (all / b2)^(1 / dim) levels needed, with 2^dim = b2 / b1: more than 4 D?
+__device__ __noinline__ bool looks_deep(const uint32_t* probe) {
+    const float b1 = (float)__ldcg(probe), b2 = (float)__ldcg(probe + 1), all = 32.0f * (float)__ldcg(probe + 2);
+    return b2 >= 1.5f * b1 && all * b1 * b1 > b2 * b2 * b2;
+}
+
 template <typename SG, typename DT, bool WEIGHTED, bool MULT, bool TABLE>
 __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4))
 lm_kernel(const LmArgs A, const int sub_log) {
@@ -486,6 +518,9 @@ lm_kernel(const LmArgs A, const int sub_log) {
         x.rb = (int64_t)tile0 * 32;
         return x;
     };
+
+    // an earlier wave proved too deep: the call reruns (only set past a barrier of this launch, if by it)
+    if (__ldcg(A.flags + FLAG_CAPACITY) != 0u) return;
 
     // With few tiles per warp a unit is a part of a tile (32 >> sub_log rows), so that a level's last and
     // fullest tiles do not leave the other warps waiting (see lm_go for the rule).
@@ -630,6 +665,24 @@ lm_kernel(const LmArgs A, const int sub_log) {
         }
         if (w & LVL_ANY) depth = D;
         if (D - depth >= wmax) break;
+        // Too deep a graph shows early: a quarter of the way the pairs reached by now and by half of that
+        // give the dimension that the balls around the sources grow with, and with it the level at which
+        // they hold every pair; past the levels provided for, the call reruns without going there first
+        // (grid 300 x 300 with weights up to 16, 500 sources: 112 -> 101 ms, 97 without the attempt).
+        // Balls that hardly grow any more belong to stragglers, not to a deep graph.
+        if (!TABLE && A.probe && (D == A.lcap / 4 || D == A.lcap / 4 + 1)) {
+            uint32_t* probe = work + 2 * A.lcap;
+            if (D == A.lcap / 4) {
+                probe_levels(A.lev, A.rows, D, wmax, bdepth, A.item_tile0 ? A.tile_item + A.tile_base : nullptr,
+                             A.item_base, A.tpb, probe);
+            } else if (looks_deep(probe)) {
+                if (blockIdx.x == 0 && threadIdx.x == 0) {
+                    atomicOr(&A.flags[FLAG_DEPTH], 1u);
+                    atomicOr(&A.flags[FLAG_CAPACITY], 1u);
+                }
+                return;
+            }
+        }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
 
@@ -839,7 +892,7 @@ cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
 
 }  // namespace
 
-int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + (int64_t)nitems * DEPTH_STRIDE + 2 * (int64_t)lcap; }
+int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + (int64_t)nitems * DEPTH_STRIDE + 2 * (int64_t)lcap + 3; }
 
 cudaError_t lm_launch(const LmArgs& A, bool narrow, bool fp32, int num_sms, cudaStream_t st) {
     if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;

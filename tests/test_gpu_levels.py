@@ -207,3 +207,37 @@ def test_source_order_small_levels(bc, k):
     g = gen.EdgeList(n=9 * k + 41, src=src.astype(np.int32), dst=dst.astype(np.int32))
     ref, _ = oracle.brandes(g, None)
     assert rel_err(bc.brandes(bc.graph_from_edgelist(g), None).cpu().numpy(), ref) <= FP64_TOL
+
+
+def with_tail(g, k):
+    """g and a path of k more nodes from its node 0."""
+    t = np.concatenate([[0], g.n + np.arange(k)]).astype(np.int32)
+    return gen.EdgeList(n=g.n + k, src=np.concatenate([g.src, t[:-1]]), dst=np.concatenate([g.dst, t[1:]]))
+
+
+DEEP_CASES = {
+    "grid-w": gen.with_weights(gen.grid(60, 60), 16, seed=41),        # given up early
+    "tail-past": gen.with_weights(with_tail(gen.erdos_renyi(600, 0.01, seed=42), 90), 9, seed=42),   # at the last level
+    "tail-within": gen.with_weights(with_tail(gen.erdos_renyi(600, 0.01, seed=43), 25), 9, seed=43),
+    "islands-w": gen.with_weights(union(gen.erdos_renyi(300, 0.03, seed=44), gen.path(60), gen.star(50)), 5, seed=44),
+    "cycle": gen.cycle(150),
+}
+
+
+@pytest.mark.parametrize("name", list(DEEP_CASES))
+def test_deep_graphs(bc, name):
+    """Calls without a bound on the levels, around the test for a deep graph at a quarter of them."""
+    g = DEEP_CASES[name]
+    S = gen.sample_targets(g.n, 45, seed=3)
+    ref, _ = oracle.brandes(g, S)
+    got = bc.brandes(bc.graph_from_edgelist(g), S, order_sources=False).cpu().numpy()
+    assert rel_err(got, ref) <= FP64_TOL
+
+
+def test_deep_graphs_batched(bc):
+    gs = [gen.erdos_renyi(80, 0.06, seed=45), gen.cycle(140), gen.grid(3, 50), gen.path(120)]
+    arena = bc.build_arena(gs)
+    got = bc.brandes_batched(arena).cpu().numpy()
+    for i, g in enumerate(gs):
+        ref, _ = oracle.brandes(g, None)
+        assert rel_err(got[arena.node_ptr_host[i]:arena.node_ptr_host[i + 1]], ref) <= FP64_TOL, i
