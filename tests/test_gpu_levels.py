@@ -241,3 +241,16 @@ def test_deep_graphs_batched(bc):
     for i, g in enumerate(gs):
         ref, _ = oracle.brandes(g, None)
         assert rel_err(got[arena.node_ptr_host[i]:arena.node_ptr_host[i + 1]], ref) <= FP64_TOL, i
+
+
+@pytest.mark.parametrize("rungs", [97, 98, 99, 140])
+@pytest.mark.parametrize("every", [1, 4, 5])
+def test_long_graphs_by_density_of_targets(bc, rungs, every):
+    """A ladder around the depth past which calls with many targets run on the lockstep kernel."""
+    g = gen.grid(2, rungs)
+    S = np.arange(0, g.n, every, dtype=np.int32)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    assert rel_err(bc.brandes(G, S).cpu().numpy(), ref) <= FP64_TOL
+    part = (np.arange(g.n) % rungs // 10).astype(np.int32)
+    assert rel_err(bc.brandes_pp(G, S, part).cpu().numpy(), ref) <= FP64_TOL
