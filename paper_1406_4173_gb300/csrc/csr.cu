@@ -117,7 +117,24 @@ __device__ __forceinline__ void bitonic(T* x, int size, int t, int nt, S&& sync)
         }
 }
 
-// One warp per row; rows above CSR_WARP_ROW go on the list.
+// Sorts the keys of each group of G lanes (G a power of two; at least `most` of them used, the others ~0).
+template <int G, typename T>
+__device__ __forceinline__ T sort_lanes(T k, int lane, int most) {
+    const int l = lane & (G - 1);
+#pragma unroll
+    for (int s = 2; s <= G; s <<= 1) {
+        if (s >= 2 * most) break;
+#pragma unroll
+        for (int j = s >> 1; j > 0; j >>= 1) {
+            const T y = __shfl_xor_sync(FULL, k, j);
+            k = ((l & j) == 0) == ((l & s) == 0) ? min(k, y) : max(k, y);
+        }
+    }
+    return k;
+}
+
+// One warp per two rows, side by side when both have up to 16 arcs (8 M edges on 1 M nodes: 706 -> 683 us against a
+// row at a time; the longer rows in shared memory take most of what is left); rows above CSR_WARP_ROW go on the list.
 template <bool W>
 __global__ void __launch_bounds__(CSR_SORT_WARPS * 32)
 csr_sort_rows_kernel(int32_t n, const int64_t* __restrict__ rp, int32_t* col, uint32_t* w, int32_t* longrows,
@@ -128,20 +145,28 @@ csr_sort_rows_kernel(int32_t n, const int64_t* __restrict__ rp, int32_t* col, ui
     const int lane = threadIdx.x & 31;
     T* x = s_x[threadIdx.x >> 5];
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
+    for (int64_t u0 = 2 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); u0 < n; u0 += 2 * nw) {
+        const int64_t own = u0 + (lane >> 4);
+        const int64_t own0 = own < n ? rp[own] : 0;
+        const int64_t ownd = own < n ? rp[own + 1] - own0 : 0;
+        const unsigned most = __reduce_max_sync(FULL, (unsigned)min(ownd, (int64_t)17));
+        if (most < 2) continue;
+        if (most <= 16) {
+            const int l = lane & 15;
+            const T k = sort_lanes<16>(l < ownd ? K::load(col, w, own0 + l) : ~(T)0, lane, (int)most);
+            const uint32_t before = __shfl_up_sync(FULL, K::head(k), 1);
+            if (l < ownd) {
+                K::store(col, w, own0 + l, k);
+                if (l > 0 && before == K::head(k)) flag_invalid(flags, WHY_DUPLICATE);
+            }
+            continue;
+        }
+        for (int64_t u = u0; u < min((int64_t)n, u0 + 2); u++) {
         const int64_t a0 = rp[u];
         const int64_t deg = rp[u + 1] - a0;
         if (deg < 2) continue;
         if (deg <= 32) {
-            T k = lane < deg ? K::load(col, w, a0 + lane) : ~(T)0;
-#pragma unroll
-            for (int s = 2; s <= 32; s <<= 1) {
-#pragma unroll
-                for (int j = s >> 1; j > 0; j >>= 1) {
-                    const T y = __shfl_xor_sync(FULL, k, j);
-                    k = ((lane & j) == 0) == ((lane & s) == 0) ? min(k, y) : max(k, y);
-                }
-            }
+            const T k = sort_lanes<32>(lane < deg ? K::load(col, w, a0 + lane) : ~(T)0, lane, (int)deg);
             const uint32_t before = __shfl_up_sync(FULL, K::head(k), 1);
             if (lane < deg) {
                 K::store(col, w, a0 + lane, k);
@@ -160,6 +185,7 @@ csr_sort_rows_kernel(int32_t n, const int64_t* __restrict__ rp, int32_t* col, ui
             __syncwarp();
         } else if (lane == 0) {
             longrows[atomicAdd(nlong, 1u)] = (int32_t)u;
+        }
         }
     }
 }
@@ -350,7 +376,7 @@ void csr_scatter(int64_t m, const int32_t* eu, const int32_t* ev, const uint32_t
 template <bool W>
 static cudaError_t csr_sort_t(int32_t n, uint32_t longest, const int64_t* rp, int32_t* col, uint32_t* w, int32_t* longrows,
                               uint32_t* nlong, uint32_t* flags, cudaStream_t st) {
-    csr_sort_rows_kernel<W><<<grid_for((int64_t)n * 32, CSR_SORT_WARPS * 32, 152 * 64), CSR_SORT_WARPS * 32, 0, st>>>(
+    csr_sort_rows_kernel<W><<<grid_for((int64_t)n * 16, CSR_SORT_WARPS * 32, 152 * 64), CSR_SORT_WARPS * 32, 0, st>>>(
         n, rp, col, w, longrows, nlong, flags);
     if (longest <= (uint32_t)CSR_WARP_ROW) return cudaSuccess;
     size_t size = 2 * CSR_WARP_ROW;

@@ -68,3 +68,30 @@ def test_build_refuses(bc, deg, what):
     for directed in (False, True):
         with pytest.raises(bc.BcppError):
             bc.csr_build(n, src, dst, w, directed)
+
+
+@pytest.mark.parametrize("a", [0, 1, 2, 3, 8, 9, 15, 16, 17, 32, 33])
+@pytest.mark.parametrize("b", [0, 1, 5, 16, 17])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_build_pairs_of_rows(bc, a, b, weighted):
+    """Two rows to a warp: lengths a and b side by side, an odd number of rows, one repeated head at a time."""
+    rng = np.random.default_rng(100 * a + b)
+    n = 41
+    src = np.concatenate([np.full(a if u % 2 == 0 else b, u) for u in range(n)]).astype(np.int32)
+    dst = np.concatenate([rng.choice(np.delete(np.arange(n), u), a if u % 2 == 0 else b, replace=False)
+                          for u in range(n)]).astype(np.int32)
+    o = rng.permutation(src.size)
+    src, dst = src[o], dst[o]
+    w = rng.integers(1, 1000, src.size).astype(np.uint32)
+    G = bc.csr_build(n, src, dst, w if weighted else None, True)
+    rp, col, wo = host_csr(n, src, dst, w, True)
+    assert np.array_equal(G.row_ptr.cpu().numpy(), rp)
+    assert np.array_equal(G.col.cpu().numpy(), col)
+    if weighted:
+        assert np.array_equal(G.w.cpu().numpy().view(np.uint32), wo)
+    for u in (0, 1):
+        at = np.nonzero(src == u)[0]
+        if at.size:
+            with pytest.raises(bc.BcppError):
+                bc.csr_build(n, np.append(src, np.int32(u)), np.append(dst, dst[at[0]]),
+                             np.append(w, np.uint32(7)) if weighted else None, True)
