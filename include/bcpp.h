@@ -139,6 +139,12 @@ void bcpp_destroy(bcpp_ctx *ctx);
 /* Workspace bytes currently held by the context (device). */
 int64_t bcpp_workspace_bytes(const bcpp_ctx *ctx);
 
+/* Which kernel the source batches of the context's last evaluation (bcpp_brandes, the Brandes++ calls,
+ * bcpp_brandes_batched, bcpp_sssp, bcpp_plan_launch) ran on: out[0] (host, int64[3]) = batches finished by
+ * the level-mask kernel, out[1] = by the lockstep kernel, out[2] = those of out[1] that the level-mask kernel
+ * had begun and given back (more distance levels than it provides for, or a path count of 2^32). */
+int bcpp_last_batches(const bcpp_ctx *ctx, int64_t *out);
+
 /* CSR build and validation (the input graph G(V,E,W) of Sec. 3).  From m edges
  * (eu[i], ev[i], weight ew[i] or unit if ew == NULL) build the CSR: row_ptr_out[n+1],
  * col_out and w_out (w_out may be NULL when ew is NULL) of capacity 2m (undirected: every

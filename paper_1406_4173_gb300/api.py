@@ -58,7 +58,7 @@ EXPORTS = ["bcpp_default_opts", "bcpp_strerror", "bcpp_create", "bcpp_destroy", 
            "bcpp_csr_build", "bcpp_csr_validate", "bcpp_brandes", "bcpp_brandes_pp", "bcpp_brandes_batched",
            "bcpp_sssp", "bcpp_skeleton", "bcpp_brandes_noalloc", "bcpp_brandes_pp_st", "bcpp_brandes_pp_all",
            "bcpp_plan_brandes", "bcpp_plan_brandes_pp", "bcpp_plan_launch", "bcpp_plan_destroy", "bcpp_autotune",
-           "bcpp_partition_lp", "bcpp_shard_bounds", "bcpp_autotune_batched"]
+           "bcpp_partition_lp", "bcpp_shard_bounds", "bcpp_autotune_batched", "bcpp_last_batches"]
 
 _lib = None
 _lock = threading.Lock()
@@ -83,6 +83,7 @@ def load_library(path: str | None = None):
             "bcpp_create": (ctypes.c_int, [ctypes.POINTER(ctypes.c_void_p), P]),
             "bcpp_destroy": (None, [P]),
             "bcpp_workspace_bytes": (i64, [P]),
+            "bcpp_last_batches": (ctypes.c_int, [P, ctypes.POINTER(i64)]),
             "bcpp_csr_build": (ctypes.c_int, [P, i32, i64, P, P, P, i32, P, P, P, ctypes.POINTER(i64)]),
             "bcpp_csr_validate": (ctypes.c_int, [P, G]),
             "bcpp_brandes": (ctypes.c_int, [P, G, P, i32, O, P, ST]),
@@ -155,6 +156,12 @@ class Context:
 
     def workspace_bytes(self) -> int:
         return int(load_library().bcpp_workspace_bytes(self.handle))
+
+    def last_batches(self) -> dict:
+        """Source batches of the last evaluation by kernel (bcpp_last_batches)."""
+        out = (ctypes.c_int64 * 3)()
+        _check(load_library().bcpp_last_batches(self.handle, out))
+        return dict(zip(("levels", "lockstep", "given_back"), map(int, out)))
 
 
 _default_ctx: dict = {}

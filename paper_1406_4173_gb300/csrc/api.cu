@@ -35,6 +35,7 @@ struct bcpp_ctx {
     unsigned long long* phase = nullptr;    // device [2]: forward / backward batch time (ns)
     int64_t launches = 0;
     int order_factor = 8;            // settled-entry capacity per node of a batch (retry: worst case)
+    int64_t ran[3] = {};             // bcpp_last_batches of the last call
     cudaEvent_t ev[8] = {};
 
     void* acquire(size_t bytes) {
@@ -332,6 +333,11 @@ struct SlotWs {
     int sum_slots = 0;          // partial-sum sets (one per slot, or per item)
     int64_t rows = 0;
     bool narrow = false;        // one-byte distance rows (0xff = unreached)
+
+    void release() {
+        d.free(); sg.free(); dl.free(); order.free(); step_d.free(); step_beg.free(); hdr.free(); bm.free();
+        bflag.free(); bcs.free(); bcc.free(); bcb.free(); counter.free();
+    }
 };
 
 // One-byte distance rows for unit-weight Brandes passes, except on the worst-case retry (which
@@ -538,6 +544,16 @@ struct Timer {
     }
 };
 
+// Batches of a pass for bcpp_last_batches, once it is done.
+void count_batches(bcpp_ctx* c, bool levels, int64_t nitems, bool given_back) {
+    c->ran[levels ? 0 : 1] += nitems;
+    if (given_back) c->ran[2] += nitems;
+}
+
+// Status of a pass that the level-mask kernel gave back (finish_status): the caller runs it on the lockstep
+// kernel, with what it has prepared.  Never returned to the user.
+constexpr int RC_GIVEN_BACK = 100;
+
 int finish_status(bcpp_ctx* c, bcpp_stats* st) {
     CK_RC(sync_flags(c));
     if (st) {
@@ -548,9 +564,34 @@ int finish_status(bcpp_ctx* c, bcpp_stats* st) {
     }
     if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
     if (c->hflags[FLAG_TIMEOUT]) return BCPP_ETIMEOUT;
+    if (c->hflags[FLAG_MASKS]) return RC_GIVEN_BACK;
     if (c->hflags[FLAG_CAPACITY]) return BCPP_ECAPACITY;
     if (c->hflags[FLAG_SIGMA_OVF]) return BCPP_EOVERFLOW_SIGMA;
     return BCPP_OK;
+}
+
+// Whether the usual lockstep rows would give up on a pass given back as well: they hold distances below 254
+// and 32-bit counts.  lcap: levels that the masks provided for.  (20,000 random nodes beside a path of 300,
+// every node a target: 116 ms straight on the worst-case rows, 204 on the usual ones first.)
+bool past_usual_rows(const bcpp_ctx* c, int lcap) { return (c->hflags[FLAG_MASKS] & MASKS_COUNT) || lcap >= 254; }
+
+// A pass that the level-mask kernel gave back, on the lockstep kernel: run() sets its workspace up and queues it.  The
+// usual rows and lists first, unless `worst`, and the worst case when they prove too small.
+template <class F>
+int run_in_lockstep(bcpp_ctx* c, bcpp_stats* st, bool worst, F&& run) {
+    int rc = BCPP_OK;
+    const int usual = c->order_factor;
+    for (int factor : {usual, 64}) {
+        if (worst && factor != 64) continue;
+        c->order_factor = factor;
+        for (int f : {FLAG_MASKS, FLAG_CAPACITY, FLAG_DEPTH})
+            CK_CUDA(cudaMemsetAsync(c->flags + f, 0, sizeof(uint32_t), c->stream));
+        rc = run();
+        if (rc == BCPP_OK) rc = finish_status(c, st);
+        if (rc != BCPP_ECAPACITY) break;
+    }
+    c->order_factor = usual;
+    return rc;
 }
 
 // in-CSR (transpose) of a graph with uint32 weights
@@ -821,6 +862,12 @@ struct LmWs {
     DBuf<double> dsum, bcs, bcc;
     DBuf<int32_t> tile0, tile_item;
     DBuf<LmRun> runs;
+
+    void release() {
+        waves.clear();
+        lev.free(); seen.free(); ctl.free(); sg.free(); cc.free(); dsum.free(); bcs.free(); bcc.free();
+        tile0.free(); tile_item.free(); runs.free();
+    }
 };
 
 // Row state kept in flight at most: enough rows that a level's work hides its barrier and its last
@@ -838,9 +885,8 @@ int64_t free_bytes(bcpp_ctx* c) {
 
 // Calls the level-mask kernel serves: batches of 32 sources, weights up to LM_MAX_WEIGHT, 32-bit arc offsets, FP64
 // dependencies, or FP32 ones on unit weights without a skeleton (fp32_too; there it adds in the lockstep
-// kernel's order, since FP32 sums in another order differ in the 8th digit).  A call whose batches prove too
-// deep, or whose path counts outgrow 32 bits, reruns with order_factor 64, which the lockstep kernel
-// serves.
+// kernel's order, since FP32 sums in another order differ in the 8th digit).  What proves too deep, or has
+// path counts past 32 bits, is given back (RC_GIVEN_BACK) and runs on the lockstep kernel.
 bool lm_serves(const bcpp_ctx* c, const bcpp_opts& o, int spl, int32_t n, int64_t arcs, uint64_t wmax,
                bool fp32_too = false) {
     return (o.precision != BCPP_FP32_DELTA || (fp32_too && wmax == 1)) && spl == 1 && c->order_factor < 64 && arcs < (1ll << 31) &&
@@ -1025,6 +1071,7 @@ struct PlainRun {
     SlotWs ws;
     LmWs lm;
     bool levels = false;           // on the level-mask kernel
+    int64_t s0 = 0, s1 = 0;        // source positions of this call's shard
     int nitems = 0, slots = 0, spl = 1, cl = 1, nb = 2;
     LsArena A{};
     LsParams P{};
@@ -1054,6 +1101,42 @@ int plain_emit_checks(bcpp_ctx* c, PlainRun& r) {
         c->launches++;
     }
     CK_CUDA(cudaGetLastError());
+    return BCPP_OK;
+}
+
+// Batches of 32 sources (of the ordered targets) and the workspace of their passes: on the level-mask kernel where
+// it serves them, unless masks = false, else on the lockstep kernel.
+int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks) {
+    const bcpp_graph* g = &r.g;
+    const int32_t n = g->n;
+    const bcpp_opts& o = r.o;
+    const bool fp32 = o.precision == BCPP_FP32_DELTA;
+    r.levels = false;
+    r.lm.release();
+    r.ws.release();
+    std::vector<LsItem> hitems = make_items(0, r.s0, r.s1, 32 * r.spl);
+    r.cl = r.spl == 1 ? choose_cluster(c, (int)hitems.size(), o) : 1;
+    const int width = r.spl == 1 ? balanced_width(r.s1 - r.s0, slot_capacity(c, o, r.cl), 32) : 32;
+    // (FP32 dependencies: the batches of the lockstep kernel, whose order of additions depends on them)
+    if (fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
+    r.lm.fp32 = fp32;
+    r.lm.mean_degree = (double)g->num_arcs / n;
+    r.lm.probe = !lm_bounded(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr);
+    if (masks && lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) &&
+        !(r.ordered && lm_dense_deep(r.ord, r.ns, n)))
+        CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
+                       lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
+    if (!r.levels && width < 32) hitems = make_items(0, r.s0, r.s1, width);
+    r.nitems = (int)hitems.size();
+    CK_ALLOC(r.items.alloc(c, r.nitems));
+    CK_RC(to_dev(c, r.items.p, hitems.data(), r.nitems));
+    if (!r.levels) {
+        const int ef = entry_factor(c, g->w != nullptr, r.spl);
+        r.slots = choose_slots(c, r.nitems, o.ctas_per_sm, slot_bytes(n, r.nb, fp32, ef, r.spl), (int64_t)n * 24, r.cl);
+        CK_RC(alloc_slots(c, r.ws, r.slots, n, r.nb, fp32, n, r.spl, ef, false));
+        r.ws.narrow = use_narrow(c, g->w != nullptr);
+        r.P.item_counter = r.ws.counter.p;
+    }
     return BCPP_OK;
 }
 
@@ -1098,36 +1181,13 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
         r.ordered = true;
         srcs = r.ord.out.p;
     }
-    // items: batches of 32 targets (ordered when requested)
-    int64_t s0, s1;
-    shard_sources(o, r.ns, s0, s1);
-    r.spl = choose_spl(c, s1 - s0, o);
-    std::vector<LsItem> hitems = make_items(0, s0, s1, 32 * r.spl);
-    r.cl = r.spl == 1 ? choose_cluster(c, (int)hitems.size(), o) : 1;
-    const int width = r.spl == 1 ? balanced_width(s1 - s0, slot_capacity(c, o, r.cl), 32) : 32;
-    // (FP32 dependencies: the batches of the lockstep kernel, whose order of additions depends on them)
-    if (fp32 && width < 32) hitems = make_items(0, s0, s1, width);
-    r.lm.fp32 = fp32;
-    r.lm.mean_degree = (double)g->num_arcs / n;
-    r.lm.probe = !lm_bounded(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr);
-    if (lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) && !(r.ordered && lm_dense_deep(r.ord, r.ns, n)))
-        CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
-                       lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
-    if (!r.levels && width < 32) hitems = make_items(0, s0, s1, width);
-    r.nitems = (int)hitems.size();
-    if (r.nitems <= 0) return BCPP_OK;
-    CK_ALLOC(r.items.alloc(c, r.nitems));
+    shard_sources(o, r.ns, r.s0, r.s1);
+    r.spl = choose_spl(c, r.s1 - r.s0, o);
+    if (r.s1 <= r.s0) return BCPP_OK;
     CK_ALLOC(r.node_off.alloc(c, 2));
-    CK_RC(to_dev(c, r.items.p, hitems.data(), r.nitems));
     const int64_t hoff[2] = {0, n};
     CK_RC(to_dev(c, r.node_off.p, hoff, 2));
     r.nb = g->w ? (int)r.wmax + 1 : 2;
-    if (!r.levels) {
-        const int ef = entry_factor(c, g->w != nullptr, r.spl);
-        r.slots = choose_slots(c, r.nitems, o.ctas_per_sm, slot_bytes(n, r.nb, fp32, ef, r.spl), (int64_t)n * 24, r.cl);
-        CK_RC(alloc_slots(c, r.ws, r.slots, n, r.nb, fp32, n, r.spl, ef, false));
-        r.ws.narrow = use_narrow(c, g->w != nullptr);
-    }
     LsArena& A = r.A;
     A.rp = g->row_ptr; A.col = g->col; A.w = (const int32_t*)g->w; A.mu = nullptr;
     if (g->directed) {
@@ -1143,14 +1203,32 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     P.srcs = srcs;
     P.in_s = nS > 0 ? r.in_s.p : nullptr;
     P.items_static = 0;
-    P.item_counter = r.ws.counter.p;
     P.flags = c->flags;
     P.phase_ns = c->phase;
+    return plain_batches(c, r, true);
+}
+
+// The passes themselves over the batches of plain_batches.
+int plain_emit_passes(bcpp_ctx* c, PlainRun& r, Timer* tb) {
+    const bcpp_graph* g = &r.g;
+    const int32_t n = g->n;
+    const double scale = !g->directed && r.o.halve_undirected != 0 ? 0.5 : 1.0;
+    if (r.levels) return lm_emit(c, r.lm, r.A, r.P, r.items.p, g->w ? r.wmax : 1, scale, r.bc_out, tb);
+    CK_RC(init_slots(c, r.ws));
+    if (tb) tb->start();
+    ls_launch(r.o.precision == BCPP_FP32_DELTA, !g->directed, r.A, r.P, r.ws.W, r.items.p, r.nitems, r.slots,
+              c->stream, r.spl, r.cl, r.ws.narrow);
+    c->launches++;
+    if (tb) tb->stop();
+    CK_CUDA(cudaGetLastError());
+    combine_launch(r.ws.W.bc_sum, r.ws.W.bc_cmp, r.slots, n, n, scale, r.bc_out, c->stream);
+    c->launches++;
+    CK_CUDA(cudaGetLastError());
     return BCPP_OK;
 }
 
 // Device work of one evaluation (no host synchronization).  tb (may be null) times the
-// lockstep launch.
+// shortest-path launches.
 int plain_emit(bcpp_ctx* c, PlainRun& r, Timer* tb) {
     const bcpp_graph* g = &r.g;
     const int32_t n = g->n;
@@ -1164,19 +1242,16 @@ int plain_emit(bcpp_ctx* c, PlainRun& r, Timer* tb) {
     }
     if (g->directed) CK_RC(in_csr_emit(c, g, r.T));
     if (r.ordered) CK_RC(order_emit(c, r.ord, g->directed != 0));
-    const bool halve = !g->directed && r.o.halve_undirected != 0;
-    if (r.levels) return lm_emit(c, r.lm, r.A, r.P, r.items.p, g->w ? r.wmax : 1, halve ? 0.5 : 1.0, r.bc_out, tb);
-    CK_RC(init_slots(c, r.ws));
-    if (tb) tb->start();
-    ls_launch(r.o.precision == BCPP_FP32_DELTA, !g->directed, r.A, r.P, r.ws.W, r.items.p, r.nitems, r.slots,
-              c->stream, r.spl, r.cl, r.ws.narrow);
-    c->launches++;
-    if (tb) tb->stop();
-    CK_CUDA(cudaGetLastError());
-    combine_launch(r.ws.W.bc_sum, r.ws.W.bc_cmp, r.slots, n, n, halve ? 0.5 : 1.0, r.bc_out, c->stream);
-    c->launches++;
-    CK_CUDA(cudaGetLastError());
-    return BCPP_OK;
+    return plain_emit_passes(c, r, tb);
+}
+
+// The passes again on the lockstep kernel, after the level-mask kernel gave them back.
+int plain_in_lockstep(bcpp_ctx* c, PlainRun& r, Timer* tb, bcpp_stats* st) {
+    const bool worst = past_usual_rows(c, r.lm.lcap);
+    return run_in_lockstep(c, st, worst, [&] {
+        CK_RC(plain_batches(c, r, false));
+        return plain_emit_passes(c, r, tb);
+    });
 }
 
 int brandes_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS, const bcpp_opts& o, double* bc_out,
@@ -1187,6 +1262,9 @@ int brandes_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS, 
     CK_RC(plain_prepare(c, g, S, nS, o, bc_out, r));
     CK_RC(plain_emit(c, r, &tb));
     int rc = finish_status(c, st);
+    const bool back = rc == RC_GIVEN_BACK;
+    if (back) rc = plain_in_lockstep(c, r, &tb, st);
+    count_batches(c, r.levels, r.nitems, back);
     tt.stop();
     if (st) {
         st->ms_brandes_sk = tb.acc;
@@ -1264,9 +1342,8 @@ int tables_levels(bcpp_ctx* c, const LsArena& A, const LsParams& P, const std::v
     }
     CK_RC(sync_flags(c));
     if (c->hflags[FLAG_TIMEOUT]) return BCPP_ETIMEOUT;
-    if (c->hflags[FLAG_CAPACITY]) {
-        CK_CUDA(cudaMemsetAsync(c->flags + FLAG_CAPACITY, 0, sizeof(uint32_t), c->stream));
-        CK_CUDA(cudaMemsetAsync(c->flags + FLAG_DEPTH, 0, sizeof(uint32_t), c->stream));
+    if (c->hflags[FLAG_MASKS]) {
+        CK_CUDA(cudaMemsetAsync(c->flags + FLAG_MASKS, 0, sizeof(uint32_t), c->stream));
         return BCPP_OK;
     }
     *done = true;
@@ -1487,6 +1564,8 @@ struct PpRun {
     bool rows_by_item = false;   // Brandes_SK in one dynamic pass with a row set per batch
     bool levels = false;         // Brandes_SK on the level-mask kernel
     LmWs lm;
+    int64_t s0 = 0, s1 = 0;      // source positions of this call's shard
+    bool ordered = false;
     int nb = 2, spl = 1, nitems = 0, cl = 1, slots = 1;
     std::vector<CentralityUnit> hunits;
     struct Lists {           // Centrality: frontiers of each non-frontier node (entries, exits)
@@ -1610,55 +1689,23 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
     return BCPP_OK;
 }
 
-int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin, const int32_t* Ssing,
-               int32_t nsing, const int32_t* Ssrc, int32_t nsrc, const uint8_t* dflag, const int32_t* part, int32_t k,
-               const bcpp_opts& o, double scale, double* bc_out, PpRun& r, Timer* tb,
-               const Skeleton* reuse = nullptr) {
-    const int32_t n = g->n;
+// Batches of 32 targets and the workspace of Brandes_SK and Centrality: on the level-mask kernel where it serves them,
+// unless masks = false, else on the lockstep kernel.
+int pp_batches(bcpp_ctx* c, PpRun& r, bool masks) {
+    const bcpp_graph* g = &r.g;
+    const bcpp_opts& o = r.o;
+    const Skeleton& K = r.K;
+    const int32_t n = g->n, N = K.N;
+    const int64_t ns = r.nt;
     const bool fp32 = o.precision == BCPP_FP32_DELTA;
-    const int64_t ns = nsrc;
-    r.g = *g; r.o = o; r.scale = scale; r.bc_out = bc_out; r.dflag = dflag;
-    // Step 1: Build_SK on P' (every node of Ssing a singleton part)
-    if (tb) tb->start();
-    Skeleton& K = r.K;
-    CK_RC(build_sk(c, g, Ssing, nsing, part, k, wmax, Tin, o, K, reuse));
-    if (tb) tb->stop();
-    const int32_t N = K.N;
-    // targets in batch order (grouped by their original part when requested), as skeleton ids
-    CK_ALLOC(r.tsk.alloc(c, ns));
-    {
-        const int32_t* Suse = Ssrc;
-        if (o.order_sources && ns > 2 * LS_LANES) {
-            CK_RC(order_targets(c, g, g->directed ? Tin->rp.p : g->row_ptr, g->directed ? Tin->col.p : g->col,
-                                g->directed ? (g->w ? Tin->w.p : nullptr) : g->w, wmax, Ssrc, ns, part, k, r.ord));
-            Suse = r.ord.out.p;
-        }
-        sk_target_ids(Suse, (int32_t)ns, K.skid.p, r.tsk.p, c->stream);
-        c->launches++;
-    }
-    r.nt = (int32_t)ns;
-    r.unit = K.wmax_sk == 1;
-    r.mult = K.mmax_sk > 1;
-    r.nb = (int)K.wmax_sk + 1;
-    int64_t s0, s1;
-    shard_sources(o, r.nt, s0, s1);
-    // Centrality work units: chunks of 64 non-frontier nodes of parts with frontiers
-    int32_t interior = 0;
-    for (int32_t i = 0; i < K.kp; i++) {
-        const int32_t sz = K.h_pstart[i + 1] - K.h_pstart[i];
-        if (K.h_nf[i] < 1 || sz <= K.h_nf[i]) continue;
-        for (int32_t v0 = K.h_nf[i]; v0 < sz; v0 += 64) {
-            r.hunits.push_back({i, v0, std::min(sz, v0 + 64), interior});
-            interior += std::min(sz, v0 + 64) - v0;
-        }
-    }
-    // without non-frontier nodes Brandes_SK runs alone and may use 64-source batches
-    r.spl = r.hunits.empty() ? choose_spl(c, s1 - s0, o) : 1;
-    std::vector<LsItem> hitems = make_items(0, s0, s1, 32 * r.spl);
-    if (N > 0 && !hitems.empty() && lm_serves(c, o, r.spl, N, K.arcs, K.wmax_sk)) {
+    r.levels = r.rows_by_item = false;
+    r.lm.release();
+    r.ws.release();
+    std::vector<LsItem> hitems = make_items(0, r.s0, r.s1, 32 * r.spl);
+    if (masks && N > 0 && !hitems.empty() && lm_serves(c, o, r.spl, N, K.arcs, K.wmax_sk)) {
         r.lm.mean_degree = (double)K.arcs / N;
         // skeleton distances are the distances in G
-        const OrderWs* ord = o.order_sources && ns > 2 * LS_LANES ? &r.ord : nullptr;
+        const OrderWs* ord = r.ordered ? &r.ord : nullptr;
         const int lcap = lm_levels(g->w != nullptr, g->directed != 0, ord);
         r.lm.probe = !lm_bounded(g->w != nullptr, g->directed != 0, ord);
         if (r.hunits.empty() && r.unit && ord && lm_dense_deep(*ord, ns, n))
@@ -1671,8 +1718,8 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
     r.cl = (!hitems.empty() && r.spl == 1) ? choose_cluster(c, (int)hitems.size(), o) : 1;
     if (r.spl == 1 && r.hunits.empty() && !r.levels) {
         // without a Centrality step (whose cost grows with the batch count, not their width)
-        const int b = balanced_width(s1 - s0, slot_capacity(c, o, r.cl), 32);
-        if (b < 32) hitems = make_items(0, s0, s1, b);
+        const int b = balanced_width(r.s1 - r.s0, slot_capacity(c, o, r.cl), 32);
+        if (b < 32) hitems = make_items(0, r.s0, r.s1, b);
     }
     r.nitems = (int)hitems.size();
     const int ef = entry_factor(c, !r.unit, r.spl);
@@ -1709,6 +1756,58 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
                           r.rows_by_item ? r.nitems : 0, r.rows_by_item ? r.nitems : 0));
     r.ws.narrow = r.hunits.empty() && use_narrow(c, !r.unit);   // Centrality reads int32 rows
     if (r.nitems > 0) {
+        CK_ALLOC(r.items.alloc(c, r.nitems));
+        CK_RC(to_dev(c, r.items.p, hitems.data(), r.nitems));
+    }
+    return BCPP_OK;
+}
+
+int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin, const int32_t* Ssing,
+               int32_t nsing, const int32_t* Ssrc, int32_t nsrc, const uint8_t* dflag, const int32_t* part, int32_t k,
+               const bcpp_opts& o, double scale, double* bc_out, PpRun& r, Timer* tb,
+               const Skeleton* reuse = nullptr) {
+    const int32_t n = g->n;
+    const bool fp32 = o.precision == BCPP_FP32_DELTA;
+    const int64_t ns = nsrc;
+    r.g = *g; r.o = o; r.scale = scale; r.bc_out = bc_out; r.dflag = dflag;
+    // Step 1: Build_SK on P' (every node of Ssing a singleton part)
+    if (tb) tb->start();
+    Skeleton& K = r.K;
+    CK_RC(build_sk(c, g, Ssing, nsing, part, k, wmax, Tin, o, K, reuse));
+    if (tb) tb->stop();
+    const int32_t N = K.N;
+    // targets in batch order (grouped by their original part when requested), as skeleton ids
+    CK_ALLOC(r.tsk.alloc(c, ns));
+    {
+        const int32_t* Suse = Ssrc;
+        if (o.order_sources && ns > 2 * LS_LANES) {
+            CK_RC(order_targets(c, g, g->directed ? Tin->rp.p : g->row_ptr, g->directed ? Tin->col.p : g->col,
+                                g->directed ? (g->w ? Tin->w.p : nullptr) : g->w, wmax, Ssrc, ns, part, k, r.ord));
+            Suse = r.ord.out.p;
+            r.ordered = true;
+        }
+        sk_target_ids(Suse, (int32_t)ns, K.skid.p, r.tsk.p, c->stream);
+        c->launches++;
+    }
+    r.nt = (int32_t)ns;
+    r.unit = K.wmax_sk == 1;
+    r.mult = K.mmax_sk > 1;
+    r.nb = (int)K.wmax_sk + 1;
+    shard_sources(o, r.nt, r.s0, r.s1);
+    // Centrality work units: chunks of 64 non-frontier nodes of parts with frontiers
+    int32_t interior = 0;
+    for (int32_t i = 0; i < K.kp; i++) {
+        const int32_t sz = K.h_pstart[i + 1] - K.h_pstart[i];
+        if (K.h_nf[i] < 1 || sz <= K.h_nf[i]) continue;
+        for (int32_t v0 = K.h_nf[i]; v0 < sz; v0 += 64) {
+            r.hunits.push_back({i, v0, std::min(sz, v0 + 64), interior});
+            interior += std::min(sz, v0 + 64) - v0;
+        }
+    }
+    // without non-frontier nodes Brandes_SK runs alone and may use 64-source batches
+    r.spl = r.hunits.empty() ? choose_spl(c, r.s1 - r.s0, o) : 1;
+    CK_RC(pp_batches(c, r, true));
+    if (r.nitems > 0) {
         CK_ALLOC(r.sk_in_s.alloc(c, N));
         if (g->directed) {   // skeleton in-arcs
             CK_ALLOC(r.icnt.alloc(c, (int64_t)N + 1));
@@ -1743,8 +1842,6 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
             CK_RC(centrality_lists(c, r, interior, false, r.entry));
             if (g->directed) CK_RC(centrality_lists(c, r, interior, true, r.exit));
         }
-        CK_ALLOC(r.items.alloc(c, r.nitems));
-        CK_RC(to_dev(c, r.items.p, hitems.data(), r.nitems));
     }
     return BCPP_OK;
 }
@@ -1860,6 +1957,16 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
     return BCPP_OK;
 }
 
+// The same again on the lockstep kernel, after the level-mask kernel gave the batches back; the skeleton, the order
+// of the targets and the frontier lists stay.
+int pp_in_lockstep(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce, bcpp_stats* st) {
+    const bool worst = past_usual_rows(c, r.lm.lcap);
+    return run_in_lockstep(c, st, worst, [&] {
+        CK_RC(pp_batches(c, r, false));
+        return pp_emit(c, r, tbr, tce);
+    });
+}
+
 void pp_fill_stats(const PpRun& r, bcpp_stats* st) {
     if (!st) return;
     st->skel_nodes = r.K.N;
@@ -1876,8 +1983,7 @@ void pp_fill_stats(const PpRun& r, bcpp_stats* st) {
 int brandes_pp_core(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin, const int32_t* Ssing,
                     int32_t nsing, const int32_t* Ssrc, int32_t nsrc, const uint8_t* dflag, const int32_t* part,
                     int32_t k, const bcpp_opts& o, double scale, double* bc_out, bcpp_stats* st, Timer& tb, Timer& tbr,
-                    Timer& tce, const Skeleton* reuse = nullptr) {
-    PpRun r;
+                    Timer& tce, PpRun& r, const Skeleton* reuse = nullptr) {
     CK_RC(pp_prepare(c, g, wmax, Tin, Ssing, nsing, Ssrc, nsrc, dflag, part, k, o, scale, bc_out, r, &tb, reuse));
     CK_RC(pp_emit(c, r, &tbr, &tce));
     pp_fill_stats(r, st);
@@ -1952,6 +2058,9 @@ int brandes_pp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t n
     CK_RC(pp_top_emit(c, t, &tbr, &tce));
     if (!t.trivial) pp_fill_stats(t.run, st);
     int rc = finish_status(c, st);
+    const bool back = rc == RC_GIVEN_BACK;
+    if (back) rc = pp_in_lockstep(c, t.run, &tbr, &tce, st);
+    count_batches(c, t.run.levels, t.run.nitems, back);
     tt.stop();
     if (st) {
         st->ms_build_sk = tb.acc;
@@ -2009,10 +2118,13 @@ int brandes_pp_st_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* Ssrc, int
     if (g->directed) CK_RC(build_in_csr(c, g, Tin));
     Timer tb(c), tbr(c), tce(c);
     const bool halve = !g->directed && o.halve_undirected != 0;
-    int rc = brandes_pp_core(c, g, wmax, &Tin, uni.p, (int32_t)nuni, Ssrc, nsrc, dflag.p, part, k, o,
-                             halve ? 0.5 : 1.0, bc_out, st, tb, tbr, tce);
-    if (rc) return rc;
-    rc = finish_status(c, st);
+    PpRun run;
+    CK_RC(brandes_pp_core(c, g, wmax, &Tin, uni.p, (int32_t)nuni, Ssrc, nsrc, dflag.p, part, k, o,
+                          halve ? 0.5 : 1.0, bc_out, st, tb, tbr, tce, run));
+    int rc = finish_status(c, st);
+    const bool back = rc == RC_GIVEN_BACK;
+    if (back) rc = pp_in_lockstep(c, run, &tbr, &tce, st);
+    count_batches(c, run.levels, run.nitems, back);
     tt.stop();
     if (st) {
         st->ms_build_sk = tb.acc;
@@ -2056,8 +2168,25 @@ struct PairLane {
     DBuf<uint8_t> dflag;
     DBuf<double> tmp, sum, comp;
     std::unique_ptr<Timer> tb, tbr, tce;
+    std::unique_ptr<PpRun> run;     // the pair in flight
     int64_t calls = 0;
 };
+
+// The lane's pair in flight into its running sums (waits for the lane's stream).
+int finish_pair(PairLane& L, int32_t n) {
+    if (!L.run) return BCPP_OK;
+    bcpp_ctx* lc = L.sc.c;
+    int rc = finish_status(lc, nullptr);
+    const bool back = rc == RC_GIVEN_BACK;
+    if (back) rc = pp_in_lockstep(lc, *L.run, L.tbr.get(), L.tce.get(), nullptr);
+    count_batches(lc, L.run->levels, L.run->nitems, back);
+    if (rc != BCPP_OK && rc != BCPP_EOVERFLOW_SIGMA) return rc;
+    L.run.reset();
+    accumulate_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 8192), 256, 0, lc->stream>>>(L.tmp.p, n, L.sum.p, L.comp.p);
+    lc->launches++;
+    L.calls++;
+    return BCPP_OK;
+}
 
 // Brandes++All (Alg. 3): Build_SK once on P, then for every ordered pair (i, j) of non-empty
 // parts Brandes_SK with S_sc = P_i and S_dest = P_j (both expanded into singletons) and
@@ -2145,6 +2274,7 @@ int brandes_pp_all_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* part, in
             if (ni == 0 || (i == j && ni < 2)) continue;
             PairLane& L = lanes[p++ % ALL_LANES];
             bcpp_ctx* lc = L.sc.c;
+            CK_RC(finish_pair(L, n));
             part_flag_kernel<<<blocks, 256, 0, lc->stream>>>(part, n, j, L.dflag.p);
             lc->launches++;
             // singletons: P_i followed by P_j (P_i alone when i == j)
@@ -2155,11 +2285,10 @@ int brandes_pp_all_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* part, in
                                         lc->stream));
                 nsing += nj;
             }
+            L.run.reset(new (std::nothrow) PpRun());
+            if (!L.run) return BCPP_ENOMEM;
             CK_RC(brandes_pp_core(lc, g, wmax, &Tin, L.pair.p, nsing, L.pair.p, ni, L.dflag.p, part, k, o, 1.0,
-                                  L.tmp.p, nullptr, *L.tb, *L.tbr, *L.tce, &K0));
-            accumulate_kernel<<<blocks, 256, 0, lc->stream>>>(L.tmp.p, n, L.sum.p, L.comp.p);
-            lc->launches++;
-            L.calls++;
+                                  L.tmp.p, nullptr, *L.tb, *L.tbr, *L.tce, *L.run, &K0));
         }
     }
     // join: the lanes' sums (and compensations) in lane order, and their status flags
@@ -2168,7 +2297,9 @@ int brandes_pp_all_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* part, in
     int64_t calls = 0;
     for (PairLane& L : lanes) {
         bcpp_ctx* lc = L.sc.c;
+        CK_RC(finish_pair(L, n));
         CK_RC(sync_flags(lc));   // waits for the lane's stream
+        for (int i = 0; i < 3; i++) c->ran[i] += lc->ran[i];
         for (int f = 0; f < FLAG_COUNT; f++) merged[f] |= lc->hflags[f];
         accumulate_kernel<<<blocks, 256, 0, c->stream>>>(L.sum.p, n, sum.p, comp.p);
         accumulate_kernel<<<blocks, 256, 0, c->stream>>>(L.comp.p, n, sum.p, comp.p);
@@ -2271,32 +2402,35 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
     P.srcs = srcs.p;
     P.flags = c->flags;
     P.phase_ns = c->phase;
-    if (levels) {
-        CK_RC(lm_emit(c, lm, A, P, items.p, g->w ? wmax : 1, o.halve_undirected ? 0.5 : 1.0, bc_out, &tb));
-        int rc = finish_status(c, st);
-        tt.stop();
-        if (st) {
-            st->ms_brandes_sk = tb.acc;
-            st->ms_total = tt.acc;
-        }
-        return rc;
-    }
-    const int slots =
-        choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxn, nb, fp32, entry_factor(c, g->w != nullptr, spl), spl),
-                     (int64_t)n * 24);
+    const double scale = o.halve_undirected ? 0.5 : 1.0;
     SlotWs ws;
-    CK_RC(alloc_slots(c, ws, slots, maxn, nb, fp32, n, spl, entry_factor(c, g->w != nullptr, spl), false));
-    ws.narrow = use_narrow(c, g->w != nullptr);
-    CK_RC(init_slots(c, ws));
-    P.item_counter = ws.counter.p;
-    tb.start();
-    ls_launch(fp32, true, A, P, ws.W, items.p, nitems, slots, c->stream, spl, 1, ws.narrow);
-    c->launches++;
-    CK_CUDA(cudaGetLastError());
-    combine_launch(ws.W.bc_sum, ws.W.bc_cmp, slots, n, n, o.halve_undirected ? 0.5 : 1.0, bc_out, c->stream);
-    c->launches++;
-    tb.stop();
+    auto lockstep = [&] {
+        lm.release();
+        ws.release();
+        const int ef = entry_factor(c, g->w != nullptr, spl);
+        const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxn, nb, fp32, ef, spl), (int64_t)n * 24);
+        CK_RC(alloc_slots(c, ws, slots, maxn, nb, fp32, n, spl, ef, false));
+        ws.narrow = use_narrow(c, g->w != nullptr);
+        CK_RC(init_slots(c, ws));
+        P.item_counter = ws.counter.p;
+        tb.start();
+        ls_launch(fp32, true, A, P, ws.W, items.p, nitems, slots, c->stream, spl, 1, ws.narrow);
+        c->launches++;
+        CK_CUDA(cudaGetLastError());
+        combine_launch(ws.W.bc_sum, ws.W.bc_cmp, slots, n, n, scale, bc_out, c->stream);
+        c->launches++;
+        tb.stop();
+        return BCPP_OK;
+    };
+    if (levels) {
+        CK_RC(lm_emit(c, lm, A, P, items.p, g->w ? wmax : 1, scale, bc_out, &tb));
+    } else {
+        CK_RC(lockstep());
+    }
     int rc = finish_status(c, st);
+    const bool back = rc == RC_GIVEN_BACK;
+    if (back) rc = run_in_lockstep(c, st, past_usual_rows(c, lm.lcap), lockstep);
+    count_batches(c, levels && !back, nitems, back);
     tt.stop();
     if (st) {
         st->ms_brandes_sk = tb.acc;
@@ -2431,31 +2565,41 @@ int sssp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* src, int32_t nsrc,
         A.irp = g->row_ptr; A.icol = g->col; A.iw = (const int32_t*)g->w;
     }
     A.node_off = node_off.p;
+    bool done = false;
     if (lm_serves(c, o, 1, n, g->num_arcs, g->w ? wmax : 1)) {
-        bool done = false;
         CK_RC(sssp_levels(c, g, A, items.p, nitems, src, wmax, dist_out, sigma_out, &done));
-        if (done) return finish_status(c, nullptr);
+        if (done) {
+            const int rc = finish_status(c, nullptr);
+            if (rc != RC_GIVEN_BACK) {
+                count_batches(c, true, nitems, false);
+                return rc;
+            }
+        }
     }
     // a batch holds each source at most once: split repeated sources across batches is not
     // needed because LS_SSSP lanes are independent rows (a repeat only repeats the row)
-    const int nb = g->w ? (int)wmax + 1 : 2;
-    const int ef = entry_factor(c, g->w != nullptr, 1);
-    const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(n, nb, false, ef), 0);
-    SlotWs ws;
-    CK_RC(alloc_slots(c, ws, slots, n, nb, false, 0, 1, ef));
-    LsParams P{};
-    P.mode = LS_SSSP;
-    P.nb = nb;
-    P.srcs = src;
-    P.dbg_d = dist_out;
-    P.dbg_s = sigma_out;
-    P.dbg_n = n;
-    P.item_counter = ws.counter.p;
-    P.flags = c->flags;
-    ls_launch(false, !g->directed, A, P, ws.W, items.p, nitems, slots, c->stream);
-    c->launches++;
-    CK_CUDA(cudaGetLastError());
-    return finish_status(c, nullptr);
+    count_batches(c, false, nitems, done);
+    // (rows are of full width here, and only the lists could prove too small: the worst case at once for deep graphs)
+    return run_in_lockstep(c, nullptr, done, [&] {
+        const int nb = g->w ? (int)wmax + 1 : 2;
+        const int ef = entry_factor(c, g->w != nullptr, 1);
+        const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(n, nb, false, ef), 0);
+        SlotWs ws;
+        CK_RC(alloc_slots(c, ws, slots, n, nb, false, 0, 1, ef));
+        LsParams P{};
+        P.mode = LS_SSSP;
+        P.nb = nb;
+        P.srcs = src;
+        P.dbg_d = dist_out;
+        P.dbg_s = sigma_out;
+        P.dbg_n = n;
+        P.item_counter = ws.counter.p;
+        P.flags = c->flags;
+        ls_launch(false, !g->directed, A, P, ws.W, items.p, nitems, slots, c->stream);
+        c->launches++;
+        CK_CUDA(cudaGetLastError());
+        return BCPP_OK;
+    });
 }
 
 int skeleton_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS, const int32_t* part, int32_t k,
@@ -2675,8 +2819,26 @@ int plan_build(bcpp_plan* p) {
     return rc;
 }
 
+// The evaluation captured again on the lockstep kernel; checks, order, skeleton and lists stay.
+int plan_to_lockstep(bcpp_plan* p) {
+    bcpp_ctx* c = p->c;
+    if (p->run) cudaGraphExecDestroy(p->run);
+    p->run = nullptr;
+    if (p->order_factor < 64 && past_usual_rows(c, p->kind == 1 ? p->plain->lm.lcap : p->pp->run.lm.lcap))
+        p->order_factor = 64;
+    c->order_factor = p->order_factor;
+    int rc = p->kind == 1 ? plain_batches(c, *p->plain, false) : pp_batches(c, p->pp->run, false);
+    if (!rc)
+        rc = capture_graph(c, p->cs, [&] {
+            return p->kind == 1 ? plain_emit(c, *p->plain, nullptr) : pp_top_emit(c, *p->pp, nullptr, nullptr);
+        }, &p->run, &p->run_kernels);
+    c->order_factor = 8;
+    return rc;
+}
+
 int plan_replay(bcpp_plan* p, bcpp_stats* st) {
     bcpp_ctx* c = p->c;
+    if (!p->run) return BCPP_ECUDA;   // an earlier rebuild failed
     if (p->check) {
         CK_CUDA(cudaGraphLaunch(p->check, c->stream));
         CK_RC(sync_flags(c));
@@ -2725,9 +2887,11 @@ int plan_create(bcpp_ctx* c, int kind, const bcpp_graph* g, const int32_t* S, in
 template <class F>
 int with_capacity_retry(bcpp_ctx* c, F&& f) {
     c->order_factor = 8;
+    std::fill(c->ran, c->ran + 3, 0);
     int rc = f();
     if (rc == BCPP_ECAPACITY) {
         c->order_factor = 64;
+        std::fill(c->ran, c->ran + 3, 0);
         rc = f();
         c->order_factor = 8;
     }
@@ -2810,6 +2974,12 @@ void bcpp_destroy(bcpp_ctx* c) {
 }
 
 int64_t bcpp_workspace_bytes(const bcpp_ctx* c) { return c ? c->held() : 0; }
+
+int bcpp_last_batches(const bcpp_ctx* c, int64_t* out) {
+    if (!c || !out) return BCPP_EINVAL;
+    std::copy(c->ran, c->ran + 3, out);
+    return BCPP_OK;
+}
 
 int bcpp_csr_build(bcpp_ctx* c, int32_t n, int64_t m, const int32_t* eu, const int32_t* ev, const uint32_t* ew,
                    int32_t directed, int64_t* row_ptr_out, int32_t* col_out, uint32_t* w_out, int64_t* num_arcs_out) {
@@ -3028,12 +3198,20 @@ int bcpp_plan_launch(bcpp_plan* p, bcpp_stats* stats) {
     Timer tt(c);
     tt.start();
     int rc = plan_replay(p, stats);
+    const bool back = rc == RC_GIVEN_BACK;
+    if (back) {
+        rc = plan_to_lockstep(p);
+        if (rc == BCPP_OK) rc = plan_replay(p, stats);
+    }
     if (rc == BCPP_ECAPACITY && p->order_factor < 64) {
         // a batch outgrew the settled-entry list: rebuild once with the worst-case capacity
         p->order_factor = 64;
-        rc = plan_build(p);
+        rc = plan_to_lockstep(p);
         if (rc == BCPP_OK) rc = plan_replay(p, stats);
     }
+    std::fill(c->ran, c->ran + 3, 0);
+    if (p->plain) count_batches(c, p->plain->levels, p->plain->nitems, back);
+    if (p->pp) count_batches(c, p->pp->run.levels, p->pp->run.nitems, back);
     tt.stop();
     if (stats) {
         const uint32_t ovf = stats->sigma_overflow;

@@ -19,8 +19,12 @@ enum : int {
     FLAG_INVALID_WHY = 3,   // first reason code of an invalid input
     FLAG_DEPTH = 4,         // a one-byte distance or 32-bit path count would overflow (rerun with wide rows)
     FLAG_TIMEOUT = 5,       // a grid barrier gave up waiting
+    FLAG_MASKS = 6,         // the level-mask kernel gave batches back: MASKS_* bits
     FLAG_COUNT = 8
 };
+
+// FLAG_MASKS: more distance levels than provided for; a path count past 32 bits
+enum : uint32_t { MASKS_DEEP = 1, MASKS_COUNT = 2 };
 
 // reason codes written into FLAG_INVALID_WHY
 enum : uint32_t {

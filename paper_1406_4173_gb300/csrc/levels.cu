@@ -519,8 +519,8 @@ lm_kernel(const LmArgs A, const int sub_log) {
         return x;
     };
 
-    // an earlier wave proved too deep: the call reruns (only set past a barrier of this launch, if by it)
-    if (__ldcg(A.flags + FLAG_CAPACITY) != 0u) return;
+    // an earlier wave was given back, and with it the call (only set past a barrier of this launch, if by it)
+    if (__ldcg(A.flags + FLAG_MASKS) != 0u) return;
 
     // With few tiles per warp a unit is a part of a tile (32 >> sub_log rows), so that a level's last and
     // fullest tiles do not leave the other warps waiting (see lm_go for the rule).
@@ -585,11 +585,8 @@ lm_kernel(const LmArgs A, const int sub_log) {
     int depth = 0;
     for (int D = 1;; D++) {
         if (D >= A.lcap) {
-            // a later level than the masks provide for (or the last one, unseen): the call reruns
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                atomicOr(&A.flags[FLAG_DEPTH], 1u);
-                atomicOr(&A.flags[FLAG_CAPACITY], 1u);
-            }
+            // a later level than the masks provide for (or the last one, unseen): the pass is given back
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&A.flags[FLAG_MASKS], MASKS_DEEP);
             return;
         }
         bool any = false, wide = false, ovf = false;
@@ -656,18 +653,15 @@ lm_kernel(const LmArgs A, const int sub_log) {
         // every block reads the same word: nobody writes level D's status any more
         const uint32_t w = __ldcg(lvl + D);
         if (w & LVL_ERR) {
-            // a path count past 32 bits: the call reruns with 64-bit rows
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                atomicOr(&A.flags[FLAG_DEPTH], 1u);
-                atomicOr(&A.flags[FLAG_CAPACITY], 1u);
-            }
+            // a path count past 32 bits: the pass is given back
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&A.flags[FLAG_MASKS], MASKS_COUNT);
             return;
         }
         if (w & LVL_ANY) depth = D;
         if (D - depth >= wmax) break;
         // Too deep a graph shows early: a quarter of the way the pairs reached by now and by half of that
         // give the dimension that the balls around the sources grow with, and with it the level at which
-        // they hold every pair; past the levels provided for, the call reruns without going there first
+        // they hold every pair; past the levels provided for, the pass is given back without going there first
         // (grid 300 x 300 with weights up to 16, 500 sources: 112 -> 101 ms, 97 without the attempt).
         // Balls that hardly grow any more belong to stragglers, not to a deep graph.
         if (!TABLE && A.probe && (D == A.lcap / 4 || D == A.lcap / 4 + 1)) {
@@ -676,10 +670,7 @@ lm_kernel(const LmArgs A, const int sub_log) {
                 probe_levels(A.lev, A.rows, D, wmax, bdepth, A.item_tile0 ? A.tile_item + A.tile_base : nullptr,
                              A.item_base, A.tpb, probe);
             } else if (looks_deep(probe)) {
-                if (blockIdx.x == 0 && threadIdx.x == 0) {
-                    atomicOr(&A.flags[FLAG_DEPTH], 1u);
-                    atomicOr(&A.flags[FLAG_CAPACITY], 1u);
-                }
+                if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&A.flags[FLAG_MASKS], MASKS_DEEP);
                 return;
             }
         }

@@ -6,8 +6,8 @@
 
 namespace bcpp {
 
-// Distance levels a launch provides for; a batch that reaches a later one aborts with FLAG_DEPTH and
-// FLAG_CAPACITY and the call reruns on the lockstep kernel.
+// Distance levels a launch provides for; a batch that reaches a later one ends the pass with FLAG_MASKS, and the
+// caller runs it on the lockstep kernel.
 constexpr int LM_MAX_LEVELS = 256;
 // Largest arc weight: every row that is not settled on all its sources looks at its in-arcs once per
 // distance value, so the forward cost grows with the number of distance values.
