@@ -641,6 +641,7 @@ struct OrderWs {
     int64_t ns = 0;
     int32_t n = 0, k = 0;
     int32_t depth = 0;        // deepest level from the hub
+    int32_t rest = 0;         // nodes outside the hub's component with two arcs or more (unit weights)
     const int32_t* S = nullptr;
     const int32_t* part = nullptr;
     DBuf<int32_t> queue;      // unit weights: [n] nodes in discovery order
@@ -714,7 +715,7 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
         CK_ALLOC(w.tmp.alloc(c, scan_tmp_elems(n)));
     }
     if (!g->w) {
-        DBuf<int32_t> par(c, n), depth(c, 1);
+        DBuf<int32_t> par(c, n), depth(c, 2);
         DBuf<uint32_t> ctl(c, order_ctl_words(c->num_sms));
         CK_ALLOC(par); CK_ALLOC(depth); CK_ALLOC(ctl);
         if (!all || part) CK_ALLOC(w.queue.alloc(c, n));
@@ -724,7 +725,11 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
         CK_CUDA(order_bfs_launch(n, g->row_ptr, g->col, par.p, all && !part ? w.out.p : w.queue.p, ctl.p, depth.p,
                                  c->flags, c->num_sms, c->stream));
         c->launches++;
-        return to_host(c, &w.depth, depth.p, 1);
+        int32_t h[2] = {0, 0};
+        CK_RC(to_host(c, h, depth.p, 2));
+        w.depth = h[0];
+        w.rest = h[1];
+        return BCPP_OK;
     }
     // levels from the hub (the node of largest degree)
     DBuf<unsigned long long> best(c, 1);
@@ -851,7 +856,7 @@ struct LmWave {
 struct LmWs {
     std::vector<LmWave> waves;
     int lcap = 0;
-    bool probe = true;         // no bound on the levels
+    bool bounded = false;      // the levels are proven to be enough (lm_bounded)
     bool narrow = true;
     bool fp32 = false;         // FP32 dependencies
     double mean_degree = 16;   // arcs per node
@@ -893,16 +898,24 @@ bool lm_serves(const bcpp_ctx* c, const bcpp_opts& o, int spl, int32_t n, int64_
            n < (1 << 25) && wmax <= LM_MAX_WEIGHT;
 }
 
-// Levels to provide for: with unit weights on an undirected graph whose levels from the hub are known,
-// no node of the hub's component is further from another than twice the deepest level.
+// Largest distance of an undirected unit-weight graph whose levels from the hub are known: no node of the hub's
+// component is further from another than twice the deepest level, and the inner nodes of a shortest path in another
+// component all have two arcs.
+int64_t lm_diameter(const OrderWs& ord) { return std::max<int64_t>(2 * (int64_t)ord.depth, (int64_t)ord.rest + 1); }
+
+// Whether that bounds the levels (not when many nodes lie in other components, where it says little).
+bool lm_bounded(bool weighted, bool directed, const OrderWs* ord) {
+    return !weighted && !directed && ord && ord->depth <= LM_MAX_LEVELS &&
+           lm_diameter(*ord) <= std::max<int64_t>(60, 2 * (int64_t)ord->depth);
+}
+
+// Levels to provide for.
 int lm_levels(bool weighted, bool directed, const OrderWs* ord) {
     if (weighted) return LM_MAX_LEVELS;
     if (!ord) return 64;
-    return std::max(directed ? 64 : 24, 2 * std::min(ord->depth, LM_MAX_LEVELS) + 4);
+    if (lm_bounded(weighted, directed, ord)) return (int)std::max<int64_t>(24, lm_diameter(*ord) + 4);
+    return std::max(64, 2 * std::min(ord->depth, LM_MAX_LEVELS) + 4);
 }
-
-// ... and then the masks are known to be enough.
-bool lm_bounded(bool weighted, bool directed, const OrderWs* ord) { return !weighted && !directed && ord; }
 
 // Many levels and many targets: batches of neighbours, which the lockstep kernel finds at few distances from each node,
 // while every level here looks at every row that is still open.  Random communities of 1,000 in a chain, every
@@ -1017,7 +1030,8 @@ LmArgs lm_wave_args(const LmWs& L, const LmWave& w, const LsArena& A, const LsPa
     a.lev = L.lev.p; a.seen = L.seen.p; a.sg = L.sg.p; a.cc = L.cc.p; a.dsum = L.dsum.p;
     a.rows = (int64_t)w.ntiles * 32;
     a.lcap = L.lcap;
-    a.probe = L.probe;
+    a.bounded = L.bounded && wmax > 1;   // (unit weights end at an empty level, also when a plan's graph has changed)
+    a.probe = !L.bounded;
     a.wmax = (int32_t)wmax;
     a.mean_degree = L.mean_degree;
     a.ctl = L.ctl.p;
@@ -1121,7 +1135,7 @@ int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks) {
     if (fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.lm.fp32 = fp32;
     r.lm.mean_degree = (double)g->num_arcs / n;
-    r.lm.probe = !lm_bounded(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr);
+    r.lm.bounded = lm_bounded(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr);
     if (masks && lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) &&
         !(r.ordered && lm_dense_deep(r.ord, r.ns, n)))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
@@ -1667,7 +1681,8 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         a.dsum = r.lm.dsum.p; a.drow = W.d;
         a.rows = (int64_t)a.ntiles * 32;
         a.lcap = r.lm.lcap;
-        a.probe = r.lm.probe;
+        a.bounded = r.lm.bounded;
+        a.probe = !r.lm.bounded;
         a.wmax = (int32_t)K.wmax_sk;
         a.mean_degree = r.lm.mean_degree;
         a.ctl = r.lm.ctl.p;
@@ -1707,7 +1722,7 @@ int pp_batches(bcpp_ctx* c, PpRun& r, bool masks) {
         // skeleton distances are the distances in G
         const OrderWs* ord = r.ordered ? &r.ord : nullptr;
         const int lcap = lm_levels(g->w != nullptr, g->directed != 0, ord);
-        r.lm.probe = !lm_bounded(g->w != nullptr, g->directed != 0, ord);
+        r.lm.bounded = lm_bounded(g->w != nullptr, g->directed != 0, ord);
         if (r.hunits.empty() && r.unit && ord && lm_dense_deep(*ord, ns, n))
             ;   // on the lockstep kernel
         else if (r.hunits.empty())

@@ -585,6 +585,7 @@ lm_kernel(const LmArgs A, const int sub_log) {
     int depth = 0;
     for (int D = 1;; D++) {
         if (D >= A.lcap) {
+            if (A.bounded) break;   // (the empty levels up to the largest weight are cut short)
             // a later level than the masks provide for (or the last one, unseen): the pass is given back
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&A.flags[FLAG_MASKS], MASKS_DEEP);
             return;

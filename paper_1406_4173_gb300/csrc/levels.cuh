@@ -47,6 +47,7 @@ struct LmArgs {
     const int32_t* bc_map;      // global node -> index of the sums over sources (nullptr = same)
     int64_t rows;               // 32 ntiles
     int32_t lcap;               // levels provided for
+    bool bounded;               // no distance reaches lcap: a pass that ends there is complete
     bool probe;                 // no bound on the levels is known: give up early on a graph that looks too deep
     int32_t wmax;
     double mean_degree;         // arcs per node

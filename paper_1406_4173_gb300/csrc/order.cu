@@ -251,17 +251,28 @@ order_bfs_kernel(int32_t n, const int64_t* __restrict__ rp, const int32_t* __res
         qe += all;
         if (!grid_barrier(ctl, flags)) return;
     }
-    if (tid == 0) *depth = L;
+    if (tid == 0) {
+        depth[0] = L;
+        depth[1] = 0;
+    }
     if (qe >= n) return;
     // the nodes not placed, by id
     const int64_t per = ((int64_t)n + nw - 1) / nw;
     const int64_t v0 = min((int64_t)n, wid * per), v1 = min((int64_t)n, v0 + per);
-    int c = 0;
-    for (int64_t v = v0 + lane; v < v1; v += 32) c += __ldcg(par + v) == INT32_MAX;
+    int c = 0, c2 = 0;
+    for (int64_t v = v0 + lane; v < v1; v += 32) {
+        const bool on = __ldcg(par + v) == INT32_MAX;
+        c += on;
+        c2 += on && __ldg(rp + v + 1) - __ldg(rp + v) >= 2;
+    }
     c = warp_sum(c);
+    c2 = warp_sum(c2);
     // (every block has read the last level's totals: it passed unit_prefix before or after the barrier below)
     if (!grid_barrier(ctl, flags)) return;
-    if (lane == 0) __stcg(tot + wid, c);
+    if (lane == 0) {
+        __stcg(tot + wid, c);
+        if (c2) atomicAdd(depth + 1, c2);
+    }
     if (!grid_barrier(ctl, flags)) return;
     int64_t before, all;
     unit_prefix(tot, before, all);

@@ -7,7 +7,8 @@ namespace bcpp {
 int64_t order_ctl_words(int num_sms);   // control block of order_bfs_launch, in 32-bit words
 
 // queue[0 .. n) = the nodes in breadth-first discovery order from the node of largest degree (unit weights; smallest id
-// on ties), the unreached ones behind them by id; *depth = the deepest level.  par: n words of scratch.
+// on ties), the unreached ones behind them by id; depth[0] = the deepest level, depth[1] = unreached nodes with two arcs
+// or more.  par: n words of scratch.
 // Levels past ORDER_MAX_LEVELS count as unreached.
 constexpr int ORDER_MAX_LEVELS = 4096;
 cudaError_t order_bfs_launch(int32_t n, const int64_t* rp, const int32_t* col, int32_t* par, int32_t* queue,

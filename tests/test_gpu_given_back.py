@@ -123,3 +123,76 @@ def test_plan_moves_once(bc, ctx, pp):
             assert b["levels"] == 0 and (b["given_back"] > 0) == (given_back > 0)
     finally:
         plan.close()
+
+
+# ---------------------------------------------------------------------------- levels that are known to be enough
+def tree(n, b):
+    v = np.arange(1, n, dtype=np.int32)
+    return gen.EdgeList(n=n, src=((v - 1) // b).astype(np.int32), dst=v)
+
+
+def subtrees(n, b, level):
+    """Part 0: the top of the tree; then one part per subtree hanging at the level."""
+    first = (b ** level - 1) // (b - 1)
+    anc = np.arange(n)
+    while (anc >= first * b + 1).any():
+        anc = np.where(anc >= first * b + 1, (anc - 1) // b, anc)
+    return np.where(np.arange(n) < first, 0, anc - first + 1).astype(np.int32)
+
+
+def star_beside_path(leaves, k):
+    i = np.arange(1, leaves + 1)
+    p = leaves + 1 + np.arange(k)
+    return gen.EdgeList(n=leaves + 1 + k, src=np.concatenate([np.zeros(leaves, np.int64), p[:-1]]).astype(np.int32),
+                        dst=np.concatenate([i, p[1:]]).astype(np.int32))
+
+
+def hub_between_chains(side, com):
+    """`side` communities (complete graphs) in a row on either side of a hub of many leaves."""
+    src, dst, off = [], [], 0
+    for _ in range(2 * side):
+        a, b = np.triu_indices(com, 1)
+        src.append(a + off), dst.append(b + off)
+        if off:
+            src.append([off - 1]), dst.append([off])
+        off += com
+    hub, mid = off, side * com
+    src += [[hub, hub], np.full(60, hub)]
+    dst += [[mid - 1, mid], hub + 1 + np.arange(60)]
+    return gen.EdgeList(n=hub + 61, src=np.concatenate(src).astype(np.int32), dst=np.concatenate(dst).astype(np.int32),
+                        part=np.minimum(np.arange(hub + 61) // com, 2 * side).astype(np.int32))
+
+
+BOUNDED = {
+    # levels provided 32, deepest 26, skeleton weights up to 16
+    "binary-tree": (tree(16383, 2), subtrees(16383, 2, 4), 100),
+    "ternary-tree": (tree(29524, 3), subtrees(29524, 3, 3), 100),
+    "hub-between-chains": (hub_between_chains(6, 12), None, 70),
+    # levels from the hub: 1; the path beside it: 39, and one more than the 60 that are provided for it at most
+    "star-path-40": (star_beside_path(100, 40), np.arange(141) % 3, 100),
+    "star-path-60": (star_beside_path(100, 60), np.arange(161) % 3, 100),
+}
+
+
+@pytest.mark.parametrize("name", list(BOUNDED))
+def test_bounded_levels_are_enough(bc, ctx, name):
+    g, part, k = BOUNDED[name]
+    part = (g.part if part is None else part).astype(np.int32)
+    S = gen.sample_targets(g.n, k, seed=5)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    for run in (lambda: bc.brandes(G, S, ctx=ctx), lambda: bc.brandes_pp(G, S, part, ctx=ctx)):
+        assert rel_err(run(), ref) <= FP64_TOL
+        b = ctx.last_batches()
+        assert b["levels"] > 0 and b["lockstep"] == 0, b
+
+
+def test_many_small_components(bc, ctx):
+    """Most nodes outside the hub's component: their count says little about the distances."""
+    k, m = 300, 12
+    src = (np.arange(k)[:, None] * m + np.arange(m - 1)).ravel()
+    g = gen.EdgeList(n=k * m + 9, src=np.concatenate([src, np.full(8, k * m)]).astype(np.int32),
+                     dst=np.concatenate([src + 1, k * m + 1 + np.arange(8)]).astype(np.int32))
+    ref, _ = oracle.brandes(g, None)
+    assert rel_err(bc.brandes(bc.graph_from_edgelist(g), None, ctx=ctx), ref) <= FP64_TOL
+    assert ctx.last_batches()["lockstep"] == 0
