@@ -545,10 +545,12 @@ struct Timer {
 };
 
 // Batches of a pass for bcpp_last_batches, once it is done.
-void count_batches(bcpp_ctx* c, bool levels, int64_t nitems, bool given_back) {
-    c->ran[levels ? 0 : 1] += nitems;
-    if (given_back) c->ran[2] += nitems;
+void count_batches(bcpp_ctx* c, int64_t levels, int64_t lockstep, int64_t given_back) {
+    c->ran[0] += levels;
+    c->ran[1] += lockstep;
+    c->ran[2] += given_back;
 }
+void count_batches(bcpp_ctx* c, bool levels, int64_t nitems) { count_batches(c, levels ? nitems : 0, levels ? 0 : nitems, 0); }
 
 // Status of a pass that the level-mask kernel gave back (finish_status): the caller runs it on the lockstep
 // kernel, with what it has prepared.  Never returned to the user.
@@ -593,6 +595,30 @@ int run_in_lockstep(bcpp_ctx* c, bcpp_stats* st, bool worst, F&& run) {
     c->order_factor = usual;
     return rc;
 }
+
+// The sums of a pass's finished batches, while those given back run on the lockstep kernel into the same output.
+__global__ void add_kernel(const double* x, int64_t n, double* out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] += x[i];
+}
+struct KeptSums {
+    DBuf<double> x;
+    int64_t n = 0;
+    explicit operator bool() const { return x.p != nullptr; }
+    int keep(bcpp_ctx* c, const double* out, int64_t count) {
+        CK_ALLOC(x.alloc(c, count));
+        n = count;
+        CK_CUDA(cudaMemcpyAsync(x.p, out, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
+        return BCPP_OK;
+    }
+    int add_to(bcpp_ctx* c, double* out) const {
+        if (!x.p) return BCPP_OK;
+        add_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 8192), 256, 0, c->stream>>>(x.p, n, out);
+        c->launches++;
+        CK_CUDA(cudaGetLastError());
+        return BCPP_OK;
+    }
+};
 
 // in-CSR (transpose) of a graph with uint32 weights
 struct InCsr {
@@ -863,6 +889,7 @@ struct LmWs {
     int32_t tpb = 0;           // uniform layout: tiles per batch
     int64_t nodes = 0;         // global nodes
     DBuf<uint32_t> lev, seen, ctl;
+    DBuf<uint32_t> back;       // per batch: given back
     DBuf<char> sg, cc;
     DBuf<double> dsum, bcs, bcc;
     DBuf<int32_t> tile0, tile_item;
@@ -870,7 +897,7 @@ struct LmWs {
 
     void release() {
         waves.clear();
-        lev.free(); seen.free(); ctl.free(); sg.free(); cc.free(); dsum.free(); bcs.free(); bcc.free();
+        lev.free(); seen.free(); ctl.free(); back.free(); sg.free(); cc.free(); dsum.free(); bcs.free(); bcc.free();
         tile0.free(); tile_item.free(); runs.free();
     }
 };
@@ -986,6 +1013,7 @@ int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_gr
     CK_ALLOC(L.sg.alloc(c, rows * 32 * (narrow ? 4 : 8)));
     CK_ALLOC(L.dsum.alloc(c, rows));
     CK_ALLOC(L.ctl.alloc(c, lm_ctl_words(lcap, most_items)));
+    CK_ALLOC(L.back.alloc(c, nitems));
     if (!forward) {
         CK_ALLOC(L.cc.alloc(c, rows * 32 * (L.fp32 ? 4 : 8)));
         CK_ALLOC(L.bcs.alloc(c, nodes));
@@ -1034,10 +1062,21 @@ LmArgs lm_wave_args(const LmWs& L, const LmWave& w, const LsArena& A, const LsPa
     a.probe = !L.bounded;
     a.wmax = (int32_t)wmax;
     a.mean_degree = L.mean_degree;
+    a.back = L.back.p + w.i0;
     a.ctl = L.ctl.p;
     a.flags = P.flags;
     a.phase_ns = P.phase_ns;
     return a;
+}
+
+// Which of nitems batches were given back, in order (waits for the stream).
+int lm_given_back(bcpp_ctx* c, const DBuf<uint32_t>& back, const std::vector<LsItem>& items, std::vector<LsItem>& out) {
+    std::vector<uint32_t> h(items.size());
+    CK_RC(to_host(c, h.data(), back.p, (int64_t)h.size()));
+    out.clear();
+    for (size_t i = 0; i < h.size(); i++)
+        if (h[i]) out.push_back(items[i]);
+    return BCPP_OK;
 }
 
 // All waves and the sum over sources (device work only): out = scale * sum.
@@ -1045,6 +1084,7 @@ int lm_emit(bcpp_ctx* c, LmWs& L, const LsArena& A, const LsParams& P, const LsI
             double scale, double* out, Timer* tb) {
     CK_CUDA(cudaMemsetAsync(L.bcs.p, 0, (size_t)L.nodes * sizeof(double), c->stream));
     CK_CUDA(cudaMemsetAsync(L.bcc.p, 0, (size_t)L.nodes * sizeof(double), c->stream));
+    CK_CUDA(cudaMemsetAsync(L.back.p, 0, (size_t)L.back.n * sizeof(uint32_t), c->stream));
     if (tb) tb->start();
     for (const LmWave& w : L.waves) {
         const LmArgs a = lm_wave_args(L, w, A, P, items, wmax);
@@ -1086,6 +1126,7 @@ struct PlainRun {
     LmWs lm;
     bool levels = false;           // on the level-mask kernel
     int64_t s0 = 0, s1 = 0;        // source positions of this call's shard
+    std::vector<LsItem> hitems;    // the batches
     int nitems = 0, slots = 0, spl = 1, cl = 1, nb = 2;
     LsArena A{};
     LsParams P{};
@@ -1119,8 +1160,8 @@ int plain_emit_checks(bcpp_ctx* c, PlainRun& r) {
 }
 
 // Batches of 32 sources (of the ordered targets) and the workspace of their passes: on the level-mask kernel where
-// it serves them, unless masks = false, else on the lockstep kernel.
-int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks) {
+// it serves them, unless masks = false, else on the lockstep kernel.  only: these batches instead of all.
+int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks, const std::vector<LsItem>* only = nullptr) {
     const bcpp_graph* g = &r.g;
     const int32_t n = g->n;
     const bcpp_opts& o = r.o;
@@ -1128,9 +1169,10 @@ int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks) {
     r.levels = false;
     r.lm.release();
     r.ws.release();
-    std::vector<LsItem> hitems = make_items(0, r.s0, r.s1, 32 * r.spl);
+    std::vector<LsItem>& hitems = r.hitems;
+    hitems = only ? *only : make_items(0, r.s0, r.s1, 32 * r.spl);
     r.cl = r.spl == 1 ? choose_cluster(c, (int)hitems.size(), o) : 1;
-    const int width = r.spl == 1 ? balanced_width(r.s1 - r.s0, slot_capacity(c, o, r.cl), 32) : 32;
+    const int width = r.spl == 1 && !only ? balanced_width(r.s1 - r.s0, slot_capacity(c, o, r.cl), 32) : 32;
     // (FP32 dependencies: the batches of the lockstep kernel, whose order of additions depends on them)
     if (fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.lm.fp32 = fp32;
@@ -1140,7 +1182,7 @@ int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks) {
         !(r.ordered && lm_dense_deep(r.ord, r.ns, n)))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
                        lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
-    if (!r.levels && width < 32) hitems = make_items(0, r.s0, r.s1, width);
+    if (!r.levels && !fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.nitems = (int)hitems.size();
     CK_ALLOC(r.items.alloc(c, r.nitems));
     CK_RC(to_dev(c, r.items.p, hitems.data(), r.nitems));
@@ -1259,13 +1301,21 @@ int plain_emit(bcpp_ctx* c, PlainRun& r, Timer* tb) {
     return plain_emit_passes(c, r, tb);
 }
 
-// The passes again on the lockstep kernel, after the level-mask kernel gave them back.
+// The batches that the level-mask kernel gave back, on the lockstep kernel; the sums of the others stay.
 int plain_in_lockstep(bcpp_ctx* c, PlainRun& r, Timer* tb, bcpp_stats* st) {
     const bool worst = past_usual_rows(c, r.lm.lcap);
-    return run_in_lockstep(c, st, worst, [&] {
-        CK_RC(plain_batches(c, r, false));
-        return plain_emit_passes(c, r, tb);
+    const int all = r.nitems;
+    std::vector<LsItem> some;
+    CK_RC(lm_given_back(c, r.lm.back, r.hitems, some));
+    KeptSums kept;
+    if ((int)some.size() < all) CK_RC(kept.keep(c, r.bc_out, r.g.n));
+    const int rc = run_in_lockstep(c, st, worst, [&] {
+        CK_RC(plain_batches(c, r, false, kept ? &some : nullptr));
+        CK_RC(plain_emit_passes(c, r, tb));
+        return kept.add_to(c, r.bc_out);
     });
+    count_batches(c, all - (int)some.size(), kept ? (int)some.size() : r.nitems, (int)some.size());
+    return rc;
 }
 
 int brandes_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS, const bcpp_opts& o, double* bc_out,
@@ -1276,9 +1326,8 @@ int brandes_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS, 
     CK_RC(plain_prepare(c, g, S, nS, o, bc_out, r));
     CK_RC(plain_emit(c, r, &tb));
     int rc = finish_status(c, st);
-    const bool back = rc == RC_GIVEN_BACK;
-    if (back) rc = plain_in_lockstep(c, r, &tb, st);
-    count_batches(c, r.levels, r.nitems, back);
+    if (rc == RC_GIVEN_BACK) rc = plain_in_lockstep(c, r, &tb, st);
+    else count_batches(c, r.levels, r.nitems);
     tt.stop();
     if (st) {
         st->ms_brandes_sk = tb.acc;
@@ -1336,10 +1385,10 @@ int build_local_csr(bcpp_ctx* c, const Skeleton& K, const int64_t* rp, const int
     return BCPP_OK;
 }
 
-// Dijkstra_SK on the level-mask kernel.  *done stays false when the batches do not fit into memory or prove
-// too deep for it (or a count outgrows 32 bits): the lockstep kernel then fills the tables.
-int tables_levels(bcpp_ctx* c, const LsArena& A, const LsParams& P, const std::vector<LsItem>& hitems,
-                  const LsItem* items, const std::vector<int32_t>& pstart, uint64_t wmax, int64_t entries, bool* done) {
+// Dijkstra_SK on the level-mask kernel.  hitems keeps the batches that are left for the lockstep kernel: all when one
+// does not fit into memory, else those that proved too deep (or have a count past 32 bits).
+int tables_levels(bcpp_ctx* c, const LsArena& A, const LsParams& P, std::vector<LsItem>& hitems,
+                  const LsItem* items, const std::vector<int32_t>& pstart, uint64_t wmax, int64_t entries) {
     LmWs L;
     bool fits = false;
     CK_RC(lm_alloc(c, L, hitems, false, [&](int32_t i) { return (int64_t)(pstart[i + 1] - pstart[i]); }, 0,
@@ -1347,6 +1396,7 @@ int tables_levels(bcpp_ctx* c, const LsArena& A, const LsParams& P, const std::v
     if (!fits) return BCPP_OK;
     fill_i32(P.td, DINF, entries, c->stream);
     CK_CUDA(cudaMemsetAsync(P.ts, 0, (size_t)entries * sizeof(uint64_t), c->stream));
+    CK_CUDA(cudaMemsetAsync(L.back.p, 0, (size_t)L.back.n * sizeof(uint32_t), c->stream));
     c->launches++;
     for (const LmWave& w : L.waves) {
         const LmArgs a = lm_wave_args(L, w, A, P, items, wmax);
@@ -1356,12 +1406,13 @@ int tables_levels(bcpp_ctx* c, const LsArena& A, const LsParams& P, const std::v
     }
     CK_RC(sync_flags(c));
     if (c->hflags[FLAG_TIMEOUT]) return BCPP_ETIMEOUT;
-    if (c->hflags[FLAG_MASKS]) {
-        CK_CUDA(cudaMemsetAsync(c->flags + FLAG_MASKS, 0, sizeof(uint32_t), c->stream));
+    if (!c->hflags[FLAG_MASKS]) {
+        hitems.clear();
         return BCPP_OK;
     }
-    *done = true;
-    return BCPP_OK;
+    CK_CUDA(cudaMemsetAsync(c->flags + FLAG_MASKS, 0, sizeof(uint32_t), c->stream));
+    const std::vector<LsItem> all = hitems;
+    return lm_given_back(c, L.back, all, hitems);
 }
 
 // reuse (may be null): a skeleton of the same graph built for `part` without singletons.  Every
@@ -1510,17 +1561,23 @@ int build_sk(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS_eff,
             P.td = dir == 0 ? K.td.p : K.tdr.p;
             P.ts = dir == 0 ? K.ts.p : K.tsr.p;
             P.flags = c->flags;
-            bool done = false;
+            std::vector<LsItem> left = hitems;
             if (lm_serves(c, bcpp_opts{}, 1, maxpart_tab, g->num_arcs, g->w ? wmax : 1))
-                CK_RC(tables_levels(c, A, P, hitems, items.p, K.h_pstart, g->w ? wmax : 1, tofs, &done));
-            if (done) continue;
+                CK_RC(tables_levels(c, A, P, left, items.p, K.h_pstart, g->w ? wmax : 1, tofs));
+            if (left.empty()) continue;
+            DBuf<LsItem> litems;
+            if ((int)left.size() < nitems) {
+                CK_ALLOC(litems.alloc(c, (int64_t)left.size()));
+                CK_RC(to_dev(c, litems.p, left.data(), (int64_t)left.size()));
+            }
             // parts are small: provide the worst case (one entry per node and frontier source)
             const int ef = entry_factor(c, true, 1);
-            const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxpart_tab, nb, false, ef), 0);
+            const int nleft = (int)left.size();
+            const int slots = choose_slots(c, nleft, o.ctas_per_sm, slot_bytes(maxpart_tab, nb, false, ef), 0);
             SlotWs ws;
             CK_RC(alloc_slots(c, ws, slots, maxpart_tab, nb, false, 0, 1, ef));
             P.item_counter = ws.counter.p;
-            ls_launch(false, !g->directed, A, P, ws.W, items.p, nitems, slots, c->stream);
+            ls_launch(false, !g->directed, A, P, ws.W, litems.p ? litems.p : items.p, nleft, slots, c->stream);
             c->launches++;
             CK_CUDA(cudaGetLastError());
             // A batch whose settle list outgrew its bound leaves its table rows unwritten: stop
@@ -1580,6 +1637,7 @@ struct PpRun {
     LmWs lm;
     int64_t s0 = 0, s1 = 0;      // source positions of this call's shard
     bool ordered = false;
+    std::vector<LsItem> hitems;  // the batches
     int nb = 2, spl = 1, nitems = 0, cl = 1, slots = 1;
     std::vector<CentralityUnit> hunits;
     struct Lists {           // Centrality: frontiers of each non-frontier node (entries, exits)
@@ -1644,6 +1702,7 @@ int pp_levels_alloc(bcpp_ctx* c, PpRun& r, int nitems, int lcap) {
     CK_ALLOC(r.lm.seen.alloc(c, rows));
     CK_ALLOC(r.lm.dsum.alloc(c, rows));
     CK_ALLOC(r.lm.ctl.alloc(c, lm_ctl_words(lcap, (int)chunk)));
+    CK_ALLOC(r.lm.back.alloc(c, nitems));
     r.lm.lcap = lcap;
     r.lm.narrow = false;
     r.lm.tpb = (int32_t)(cap_n / 32);
@@ -1663,6 +1722,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
     const SkTables T = K.tables();
     CK_CUDA(cudaMemsetAsync(W.bc_sum, 0, (size_t)r.slots * W.cap_bc * sizeof(double), c->stream));
     CK_CUDA(cudaMemsetAsync(W.bc_cmp, 0, (size_t)r.slots * W.cap_bc * sizeof(double), c->stream));
+    CK_CUDA(cudaMemsetAsync(r.lm.back.p, 0, (size_t)r.nitems * sizeof(uint32_t), c->stream));
     for (int c0 = 0; c0 < r.nitems; c0 += r.slots) {
         const int cn = std::min(r.slots, r.nitems - c0);
         LmArgs a{};
@@ -1685,6 +1745,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         a.probe = !r.lm.bounded;
         a.wmax = (int32_t)K.wmax_sk;
         a.mean_degree = r.lm.mean_degree;
+        a.back = r.lm.back.p + c0;
         a.ctl = r.lm.ctl.p;
         a.flags = c->flags;
         a.phase_ns = c->phase;
@@ -1696,7 +1757,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         if (tbr) tbr->stop();
         if (tce) tce->start();
         centrality_launch(false, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, r.entries(), r.exits(), W.d, W.sg,
-                          W.dl, W.cap_n, W.bc_sum, W.bc_cmp, W.cap_bc, c->flags, c->stream);
+                          W.dl, W.cap_n, W.bc_sum, W.bc_cmp, W.cap_bc, a.back, c->flags, c->stream);
         c->launches++;
         if (tce) tce->stop();
         CK_CUDA(cudaGetLastError());
@@ -1705,8 +1766,8 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
 }
 
 // Batches of 32 targets and the workspace of Brandes_SK and Centrality: on the level-mask kernel where it serves them,
-// unless masks = false, else on the lockstep kernel.
-int pp_batches(bcpp_ctx* c, PpRun& r, bool masks) {
+// unless masks = false, else on the lockstep kernel.  only: these batches instead of all.
+int pp_batches(bcpp_ctx* c, PpRun& r, bool masks, const std::vector<LsItem>* only = nullptr) {
     const bcpp_graph* g = &r.g;
     const bcpp_opts& o = r.o;
     const Skeleton& K = r.K;
@@ -1716,7 +1777,8 @@ int pp_batches(bcpp_ctx* c, PpRun& r, bool masks) {
     r.levels = r.rows_by_item = false;
     r.lm.release();
     r.ws.release();
-    std::vector<LsItem> hitems = make_items(0, r.s0, r.s1, 32 * r.spl);
+    std::vector<LsItem>& hitems = r.hitems;
+    hitems = only ? *only : make_items(0, r.s0, r.s1, 32 * r.spl);
     if (masks && N > 0 && !hitems.empty() && lm_serves(c, o, r.spl, N, K.arcs, K.wmax_sk)) {
         r.lm.mean_degree = (double)K.arcs / N;
         // skeleton distances are the distances in G
@@ -1731,7 +1793,7 @@ int pp_batches(bcpp_ctx* c, PpRun& r, bool masks) {
             CK_RC(pp_levels_alloc(c, r, (int)hitems.size(), lcap));
     }
     r.cl = (!hitems.empty() && r.spl == 1) ? choose_cluster(c, (int)hitems.size(), o) : 1;
-    if (r.spl == 1 && r.hunits.empty() && !r.levels) {
+    if (r.spl == 1 && r.hunits.empty() && !r.levels && !only) {
         // without a Centrality step (whose cost grows with the batch count, not their width)
         const int b = balanced_width(r.s1 - r.s0, slot_capacity(c, o, r.cl), 32);
         if (b < 32) hitems = make_items(0, r.s0, r.s1, b);
@@ -1934,7 +1996,7 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tce) tce->start();
             centrality_launch(fp32, r.units.p, (int)r.hunits.size(), r.nitems, T, K.pnodes.p, r.entries(), r.exits(),
                               r.ws.W.d, r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
-                              c->flags, c->stream);
+                              nullptr, c->flags, c->stream);
             c->launches++;
             if (tce) tce->stop();
             CK_CUDA(cudaGetLastError());
@@ -1958,7 +2020,7 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tce) tce->start();
             centrality_launch(fp32, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, r.entries(), r.exits(),
                               r.ws.W.d, r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
-                              c->flags, c->stream);
+                              nullptr, c->flags, c->stream);
             c->launches++;
             if (tce) tce->stop();
             CK_CUDA(cudaGetLastError());
@@ -1972,14 +2034,22 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
     return BCPP_OK;
 }
 
-// The same again on the lockstep kernel, after the level-mask kernel gave the batches back; the skeleton, the order
-// of the targets and the frontier lists stay.
+// The batches that the level-mask kernel gave back, on the lockstep kernel; the sums of the others, the skeleton, the
+// order of the targets and the frontier lists stay.
 int pp_in_lockstep(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce, bcpp_stats* st) {
     const bool worst = past_usual_rows(c, r.lm.lcap);
-    return run_in_lockstep(c, st, worst, [&] {
-        CK_RC(pp_batches(c, r, false));
-        return pp_emit(c, r, tbr, tce);
+    const int all = r.nitems;
+    std::vector<LsItem> some;
+    CK_RC(lm_given_back(c, r.lm.back, r.hitems, some));
+    KeptSums kept;
+    if ((int)some.size() < all) CK_RC(kept.keep(c, r.bc_out, r.g.n));
+    const int rc = run_in_lockstep(c, st, worst, [&] {
+        CK_RC(pp_batches(c, r, false, kept ? &some : nullptr));
+        CK_RC(pp_emit(c, r, tbr, tce));
+        return kept.add_to(c, r.bc_out);
     });
+    count_batches(c, all - (int)some.size(), kept ? (int)some.size() : r.nitems, (int)some.size());
+    return rc;
 }
 
 void pp_fill_stats(const PpRun& r, bcpp_stats* st) {
@@ -2073,9 +2143,8 @@ int brandes_pp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t n
     CK_RC(pp_top_emit(c, t, &tbr, &tce));
     if (!t.trivial) pp_fill_stats(t.run, st);
     int rc = finish_status(c, st);
-    const bool back = rc == RC_GIVEN_BACK;
-    if (back) rc = pp_in_lockstep(c, t.run, &tbr, &tce, st);
-    count_batches(c, t.run.levels, t.run.nitems, back);
+    if (rc == RC_GIVEN_BACK) rc = pp_in_lockstep(c, t.run, &tbr, &tce, st);
+    else count_batches(c, t.run.levels, t.run.nitems);
     tt.stop();
     if (st) {
         st->ms_build_sk = tb.acc;
@@ -2137,9 +2206,8 @@ int brandes_pp_st_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* Ssrc, int
     CK_RC(brandes_pp_core(c, g, wmax, &Tin, uni.p, (int32_t)nuni, Ssrc, nsrc, dflag.p, part, k, o,
                           halve ? 0.5 : 1.0, bc_out, st, tb, tbr, tce, run));
     int rc = finish_status(c, st);
-    const bool back = rc == RC_GIVEN_BACK;
-    if (back) rc = pp_in_lockstep(c, run, &tbr, &tce, st);
-    count_batches(c, run.levels, run.nitems, back);
+    if (rc == RC_GIVEN_BACK) rc = pp_in_lockstep(c, run, &tbr, &tce, st);
+    else count_batches(c, run.levels, run.nitems);
     tt.stop();
     if (st) {
         st->ms_build_sk = tb.acc;
@@ -2192,9 +2260,8 @@ int finish_pair(PairLane& L, int32_t n) {
     if (!L.run) return BCPP_OK;
     bcpp_ctx* lc = L.sc.c;
     int rc = finish_status(lc, nullptr);
-    const bool back = rc == RC_GIVEN_BACK;
-    if (back) rc = pp_in_lockstep(lc, *L.run, L.tbr.get(), L.tce.get(), nullptr);
-    count_batches(lc, L.run->levels, L.run->nitems, back);
+    if (rc == RC_GIVEN_BACK) rc = pp_in_lockstep(lc, *L.run, L.tbr.get(), L.tce.get(), nullptr);
+    else count_batches(lc, L.run->levels, L.run->nitems);
     if (rc != BCPP_OK && rc != BCPP_EOVERFLOW_SIGMA) return rc;
     L.run.reset();
     accumulate_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 8192), 256, 0, lc->stream>>>(L.tmp.p, n, L.sum.p, L.comp.p);
@@ -2419,23 +2486,25 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
     P.phase_ns = c->phase;
     const double scale = o.halve_undirected ? 0.5 : 1.0;
     SlotWs ws;
+    KeptSums kept;
+    int run_items = nitems;
     auto lockstep = [&] {
         lm.release();
         ws.release();
         const int ef = entry_factor(c, g->w != nullptr, spl);
-        const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(maxn, nb, fp32, ef, spl), (int64_t)n * 24);
+        const int slots = choose_slots(c, run_items, o.ctas_per_sm, slot_bytes(maxn, nb, fp32, ef, spl), (int64_t)n * 24);
         CK_RC(alloc_slots(c, ws, slots, maxn, nb, fp32, n, spl, ef, false));
         ws.narrow = use_narrow(c, g->w != nullptr);
         CK_RC(init_slots(c, ws));
         P.item_counter = ws.counter.p;
         tb.start();
-        ls_launch(fp32, true, A, P, ws.W, items.p, nitems, slots, c->stream, spl, 1, ws.narrow);
+        ls_launch(fp32, true, A, P, ws.W, items.p, run_items, slots, c->stream, spl, 1, ws.narrow);
         c->launches++;
         CK_CUDA(cudaGetLastError());
         combine_launch(ws.W.bc_sum, ws.W.bc_cmp, slots, n, n, scale, bc_out, c->stream);
         c->launches++;
         tb.stop();
-        return BCPP_OK;
+        return kept.add_to(c, bc_out);
     };
     if (levels) {
         CK_RC(lm_emit(c, lm, A, P, items.p, g->w ? wmax : 1, scale, bc_out, &tb));
@@ -2443,9 +2512,20 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
         CK_RC(lockstep());
     }
     int rc = finish_status(c, st);
-    const bool back = rc == RC_GIVEN_BACK;
-    if (back) rc = run_in_lockstep(c, st, past_usual_rows(c, lm.lcap), lockstep);
-    count_batches(c, levels && !back, nitems, back);
+    if (rc == RC_GIVEN_BACK) {
+        // only the batches that were given back; the sums of the others stay
+        std::vector<LsItem> some;
+        CK_RC(lm_given_back(c, lm.back, hitems, some));
+        run_items = (int)some.size();
+        maxn = 0;
+        for (const LsItem& it : some) maxn = std::max(maxn, off[it.g + 1] - off[it.g]);
+        CK_RC(to_dev(c, items.p, some.data(), run_items));
+        if (run_items < nitems) CK_RC(kept.keep(c, bc_out, n));
+        rc = run_in_lockstep(c, st, past_usual_rows(c, lm.lcap), lockstep);
+        count_batches(c, nitems - run_items, run_items, run_items);
+    } else {
+        count_batches(c, levels, nitems);
+    }
     tt.stop();
     if (st) {
         st->ms_brandes_sk = tb.acc;
@@ -2501,9 +2581,10 @@ int partition_lp_dev(bcpp_ctx* c, const bcpp_graph* g, int32_t max_rounds, int32
 
 // --------------------------------------------------------------------------- inspection
 // Distances and counts on the level-mask kernel: forward passes with distance rows, turned around into
-// the caller's [source][node] arrays.  *done stays false when not even one batch fits into memory.
+// the caller's [source][node] arrays.  *done stays false when not even one batch fits into memory; back: see LmArgs.
 int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem* items, int nitems,
-                const int32_t* src, uint64_t wmax, int32_t* dist_out, uint64_t* sigma_out, bool* done) {
+                const int32_t* src, uint64_t wmax, int32_t* dist_out, uint64_t* sigma_out, DBuf<uint32_t>& back,
+                bool* done) {
     const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr);
     const int64_t tpb = ((int64_t)g->n + 31) / 32, cap_n = tpb * 32;
     const int64_t each = cap_n * (32 * (4 + 8) + 8 + 4 + 4ll * lcap);
@@ -2516,6 +2597,8 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
     DBuf<uint32_t> lev(c, rows * lcap), seen(c, rows), ctl(c, lm_ctl_words(lcap, (int)chunk));
     DBuf<double> dsum(c, rows);
     CK_ALLOC(d); CK_ALLOC(sg); CK_ALLOC(lev); CK_ALLOC(seen); CK_ALLOC(ctl); CK_ALLOC(dsum);
+    CK_ALLOC(back.alloc(c, nitems));
+    CK_CUDA(cudaMemsetAsync(back.p, 0, (size_t)nitems * sizeof(uint32_t), c->stream));
     for (int c0 = 0; c0 < nitems; c0 += (int)chunk) {
         const int cn = (int)std::min<int64_t>(chunk, nitems - c0);
         LmArgs a{};
@@ -2533,6 +2616,7 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
         a.probe = true;
         a.wmax = (int32_t)wmax;
         a.mean_degree = (double)g->num_arcs / g->n;
+        a.back = back.p + c0;
         a.ctl = ctl.p;
         a.flags = c->flags;
         CK_CUDA(cudaMemsetAsync(ctl.p, 0, (size_t)lm_ctl_words(lcap, cn) * sizeof(uint32_t), c->stream));
@@ -2582,23 +2666,28 @@ int sssp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* src, int32_t nsrc,
     A.node_off = node_off.p;
     bool done = false;
     if (lm_serves(c, o, 1, n, g->num_arcs, g->w ? wmax : 1)) {
-        CK_RC(sssp_levels(c, g, A, items.p, nitems, src, wmax, dist_out, sigma_out, &done));
+        DBuf<uint32_t> back;
+        CK_RC(sssp_levels(c, g, A, items.p, nitems, src, wmax, dist_out, sigma_out, back, &done));
         if (done) {
             const int rc = finish_status(c, nullptr);
             if (rc != RC_GIVEN_BACK) {
-                count_batches(c, true, nitems, false);
+                count_batches(c, true, nitems);
                 return rc;
             }
+            const std::vector<LsItem> all = hitems;
+            CK_RC(lm_given_back(c, back, all, hitems));
+            CK_RC(to_dev(c, items.p, hitems.data(), (int64_t)hitems.size()));
         }
     }
+    const int left = (int)hitems.size();
+    count_batches(c, nitems - left, left, done ? left : 0);
     // a batch holds each source at most once: split repeated sources across batches is not
     // needed because LS_SSSP lanes are independent rows (a repeat only repeats the row)
-    count_batches(c, false, nitems, done);
     // (rows are of full width here, and only the lists could prove too small: the worst case at once for deep graphs)
     return run_in_lockstep(c, nullptr, done, [&] {
         const int nb = g->w ? (int)wmax + 1 : 2;
         const int ef = entry_factor(c, g->w != nullptr, 1);
-        const int slots = choose_slots(c, nitems, o.ctas_per_sm, slot_bytes(n, nb, false, ef), 0);
+        const int slots = choose_slots(c, left, o.ctas_per_sm, slot_bytes(n, nb, false, ef), 0);
         SlotWs ws;
         CK_RC(alloc_slots(c, ws, slots, n, nb, false, 0, 1, ef));
         LsParams P{};
@@ -2610,7 +2699,7 @@ int sssp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* src, int32_t nsrc,
         P.dbg_n = n;
         P.item_counter = ws.counter.p;
         P.flags = c->flags;
-        ls_launch(false, !g->directed, A, P, ws.W, items.p, nitems, slots, c->stream);
+        ls_launch(false, !g->directed, A, P, ws.W, items.p, left, slots, c->stream);
         c->launches++;
         CK_CUDA(cudaGetLastError());
         return BCPP_OK;
@@ -3225,8 +3314,9 @@ int bcpp_plan_launch(bcpp_plan* p, bcpp_stats* stats) {
         if (rc == BCPP_OK) rc = plan_replay(p, stats);
     }
     std::fill(c->ran, c->ran + 3, 0);
-    if (p->plain) count_batches(c, p->plain->levels, p->plain->nitems, back);
-    if (p->pp) count_batches(c, p->pp->run.levels, p->pp->run.nitems, back);
+    if (p->plain) count_batches(c, p->plain->levels, p->plain->nitems);
+    if (p->pp) count_batches(c, p->pp->run.levels, p->pp->run.nitems);
+    if (back) c->ran[2] = c->ran[1];
     tt.stop();
     if (stats) {
         const uint32_t ovf = stats->sigma_overflow;

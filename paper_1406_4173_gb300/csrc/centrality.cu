@@ -88,13 +88,14 @@ __global__ void __launch_bounds__(CT_WARPS * 32, 5)
 centrality_kernel(const CentralityUnit* __restrict__ units, int nslots, SkTables T, const uint32_t* __restrict__ pnodes,
                   CentralityLists E, CentralityLists X, const int32_t* __restrict__ d_all,
                   const uint64_t* __restrict__ sg_all, const DT* __restrict__ dl_all, int64_t cap_n, double* bc_sum,
-                  double* bc_cmp, int64_t cap_bc, uint32_t* flags) {
+                  double* bc_cmp, int64_t cap_bc, const uint32_t* __restrict__ skip, uint32_t* flags) {
     __shared__ CtSm<DT> s_warp[CT_WARPS];
     CtSm<DT>& sm = s_warp[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const CentralityUnit U = units[blockIdx.x];
     bool ovf = false;
     for (int slot = blockIdx.y; slot < nslots; slot += gridDim.y) {
+        if (skip && __ldg(skip + slot)) continue;   // a batch without rows
         // rows of this slot, this lane's source
         const int32_t* dr = d_all + (int64_t)slot * cap_n * 32 + lane;
         const uint64_t* sr = sg_all + (int64_t)slot * cap_n * 32 + lane;
@@ -219,16 +220,16 @@ void ct_fill(const CentralityUnit* units, int nunits, SkTables T, bool exits, co
 void centrality_launch(bool fp32_delta, const CentralityUnit* units, int nunits, int nslots, SkTables T,
                        const uint32_t* pnodes, CentralityLists E, CentralityLists X, const int32_t* d,
                        const uint64_t* sg, const void* dl, int64_t cap_n, double* bc_sum, double* bc_cmp,
-                       int64_t cap_bc, uint32_t* flags, cudaStream_t st) {
+                       int64_t cap_bc, const uint32_t* skip, uint32_t* flags, cudaStream_t st) {
     if (nunits <= 0 || nslots <= 0) return;
     // neighbouring blocks take one batch's neighbouring nodes: their frontier rows are shared in L2
     const dim3 grid((unsigned)nunits, (unsigned)std::min(nslots, 65535));
     if (fp32_delta)
         centrality_kernel<float><<<grid, CT_WARPS * 32, 0, st>>>(units, nslots, T, pnodes, E, X, d, sg, (const float*)dl,
-                                                                cap_n, bc_sum, bc_cmp, cap_bc, flags);
+                                                                cap_n, bc_sum, bc_cmp, cap_bc, skip, flags);
     else
         centrality_kernel<double><<<grid, CT_WARPS * 32, 0, st>>>(units, nslots, T, pnodes, E, X, d, sg,
-                                                                 (const double*)dl, cap_n, bc_sum, bc_cmp, cap_bc, flags);
+                                                                 (const double*)dl, cap_n, bc_sum, bc_cmp, cap_bc, skip, flags);
 }
 
 }  // namespace bcpp

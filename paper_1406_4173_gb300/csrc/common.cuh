@@ -23,8 +23,9 @@ enum : int {
     FLAG_COUNT = 8
 };
 
-// FLAG_MASKS: more distance levels than provided for; a path count past 32 bits
-enum : uint32_t { MASKS_DEEP = 1, MASKS_COUNT = 2 };
+// FLAG_MASKS: some batch with more distance levels than provided for; with a path count past 32 bits; a whole
+// wave looked too deep (later waves of the pass are not begun)
+enum : uint32_t { MASKS_DEEP = 1, MASKS_COUNT = 2, MASKS_ALL = 4 };
 
 // reason codes written into FLAG_INVALID_WHY
 enum : uint32_t {

@@ -54,12 +54,13 @@ template <bool WEIGHTED>
 constexpr int LM_GATHERS = WEIGHTED ? 3 : 2;
 constexpr int LM_MAX_SUB = 3;      // units of 4 rows at least
 constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of larger degree go one by one)
+constexpr int CTL_WIDE = 3, CTL_BACK = 4;   // batches with a path count past 32 bits; batches given back
 constexpr int CTL_LVL = CTL_WORDS;
+constexpr unsigned LVL_ANY = 1u, LVL_STOP = 2u;
 // Words between two batches' depths: a 128-byte line each, since every SM stores to them once per level (side by
 // side, stores of 152 SMs to a few lines held up everyone's loads: n = 10,000, every node a target 7.4 -> 6.3 ms,
 // Brandes++ at n = 100,000 8.6 -> 7.8 ms).
 constexpr int DEPTH_STRIDE = 32;
-constexpr unsigned LVL_ANY = 1u, LVL_ERR = 2u;
 
 // 1/x for small path counts, correctly rounded by the compiler
 constexpr int RCP_N = 1024;
@@ -445,15 +446,16 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, SM& sm, int lane, uin
     }
 }
 
-// Pairs reached by level D and by D / 2, and rows, of a sample of the unfinished batches' rows.  (Its own function:
-// inlined, it cost the kernel's loops registers, n = 10,000: 6.1 -> 6.9 ms.)
+// Pairs reached by level D and by D / 2, and rows, of a sample of the unfinished batches' rows, and all rows sampled.
+// (Its own function: inlined, it cost the kernel's loops registers, n = 10,000: 6.1 -> 6.9 ms.)
 __device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int D, int wmax, const uint32_t* bdepth,
                                           const int32_t* tile_item, int32_t item_base, int32_t tpb, uint32_t* probe) {
     const int64_t nt = (int64_t)gridDim.x * LM_THREADS, step = max((int64_t)1, rows / nt);
-    uint32_t b1 = 0, b2 = 0, all = 0;
+    uint32_t b1 = 0, b2 = 0, all = 0, total = 0;
     for (int64_t row = ((int64_t)blockIdx.x * LM_THREADS + threadIdx.x) * step; row < rows; row += nt * step) {
         const int32_t t = (int32_t)(row >> 5);
         const int it = tile_item ? __ldg(tile_item + t) - item_base : t / tpb;
+        total++;
         if ((int)bdepth[it * DEPTH_STRIDE] + wmax < D) continue;   // (a batch that is done has no masks there)
         all++;
         for (int l = 0; l <= D; l++) {
@@ -465,10 +467,12 @@ __device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int
     b1 = __reduce_add_sync(FULL, b1);
     b2 = __reduce_add_sync(FULL, b2);
     all = __reduce_add_sync(FULL, all);
-    if ((threadIdx.x & 31) == 0 && all) {
+    total = __reduce_add_sync(FULL, total);
+    if ((threadIdx.x & 31) == 0 && total) {
         atomicAdd(probe, b1);
         atomicAdd(probe + 1, b2);
         atomicAdd(probe + 2, all);
+        atomicAdd(probe + 3, total);
     }
 }
 // D (all / b2)^(1 / dim) levels needed, with 2^dim = b2 / b1: more than 4 D?
@@ -477,11 +481,33 @@ __device__ __noinline__ bool looks_deep(const uint32_t* probe) {
     return b2 >= 1.5f * b1 && all * b1 * b1 > b2 * b2 * b2;
 }
 
+// Marks the batches that are given back: those deeper than `most`, which could still grow past the level where the
+// pass was cut, and those with a path count past 32 bits.  The backward pass takes them for empty.
+__device__ __noinline__ void mark_back(uint32_t* bdepth, int nitems, int most, uint32_t* back, uint32_t* ctl,
+                                       uint32_t* flags) {
+    for (int it = blockIdx.x * LM_THREADS + threadIdx.x; it < nitems; it += gridDim.x * LM_THREADS) {
+        uint32_t* b = bdepth + (int64_t)it * DEPTH_STRIDE;
+        const uint32_t why = ((int)b[0] > most ? MASKS_DEEP : 0u) | (b[1] ? MASKS_COUNT : 0u);
+        if (why) {
+            b[0] = 0u;
+            back[it] = 1u;
+            atomicOr(&flags[FLAG_MASKS], why);
+            atomicAdd(ctl + CTL_BACK, 1u);
+        }
+    }
+}
+
+// A batch has a path count past 32 bits; most of them: the level is the last.
+__device__ __forceinline__ void note_wide(uint32_t* b, uint32_t* ctl, uint32_t* lvl, int nitems) {
+    if (atomicExch(b + 1, 1u) == 0u && 2 * (int)(atomicAdd(ctl + CTL_WIDE, 1u) + 1u) > nitems) atomicOr(lvl, LVL_STOP);
+}
+
 template <typename SG, typename DT, bool WEIGHTED, bool MULT, bool TABLE>
 __global__ void __launch_bounds__(LM_THREADS, lm_min_blocks(sizeof(SG) == 4))
 lm_kernel(const LmArgs A, const int sub_log) {
     using Sm = WarpSm<MULT, std::is_same<DT, float>::value>;
     __shared__ Sm s_warp[LM_WARPS];
+    __shared__ int s_last;   // last level of the forward pass
     const int lane = threadIdx.x & 31;
     Sm& sm = s_warp[threadIdx.x >> 5];
     const int wid = blockIdx.x * LM_WARPS + (threadIdx.x >> 5);
@@ -519,8 +545,11 @@ lm_kernel(const LmArgs A, const int sub_log) {
         return x;
     };
 
-    // an earlier wave was given back, and with it the call (only set past a barrier of this launch, if by it)
-    if (__ldcg(A.flags + FLAG_MASKS) != 0u) return;
+    // an earlier wave of the pass looked too deep (only set past a barrier of this launch, if by it)
+    if (__ldcg(A.flags + FLAG_MASKS) & MASKS_ALL) {
+        for (int it = blockIdx.x * LM_THREADS + threadIdx.x; it < A.nitems; it += gridDim.x * LM_THREADS) A.back[it] = 1u;
+        return;
+    }
 
     // With few tiles per warp a unit is a part of a tile (32 >> sub_log rows), so that a level's last and
     // fullest tiles do not leave the other warps waiting (see lm_go for the rule).
@@ -582,15 +611,12 @@ lm_kernel(const LmArgs A, const int sub_log) {
     if (!grid_barrier(A.ctl, A.flags)) return;
 
     // ------------------------------------------------------------------ forward
+    // A batch that may reach a later level when the pass is cut, and one with a path count past 32 bits (second word
+    // beside its depth), is given back; the others go on.
+    // (The last level is kept in shared memory: a register for it cost the weighted instances 1 to 3%.)
     int depth = 0;
-    for (int D = 1;; D++) {
-        if (D >= A.lcap) {
-            if (A.bounded) break;   // (the empty levels up to the largest weight are cut short)
-            // a later level than the masks provide for (or the last one, unseen): the pass is given back
-            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&A.flags[FLAG_MASKS], MASKS_DEEP);
-            return;
-        }
-        bool any = false, wide = false, ovf = false;
+    for (int D = 1; D < A.lcap; D++) {
+        bool any = false, ovf = false;
         for_units(work + D, [&](int unit) {
             const int t = unit >> sub_log;
             const bool mine = lane >> (5 - sub_log) == (unit & ((1 << sub_log) - 1));
@@ -627,7 +653,7 @@ lm_kernel(const LmArgs A, const int sub_log) {
                         A.ts[tab + (int64_t)r * nf + s] = acc;
                     }
                     if (drow) drow[r * 32 + s] = D;
-                    if constexpr (sizeof(SG) == 4) wide |= (acc >> 32) != 0;
+                    if (sizeof(SG) == 4 && (acc >> 32) != 0) note_wide(bdepth + x.it * DEPTH_STRIDE, A.ctl, lvl + D, A.nitems);
                 }
             };
             tile_sums<true, WEIGHTED, MULT, TABLE, SG, uint64_t>(
@@ -645,25 +671,18 @@ lm_kernel(const LmArgs A, const int sub_log) {
             __syncwarp();
         });
         if (sizeof(SG) == 8 && __any_sync(FULL, ovf) && lane == 0) atomicOr(&A.flags[FLAG_SIGMA_OVF], 1u);
-        if (__any_sync(FULL, wide)) {
-            if (lane == 0) atomicOr(lvl + D, LVL_ERR | LVL_ANY);
-        } else if (any && lane == 0 && (__ldcg(lvl + D) & LVL_ANY) == 0u) {
-            atomicOr(lvl + D, LVL_ANY);
-        }
+        if (any && lane == 0 && __ldcg(lvl + D) == 0u) atomicOr(lvl + D, LVL_ANY);
+        if (threadIdx.x == 0) s_last = D;
         if (!grid_barrier(A.ctl, A.flags)) return;
         // every block reads the same word: nobody writes level D's status any more
         const uint32_t w = __ldcg(lvl + D);
-        if (w & LVL_ERR) {
-            // a path count past 32 bits: the pass is given back
-            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&A.flags[FLAG_MASKS], MASKS_COUNT);
-            return;
-        }
         if (w & LVL_ANY) depth = D;
-        if (D - depth >= wmax) break;
+        if (D - depth >= wmax || (sizeof(SG) == 4 && (w & LVL_STOP))) break;
         // Too deep a graph shows early: a quarter of the way the pairs reached by now and by half of that
         // give the dimension that the balls around the sources grow with, and with it the level at which
-        // they hold every pair; past the levels provided for, the pass is given back without going there first
-        // (grid 300 x 300 with weights up to 16, 500 sources: 112 -> 101 ms, 97 without the attempt).
+        // they hold every pair; past the levels provided for, the unfinished batches are given back without going there
+        // first (grid 300 x 300 with weights up to 16, 500 sources: 112 -> 101 ms, 97 without the attempt), and
+        // with them the later waves of a graph, when they are most of the wave.
         // Balls that hardly grow any more belong to stragglers, not to a deep graph.
         if (!TABLE && A.probe && (D == A.lcap / 4 || D == A.lcap / 4 + 1)) {
             uint32_t* probe = work + 2 * A.lcap;
@@ -671,10 +690,18 @@ lm_kernel(const LmArgs A, const int sub_log) {
                 probe_levels(A.lev, A.rows, D, wmax, bdepth, A.item_tile0 ? A.tile_item + A.tile_base : nullptr,
                              A.item_base, A.tpb, probe);
             } else if (looks_deep(probe)) {
-                if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&A.flags[FLAG_MASKS], MASKS_DEEP);
-                return;
+                if (blockIdx.x == 0 && threadIdx.x == 0 && !A.item_tile0 && 2 * __ldcg(probe + 2) > __ldcg(probe + 3))
+                    atomicOr(&A.flags[FLAG_MASKS], MASKS_ALL);
+                break;
             }
         }
+    }
+    // Cut: the batches could still grow.  (With a bound, weighted skeletons, only empty levels are missing.)
+    const uint32_t nwide = sizeof(SG) == 4 ? __ldcg(A.ctl + CTL_WIDE) : 0u;
+    const bool cut = s_last - depth < wmax && (sizeof(SG) == 4 || !A.bounded);
+    if (cut || nwide) {
+        mark_back(bdepth, A.nitems, 2 * nwide > (uint32_t)A.nitems ? -1 : cut ? s_last - wmax : INT32_MAX, A.back, A.ctl, A.flags);
+        if (!grid_barrier(A.ctl, A.flags) || __ldcg(A.ctl + CTL_BACK) == (uint32_t)A.nitems) return;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
 
@@ -884,7 +911,7 @@ cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
 
 }  // namespace
 
-int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + (int64_t)nitems * DEPTH_STRIDE + 2 * (int64_t)lcap + 3; }
+int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + (int64_t)nitems * DEPTH_STRIDE + 2 * (int64_t)lcap + 4; }
 
 cudaError_t lm_launch(const LmArgs& A, bool narrow, bool fp32, int num_sms, cudaStream_t st) {
     if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;

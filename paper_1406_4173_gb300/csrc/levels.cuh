@@ -6,8 +6,8 @@
 
 namespace bcpp {
 
-// Distance levels a launch provides for; a batch that reaches a later one ends the pass with FLAG_MASKS, and the
-// caller runs it on the lockstep kernel.
+// Distance levels a launch provides for.  A batch that reaches a later one is given back (LmArgs::back, FLAG_MASKS), and
+// the caller runs it on the lockstep kernel.
 constexpr int LM_MAX_LEVELS = 256;
 // Largest arc weight: every row that is not settled on all its sources looks at its in-arcs once per
 // distance value, so the forward cost grows with the number of distance values.
@@ -51,6 +51,7 @@ struct LmArgs {
     bool probe;                 // no bound on the levels is known: give up early on a graph that looks too deep
     int32_t wmax;
     double mean_degree;         // arcs per node
+    uint32_t* back;             // [nitems], zeroed: set for the batches given back (their dsum stays 0)
     uint32_t* ctl;              // lm_ctl_words() zeroed words: barrier, level status, depth of each batch
     uint32_t* flags;
     unsigned long long* phase_ns;
@@ -59,7 +60,7 @@ struct LmArgs {
 int64_t lm_ctl_words(int lcap, int nitems);
 
 // Forward and backward pass of every batch of the wave; one cooperative launch.  narrow: 32-bit path
-// counts (a count of 2^32 or more aborts like a late level).  fp32: FP32 dependencies (unit weights, narrow).
+// counts (a batch with a count of 2^32 or more is given back).  fp32: FP32 dependencies (unit weights, narrow).
 cudaError_t lm_launch(const LmArgs& A, bool narrow, bool fp32, int num_sms, cudaStream_t st);
 
 // Dijkstra_SK (Eq. 10): forward pass of every batch (sources: frontiers aux .. aux + nsrc - 1 of graph g, cc =

@@ -64,11 +64,12 @@ struct CentralityLists {
 void ct_count(const CentralityUnit* units, int nunits, SkTables T, bool exits, int64_t* cnt, cudaStream_t st);
 void ct_fill(const CentralityUnit* units, int nunits, SkTables T, bool exits, const int32_t* skbase, const int64_t* rp,
              int2* ft, uint64_t* mu, cudaStream_t st);
-// all units for the slots of one Brandes_SK chunk; E, X: entry and exit lists (undirected: the same)
+// all units for the slots of one Brandes_SK chunk; E, X: entry and exit lists (undirected: the same); skip (may be null):
+// non-zero for the slots to leave out
 void centrality_launch(bool fp32_delta, const CentralityUnit* units, int nunits, int nslots, SkTables T,
                        const uint32_t* pnodes, CentralityLists E, CentralityLists X, const int32_t* d,
                        const uint64_t* sg, const void* dl, int64_t cap_n, double* bc_sum, double* bc_cmp,
-                       int64_t cap_bc, uint32_t* flags, cudaStream_t st);
+                       int64_t cap_bc, const uint32_t* skip, uint32_t* flags, cudaStream_t st);
 
 // bc_out[v] = scale * sum over slots of (bc_sum + bc_cmp), Neumaier over slots
 void combine_launch(const double* bc_sum, const double* bc_cmp, int nslots, int64_t cap_bc, int64_t n, double scale,

@@ -62,7 +62,7 @@ def test_plain_keeps_what_it_prepared(bc, ctx):
     got, st = bc.brandes(G, S, stats=True, ctx=ctx)
     assert rel_err(got, ref) <= FP64_TOL
     b = ctx.last_batches()
-    assert b["levels"] == 0 and b["lockstep"] == b["given_back"] > 0
+    assert b["levels"] == 0 and b["given_back"] == 3 and b["lockstep"] > 0
     _, st32 = bc.brandes(G, S, precision="fp32", stats=True, ctx=ctx)
     assert ctx.last_batches()["given_back"] == 0
     assert st["kernel_launches"] <= st32["kernel_launches"] + ATTEMPT
@@ -196,3 +196,91 @@ def test_many_small_components(bc, ctx):
     ref, _ = oracle.brandes(g, None)
     assert rel_err(bc.brandes(bc.graph_from_edgelist(g), None, ctx=ctx), ref) <= FP64_TOL
     assert ctx.last_batches()["lockstep"] == 0
+
+
+# ---------------------------------------------------------------------------- only the batches that do not fit
+def beside(g, h):
+    """Disjoint union of two graphs with parts."""
+    part = None if g.part is None else np.concatenate([g.part, h.part + g.part.max() + 1]).astype(np.int32)
+    return gen.EdgeList(n=g.n + h.n, src=np.concatenate([g.src, h.src + g.n]).astype(np.int32),
+                        dst=np.concatenate([g.dst, h.dst + g.n]).astype(np.int32), part=part)
+
+
+def layers(count, width):
+    """Layers of nodes, neighbouring ones completely joined: width^(d - 1) paths at distance d."""
+    a, b = (x.ravel() for x in np.meshgrid(np.arange(width), np.arange(width)))
+    src = np.concatenate([a + i * width for i in range(count - 1)])
+    dst = np.concatenate([b + (i + 1) * width for i in range(count - 1)])
+    return gen.EdgeList(n=count * width, src=src.astype(np.int32), dst=dst.astype(np.int32))
+
+
+# path of 100: four batches, each too deep for the 64 levels of a batched call; 16 layers of eight nodes: 8^11 = 2^33
+# paths and more from the first and the last 32 nodes only
+@pytest.mark.parametrize("odd,back", [(gen.path(100), 4), (layers(16, 8), 2)], ids=["deep", "counts"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_batched_keeps_the_other_graphs(bc, ctx, odd, back, precision):
+    gs = [gen.erdos_renyi(n, min(1.0, 6.0 / n), seed=n) for n in (40, 64, 65, 200)] + [odd]
+    arena = bc.build_arena(gs)
+    got = bc.brandes_batched(arena, precision=precision, ctx=ctx).cpu().numpy()
+    for i, g in enumerate(gs):
+        ref, _ = oracle.brandes(g, None)
+        x = got[arena.node_ptr_host[i]:arena.node_ptr_host[i + 1]]
+        assert rel_err(x, ref) <= (FP64_TOL if precision == "fp64" else 2e-6), i
+    total = sum(-(-g.n // 32) for g in gs)
+    assert ctx.last_batches() == {"levels": total - back, "lockstep": back, "given_back": back}
+
+
+def two_components():
+    g = gen.planted_partition(600, 6, 0.06, 0.004, seed=51)
+    p = gen.path(300)
+    p.part = (np.arange(300) // 30).astype(np.int32)
+    return beside(g, p)
+
+
+@pytest.mark.parametrize("method", ["plain", "plain-fp32", "pp", "pp-chunks", "pp-st", "plan"])
+def test_targets_of_a_deep_component(bc, ctx, method):
+    g = two_components()
+    S = np.concatenate([np.arange(0, 600, 3), np.arange(600, 900, 4)]).astype(np.int32)   # 200 and 75 targets
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    if method.startswith("plain"):
+        got = bc.brandes(G, S, precision="fp32" if "32" in method else "fp64", ctx=ctx)
+    elif method == "pp-st":
+        got = bc.brandes_pp_st(G, S, S, g.part, ctx=ctx)
+    elif method == "plan":
+        plan = bc.plan_brandes(G, S, ctx=ctx)
+        got = plan.launch().cpu().numpy()
+        plan.close()
+    else:
+        got = bc.brandes_pp(G, S, g.part, pp_chunks=int("chunks" in method), ctx=ctx)
+    assert rel_err(got, ref) <= (2e-6 if "32" in method else FP64_TOL)
+    b = ctx.last_batches()
+    if method == "plan":        # moves as a whole
+        assert b["levels"] == 0 and b["given_back"] == b["lockstep"] > 0
+    else:
+        assert b["given_back"] == b["lockstep"] and 3 <= b["lockstep"] <= 3 + (method == "plain-fp32") * 80
+        assert b["levels"] >= 6
+
+
+def test_paths_from_a_deep_component(bc, ctx):
+    g = two_components()
+    src = np.concatenate([np.arange(32), 600 + 9 * np.arange(32)]).astype(np.int32)
+    d, s = bc.sssp(bc.graph_from_edgelist(g), src, ctx=ctx)
+    assert ctx.last_batches() == {"levels": 1, "lockstep": 1, "given_back": 1}
+    for i, v in enumerate(src):
+        rd, rs, _ = oracle.sssp(g, int(v))
+        assert np.array_equal(d[i].cpu().numpy(), rd)
+        assert np.array_equal(s[i].cpu().numpy().view(np.uint64), rs)
+
+
+def test_tables_of_a_deep_part(bc):
+    """One part (a path of 300) is too deep for the Dijkstra_SK masks, the others are not."""
+    g = two_components()
+    part = np.minimum(g.part, 6).astype(np.int32)
+    S = np.array([3, 100, 350, 610, 750, 890], np.int32)
+    nodes, (u, v, w, mu) = bc.skeleton(bc.graph_from_edgelist(g), S, part)
+    rn, (ru, rv, rw, rmu), _ = oracle.skeleton(g, S, part)
+    o, ro = np.lexsort((v, u)), np.lexsort((rv, ru))
+    assert np.array_equal(np.sort(nodes), np.sort(rn))
+    for x, rx in ((u, ru), (v, rv), (w, rw), (mu, rmu)):
+        assert np.array_equal(np.asarray(x)[o].astype(np.uint64), np.asarray(rx)[ro].astype(np.uint64))
