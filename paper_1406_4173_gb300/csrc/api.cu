@@ -722,6 +722,20 @@ __global__ void parent_keys_kernel(const uint32_t* nodes, int64_t count, const i
     }
 }
 
+// Unit weights: all nodes in discovery order from the hub, and the levels of the search.
+int hub_search(bcpp_ctx* c, const bcpp_graph* g, int32_t* queue, OrderWs& w) {
+    DBuf<int32_t> par(c, g->n), depth(c, 2);
+    DBuf<uint32_t> ctl(c, order_ctl_words(c->num_sms));
+    CK_ALLOC(par); CK_ALLOC(depth); CK_ALLOC(ctl);
+    CK_CUDA(order_bfs_launch(g->n, g->row_ptr, g->col, par.p, queue, ctl.p, depth.p, c->flags, c->num_sms, c->stream));
+    c->launches++;
+    int32_t h[2] = {0, 0};
+    CK_RC(to_host(c, h, depth.p, 2));
+    w.depth = h[0];
+    w.rest = h[1];
+    return BCPP_OK;
+}
+
 int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const int32_t* icol, const uint32_t* iw,
                   uint64_t wmax, const int32_t* S, int64_t ns, const int32_t* part, int32_t k, OrderWs& w) {
     const int32_t n = g->n;
@@ -741,21 +755,11 @@ int order_prepare(bcpp_ctx* c, const bcpp_graph* g, const int64_t* irp, const in
         CK_ALLOC(w.tmp.alloc(c, scan_tmp_elems(n)));
     }
     if (!g->w) {
-        DBuf<int32_t> par(c, n), depth(c, 2);
-        DBuf<uint32_t> ctl(c, order_ctl_words(c->num_sms));
-        CK_ALLOC(par); CK_ALLOC(depth); CK_ALLOC(ctl);
         if (!all || part) CK_ALLOC(w.queue.alloc(c, n));
         if (!all) {
             CK_ALLOC(w.mem.alloc(c, n)); CK_ALLOC(w.flag.alloc(c, n)); CK_ALLOC(w.place.alloc(c, n));
         }
-        CK_CUDA(order_bfs_launch(n, g->row_ptr, g->col, par.p, all && !part ? w.out.p : w.queue.p, ctl.p, depth.p,
-                                 c->flags, c->num_sms, c->stream));
-        c->launches++;
-        int32_t h[2] = {0, 0};
-        CK_RC(to_host(c, h, depth.p, 2));
-        w.depth = h[0];
-        w.rest = h[1];
-        return BCPP_OK;
+        return hub_search(c, g, all && !part ? w.out.p : w.queue.p, w);
     }
     // levels from the hub (the node of largest degree)
     DBuf<unsigned long long> best(c, 1);
@@ -936,10 +940,13 @@ bool lm_bounded(bool weighted, bool directed, const OrderWs* ord) {
            lm_diameter(*ord) <= std::max<int64_t>(60, 2 * (int64_t)ord->depth);
 }
 
-// Levels to provide for.
-int lm_levels(bool weighted, bool directed, const OrderWs* ord) {
+// Levels to provide for.  Nothing is known about them (no search, not bounded): all that the masks can hold while
+// those take up to 2 GB, as few batches lose little by many levels (chain of 30 x 1,000 random nodes, 60 targets:
+// 2.2 ms, 3.5 in lockstep, 4.8 with 64 levels and then in lockstep), else 64.
+bool lm_all_levels(int64_t rows) { return rows * LM_MAX_LEVELS <= (2ll << 30) / 4; }
+int lm_levels(bool weighted, bool directed, const OrderWs* ord, int64_t rows) {
     if (weighted) return LM_MAX_LEVELS;
-    if (!ord) return 64;
+    if (!ord) return lm_all_levels(rows) ? LM_MAX_LEVELS : 64;
     if (lm_bounded(weighted, directed, ord)) return (int)std::max<int64_t>(24, lm_diameter(*ord) + 4);
     return std::max(64, 2 * std::min(ord->depth, LM_MAX_LEVELS) + 4);
 }
@@ -1119,7 +1126,7 @@ struct PlainRun {
     DBuf<int32_t> all;
     InCsr T;
     OrderWs ord;
-    bool ordered = false;
+    bool ordered = false, searched = false;   // ord holds the order; the levels from the hub
     DBuf<LsItem> items;
     DBuf<int64_t> node_off;
     SlotWs ws;
@@ -1172,16 +1179,17 @@ int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks, const std::vector<LsItem
     std::vector<LsItem>& hitems = r.hitems;
     hitems = only ? *only : make_items(0, r.s0, r.s1, 32 * r.spl);
     r.cl = r.spl == 1 ? choose_cluster(c, (int)hitems.size(), o) : 1;
+    const OrderWs* ord = r.searched ? &r.ord : nullptr;
+    const int64_t rows = (int64_t)hitems.size() * n;
     const int width = r.spl == 1 && !only ? balanced_width(r.s1 - r.s0, slot_capacity(c, o, r.cl), 32) : 32;
     // (FP32 dependencies: the batches of the lockstep kernel, whose order of additions depends on them)
     if (fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.lm.fp32 = fp32;
     r.lm.mean_degree = (double)g->num_arcs / n;
-    r.lm.bounded = lm_bounded(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr);
-    if (masks && lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) &&
-        !(r.ordered && lm_dense_deep(r.ord, r.ns, n)))
+    r.lm.bounded = lm_bounded(g->w != nullptr, g->directed != 0, ord);
+    if (masks && lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) && !(ord && lm_dense_deep(*ord, r.ns, n)))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
-                       lm_levels(g->w != nullptr, g->directed != 0, r.ordered ? &r.ord : nullptr), true, &r.levels));
+                       lm_levels(g->w != nullptr, g->directed != 0, ord, rows), true, &r.levels));
     if (!r.levels && !fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.nitems = (int)hitems.size();
     CK_ALLOC(r.items.alloc(c, r.nitems));
@@ -1234,12 +1242,23 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     if (o.order_sources && r.ns > 2 * LS_LANES && !g->w) {   // measured to help on unit weights only
         CK_RC(order_prepare(c, g, g->directed ? r.T.rp.p : g->row_ptr, g->directed ? r.T.col.p : g->col,
                             g->directed ? (g->w ? r.T.w.p : nullptr) : g->w, r.wmax, srcs, r.ns, nullptr, 0, r.ord));
-        r.ordered = true;
+        r.ordered = r.searched = true;
         srcs = r.ord.out.p;
     }
     shard_sources(o, r.ns, r.s0, r.s1);
     r.spl = choose_spl(c, r.s1 - r.s0, o);
     if (r.s1 <= r.s0) return BCPP_OK;
+    const int64_t rows = div_up(r.s1 - r.s0, LS_LANES) * (int64_t)n;
+    if (!r.ordered && !g->w && (!lm_all_levels(rows) || (rows >= (1 << 18) && 4 * r.ns >= n)) &&
+        lm_serves(c, o, r.spl, n, g->num_arcs, 1, true)) {
+        // A large call in the given order, or one with many targets: the levels decide on the kernel.  (Chains of random
+        // communities, every node a target, in lockstep 118 ms at 30 x 1,000 and 3.3 at 16 x 200, begun on masks 197
+        // and 4.5; the search takes 0.1 to 0.4 ms.)
+        DBuf<int32_t> queue(c, n);
+        CK_ALLOC(queue);
+        CK_RC(hub_search(c, g, queue.p, r.ord));
+        r.searched = true;
+    }
     CK_ALLOC(r.node_off.alloc(c, 2));
     const int64_t hoff[2] = {0, n};
     CK_RC(to_dev(c, r.node_off.p, hoff, 2));
@@ -1391,8 +1410,10 @@ int tables_levels(bcpp_ctx* c, const LsArena& A, const LsParams& P, std::vector<
                   const LsItem* items, const std::vector<int32_t>& pstart, uint64_t wmax, int64_t entries) {
     LmWs L;
     bool fits = false;
+    int64_t rows = 0;
+    for (const LsItem& it : hitems) rows += pstart[it.g + 1] - pstart[it.g];
     CK_RC(lm_alloc(c, L, hitems, false, [&](int32_t i) { return (int64_t)(pstart[i + 1] - pstart[i]); }, 0,
-                   lm_levels(A.w != nullptr, true, nullptr), true, &fits, true));
+                   lm_levels(A.w != nullptr, true, nullptr, rows), true, &fits, true));
     if (!fits) return BCPP_OK;
     fill_i32(P.td, DINF, entries, c->stream);
     CK_CUDA(cudaMemsetAsync(P.ts, 0, (size_t)entries * sizeof(uint64_t), c->stream));
@@ -1783,7 +1804,7 @@ int pp_batches(bcpp_ctx* c, PpRun& r, bool masks, const std::vector<LsItem>* onl
         r.lm.mean_degree = (double)K.arcs / N;
         // skeleton distances are the distances in G
         const OrderWs* ord = r.ordered ? &r.ord : nullptr;
-        const int lcap = lm_levels(g->w != nullptr, g->directed != 0, ord);
+        const int lcap = lm_levels(g->w != nullptr, g->directed != 0, ord, (int64_t)hitems.size() * N);
         r.lm.bounded = lm_bounded(g->w != nullptr, g->directed != 0, ord);
         if (r.hunits.empty() && r.unit && ord && lm_dense_deep(*ord, ns, n))
             ;   // on the lockstep kernel
@@ -2471,9 +2492,11 @@ int batched_dev(bcpp_ctx* c, int32_t ngraphs, const int64_t* node_ptr_dev, const
     LmWs lm;
     lm.fp32 = fp32;
     lm.mean_degree = (double)g->num_arcs / n;
+    // (Every level looks at the tiles of all graphs, so the levels of a long one are better left to the lockstep kernel:
+    // 512 graphs of 200 nodes and a path of 100, 3.6 ms with 64 levels, 5.9 with 256.)
+    const int lcap = g->w ? LM_MAX_LEVELS : 64;
     if (lm_serves(c, o, spl, (int32_t)maxn, g->num_arcs, g->w ? wmax : 1, !g->w))
-        CK_RC(lm_alloc(c, lm, hitems, false, [&](int32_t gi) { return off[gi + 1] - off[gi]; }, n,
-                       lm_levels(g->w != nullptr, false, nullptr), true, &levels));
+        CK_RC(lm_alloc(c, lm, hitems, false, [&](int32_t gi) { return off[gi + 1] - off[gi]; }, n, lcap, true, &levels));
     LsArena A{};
     A.rp = g->row_ptr; A.col = lcol.p; A.w = (const int32_t*)g->w;
     A.irp = g->row_ptr; A.icol = lcol.p; A.iw = (const int32_t*)g->w;
@@ -2585,8 +2608,8 @@ int partition_lp_dev(bcpp_ctx* c, const bcpp_graph* g, int32_t max_rounds, int32
 int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem* items, int nitems,
                 const int32_t* src, uint64_t wmax, int32_t* dist_out, uint64_t* sigma_out, DBuf<uint32_t>& back,
                 bool* done) {
-    const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr);
     const int64_t tpb = ((int64_t)g->n + 31) / 32, cap_n = tpb * 32;
+    const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr, nitems * cap_n);
     const int64_t each = cap_n * (32 * (4 + 8) + 8 + 4 + 4ll * lcap);
     int64_t chunk = std::min<int64_t>(nitems, std::min(free_bytes(c), std::max(LM_WAVE_BYTES, each)) / each);
     chunk = std::min<int64_t>(chunk, ((1ll << 31) - 1) / cap_n);

@@ -284,3 +284,35 @@ def test_tables_of_a_deep_part(bc):
     assert np.array_equal(np.sort(nodes), np.sort(rn))
     for x, rx in ((u, ru), (v, rv), (w, rw), (mu, rmu)):
         assert np.array_equal(np.asarray(x)[o].astype(np.uint64), np.asarray(rx)[ro].astype(np.uint64))
+
+
+# ---------------------------------------------------------------------------- levels without an order of the targets
+def community_chain(count, size):
+    g = [gen.erdos_renyi(size, 8.0 / size, seed=60 + i) for i in range(count)]
+    src = [x.src + i * size for i, x in enumerate(g)] + [np.arange(1, count) * size]
+    dst = [x.dst + i * size for i, x in enumerate(g)] + [np.arange(1, count) * size - 1]
+    lo, hi = (f(np.concatenate(src), np.concatenate(dst)).astype(np.int32) for f in (np.minimum, np.maximum))
+    return gen.EdgeList(n=count * size, src=lo, dst=hi)
+
+
+def test_few_unordered_targets_of_a_long_graph(bc, ctx):
+    """More than 64 levels, nothing known about them, few batches: the masks hold them all."""
+    g = community_chain(20, 60)
+    G = bc.graph_from_edgelist(g)
+    for S, kw in ((gen.sample_targets(g.n, 60, seed=5), {}), (gen.sample_targets(g.n, 200, seed=5), {"order_sources": False})):
+        ref, _ = oracle.brandes(g, S)
+        assert max(x for x in oracle.sssp(g, int(S[0]))[0] if x < 2**31 - 1) > 64
+        assert rel_err(bc.brandes(G, S, ctx=ctx, **kw), ref) <= FP64_TOL
+        assert ctx.last_batches()["lockstep"] == 0
+
+
+@pytest.mark.parametrize("count,size,route", [(30, 310, "lockstep"), (8, 1100, "levels")])
+def test_many_unordered_targets(bc, ctx, count, size, route):
+    """Large calls in the given order: the levels from the hub decide as they do for ordered calls."""
+    g = community_chain(count, size)
+    S = None
+    ref, _ = oracle.brandes(g, S)
+    got = bc.brandes(bc.graph_from_edgelist(g), S, order_sources=False, ctx=ctx)
+    assert rel_err(got, ref) <= FP64_TOL
+    b = ctx.last_batches()
+    assert b["given_back"] == 0 and b[route] > 0 and sum(b.values()) == b[route]
