@@ -36,6 +36,7 @@ struct bcpp_ctx {
     int64_t launches = 0;
     int order_factor = 8;            // settled-entry capacity per node of a batch (retry: worst case)
     int64_t ran[3] = {};             // bcpp_last_batches of the last call
+    int64_t tile_arcs = 0;           // of the graph checked last (validate_csr)
     cudaEvent_t ev[8] = {};
 
     void* acquire(size_t bytes) {
@@ -296,17 +297,20 @@ int check_graph_struct(const bcpp_graph* g) {
     return BCPP_OK;
 }
 
-// Validate a CSR; on success *wmax_out = max weight (1 for unit weights).
+// Validate a CSR; on success *wmax_out = max weight (1 for unit weights), and c->tile_arcs = the most arcs of 32
+// consecutive rows.
 int validate_csr(bcpp_ctx* c, const bcpp_graph* g, uint64_t* wmax_out, const int64_t* node_off = nullptr,
                  int32_t ngraphs = 0) {
-    DBuf<unsigned long long> wmax(c, 1);
+    DBuf<unsigned long long> wmax(c, 2);
     CK_ALLOC(wmax);
-    CK_CUDA(cudaMemsetAsync(wmax.p, 0, sizeof(unsigned long long), c->stream));
+    CK_CUDA(cudaMemsetAsync(wmax.p, 0, 2 * sizeof(unsigned long long), c->stream));
     csr_check(g->n, g->num_arcs, g->row_ptr, g->col, g->w, g->directed, c->flags, wmax.p, c->stream, node_off,
-              ngraphs);
+              ngraphs, wmax.p + 1);
     c->launches++;
-    unsigned long long hw = 0;
-    CK_RC(to_host(c, &hw, (const unsigned long long*)wmax.p, 1));
+    unsigned long long h[2] = {0, 0};
+    CK_RC(to_host(c, h, (const unsigned long long*)wmax.p, 2));
+    unsigned long long hw = h[0];
+    c->tile_arcs = (int64_t)h[1];
     CK_RC(sync_flags(c));
     if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
     if (hw == 0) hw = 1;
@@ -890,6 +894,7 @@ struct LmWs {
     bool narrow = true;
     bool fp32 = false;         // FP32 dependencies
     double mean_degree = 16;   // arcs per node
+    int64_t tile_arcs = 0;     // most arcs of 32 consecutive rows (0: not known)
     int32_t tpb = 0;           // uniform layout: tiles per batch
     int64_t nodes = 0;         // global nodes
     DBuf<uint32_t> lev, seen, ctl;
@@ -943,10 +948,12 @@ bool lm_bounded(bool weighted, bool directed, const OrderWs* ord) {
 // Levels to provide for.  Nothing is known about them (no search, not bounded): all that the masks can hold while
 // those take up to 2 GB, as few batches lose little by many levels (chain of 30 x 1,000 random nodes, 60 targets:
 // 2.2 ms, 3.5 in lockstep, 4.8 with 64 levels and then in lockstep), else 64.
+// Nor where single tiles hold most arcs, for which every level waits (tile_arcs, see LmArgs; 50,000 nodes on 200 hubs in
+// a row, neighbouring ids, 64 targets: 12.6 ms on 111 levels, 6.3 in lockstep, 7.5 with 64 levels and then in lockstep).
 bool lm_all_levels(int64_t rows) { return rows * LM_MAX_LEVELS <= (2ll << 30) / 4; }
-int lm_levels(bool weighted, bool directed, const OrderWs* ord, int64_t rows) {
+int lm_levels(bool weighted, bool directed, const OrderWs* ord, int64_t rows, int64_t tile_arcs = 0, double mean_degree = 0) {
     if (weighted) return LM_MAX_LEVELS;
-    if (!ord) return lm_all_levels(rows) ? LM_MAX_LEVELS : 64;
+    if (!ord) return lm_all_levels(rows) && tile_arcs <= std::max(1024.0, 256 * mean_degree) ? LM_MAX_LEVELS : 64;
     if (lm_bounded(weighted, directed, ord)) return (int)std::max<int64_t>(24, lm_diameter(*ord) + 4);
     return std::max(64, 2 * std::min(ord->depth, LM_MAX_LEVELS) + 4);
 }
@@ -1069,6 +1076,7 @@ LmArgs lm_wave_args(const LmWs& L, const LmWave& w, const LsArena& A, const LsPa
     a.probe = !L.bounded;
     a.wmax = (int32_t)wmax;
     a.mean_degree = L.mean_degree;
+    a.tile_arcs = L.tile_arcs;
     a.back = L.back.p + w.i0;
     a.ctl = L.ctl.p;
     a.flags = P.flags;
@@ -1118,6 +1126,7 @@ struct PlainRun {
     bcpp_opts o{};
     double* bc_out = nullptr;
     uint64_t wmax = 1;
+    int64_t tile_arcs = 0;         // of g (see LmArgs)
     int64_t ns = 0;
     bool trivial = false;          // |S| < 2 or n == 0: all zeros
     DBuf<uint8_t> in_s;
@@ -1186,10 +1195,11 @@ int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks, const std::vector<LsItem
     if (fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.lm.fp32 = fp32;
     r.lm.mean_degree = (double)g->num_arcs / n;
+    r.lm.tile_arcs = r.tile_arcs;
     r.lm.bounded = lm_bounded(g->w != nullptr, g->directed != 0, ord);
     if (masks && lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) && !(ord && lm_dense_deep(*ord, r.ns, n)))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
-                       lm_levels(g->w != nullptr, g->directed != 0, ord, rows), true, &r.levels));
+                       lm_levels(g->w != nullptr, g->directed != 0, ord, rows, r.tile_arcs, r.lm.mean_degree), true, &r.levels));
     if (!r.levels && !fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.nitems = (int)hitems.size();
     CK_ALLOC(r.items.alloc(c, r.nitems));
@@ -1213,6 +1223,7 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     r.g = *g; r.S = S; r.nS = nS; r.o = o; r.bc_out = bc_out;
     CK_RC(reset_flags(c));
     CK_RC(validate_csr(c, g, &r.wmax));
+    r.tile_arcs = c->tile_arcs;
     CK_ALLOC(r.wmaxd.alloc(c, 1));
     if (nS > 0) {
         CK_ALLOC(r.in_s.alloc(c, n));
@@ -2609,7 +2620,7 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
                 const int32_t* src, uint64_t wmax, int32_t* dist_out, uint64_t* sigma_out, DBuf<uint32_t>& back,
                 bool* done) {
     const int64_t tpb = ((int64_t)g->n + 31) / 32, cap_n = tpb * 32;
-    const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr, nitems * cap_n);
+    const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr, nitems * cap_n, c->tile_arcs, (double)g->num_arcs / g->n);
     const int64_t each = cap_n * (32 * (4 + 8) + 8 + 4 + 4ll * lcap);
     int64_t chunk = std::min<int64_t>(nitems, std::min(free_bytes(c), std::max(LM_WAVE_BYTES, each)) / each);
     chunk = std::min<int64_t>(chunk, ((1ll << 31) - 1) / cap_n);
@@ -2639,6 +2650,7 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
         a.probe = true;
         a.wmax = (int32_t)wmax;
         a.mean_degree = (double)g->num_arcs / g->n;
+        a.tile_arcs = c->tile_arcs;
         a.back = back.p + c0;
         a.ctl = ctl.p;
         a.flags = c->flags;

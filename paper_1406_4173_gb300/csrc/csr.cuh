@@ -21,9 +21,10 @@ void csr_expand(int32_t n, int64_t m, const int32_t* eu, const int32_t* ev, cons
 // from sorted keys: col, weights, row_ptr; flags repeated arcs
 void csr_finish(const uint64_t* keys, const uint32_t* vals, int64_t na, int32_t n, int64_t* rp, int32_t* col,
                 uint32_t* w_out, uint32_t* flags, cudaStream_t st);
+// checks of a CSR: *wmax (zeroed) = largest weight, *tile_arcs (zeroed; may be null) = most arcs of 32 consecutive rows
 void csr_check(int32_t n, int64_t na, const int64_t* rp, const int32_t* col, const uint32_t* w, int directed,
                uint32_t* flags, unsigned long long* wmax, cudaStream_t st, const int64_t* node_off = nullptr,
-               int32_t ngraphs = 0);
+               int32_t ngraphs = 0, unsigned long long* tile_arcs = nullptr);
 // graph-local heads of a disjoint union (flags arcs that leave their graph)
 void csr_localize(int32_t n, const int64_t* rp, const int32_t* col, const int64_t* node_off, int32_t ngraphs,
                   int32_t* lcol, uint32_t* flags, cudaStream_t st);

@@ -51,6 +51,7 @@ struct LmArgs {
     bool probe;                 // no bound on the levels is known: give up early on a graph that looks too deep
     int32_t wmax;
     double mean_degree;         // arcs per node
+    int64_t tile_arcs;          // most arcs of 32 consecutive rows (0: not known)
     uint32_t* back;             // [nitems], zeroed: set for the batches given back (their dsum stays 0)
     uint32_t* ctl;              // lm_ctl_words() zeroed words: barrier, level status, depth of each batch
     uint32_t* flags;

@@ -316,3 +316,23 @@ def test_many_unordered_targets(bc, ctx, count, size, route):
     assert rel_err(got, ref) <= FP64_TOL
     b = ctx.last_batches()
     assert b["given_back"] == 0 and b[route] > 0 and sum(b.values()) == b[route]
+
+
+@pytest.mark.parametrize("hubs,leaves", [(8, 150), (40, 40), (70, 33)])
+@pytest.mark.parametrize("k", [40, 64, 400])
+def test_hubs_in_single_tiles(bc, ctx, hubs, leaves, k):
+    """A row of hubs with neighbouring ids: tiles of thousands of arcs among tiles of 32, taken in parts."""
+    n = hubs * (leaves + 1)
+    leaf = np.arange(hubs, n)
+    g = gen.EdgeList(n=n, src=np.concatenate([np.arange(hubs - 1), (leaf - hubs) % hubs]).astype(np.int32),
+                     dst=np.concatenate([np.arange(1, hubs), leaf]).astype(np.int32))
+    S = gen.sample_targets(n, k, seed=6)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    assert rel_err(bc.brandes(G, S, ctx=ctx), ref) <= FP64_TOL
+    assert rel_err(bc.brandes(G, S, precision="fp32", ctx=ctx), ref) <= 2e-6
+    d, s = bc.sssp(G, S[:33], ctx=ctx)
+    for i, v in enumerate(S[:33]):
+        rd, rs, _ = oracle.sssp(g, int(v))
+        assert np.array_equal(d[i].cpu().numpy(), rd)
+        assert np.array_equal(s[i].cpu().numpy().view(np.uint64), rs)
