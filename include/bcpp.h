@@ -272,8 +272,10 @@ typedef struct bcpp_plan bcpp_plan;
  * rewrite them (another target set of the same size; another graph with the same n, num_arcs,
  * directedness and weights present or absent, max weight not above the one at creation).
  * Every launch first re-checks the graph and S on the device (a separate small graph) and
- * returns BCPP_EINVAL without computing when they are invalid.  On success *plan receives the
- * plan; on error *plan = NULL and nothing is held. */
+ * returns BCPP_EINVAL without computing when they are invalid.  The choice of kernel and the
+ * distance levels provided for are those of the graph at creation: see bcpp_plan_launch for a
+ * rewritten graph that needs more.  On success *plan receives the plan; on error *plan = NULL and
+ * nothing is held. */
 int bcpp_plan_brandes(bcpp_ctx *ctx, const bcpp_graph *g, const int32_t *S, int32_t nS,
                       const bcpp_opts *opts, double *bc_out, bcpp_plan **plan);
 
@@ -286,8 +288,10 @@ int bcpp_plan_brandes_pp(bcpp_ctx *ctx, const bcpp_graph *g, const int32_t *S, i
                          bcpp_plan **plan);
 
 /* Replay the plan on the context's stream and wait for it.  Status as for the direct call
- * (a batch whose settled-entry list outgrows its bound makes the plan rebuild itself once
- * with the worst-case bound and replay, so BCPP_ECAPACITY is not returned for that).  stats
+ * (a plan that the level-mask kernel gives back is captured again within the launch: with the levels of
+ * the graph's current contents where those are more than it provides for, else on the lockstep
+ * kernel, where it stays; a batch whose settled-entry list outgrows its bound makes it move to the
+ * worst-case bound, so BCPP_ECAPACITY is not returned for that).  stats
  * (may be NULL): ms_total = device time of the launch, kernel_launches = kernels in the
  * captured graph, and for Brandes++ the skeleton sizes of creation. */
 int bcpp_plan_launch(bcpp_plan *plan, bcpp_stats *stats);

@@ -2958,6 +2958,31 @@ int plan_build(bcpp_plan* p) {
     return rc;
 }
 
+// Plain plans: the evaluation captured again on masks with the levels of the graph's current contents, if those are more
+// than it provides for.  *done = false: they are not, or the masks do not serve it.
+int plan_deepen(bcpp_plan* p, bool* done) {
+    bcpp_ctx* c = p->c;
+    *done = false;
+    if (p->kind != 1 || !p->plain->levels || !p->plain->searched) return BCPP_OK;
+    PlainRun& r = *p->plain;
+    {
+        DBuf<int32_t> queue(c, p->g.n);
+        OrderWs now;
+        CK_ALLOC(queue);
+        CK_RC(hub_search(c, &p->g, queue.p, now));
+        r.ord.depth = std::max(r.ord.depth, now.depth);
+        r.ord.rest = std::max(r.ord.rest, now.rest);
+    }
+    const int provided = r.lm.lcap;
+    if (lm_levels(false, p->g.directed != 0, &r.ord, 0) <= provided) return BCPP_OK;
+    if (p->run) cudaGraphExecDestroy(p->run);
+    p->run = nullptr;
+    CK_RC(plain_batches(c, r, true));
+    CK_RC(capture_graph(c, p->cs, [&] { return plain_emit(c, r, nullptr); }, &p->run, &p->run_kernels));
+    *done = r.levels;
+    return BCPP_OK;
+}
+
 // The evaluation captured again on the lockstep kernel; checks, order, skeleton and lists stay.
 int plan_to_lockstep(bcpp_plan* p) {
     bcpp_ctx* c = p->c;
@@ -3337,6 +3362,14 @@ int bcpp_plan_launch(bcpp_plan* p, bcpp_stats* stats) {
     Timer tt(c);
     tt.start();
     int rc = plan_replay(p, stats);
+    if (rc == RC_GIVEN_BACK) {
+        // deeper than the graph at creation: more levels first, then the lockstep kernel
+        bool deeper = false;
+        const int why = c->hflags[FLAG_MASKS];
+        if (!(why & MASKS_COUNT)) rc = plan_deepen(p, &deeper);
+        if (deeper && rc == BCPP_OK) rc = plan_replay(p, stats);
+        else if (rc == BCPP_OK) rc = RC_GIVEN_BACK;
+    }
     const bool back = rc == RC_GIVEN_BACK;
     if (back) {
         rc = plan_to_lockstep(p);

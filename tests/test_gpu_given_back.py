@@ -336,3 +336,39 @@ def test_hubs_in_single_tiles(bc, ctx, hubs, leaves, k):
         rd, rs, _ = oracle.sssp(g, int(v))
         assert np.array_equal(d[i].cpu().numpy(), rd)
         assert np.array_equal(s[i].cpu().numpy().view(np.uint64), rs)
+
+
+# ---------------------------------------------------------------------------- plans of a rewritten graph
+def spine(length, n):
+    """A path of `length` nodes and n - length leaves, spread over it: n - 1 edges."""
+    leaf = np.arange(length, n)
+    src = np.concatenate([np.arange(length - 1), leaf % length])
+    dst = np.concatenate([np.arange(1, length), leaf])
+    return gen.EdgeList(n=n, src=src.astype(np.int32), dst=dst.astype(np.int32))
+
+
+def rewrite(bc, G, g):
+    new = bc.graph_from_edgelist(g)
+    G.row_ptr.copy_(new.row_ptr)
+    G.col.copy_(new.col)
+
+
+@pytest.mark.parametrize("order_sources", [True, False])
+def test_plan_follows_a_deeper_graph_and_back(bc, ctx, order_sources):
+    flat, deep, deeper = gen.star(500), spine(60, 500), spine(110, 500)
+    S = gen.sample_targets(500, 90, seed=2)
+    G = bc.graph_from_edgelist(flat)
+    plan = bc.plan_brandes(G, S, order_sources=order_sources, ctx=ctx)
+    try:
+        for g in (flat, deep, deep, flat, deeper, flat, deep):
+            rewrite(bc, G, g)
+            assert rel_err(plan.launch(), oracle.brandes(g, S)[0]) <= FP64_TOL
+            b = ctx.last_batches()
+            assert b["lockstep"] == 0 and b["given_back"] == 0, b
+        # past what the masks can hold: moves to the lockstep kernel, and is right on it
+        for g in (gen.path(500), flat):
+            rewrite(bc, G, g)
+            assert rel_err(plan.launch(), oracle.brandes(g, S)[0]) <= FP64_TOL
+            assert ctx.last_batches()["levels"] == 0
+    finally:
+        plan.close()
