@@ -57,6 +57,7 @@ constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of large
 constexpr int CTL_WIDE = 3, CTL_BACK = 4;   // batches with a path count past 32 bits; batches given back
 constexpr int CTL_LVL = CTL_WORDS;
 constexpr unsigned LVL_ANY = 1u, LVL_STOP = 2u;
+constexpr int PROBE_WORDS = 5;
 // Words between two batches' depths: a 128-byte line each, since every SM stores to them once per level (side by
 // side, stores of 152 SMs to a few lines held up everyone's loads: n = 10,000, every node a target 7.4 -> 6.3 ms,
 // Brandes++ at n = 100,000 8.6 -> 7.8 ms).
@@ -446,18 +447,21 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, SM& sm, int lane, uin
     }
 }
 
-// Pairs reached by level D and by D / 2, and rows, of a sample of the unfinished batches' rows, and all rows sampled.
-// (Its own function: inlined, it cost the kernel's loops registers, n = 10,000: 6.1 -> 6.9 ms.)
+// Pairs reached by level D and by D / 2, and all pairs, of a sample of the unfinished batches' rows; rows of these
+// batches, and all rows sampled.  (Its own function: inlined, it cost the kernel's loops registers, n = 10,000:
+// 6.1 -> 6.9 ms.)
 __device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int D, int wmax, const uint32_t* bdepth,
-                                          const int32_t* tile_item, int32_t item_base, int32_t tpb, uint32_t* probe) {
+                                          const LsItem* items, const int32_t* tile_item, int32_t item_base, int32_t tpb,
+                                          uint32_t* probe) {
     const int64_t nt = (int64_t)gridDim.x * LM_THREADS, step = max((int64_t)1, rows / nt);
-    uint32_t b1 = 0, b2 = 0, all = 0, total = 0;
+    uint32_t b1 = 0, b2 = 0, pairs = 0, open = 0, total = 0;
     for (int64_t row = ((int64_t)blockIdx.x * LM_THREADS + threadIdx.x) * step; row < rows; row += nt * step) {
         const int32_t t = (int32_t)(row >> 5);
         const int it = tile_item ? __ldg(tile_item + t) - item_base : t / tpb;
         total++;
         if ((int)bdepth[it * DEPTH_STRIDE] + wmax < D) continue;   // (a batch that is done has no masks there)
-        all++;
+        open++;
+        pairs += __ldg(&items[it].nsrc);
         for (int l = 0; l <= D; l++) {
             const uint32_t c = __popc(__ldcg(lev + (int64_t)l * rows + row));
             b2 += c;
@@ -466,19 +470,23 @@ __device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int
     }
     b1 = __reduce_add_sync(FULL, b1);
     b2 = __reduce_add_sync(FULL, b2);
-    all = __reduce_add_sync(FULL, all);
+    pairs = __reduce_add_sync(FULL, pairs);
+    open = __reduce_add_sync(FULL, open);
     total = __reduce_add_sync(FULL, total);
     if ((threadIdx.x & 31) == 0 && total) {
         atomicAdd(probe, b1);
         atomicAdd(probe + 1, b2);
-        atomicAdd(probe + 2, all);
-        atomicAdd(probe + 3, total);
+        atomicAdd(probe + 2, pairs);
+        atomicAdd(probe + 3, open);
+        atomicAdd(probe + 4, total);
     }
 }
-// D (all / b2)^(1 / dim) levels needed, with 2^dim = b2 / b1: more than 4 D?
-__device__ __noinline__ bool looks_deep(const uint32_t* probe) {
-    const float b1 = (float)__ldcg(probe), b2 = (float)__ldcg(probe + 1), all = 32.0f * (float)__ldcg(probe + 2);
-    return b2 >= 1.5f * b1 && all * b1 * b1 > b2 * b2 * b2;
+// D (pairs / b2)^(1 / dim) levels needed, with 2^dim = b2 / b1: more than 2^k D?
+__device__ __noinline__ bool looks_deep(const uint32_t* probe, int k) {
+    const float b1 = (float)__ldcg(probe), b2 = (float)__ldcg(probe + 1), g = b2 / b1;
+    float x = (float)__ldcg(probe + 2) / b2;
+    for (; k > 0; k--) x /= g;
+    return b1 > 0.0f && g >= 1.5f && x > 1.0f;
 }
 
 // Marks the batches that are given back: those deeper than `most`, which could still grow past the level where the
@@ -678,19 +686,21 @@ lm_kernel(const LmArgs A, const int sub_log) {
         const uint32_t w = __ldcg(lvl + D);
         if (w & LVL_ANY) depth = D;
         if (D - depth >= wmax || (sizeof(SG) == 4 && (w & LVL_STOP))) break;
-        // Too deep a graph shows early: a quarter of the way the pairs reached by now and by half of that
+        // Too deep a graph shows early: an eighth and a quarter of the way the pairs reached by now and by half of that
         // give the dimension that the balls around the sources grow with, and with it the level at which
-        // they hold every pair; past the levels provided for, the unfinished batches are given back without going there
-        // first (grid 300 x 300 with weights up to 16, 500 sources: 112 -> 101 ms, 97 without the attempt), and
-        // with them the later waves of a graph, when they are most of the wave.
+        // they hold every pair; past the levels provided for (at an eighth: past twice as many), the unfinished batches
+        // are given back without going there first, and with them the later waves of a graph, when they are most of
+        // the wave.  (Binary tree of 131,071 nodes, weights up to 30, 512 sources: 92.7 -> 90.1 ms, 88.2 without the attempt.)
         // Balls that hardly grow any more belong to stragglers, not to a deep graph.
-        if (!TABLE && A.probe && (D == A.lcap / 4 || D == A.lcap / 4 + 1)) {
-            uint32_t* probe = work + 2 * A.lcap;
-            if (D == A.lcap / 4) {
-                probe_levels(A.lev, A.rows, D, wmax, bdepth, A.item_tile0 ? A.tile_item + A.tile_base : nullptr,
+        const int part = A.lcap / 8;
+        if (A.probe && (D == part || D == part + 1 || D == 2 * part || D == 2 * part + 1)) {
+            const bool early = D <= part + 1;
+            uint32_t* probe = work + 2 * A.lcap + (early ? 0 : PROBE_WORDS);
+            if (D == part || D == 2 * part) {
+                probe_levels(A.lev, A.rows, D, wmax, bdepth, A.items, A.item_tile0 ? A.tile_item + A.tile_base : nullptr,
                              A.item_base, A.tpb, probe);
-            } else if (looks_deep(probe)) {
-                if (blockIdx.x == 0 && threadIdx.x == 0 && !A.item_tile0 && 2 * __ldcg(probe + 2) > __ldcg(probe + 3))
+            } else if (looks_deep(probe, early ? 4 : 2)) {
+                if (blockIdx.x == 0 && threadIdx.x == 0 && !A.item_tile0 && 2 * __ldcg(probe + 3) > __ldcg(probe + 4))
                     atomicOr(&A.flags[FLAG_MASKS], MASKS_ALL);
                 break;
             }
@@ -917,7 +927,7 @@ cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
 
 }  // namespace
 
-int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + (int64_t)nitems * DEPTH_STRIDE + 2 * (int64_t)lcap + 4; }
+int64_t lm_ctl_words(int lcap, int nitems) { return CTL_LVL + lcap + 1 + (int64_t)nitems * DEPTH_STRIDE + 2 * (int64_t)lcap + 2 * PROBE_WORDS; }
 
 cudaError_t lm_launch(const LmArgs& A, bool narrow, bool fp32, int num_sms, cudaStream_t st) {
     if (A.nitems <= 0 || A.ntiles <= 0) return cudaSuccess;
