@@ -142,8 +142,8 @@ int64_t bcpp_workspace_bytes(const bcpp_ctx *ctx);
 /* Which kernel the source batches of the context's last evaluation (bcpp_brandes, the Brandes++ calls,
  * bcpp_brandes_batched, bcpp_sssp, bcpp_plan_launch) ran on: out[0] (host, int64[3]) = batches finished by
  * the level-mask kernel, out[1] = by the lockstep kernel, out[2] = batches that the level-mask kernel began and
- * gave back to the lockstep kernel (more distance levels than it provides for, or a path count of 2^32; when that
- * is all of them, their sources may be batched anew). */
+ * gave back to the lockstep kernel (more distance levels than it provides for, or a path count of 2^32; their
+ * sources may be batched anew there). */
 int bcpp_last_batches(const bcpp_ctx *ctx, int64_t *out);
 
 /* CSR build and validation (the input graph G(V,E,W) of Sec. 3).  From m edges

@@ -227,7 +227,8 @@ def test_batched_keeps_the_other_graphs(bc, ctx, odd, back, precision):
         x = got[arena.node_ptr_host[i]:arena.node_ptr_host[i + 1]]
         assert rel_err(x, ref) <= (FP64_TOL if precision == "fp64" else 2e-6), i
     total = sum(-(-g.n // 32) for g in gs)
-    assert ctx.last_batches() == {"levels": total - back, "lockstep": back, "given_back": back}
+    b = ctx.last_batches()
+    assert b["levels"] == total - back and b["given_back"] == back and b["lockstep"] >= back
 
 
 def two_components():
@@ -258,7 +259,7 @@ def test_targets_of_a_deep_component(bc, ctx, method):
     if method == "plan":        # moves as a whole
         assert b["levels"] == 0 and b["given_back"] == b["lockstep"] > 0
     else:
-        assert b["given_back"] == b["lockstep"] and 3 <= b["lockstep"] <= 3 + (method == "plain-fp32") * 80
+        assert 3 <= b["given_back"] <= 3 + (method == "plain-fp32") * 80 and b["lockstep"] >= b["given_back"]
         assert b["levels"] >= 6
 
 
@@ -372,3 +373,27 @@ def test_plan_follows_a_deeper_graph_and_back(bc, ctx, order_sources):
             assert ctx.last_batches()["levels"] == 0
     finally:
         plan.close()
+
+
+@pytest.mark.parametrize("tail", [20, 300])
+@pytest.mark.parametrize("sources", [1, 33])
+def test_early_test_for_deep_graphs(bc, ctx, tail, sources):
+    """The tests an eighth and a quarter of the way: a grid past the levels is given up, a graph with a tail within them
+    is not, also from a single source; Dijkstra_SK tables of a deep part, too."""
+    deep = gen.with_weights(gen.grid(60, 60), 16, seed=71)
+    e = gen.erdos_renyi(700, 0.01, seed=72)
+    t = np.concatenate([[0], e.n + np.arange(tail)]).astype(np.int32)
+    within = gen.with_weights(gen.EdgeList(n=e.n + tail, src=np.concatenate([e.src, t[:-1]]),
+                                           dst=np.concatenate([e.dst, t[1:]])), 9 if tail < 100 else 1, seed=73)
+    for g, served in ((deep, False), (within, tail < 100)):
+        src = np.arange(0, g.n, g.n // sources, dtype=np.int32)[:sources]
+        d, s = bc.sssp(bc.graph_from_edgelist(g), src, ctx=ctx)
+        assert (ctx.last_batches()["levels"] > 0) == served
+        for i, v in enumerate(src):
+            rd, rs, _ = oracle.sssp(g, int(v))
+            assert np.array_equal(d[i].cpu().numpy(), rd)
+            assert np.array_equal(s[i].cpu().numpy().view(np.uint64), rs)
+    part = (np.arange(deep.n) // 1200).astype(np.int32)
+    S = gen.sample_targets(deep.n, 6, seed=5)
+    ref, _ = oracle.brandes(deep, S)
+    assert rel_err(bc.brandes_pp(bc.graph_from_edgelist(deep), S, part, ctx=ctx), ref) <= FP64_TOL
