@@ -1695,7 +1695,7 @@ struct PpRun {
         CentralityLists view() const { return CentralityLists{rp.p, ft.p, mu.p}; }
     } entry, exit;
     CentralityLists entries() const { return entry.view(); }
-    CentralityLists exits() const { return exit.rp.p ? exit.view() : entry.view(); }
+    CentralityLists exits() const { return g.directed ? exit.view() : entry.view(); }
     DBuf<uint8_t> sk_in_s;
     DBuf<int64_t> irp, icnt, itmp;
     DBuf<int32_t> icol, iw;
@@ -1707,7 +1707,8 @@ struct PpRun {
     LsArena A{};
 };
 
-// Centrality's frontier lists of the non-frontier nodes, from the entry or exit tables.
+// Centrality's frontier lists of the non-frontier nodes, from the entry or exit tables.  None (L.rp stays null) when they
+// would take more than half of the memory that is left: Centrality then reads the tables.
 int centrality_lists(bcpp_ctx* c, PpRun& r, int32_t interior, bool exits, PpRun::Lists& L) {
     const SkTables T = r.K.tables();
     const int nunits = (int)r.hunits.size();
@@ -1719,10 +1720,14 @@ int centrality_lists(bcpp_ctx* c, PpRun& r, int32_t interior, bool exits, PpRun:
     exclusive_scan<int64_t>(cnt.p, L.rp.p, (int64_t)interior + 1, nullptr, tmp.p, c->stream, c->launches);
     int64_t total = 0;
     CK_RC(to_host(c, &total, L.rp.p + interior, 1));
-    CK_ALLOC(L.ft.alloc(c, total));
-    CK_ALLOC(L.mu.alloc(c, total));
+    c->launches++;
+    const int64_t bytes = total * (int64_t)(sizeof(int2) + sizeof(uint64_t));
+    if ((bytes > (256 << 20) && bytes > free_bytes(c) / 2) || !L.ft.alloc(c, total) || !L.mu.alloc(c, total)) {
+        L.rp.free(); L.ft.free(); L.mu.free();
+        return BCPP_OK;
+    }
     ct_fill(r.units.p, nunits, T, exits, r.K.skbase.p, L.rp.p, L.ft.p, L.mu.p, c->stream);
-    c->launches += 2;
+    c->launches++;
     CK_CUDA(cudaGetLastError());
     return BCPP_OK;
 }
@@ -1804,7 +1809,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         c->launches += 2;
         if (tbr) tbr->stop();
         if (tce) tce->start();
-        centrality_launch(false, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, r.entries(), r.exits(), W.d, W.sg,
+        centrality_launch(false, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, K.skbase.p, r.entries(), r.exits(), W.d, W.sg,
                           W.dl, W.cap_n, W.bc_sum, W.bc_cmp, W.cap_bc, a.back, c->flags, c->stream);
         c->launches++;
         if (tce) tce->stop();
@@ -1931,6 +1936,13 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
             interior += std::min(sz, v0 + 64) - v0;
         }
     }
+    // (the lists before the batches' workspace, which takes what memory is left)
+    if (!r.hunits.empty() && r.s1 > r.s0) {
+        CK_ALLOC(r.units.alloc(c, (int64_t)r.hunits.size()));
+        CK_RC(to_dev(c, r.units.p, r.hunits.data(), (int64_t)r.hunits.size()));
+        CK_RC(centrality_lists(c, r, interior, false, r.entry));
+        if (g->directed) CK_RC(centrality_lists(c, r, interior, true, r.exit));
+    }
     // without non-frontier nodes Brandes_SK runs alone and may use 64-source batches
     r.spl = r.hunits.empty() ? choose_spl(c, r.s1 - r.s0, o) : 1;
     CK_RC(pp_batches(c, r, true));
@@ -1963,12 +1975,6 @@ int pp_prepare(bcpp_ctx* c, const bcpp_graph* g, uint64_t wmax, const InCsr* Tin
             A.irp = A.rp; A.icol = A.col; A.iw = A.w; A.imu = A.mu;
         }
         A.node_off = r.node_off.p;
-        CK_ALLOC(r.units.alloc(c, (int64_t)r.hunits.size()));
-        CK_RC(to_dev(c, r.units.p, r.hunits.data(), (int64_t)r.hunits.size()));
-        if (!r.hunits.empty()) {
-            CK_RC(centrality_lists(c, r, interior, false, r.entry));
-            if (g->directed) CK_RC(centrality_lists(c, r, interior, true, r.exit));
-        }
     }
     return BCPP_OK;
 }
@@ -2044,7 +2050,7 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tbr) tbr->stop();
             CK_CUDA(cudaGetLastError());
             if (tce) tce->start();
-            centrality_launch(fp32, r.units.p, (int)r.hunits.size(), r.nitems, T, K.pnodes.p, r.entries(), r.exits(),
+            centrality_launch(fp32, r.units.p, (int)r.hunits.size(), r.nitems, T, K.pnodes.p, K.skbase.p, r.entries(), r.exits(),
                               r.ws.W.d, r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
                               nullptr, c->flags, c->stream);
             c->launches++;
@@ -2068,7 +2074,7 @@ int pp_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
             if (tbr) tbr->stop();
             CK_CUDA(cudaGetLastError());
             if (tce) tce->start();
-            centrality_launch(fp32, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, r.entries(), r.exits(),
+            centrality_launch(fp32, r.units.p, (int)r.hunits.size(), cn, T, K.pnodes.p, K.skbase.p, r.entries(), r.exits(),
                               r.ws.W.d, r.ws.W.sg, r.ws.W.dl, r.ws.W.cap_n, r.ws.W.bc_sum, r.ws.W.bc_cmp, r.ws.W.cap_bc,
                               nullptr, c->flags, c->stream);
             c->launches++;

@@ -83,10 +83,13 @@ __global__ void ct_fill_kernel(const CentralityUnit* __restrict__ units, int nun
     }
 }
 
-template <typename DT>
+// LISTS: both lists are there; else those that are not are read from the tables (entries without paths add nothing: their
+// distance is that of a path, their count zero).
+template <typename DT, bool LISTS>
 __global__ void __launch_bounds__(CT_WARPS * 32, 5)
 centrality_kernel(const CentralityUnit* __restrict__ units, int nslots, SkTables T, const uint32_t* __restrict__ pnodes,
-                  CentralityLists E, CentralityLists X, const int32_t* __restrict__ d_all,
+                  const int32_t* __restrict__ skbase, CentralityLists E, CentralityLists X,
+                  const int32_t* __restrict__ d_all,
                   const uint64_t* __restrict__ sg_all, const DT* __restrict__ dl_all, int64_t cap_n, double* bc_sum,
                   double* bc_cmp, int64_t cap_bc, const uint32_t* __restrict__ skip, uint32_t* flags) {
     __shared__ CtSm<DT> s_warp[CT_WARPS];
@@ -103,16 +106,19 @@ centrality_kernel(const CentralityUnit* __restrict__ units, int nslots, SkTables
         for (int32_t v = U.v0 + (threadIdx.x >> 5); v < U.v1; v += CT_WARPS) {
             const int32_t q = U.pad + v - U.v0;
             // f(entries staged) for every stage of a list; the stage of a short list stays for a second visit
-            auto staged = [&](const CentralityLists& L, bool again, auto&& f) {
-                const int64_t a0 = __ldg(L.rp + q);
-                const int cnt = (int)(__ldg(L.rp + q + 1) - a0);
+            auto staged = [&](const CentralityLists& L, bool exits, bool again, auto&& f) {
+                const bool list = LISTS || L.rp;
+                const int64_t a0 = list ? __ldg(L.rp + q) : T.toff[U.part] + (int64_t)v * T.nf[U.part];
+                const int cnt = list ? (int)(__ldg(L.rp + q + 1) - a0) : T.nf[U.part];
                 for (int c0 = 0; c0 < cnt; c0 += CT_STAGE) {
                     const int m = min(CT_STAGE, cnt - c0);
                     if (!again || cnt > CT_STAGE) {
                         __syncwarp();
                         for (int k = lane; k < m; k += 32) {
-                            sm.ft[k] = __ldg(L.ft + a0 + c0 + k);
-                            const uint64_t mu = __ldg(L.mu + a0 + c0 + k);
+                            const int64_t e = a0 + c0 + k;
+                            sm.ft[k] = list ? __ldg(L.ft + e)
+                                            : make_int2(skbase[U.part] + c0 + k, __ldg((exits ? T.tdr : T.td) + e));
+                            const uint64_t mu = __ldg((list ? L.mu : exits ? T.tsr : T.ts) + e);
                             sm.mu[k] = mu;
                             sm.md[k] = (DT)mu;
                         }
@@ -123,7 +129,7 @@ centrality_kernel(const CentralityUnit* __restrict__ units, int nslots, SkTables
             };
             // distances (two of them at most DINF = 2^31 - 1, so a sum never wraps; DINF and above: none)
             uint32_t best = (uint32_t)DINF;
-            staged(E, false, [&](int m) {
+            staged(E, false, false, [&](int m) {
                 int k = 0;
                 for (; k + 4 <= m; k += 4) {
                     uint32_t d[4];
@@ -183,11 +189,11 @@ centrality_kernel(const CentralityUnit* __restrict__ units, int nslots, SkTables
                     __syncwarp();
                 }
             };
-            if (E.ft == X.ft) {   // undirected: one list for both
-                staged(E, true, [&](int m) { sums(m, true, true); });
+            if (T.ts == T.tsr) {   // undirected: one list for both
+                staged(E, false, true, [&](int m) { sums(m, true, true); });
             } else {
-                staged(E, true, [&](int m) { sums(m, true, false); });
-                staged(X, false, [&](int m) { sums(m, false, true); });
+                staged(E, false, true, [&](int m) { sums(m, true, false); });
+                staged(X, true, false, [&](int m) { sums(m, false, true); });
             }
             double delta = (double)((DT)sv * acc);
             if (!__any_sync(FULL, delta != 0.0)) continue;
@@ -218,18 +224,26 @@ void ct_fill(const CentralityUnit* units, int nunits, SkTables T, bool exits, co
 }
 
 void centrality_launch(bool fp32_delta, const CentralityUnit* units, int nunits, int nslots, SkTables T,
-                       const uint32_t* pnodes, CentralityLists E, CentralityLists X, const int32_t* d,
+                       const uint32_t* pnodes, const int32_t* skbase, CentralityLists E, CentralityLists X, const int32_t* d,
                        const uint64_t* sg, const void* dl, int64_t cap_n, double* bc_sum, double* bc_cmp,
                        int64_t cap_bc, const uint32_t* skip, uint32_t* flags, cudaStream_t st) {
     if (nunits <= 0 || nslots <= 0) return;
     // neighbouring blocks take one batch's neighbouring nodes: their frontier rows are shared in L2
     const dim3 grid((unsigned)nunits, (unsigned)std::min(nslots, 65535));
-    if (fp32_delta)
-        centrality_kernel<float><<<grid, CT_WARPS * 32, 0, st>>>(units, nslots, T, pnodes, E, X, d, sg, (const float*)dl,
-                                                                cap_n, bc_sum, bc_cmp, cap_bc, skip, flags);
-    else
-        centrality_kernel<double><<<grid, CT_WARPS * 32, 0, st>>>(units, nslots, T, pnodes, E, X, d, sg,
-                                                                 (const double*)dl, cap_n, bc_sum, bc_cmp, cap_bc, skip, flags);
+    auto go = [&](auto kernel, auto* c) {
+        kernel<<<grid, CT_WARPS * 32, 0, st>>>(units, nslots, T, pnodes, skbase, E, X, d, sg, c, cap_n, bc_sum, bc_cmp, cap_bc,
+                                               skip, flags);
+    };
+    const bool lists = E.rp && X.rp;
+    if (fp32_delta) {
+        const float* c = static_cast<const float*>(dl);
+        if (lists) go(centrality_kernel<float, true>, c);
+        else go(centrality_kernel<float, false>, c);
+    } else {
+        const double* c = static_cast<const double*>(dl);
+        if (lists) go(centrality_kernel<double, true>, c);
+        else go(centrality_kernel<double, false>, c);
+    }
 }
 
 }  // namespace bcpp

@@ -54,7 +54,8 @@ void sk_target_ids(const int32_t* S, int32_t nS, const int32_t* skid, int32_t* o
 // Centrality (Eq. 13), see centrality.cu.  A unit is up to 64 non-frontier nodes of a part (locals
 // [v0, v1)); pad is the index of its first node among all of them.
 struct CentralityUnit { int32_t part; int32_t v0; int32_t v1; int32_t pad; };
-// per non-frontier node the frontiers with a non-zero path count: skeleton row and distance, and the count
+// per non-frontier node the frontiers with a non-zero path count: skeleton row and distance, and the count (rp null: none,
+// the node's whole table row)
 struct CentralityLists {
     const int64_t* rp;       // [nodes + 1]
     const int2* ft;
@@ -67,7 +68,7 @@ void ct_fill(const CentralityUnit* units, int nunits, SkTables T, bool exits, co
 // all units for the slots of one Brandes_SK chunk; E, X: entry and exit lists (undirected: the same); skip (may be null):
 // non-zero for the slots to leave out
 void centrality_launch(bool fp32_delta, const CentralityUnit* units, int nunits, int nslots, SkTables T,
-                       const uint32_t* pnodes, CentralityLists E, CentralityLists X, const int32_t* d,
+                       const uint32_t* pnodes, const int32_t* skbase, CentralityLists E, CentralityLists X, const int32_t* d,
                        const uint64_t* sg, const void* dl, int64_t cap_n, double* bc_sum, double* bc_cmp,
                        int64_t cap_bc, const uint32_t* skip, uint32_t* flags, cudaStream_t st);
 
