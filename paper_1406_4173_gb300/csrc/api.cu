@@ -2834,42 +2834,47 @@ int csr_build_dev(bcpp_ctx* c, int32_t n, int64_t m, const int32_t* eu, const in
     if (ew && !w_out && m > 0) return BCPP_EINVAL;
     CK_RC(reset_flags(c));
     const int64_t na = directed ? m : 2 * m;
-    if (m > 0 && n > 0) {
-        DBuf<uint32_t> counts(c, (int64_t)n + 1), place(c, na), longest(c, 2);   // longest row, long rows
-        DBuf<int64_t> stmp(c, scan_tmp_elems((int64_t)n + 1));
-        CK_ALLOC(counts); CK_ALLOC(place); CK_ALLOC(longest); CK_ALLOC(stmp);
-        CK_CUDA(cudaMemsetAsync(counts.p, 0, ((size_t)n + 1) * sizeof(uint32_t), c->stream));
-        CK_CUDA(cudaMemsetAsync(longest.p, 0, 2 * sizeof(uint32_t), c->stream));
-        csr_count(n, m, eu, ev, ew, directed, counts.p, place.p, longest.p, c->flags, c->stream);
-        c->launches += 2;
-        uint32_t hl = 0;
-        CK_CUDA(cudaMemcpyAsync(&hl, longest.p, sizeof(hl), cudaMemcpyDeviceToHost, c->stream));
-        CK_RC(sync_flags(c));
-        if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
-        if (hl <= CSR_LONG_ROW) {
-            exclusive_scan<uint32_t>(counts.p, rp, (int64_t)n + 1, nullptr, stmp.p, c->stream, c->launches);
-            csr_scatter(m, eu, ev, ew, directed, rp, place.p, col, ew ? w_out : nullptr, c->stream);
-            // (the counts are no longer needed: the list of long rows takes their place)
-            CK_CUDA(csr_sort_rows(n, hl, rp, col, ew ? w_out : nullptr, reinterpret_cast<int32_t*>(counts.p),
-                                  longest.p + 1, c->flags, c->stream));
-            c->launches += 3;
-            CK_CUDA(cudaGetLastError());
-            *num_arcs_out = na;
-            return finish_status(c, nullptr);
-        }
+    if (n == 0 && m > 0) return BCPP_EINVAL;   // no end is in range
+    if (m == 0) {
+        CK_CUDA(cudaMemsetAsync(rp, 0, ((size_t)n + 1) * sizeof(int64_t), c->stream));
+        *num_arcs_out = 0;
+        return finish_status(c, nullptr);
     }
-    DBuf<uint64_t> keys(c, na), kb(c, na);
-    DBuf<uint32_t> vals(c, na), vb(c, na);
-    DBuf<int64_t> hist(c, radix_hist_elems(na)), tmp(c, scan_tmp_elems(radix_hist_elems(na)));
-    CK_ALLOC(keys); CK_ALLOC(kb); CK_ALLOC(vals); CK_ALLOC(vb); CK_ALLOC(hist); CK_ALLOC(tmp);
-    csr_expand(n, m, eu, ev, ew, directed, keys.p, vals.p, c->flags, c->stream);
-    c->launches++;
+    uint32_t* w = ew ? w_out : nullptr;
+    const int64_t most = na / CSR_LONG_ROW + 1;   // rows above CSR_LONG_ROW, and one
+    DBuf<uint32_t> counts(c, (int64_t)n + 1), place(c, na), nlong(c, 1);
+    DBuf<CsrLong> info(c, 1);
+    DBuf<int32_t> rows(c, most);
+    DBuf<int64_t> len(c, most), stmp(c, scan_tmp_elems(std::max<int64_t>((int64_t)n + 1, most)));
+    CK_ALLOC(counts); CK_ALLOC(place); CK_ALLOC(nlong); CK_ALLOC(info); CK_ALLOC(rows); CK_ALLOC(len); CK_ALLOC(stmp);
+    CK_CUDA(cudaMemsetAsync(counts.p, 0, ((size_t)n + 1) * sizeof(uint32_t), c->stream));
+    CK_CUDA(cudaMemsetAsync(nlong.p, 0, sizeof(uint32_t), c->stream));
+    CK_CUDA(cudaMemsetAsync(info.p, 0, sizeof(CsrLong), c->stream));
+    csr_count(n, m, eu, ev, ew, directed, counts.p, place.p, info.p, rows.p, len.p, c->flags, c->stream);
+    c->launches += 2;
+    CsrLong h{};
+    CK_CUDA(cudaMemcpyAsync(&h, info.p, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     CK_RC(sync_flags(c));
     if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
-    radix_sort_pairs(keys.p, vals.p, kb.p, vb.p, na, bits_for((uint64_t)n * (uint64_t)n), hist.p, tmp.p, c->stream,
-                     c->launches);
-    csr_finish(keys.p, vals.p, na, n, rp, col, ew ? w_out : nullptr, c->flags, c->stream);
-    c->launches += 2;
+    exclusive_scan<uint32_t>(counts.p, rp, (int64_t)n + 1, nullptr, stmp.p, c->stream, c->launches);
+    csr_scatter(m, eu, ev, ew, directed, rp, place.p, col, w, c->stream);
+    // (the counts are no longer needed: the list of long rows takes their place)
+    CK_CUDA(csr_sort_rows(n, h.longest, rp, col, w, reinterpret_cast<int32_t*>(counts.p), nlong.p, c->flags, c->stream));
+    c->launches += 3;
+    if (h.rows) {
+        place.free();
+        const int64_t arcs = (int64_t)h.arcs;
+        DBuf<int64_t> off(c, (int64_t)h.rows + 1), hist(c, radix_hist_elems(arcs)), tmp(c, scan_tmp_elems(radix_hist_elems(arcs)));
+        DBuf<uint64_t> keys(c, arcs), kb(c, arcs);
+        DBuf<uint32_t> vals(c, arcs), vb(c, arcs);
+        CK_ALLOC(off); CK_ALLOC(hist); CK_ALLOC(tmp); CK_ALLOC(keys); CK_ALLOC(kb); CK_ALLOC(vals); CK_ALLOC(vb);
+        exclusive_scan<int64_t>(len.p, off.p, h.rows, off.p + h.rows, stmp.p, c->stream, c->launches);
+        csr_gather_rows(n, (int32_t)h.rows, rows.p, off.p, rp, col, w, keys.p, vals.p, c->stream);
+        radix_sort_pairs(keys.p, vals.p, kb.p, vb.p, arcs, bits_for((uint64_t)h.rows * (uint64_t)n), hist.p, tmp.p, c->stream,
+                         c->launches);
+        csr_return_rows(n, arcs, rows.p, off.p, rp, keys.p, vals.p, col, w, c->flags, c->stream);
+        c->launches += 2;
+    }
     CK_CUDA(cudaGetLastError());
     *num_arcs_out = na;
     return finish_status(c, nullptr);

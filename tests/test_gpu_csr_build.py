@@ -95,3 +95,40 @@ def test_build_pairs_of_rows(bc, a, b, weighted):
             with pytest.raises(bc.BcppError):
                 bc.csr_build(n, np.append(src, np.int32(u)), np.append(dst, dst[at[0]]),
                              np.append(w, np.uint32(7)) if weighted else None, True)
+
+
+@pytest.mark.parametrize("hubs", [1, 2, 5])
+@pytest.mark.parametrize("end", ["first", "second"])
+@pytest.mark.parametrize("shuffled", [False, True])
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_build_several_long_rows(bc, hubs, end, shuffled, directed, weighted):
+    """Rows above 16,384 arcs are sorted apart: several of them, with shorter rows between, their nodes as first or
+    second ends, grouped (a warp's edges share an end) or not."""
+    rng = np.random.default_rng(hubs)
+    n, deg = 20011, 16384 + 37
+    ids = np.sort(rng.choice(n, hubs, replace=False))
+    pairs = [np.stack([np.full(deg, h), rng.choice(np.delete(np.arange(n), ids), deg, replace=False)]) for h in ids]
+    pairs.append(rng.choice(np.delete(np.arange(n), ids), (2, 3000)))
+    a, b = np.concatenate(pairs, axis=1)
+    if end == "second":
+        a, b = b, a
+    key = np.minimum(a, b).astype(np.int64) * n + np.maximum(a, b)
+    keep = np.unique(key, return_index=True)[1]
+    keep = keep[a[keep] != b[keep]]
+    keep = rng.permutation(keep) if shuffled else np.sort(keep)
+    src, dst = a[keep].astype(np.int32), b[keep].astype(np.int32)
+    w = rng.integers(1, 1000, len(src)).astype(np.uint32)
+    G = bc.csr_build(n, src, dst, w if weighted else None, directed)
+    rp, col, ww = host_csr(n, src, dst, w, directed)
+    assert np.array_equal(G.row_ptr.cpu().numpy(), rp)
+    assert np.array_equal(G.col.cpu().numpy(), col)
+    if weighted:
+        assert np.array_equal(G.w.cpu().numpy().view(np.uint32), ww)
+
+
+def test_build_of_nothing(bc):
+    none = np.zeros(0, np.int32)
+    for n in (0, 1, 70):
+        G = bc.csr_build(n, none, none, None, False)
+        assert np.array_equal(G.row_ptr.cpu().numpy(), np.zeros(n + 1, np.int64)) and G.col.numel() == 0
