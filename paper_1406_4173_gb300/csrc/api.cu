@@ -422,7 +422,9 @@ std::vector<LsItem> spread_items(const std::vector<LsItem>& items, int64_t n, bo
     if (weighted || n > 4096) return items;
     int64_t total = 0;
     for (const LsItem& it : items) total += it.nsrc;
-    const int b = balanced_width(total, slots_cap, 32);
+    const int pieces = 32 / balanced_width(total, slots_cap, 32);
+    if (pieces <= 1) return items;
+    const int b = (32 + pieces - 1) / pieces;
     std::vector<LsItem> out;
     for (const LsItem& it : items)
         for (int32_t s = 0; s < it.nsrc; s += b) out.push_back(LsItem{it.g, it.src_off + s, std::min(b, it.nsrc - s), it.aux});
@@ -916,13 +918,13 @@ struct LmWs {
     DBuf<uint32_t> back;       // per batch: given back
     DBuf<char> sg, cc;
     DBuf<double> dsum, bcs, bcc;
-    DBuf<int32_t> tile0, tile_item;
-    DBuf<LmRun> runs;
+    DBuf<int32_t> tile0, tile_item;   // (and the runs behind tile0, in one copy)
+    LmRun* run_list = nullptr;
 
     void release() {
         waves.clear();
         lev.free(); seen.free(); ctl.free(); back.free(); sg.free(); cc.free(); dsum.free(); bcs.free(); bcc.free();
-        tile0.free(); tile_item.free(); runs.free();
+        tile0.free(); tile_item.free();
     }
 };
 
@@ -994,7 +996,7 @@ int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_gr
     const int64_t row_bytes = 32 * ((narrow ? 4 : 8) + (forward ? 0 : L.fp32 ? 4 : 8)) + 8 + 4 + 4ll * lcap;
     const int64_t budget = free_bytes(c);
     int64_t total = 0, largest = 0;
-    std::vector<int32_t> tile0;
+    std::vector<int32_t> tile0;   // first tile of each batch
     if (!one_graph) tile0.resize((size_t)nitems + 1);
     for (int i = 0; i < nitems; i++) {
         const int64_t t = (size_of(items[i].g) + 31) / 32;
@@ -1047,15 +1049,18 @@ int lm_alloc(bcpp_ctx* c, LmWs& L, const std::vector<LsItem>& items, bool one_gr
         CK_ALLOC(L.cc.alloc(c, rows * 32 * (L.fp32 ? 4 : 8)));
         CK_ALLOC(L.bcs.alloc(c, nodes));
         CK_ALLOC(L.bcc.alloc(c, nodes));
-        CK_ALLOC(L.runs.alloc(c, (int64_t)runs.size()));
-        CK_RC(to_dev(c, L.runs.p, runs.data(), (int64_t)runs.size()));
     }
-    if (one_graph) {
-        L.tpb = (int32_t)largest;
-    } else {
-        CK_ALLOC(L.tile0.alloc(c, (int64_t)nitems + 1));
+    if (one_graph) L.tpb = (int32_t)largest;
+    if (forward) runs.clear();
+    // tile0 and the runs (16-byte aligned) in one copy: each costs a wait for the stream
+    const size_t at = (tile0.size() + 3) / 4 * 4;
+    tile0.resize(at + 4 * runs.size());
+    std::memcpy(tile0.data() + at, runs.data(), runs.size() * sizeof(LmRun));
+    CK_ALLOC(L.tile0.alloc(c, (int64_t)tile0.size()));
+    CK_RC(to_dev(c, L.tile0.p, tile0.data(), (int64_t)tile0.size()));
+    L.run_list = reinterpret_cast<LmRun*>(L.tile0.p + at);
+    if (!one_graph) {
         CK_ALLOC(L.tile_item.alloc(c, total));
-        CK_RC(to_dev(c, L.tile0.p, tile0.data(), (int64_t)nitems + 1));
         lm_tile_items(L.tile0.p, nitems, (int32_t)total, L.tile_item.p, c->stream);
         c->launches++;
     }
@@ -1120,7 +1125,7 @@ int lm_emit(bcpp_ctx* c, LmWs& L, const LsArena& A, const LsParams& P, const LsI
         const LmArgs a = lm_wave_args(L, w, A, P, items, wmax);
         CK_CUDA(cudaMemsetAsync(L.ctl.p, 0, (size_t)lm_ctl_words(L.lcap, a.nitems) * sizeof(uint32_t), c->stream));
         CK_CUDA(lm_launch(a, L.narrow, L.fp32, c->num_sms, c->stream));
-        lm_accumulate(a, L.runs.p + w.run0, w.nruns, w.natiles, L.bcs.p, L.bcc.p, c->stream);
+        lm_accumulate(a, L.run_list + w.run0, w.nruns, w.natiles, L.bcs.p, L.bcc.p, c->stream);
         c->launches += 2;
     }
     if (tb) tb->stop();

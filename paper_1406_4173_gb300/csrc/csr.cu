@@ -4,7 +4,7 @@
 // and zero weights.  Arcs are counted per tail (the count's atomics also give every arc a place in
 // its row), scattered to their rows, and each row is sorted where it lies: in a warp's registers up to 32
 // arcs, in shared memory up to CSR_LONG_ROW.  Nothing but the arcs themselves and one 32-bit place per arc
-// is moved, and both fit the 129 MB L2 at 16 M arcs: 1.97 -> 0.66 ms for 8 M edges on 1 M nodes.  The arcs of longer rows
+// is moved, and both fit the 129 MB L2 at 16 M arcs: 1.97 -> 0.70 ms for 8 M edges on 1 M nodes.  The arcs of longer rows
 // are sorted together by the library's radix sort of 64-bit (row index, head) keys (all arcs of the graph that way
 // before: star of 8 M edges 2.27 -> 1.49 ms).
 #include <algorithm>
