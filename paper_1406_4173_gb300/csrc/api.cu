@@ -25,6 +25,11 @@ struct PoolBlock {
     bool used;
 };
 
+// Most arcs of 32 consecutive rows and of one row (0: not known).
+struct RowStats {
+    int64_t tile = 0, row = 0;
+};
+
 struct bcpp_ctx {
     cudaStream_t stream = nullptr;
     int device = 0;
@@ -36,7 +41,7 @@ struct bcpp_ctx {
     int64_t launches = 0;
     int order_factor = 8;            // settled-entry capacity per node of a batch (retry: worst case)
     int64_t ran[3] = {};             // bcpp_last_batches of the last call
-    int64_t tile_arcs = 0;           // of the graph checked last (validate_csr)
+    RowStats rows;                   // of the graph checked last (validate_csr)
     cudaEvent_t ev[8] = {};
 
     void* acquire(size_t bytes) {
@@ -297,20 +302,19 @@ int check_graph_struct(const bcpp_graph* g) {
     return BCPP_OK;
 }
 
-// Validate a CSR; on success *wmax_out = max weight (1 for unit weights), and c->tile_arcs = the most arcs of 32
-// consecutive rows.
+// Validate a CSR; on success *wmax_out = max weight (1 for unit weights), and c->rows.
 int validate_csr(bcpp_ctx* c, const bcpp_graph* g, uint64_t* wmax_out, const int64_t* node_off = nullptr,
                  int32_t ngraphs = 0) {
-    DBuf<unsigned long long> wmax(c, 2);
+    DBuf<unsigned long long> wmax(c, 3);
     CK_ALLOC(wmax);
-    CK_CUDA(cudaMemsetAsync(wmax.p, 0, 2 * sizeof(unsigned long long), c->stream));
+    CK_CUDA(cudaMemsetAsync(wmax.p, 0, 3 * sizeof(unsigned long long), c->stream));
     csr_check(g->n, g->num_arcs, g->row_ptr, g->col, g->w, g->directed, c->flags, wmax.p, c->stream, node_off,
               ngraphs, wmax.p + 1);
     c->launches++;
-    unsigned long long h[2] = {0, 0};
-    CK_RC(to_host(c, h, (const unsigned long long*)wmax.p, 2));
+    unsigned long long h[3] = {0, 0, 0};
+    CK_RC(to_host(c, h, (const unsigned long long*)wmax.p, 3));
     unsigned long long hw = h[0];
-    c->tile_arcs = (int64_t)h[1];
+    c->rows = RowStats{(int64_t)h[1], (int64_t)h[2]};
     CK_RC(sync_flags(c));
     if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
     if (hw == 0) hw = 1;
@@ -911,7 +915,8 @@ struct LmWs {
     bool narrow = true;
     bool fp32 = false;         // FP32 dependencies
     double mean_degree = 16;   // arcs per node
-    int64_t tile_arcs = 0;     // most arcs of 32 consecutive rows (0: not known)
+    RowStats rows;
+    bool few = false;          // see LmArgs
     int32_t tpb = 0;           // uniform layout: tiles per batch
     int64_t nodes = 0;         // global nodes
     DBuf<uint32_t> lev, seen, ctl;
@@ -939,6 +944,14 @@ int64_t free_bytes(bcpp_ctx* c) {
     for (auto& b : c->pool)
         if (!b.used) reusable += (int64_t)b.bytes;
     return (int64_t)((double)((int64_t)fr + reusable) * 0.80);
+}
+
+// Weighted passes look at a long row once per distance value, one warp at 32 x 4 arcs a step: where that takes far
+// longer than everything else of a level, the lockstep kernel is faster (star of 20,000, weights up to 30, 500
+// targets: 28.8 ms, 16.8 in lockstep; the figures below are microseconds).
+bool lm_long_row(bool weighted, const RowStats& rows, double batches, double arcs) {
+    const double row = 0.0094 * (double)rows.row, rest = 1e-5 * batches * arcs;
+    return weighted && row > 60 && row > 4 * rest;
 }
 
 // Calls the level-mask kernel serves: batches of 32 sources, weights up to LM_MAX_WEIGHT, 32-bit arc offsets, FP64
@@ -1096,7 +1109,9 @@ LmArgs lm_wave_args(const LmWs& L, const LmWave& w, const LsArena& A, const LsPa
     a.probe = !L.bounded;
     a.wmax = (int32_t)wmax;
     a.mean_degree = L.mean_degree;
-    a.tile_arcs = L.tile_arcs;
+    a.tile_arcs = L.rows.tile;
+    a.row_arcs = L.rows.row;
+    a.few = L.few;
     a.back = L.back.p + w.i0;
     a.ctl = L.ctl.p;
     a.flags = P.flags;
@@ -1146,7 +1161,7 @@ struct PlainRun {
     bcpp_opts o{};
     double* bc_out = nullptr;
     uint64_t wmax = 1;
-    int64_t tile_arcs = 0;         // of g (see LmArgs)
+    RowStats rows;                 // of g
     int64_t ns = 0;
     bool trivial = false;          // |S| < 2 or n == 0: all zeros
     DBuf<uint8_t> in_s;
@@ -1215,11 +1230,13 @@ int plain_batches(bcpp_ctx* c, PlainRun& r, bool masks, const std::vector<LsItem
     if (fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     r.lm.fp32 = fp32;
     r.lm.mean_degree = (double)g->num_arcs / n;
-    r.lm.tile_arcs = r.tile_arcs;
+    r.lm.rows = r.rows;
+    r.lm.few = (int64_t)hitems.size() <= slot_capacity(c, o, r.cl);
     r.lm.bounded = lm_bounded(g->w != nullptr, g->directed != 0, ord);
-    if (masks && lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) && !(ord && lm_dense_deep(*ord, r.ns, n)))
+    if (masks && lm_serves(c, o, r.spl, n, g->num_arcs, g->w ? r.wmax : 1, !g->w) && !(ord && lm_dense_deep(*ord, r.ns, n)) &&
+        !lm_long_row(g->w != nullptr, r.rows, (double)hitems.size(), (double)g->num_arcs))
         CK_RC(lm_alloc(c, r.lm, hitems, true, [&](int32_t) { return n; }, n,
-                       lm_levels(g->w != nullptr, g->directed != 0, ord, rows, r.tile_arcs, r.lm.mean_degree), true, &r.levels));
+                       lm_levels(g->w != nullptr, g->directed != 0, ord, rows, r.rows.tile, r.lm.mean_degree), true, &r.levels));
     if (!r.levels && !fp32 && width < 32) hitems = make_items(0, r.s0, r.s1, width);
     if (only && !fp32) hitems = spread_items(hitems, n, g->w != nullptr, slot_capacity(c, o, r.cl));
     r.nitems = (int)hitems.size();
@@ -1244,7 +1261,7 @@ int plain_prepare(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     r.g = *g; r.S = S; r.nS = nS; r.o = o; r.bc_out = bc_out;
     CK_RC(reset_flags(c));
     CK_RC(validate_csr(c, g, &r.wmax));
-    r.tile_arcs = c->tile_arcs;
+    r.rows = c->rows;
     CK_ALLOC(r.wmaxd.alloc(c, 1));
     if (nS > 0) {
         CK_ALLOC(r.in_s.alloc(c, n));
@@ -1803,6 +1820,7 @@ int pp_levels_emit(bcpp_ctx* c, PpRun& r, Timer* tbr, Timer* tce) {
         a.probe = !r.lm.bounded;
         a.wmax = (int32_t)K.wmax_sk;
         a.mean_degree = r.lm.mean_degree;
+        a.few = r.lm.few;
         a.back = r.lm.back.p + c0;
         a.ctl = r.lm.ctl.p;
         a.flags = c->flags;
@@ -1839,6 +1857,7 @@ int pp_batches(bcpp_ctx* c, PpRun& r, bool masks, const std::vector<LsItem>* onl
     hitems = only ? *only : make_items(0, r.s0, r.s1, 32 * r.spl);
     if (masks && N > 0 && !hitems.empty() && lm_serves(c, o, r.spl, N, K.arcs, K.wmax_sk)) {
         r.lm.mean_degree = (double)K.arcs / N;
+        r.lm.few = (int64_t)hitems.size() <= slot_capacity(c, o, choose_cluster(c, (int)hitems.size(), o));
         // skeleton distances are the distances in G
         const OrderWs* ord = r.ordered ? &r.ord : nullptr;
         const int lcap = lm_levels(g->w != nullptr, g->directed != 0, ord, (int64_t)hitems.size() * N);
@@ -2652,7 +2671,7 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
                 const int32_t* src, uint64_t wmax, int32_t* dist_out, uint64_t* sigma_out, DBuf<uint32_t>& back,
                 bool* done) {
     const int64_t tpb = ((int64_t)g->n + 31) / 32, cap_n = tpb * 32;
-    const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr, nitems * cap_n, c->tile_arcs, (double)g->num_arcs / g->n);
+    const int lcap = lm_levels(g->w != nullptr, g->directed != 0, nullptr, nitems * cap_n, c->rows.tile, (double)g->num_arcs / g->n);
     const int64_t each = cap_n * (32 * (4 + 8) + 8 + 4 + 4ll * lcap);
     int64_t chunk = std::min<int64_t>(nitems, std::min(free_bytes(c), std::max(LM_WAVE_BYTES, each)) / each);
     chunk = std::min<int64_t>(chunk, ((1ll << 31) - 1) / cap_n);
@@ -2682,7 +2701,8 @@ int sssp_levels(bcpp_ctx* c, const bcpp_graph* g, const LsArena& A, const LsItem
         a.probe = true;
         a.wmax = (int32_t)wmax;
         a.mean_degree = (double)g->num_arcs / g->n;
-        a.tile_arcs = c->tile_arcs;
+        a.tile_arcs = c->rows.tile;
+        a.row_arcs = c->rows.row;
         a.back = back.p + c0;
         a.ctl = ctl.p;
         a.flags = c->flags;
@@ -2732,7 +2752,8 @@ int sssp_dev(bcpp_ctx* c, const bcpp_graph* g, const int32_t* src, int32_t nsrc,
     }
     A.node_off = node_off.p;
     bool done = false;
-    if (lm_serves(c, o, 1, n, g->num_arcs, g->w ? wmax : 1)) {
+    if (lm_serves(c, o, 1, n, g->num_arcs, g->w ? wmax : 1) &&
+        !lm_long_row(g->w != nullptr, c->rows, nitems, (double)g->num_arcs)) {
         DBuf<uint32_t> back;
         CK_RC(sssp_levels(c, g, A, items.p, nitems, src, wmax, dist_out, sigma_out, back, &done));
         if (done) {

@@ -256,7 +256,7 @@ __global__ void csr_sort_long_kernel(const int64_t* __restrict__ rp, int32_t* co
 __global__ void csr_check_kernel(int32_t n, int64_t na, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                                  const uint32_t* __restrict__ w, int directed, uint32_t* flags,
                                  unsigned long long* wmax, const int64_t* __restrict__ node_off, int32_t ngraphs,
-                                 unsigned long long* tile_out) {
+                                 unsigned long long* stats) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -264,10 +264,13 @@ __global__ void csr_check_kernel(int32_t n, int64_t na, const int64_t* __restric
         if (rp[0] != 0 || rp[n] != na) flag_invalid(flags, WHY_ROWPTR);
     }
     uint32_t local_max = 0;
-    int64_t tile_arcs = 0;
+    int64_t tile_arcs = 0, row_arcs = 0;
     for (int64_t u = warp; u < n; u += nwarps) {
         const int64_t a0 = rp[u], a1 = rp[u + 1];
-        if (tile_out && (u & 31) == 0) tile_arcs = max(tile_arcs, rp[min(u + 32, (int64_t)n)] - a0);
+        if (stats) {
+            row_arcs = max(row_arcs, a1 - a0);
+            if ((u & 31) == 0) tile_arcs = max(tile_arcs, rp[min(u + 32, (int64_t)n)] - a0);
+        }
         if (a0 > a1 || a0 < 0 || a1 > na) {
             if (lane == 0) flag_invalid(flags, WHY_ROWPTR);
             continue;
@@ -306,7 +309,8 @@ __global__ void csr_check_kernel(int32_t n, int64_t na, const int64_t* __restric
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) local_max = max(local_max, __shfl_xor_sync(FULL, local_max, o));
     if (lane == 0 && local_max) atomicMax(wmax, (unsigned long long)local_max);
-    if (lane == 0 && tile_arcs > 0) atomicMax(tile_out, (unsigned long long)tile_arcs);
+    if (lane == 0 && tile_arcs > 0) atomicMax(stats, (unsigned long long)tile_arcs);
+    if (lane == 0 && row_arcs > 0) atomicMax(stats + 1, (unsigned long long)row_arcs);
 }
 
 // Targets: in range and distinct; sets in_s[v] = 1 for v in S.
@@ -421,9 +425,9 @@ cudaError_t csr_sort_rows(int32_t n, uint32_t longest, const int64_t* rp, int32_
 
 void csr_check(int32_t n, int64_t na, const int64_t* rp, const int32_t* col, const uint32_t* w, int directed,
                uint32_t* flags, unsigned long long* wmax, cudaStream_t st, const int64_t* node_off, int32_t ngraphs,
-               unsigned long long* tile_arcs) {
+               unsigned long long* stats) {
     csr_check_kernel<<<grid_for((int64_t)n * 32, 256), 256, 0, st>>>(n, na, rp, col, w, directed, flags, wmax,
-                                                                      node_off, ngraphs, tile_arcs);
+                                                                      node_off, ngraphs, stats);
 }
 
 void csr_localize(int32_t n, const int64_t* rp, const int32_t* col, const int64_t* node_off, int32_t ngraphs,

@@ -505,9 +505,9 @@ __device__ __noinline__ void mark_back(uint32_t* bdepth, int nitems, int most, u
     }
 }
 
-// A batch has a path count past 32 bits; most of them: the level is the last.
-__device__ __forceinline__ void note_wide(uint32_t* b, uint32_t* ctl, uint32_t* lvl, int nitems) {
-    if (atomicExch(b + 1, 1u) == 0u && 2 * (int)(atomicAdd(ctl + CTL_WIDE, 1u) + 1u) > nitems) atomicOr(lvl, LVL_STOP);
+// A batch has a path count past 32 bits; more than `most` of them: the level is the last.
+__device__ __forceinline__ void note_wide(uint32_t* b, uint32_t* ctl, uint32_t* lvl, int most) {
+    if (atomicExch(b + 1, 1u) == 0u && (int)(atomicAdd(ctl + CTL_WIDE, 1u) + 1u) > most) atomicOr(lvl, LVL_STOP);
 }
 
 template <typename SG, typename DT, bool WEIGHTED, bool MULT, bool TABLE>
@@ -661,7 +661,7 @@ lm_kernel(const LmArgs A, const int sub_log) {
                         A.ts[tab + (int64_t)r * nf + s] = acc;
                     }
                     if (drow) drow[r * 32 + s] = D;
-                    if (sizeof(SG) == 4 && (acc >> 32) != 0) note_wide(bdepth + x.it * DEPTH_STRIDE, A.ctl, lvl + D, A.nitems);
+                    if (sizeof(SG) == 4 && (acc >> 32) != 0) note_wide(bdepth + x.it * DEPTH_STRIDE, A.ctl, lvl + D, A.nitems / (A.few ? 3 : 2));
                 }
             };
             tile_sums<true, WEIGHTED, MULT, TABLE, SG, uint64_t>(
@@ -710,8 +710,15 @@ lm_kernel(const LmArgs A, const int sub_log) {
     const uint32_t nwide = sizeof(SG) == 4 ? __ldcg(A.ctl + CTL_WIDE) : 0u;
     const bool cut = s_last - depth < wmax && (sizeof(SG) == 4 || !A.bounded);
     if (cut || nwide) {
-        mark_back(bdepth, A.nitems, 2 * nwide > (uint32_t)A.nitems ? -1 : cut ? s_last - wmax : INT32_MAX, A.back, A.ctl, A.flags);
-        if (!grid_barrier(A.ctl, A.flags) || __ldcg(A.ctl + CTL_BACK) == (uint32_t)A.nitems) return;
+        const int some = A.nitems / (A.few ? 3 : 2);
+        mark_back(bdepth, A.nitems, (int)nwide > some ? -1 : cut ? s_last - wmax : INT32_MAX, A.back, A.ctl, A.flags);
+        if (!grid_barrier(A.ctl, A.flags)) return;
+        const int back = (int)__ldcg(A.ctl + CTL_BACK);
+        if (back == A.nitems) return;
+        if (A.few && back > some) {
+            for (int it = blockIdx.x * LM_THREADS + threadIdx.x; it < A.nitems; it += gridDim.x * LM_THREADS) A.back[it] = 1u;
+            return;
+        }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && A.phase_ns) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
 
@@ -913,7 +920,8 @@ cudaError_t lm_go(const LmArgs& A, int num_sms, cudaStream_t st) {
     while (sub_log < LM_MAX_SUB && (double)((int64_t)A.ntiles << sub_log) < goal) sub_log++;
     // And where single tiles hold far more arcs than a warp's share of a level, which would wait for their warps (with
     // many tiles the others go on meanwhile): 50,000 nodes on 60 hubs of neighbouring ids, 64 targets: 12.0 -> 5.0 ms.
-    if (A.ntiles < 2 * warps) {
+    // (Not where one row holds most of them: star of 20,000, weights up to 30, 500 targets: 28.8 ms, in parts 35.9.)
+    if (A.ntiles < 2 * warps && A.row_arcs < A.tile_arcs / 2) {
         const double share = 32.0 * A.mean_degree * A.ntiles / warps;
         while (sub_log < LM_MAX_SUB && (double)(A.tile_arcs >> sub_log) > std::max(4.0 * LM_CAP, 4.0 * share)) sub_log++;
     }

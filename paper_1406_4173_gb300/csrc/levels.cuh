@@ -48,10 +48,11 @@ struct LmArgs {
     int64_t rows;               // 32 ntiles
     int32_t lcap;               // levels provided for
     bool bounded;               // no distance reaches lcap: a pass that ends there is complete
+    bool few;                   // when more than a third of the batches are given back, all are
     bool probe;                 // no bound on the levels is known: give up early on a graph that looks too deep
     int32_t wmax;
     double mean_degree;         // arcs per node
-    int64_t tile_arcs;          // most arcs of 32 consecutive rows (0: not known)
+    int64_t tile_arcs, row_arcs;   // most arcs of 32 consecutive rows, of one row (0: not known)
     uint32_t* back;             // [nitems], zeroed: set for the batches given back (their dsum stays 0)
     uint32_t* ctl;              // lm_ctl_words() zeroed words: barrier, level status, depth of each batch
     uint32_t* flags;

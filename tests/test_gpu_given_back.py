@@ -397,3 +397,25 @@ def test_early_test_for_deep_graphs(bc, ctx, tail, sources):
     S = gen.sample_targets(deep.n, 6, seed=5)
     ref, _ = oracle.brandes(deep, S)
     assert rel_err(bc.brandes_pp(bc.graph_from_edgelist(deep), S, part, ctx=ctx), ref) <= FP64_TOL
+
+
+@pytest.mark.parametrize("method", ["plain", "pp"])
+def test_few_batches_go_together(bc, ctx, method):
+    """Three of six batches do not fit: the lockstep kernel takes all six at once."""
+    g = two_components()
+    S = np.concatenate([np.arange(0, 600, 6), np.arange(600, 900, 4)]).astype(np.int32)
+    ref, _ = oracle.brandes(g, S)
+    G = bc.graph_from_edgelist(g)
+    got = bc.brandes(G, S, ctx=ctx) if method == "plain" else bc.brandes_pp(G, S, g.part, ctx=ctx)
+    assert rel_err(got, ref) <= FP64_TOL
+    b = ctx.last_batches()
+    assert b["levels"] == 0 and b["given_back"] == 6
+
+
+def test_long_row_of_a_weighted_graph(bc, ctx):
+    g = gen.with_weights(gen.star(9000), 20, seed=9)
+    S = gen.sample_targets(g.n, 70, seed=9)
+    ref, _ = oracle.brandes(g, S)
+    assert rel_err(bc.brandes(bc.graph_from_edgelist(g), S, ctx=ctx), ref) <= FP64_TOL
+    b = ctx.last_batches()
+    assert b["levels"] == 0 and b["given_back"] == 0
