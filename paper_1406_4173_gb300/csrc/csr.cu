@@ -263,6 +263,9 @@ __global__ void csr_check_kernel(int32_t n, int64_t na, const int64_t* __restric
     if (warp == 0 && lane == 0) {
         if (rp[0] != 0 || rp[n] != na) flag_invalid(flags, WHY_ROWPTR);
     }
+    __shared__ unsigned long long s_max[3];   // weight, arcs of 32 rows, arcs of a row
+    if (threadIdx.x < 3) s_max[threadIdx.x] = 0ull;
+    __syncthreads();
     uint32_t local_max = 0;
     int64_t tile_arcs = 0, row_arcs = 0;
     for (int64_t u = warp; u < n; u += nwarps) {
@@ -308,9 +311,18 @@ __global__ void csr_check_kernel(int32_t n, int64_t na, const int64_t* __restric
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) local_max = max(local_max, __shfl_xor_sync(FULL, local_max, o));
-    if (lane == 0 && local_max) atomicMax(wmax, (unsigned long long)local_max);
-    if (lane == 0 && tile_arcs > 0) atomicMax(stats, (unsigned long long)tile_arcs);
-    if (lane == 0 && row_arcs > 0) atomicMax(stats + 1, (unsigned long long)row_arcs);
+    // the maxima of the block, then, from blocks that may raise them, those of all (65,000 warps' atomics to three
+    // addresses took 40 us each)
+    if (lane == 0) {
+        atomicMax(&s_max[0], (unsigned long long)local_max);
+        atomicMax(&s_max[1], (unsigned long long)tile_arcs);
+        atomicMax(&s_max[2], (unsigned long long)row_arcs);
+    }
+    __syncthreads();
+    if (threadIdx.x < (stats ? 3 : 1)) {
+        unsigned long long* p = threadIdx.x == 0 ? wmax : stats + threadIdx.x - 1;
+        if (s_max[threadIdx.x] > __ldcg(p)) atomicMax(p, s_max[threadIdx.x]);
+    }
 }
 
 // Targets: in range and distinct; sets in_s[v] = 1 for v in S.
