@@ -65,15 +65,20 @@ typedef struct {
 } bcpp_graph;
 
 typedef struct {
-    int32_t precision;         /* BCPP_FP64 (default) or BCPP_FP32_DELTA */
+    int32_t precision;         /* BCPP_FP64 (default) or BCPP_FP32_DELTA.  FP32 dependencies save memory,
+                                * not time: FP64 is the faster one on all measured graphs (plain Brandes
+                                * at n = 1,000,000 129 against 148 ms, Brandes++ 296 against 1,052 for
+                                * both) since the level-mask kernel adds FP32 in the lockstep kernel's order
+                                * and leaves FP32 with weights or a skeleton to that kernel */
     int32_t halve_undirected;  /* 1 (default): halve undirected results; 0: ordered-pair sums */
     int32_t batch;             /* sources per batch: 0 = default (32), 32 or 64.  64 applies to plain
                                 * Brandes passes (bcpp_brandes, bcpp_brandes_batched, Brandes++ without
                                 * non-frontier nodes); Dijkstra_SK, Brandes_SK with Centrality and
                                 * bcpp_sssp use 32. */
     int32_t ctas_per_sm;       /* resident source batches per SM of the lockstep kernel: 0 = auto (the
-                                * level-mask kernel, which serves FP64 calls with weights up to 32, takes
-                                * its own launch shape whatever this and `cluster` say) */
+                                * level-mask kernel, which serves 32-source batches with weights up to 32
+                                * in FP64, and with unit weights of plain and batched calls in FP32 too, takes its
+                                * own launch shape whatever this and `cluster` say) */
     int32_t validate;          /* reserved: the CSR, S and the partition are always checked */
     int32_t host_buffers;      /* 1: array arguments are host pointers (copied in and out) */
     int32_t order_sources;     /* 1 (default): batch the targets in order of their breadth-first level
@@ -234,7 +239,9 @@ int bcpp_skeleton(bcpp_ctx *ctx, const bcpp_graph *g, const int32_t *S, int32_t 
  * sample fills the GPU at least twice over, or is all of S), and writes into *tuned a copy of
  * *opts (NULL: defaults) whose `batch` and `cluster` are the fastest candidate's.  ms_out
  * (host, may be NULL) receives the candidates' kernel times in milliseconds
- * [BCPP_AUTOTUNE_CANDIDATES] (-1 when |S| < 2).  The tuned options apply to bcpp_brandes,
+ * [BCPP_AUTOTUNE_CANDIDATES] (-1 when |S| < 2).  Where the level-mask kernel serves the sample, the
+ * 32-source candidates are one launch, timed once and reported for each; `cluster` is then the one
+ * that 0 would choose.  The tuned options apply to bcpp_brandes,
  * bcpp_brandes_pp and the plans on the same graph.  Errors as for bcpp_brandes;
  * opts->host_buffers must be 0. */
 #define BCPP_AUTOTUNE_CANDIDATES 4
@@ -246,7 +253,8 @@ int bcpp_autotune(bcpp_ctx *ctx, const bcpp_graph *g, const int32_t *S, int32_t 
  * two or one resident batches per SM (`ctas_per_sm`), in the order (32, 2), (64, 2), (32, 1),
  * (64, 1) -- and writes into *tuned a copy of *opts (NULL: defaults) with the fastest candidate's
  * `batch` and `ctas_per_sm`.  A batched graph's batches are small and numerous, so every batch
- * runs on one CTA (no cluster candidates).  ms_out (host, may be NULL) receives the candidates'
+ * runs on one CTA (no cluster candidates).  Where the level-mask kernel serves the arena, the two
+ * 32-source candidates are one launch, timed once.  ms_out (host, may be NULL) receives the candidates'
  * kernel times in milliseconds [BCPP_AUTOTUNE_BATCHED_CANDIDATES] (-1 for an empty arena).
  * Arguments and errors as for bcpp_brandes_batched; opts->host_buffers must be 0. */
 #define BCPP_AUTOTUNE_BATCHED_CANDIDATES 4

@@ -3482,7 +3482,8 @@ int bcpp_autotune(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
     const int64_t shards = std::max<int64_t>(1, nitems / (2 * wave));
     DBuf<double> scratch(c, g->n);
     if (!scratch) return BCPP_ENOMEM;
-    float best = -1.f;
+    float best = -1.f, first = -1.f;
+    bool alike = false;
     for (int i = 0; i < BCPP_AUTOTUNE_CANDIDATES; i++) {
         bcpp_opts o = base;
         o.batch = cand[i][0];
@@ -3490,13 +3491,23 @@ int bcpp_autotune(bcpp_ctx* c, const bcpp_graph* g, const int32_t* S, int32_t nS
         o.shard_index = 0;
         o.shard_count = (int32_t)shards;
         bcpp_stats st{};
+        if (alike && cand[i][0] == 32) {
+            if (ms_out) ms_out[i] = first;
+            continue;
+        }
         rc = with_capacity_retry(c, [&] { return brandes_dev(c, g, S, nS, o, scratch.p, &st); });
         if (rc != BCPP_OK && rc != BCPP_EOVERFLOW_SIGMA) return rc;
         if (ms_out) ms_out[i] = st.ms_brandes_sk;
+        if (i == 0) {
+            // all on the level-mask kernel, which takes its own launch shape: the other 32-source candidates would
+            // run the same launches (what falls to the lockstep kernel gets the default cluster)
+            alike = c->ran[0] > 0 && c->ran[1] == 0;
+            first = st.ms_brandes_sk;
+        }
         if (best < 0.f || st.ms_brandes_sk < best) {
             best = st.ms_brandes_sk;
             tuned->batch = cand[i][0];
-            tuned->cluster = cand[i][1];
+            tuned->cluster = alike && cand[i][0] == 32 ? choose_cluster(c, (int)nitems, base) : cand[i][1];
         }
     }
     return BCPP_OK;
@@ -3519,16 +3530,25 @@ int bcpp_autotune_batched(bcpp_ctx* c, int32_t num_graphs, const int64_t* graph_
     if (rc) return rc;
     DBuf<double> scratch(c, arena->n);
     if (!scratch) return BCPP_ENOMEM;
-    float best = -1.f;
+    float best = -1.f, first = -1.f;
+    bool alike = false;
     for (int i = 0; i < BCPP_AUTOTUNE_BATCHED_CANDIDATES; i++) {
         bcpp_opts o = base;
         o.batch = cand[i][0];
         o.ctas_per_sm = cand[i][1];
         bcpp_stats st{};
+        if (alike && cand[i][0] == 32) {
+            if (ms_out) ms_out[i] = first;
+            continue;
+        }
         rc = with_capacity_retry(c, [&] { return batched_dev(c, num_graphs, graph_node_ptr, hptr.data(), arena, o,
                                                              scratch.p, &st); });
         if (rc != BCPP_OK && rc != BCPP_EOVERFLOW_SIGMA) return rc;
         if (ms_out) ms_out[i] = st.ms_brandes_sk;
+        if (i == 0) {
+            alike = c->ran[0] > 0 && c->ran[1] == 0;   // as in bcpp_autotune
+            first = st.ms_brandes_sk;
+        }
         if (best < 0.f || st.ms_brandes_sk < best) {
             best = st.ms_brandes_sk;
             tuned->batch = cand[i][0];

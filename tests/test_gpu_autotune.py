@@ -72,3 +72,20 @@ def test_autotune_batched_candidates_and_parity(bc):
     for i, g in enumerate(gs):
         ref, _ = oracle.brandes(g)
         assert rel_err(got[off[i]:off[i + 1]], ref) <= 1e-12, i
+
+
+def test_autotune_times_alike_candidates_once(bc):
+    """On the level-mask kernel the 32-source candidates are the same launch: one time for all of them, and the
+    cluster that the default would choose."""
+    g = gen.planted_partition(2000, 8, 0.03, 0.002, seed=41)
+    G = bc.graph_from_edgelist(g)
+    S = gen.sample_targets(g.n, 640, seed=4)
+    ctx = bc.Context()
+    tuned, times = bc.autotune(G, S, ctx=ctx)
+    assert times[(32, 1)] == times[(32, 2)] == times[(32, 4)] > 0
+    if tuned["batch"] == 32:
+        assert tuned["cluster"] == 4      # 20 batches
+    arena = bc.build_arena([g, gen.erdos_renyi(90, 0.08, seed=3)])
+    _, times = bc.autotune_batched(arena, ctx=ctx)
+    assert times[(32, 2)] == times[(32, 1)] > 0
+    ctx.close()
