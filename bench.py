@@ -221,11 +221,9 @@ def centrality_bytes_per_source(frontiers, interior_nodes, delta_bytes=8):
     return frontiers * (4 + 8 + delta_bytes) + interior_nodes * 8
 
 
-def kernel_name(precision, weights_above_one, skeleton=False):
-    """The shortest-path kernel that a call takes (FP64: level masks; FP32 dependencies: level masks on
-    unit weights without a skeleton, else lockstep)."""
-    levels = precision == "fp64" or not (weights_above_one or skeleton)
-    return "lm_kernel" if levels else "ls_kernel"
+def kernel_name(ran):
+    """The shortest-path kernel that most batches of a call ran on (Context.last_batches)."""
+    return "lm_kernel" if ran["levels"] >= ran["lockstep"] else "ls_kernel"
 
 
 def dist_env():
@@ -605,16 +603,20 @@ def _run_single(args, bc, g, S, ctx, flush, dev, ws, rank, pool):
     my_sources = api.shard_bounds(nS, rank, ws)
     my_ns = my_sources[1] - my_sources[0]
 
+    ran = {}
+
     def step():
         flush.fill_(1)
         st = {}
 
         def plain(r, R):
             _, st["plain"] = bc.brandes(G, Sarg, precision=prec, out=bc_plain, stats=True, ctx=ctx, shard=shard)
+            ran["plain"] = ctx.last_batches()
             return bc_plain
 
         def pp(r, R):
             _, st["pp"] = bc.brandes_pp(G, Sarg, part, precision=prec, out=bc_pp, stats=True, ctx=ctx, shard=shard)
+            ran["pp"] = ctx.last_batches()
             return bc_pp
 
         if ws > 1:
@@ -714,7 +716,7 @@ def _run_single(args, bc, g, S, ctx, flush, dev, ws, rank, pool):
     rooflines = {}
     if not args.no_roofline_model:
         D_avg = _tight_arcs(bc, G, np.linspace(0, n - 1, 32).astype(np.int32), ctx)
-        plain_kernel = kernel_name(prec, g.w is not None)
+        plain_kernel = kernel_name(ran["plain"])
         if plain_kernel == "lm_kernel":
             by_plain = model_bytes_per_source_levels(n, A, D_avg, 32, 4, delta_bytes, g.w is not None) * my_ns
         else:
@@ -727,7 +729,7 @@ def _run_single(args, bc, g, S, ctx, flush, dev, ws, rank, pool):
             sources_per_launch=my_ns)
         skm = _skeleton_model(bc, g, G, S_order, np.asarray(g.part), ctx)
         if sk_ms > 0:
-            sk_kernel = kernel_name(prec, True, skeleton=True)
+            sk_kernel = kernel_name(ran["pp"])
             if sk_kernel == "lm_kernel":
                 by_sk = model_bytes_per_source_levels(skm["N"], skm["arcs"], skm["D"], 32, 8, delta_bytes,
                                                       skm["weighted"], skm["mult"]) * my_ns
@@ -841,9 +843,12 @@ def _run_batched(args, bc, graphs, ctx, flush, dev, ws, rank):
         tuned, times = bc.autotune_batched(arena, precision=prec, ctx=ctx)
         tune = {"tuned": tuned, "candidates_ms": {f"batch{b}_cluster{c}": t for (b, c), t in times.items()}}
 
+    ran = {}
+
     def step():
         flush.fill_(1)
         _, st = bc.brandes_batched(arena, precision=prec, out=out, stats=True, ctx=ctx, **tuned)
+        ran.update(ctx.last_batches())
         return st
 
     dt, wall, logs, clocks = _timed(args, ws, dev, step)
@@ -870,13 +875,19 @@ def _run_batched(args, bc, graphs, ctx, flush, dev, ws, rank):
         fracs.append(D / max(1, Gs.num_arcs))
     tight_frac = float(np.mean(fracs))
     delta_bytes = 4 if prec == "fp32" else 8
-    bytes_launch = float(sum(g.n * model_bytes_per_source_levels(g.n, 2 * g.m, tight_frac * 2 * g.m, 32, 4, delta_bytes)
-                             for g in mine))
+    kernel = kernel_name(ran)
+
+    def model(gn, arcs):
+        if kernel == "lm_kernel":
+            return model_bytes_per_source_levels(gn, arcs, tight_frac * arcs, 32, 4, delta_bytes)
+        return model_bytes_per_source(gn, arcs, tight_frac * arcs, 32, delta_bytes)
+
+    bytes_launch = float(sum(g.n * model(g.n, 2 * g.m) for g in mine))
     hbm, _, peak_kind = measured_peaks()
     ls_ms = statistics.mean(st["ms_brandes_sk"] for st in logs)
     achieved = bytes_launch / (ls_ms / 1e3) / 1e9
     roofline = _roof("hbm", achieved, hbm, "GB/s",
-                     f"{kernel_name(prec, False)} (batched plain Brandes, forward + backward)", None,
+                     f"{kernel} (batched plain Brandes, forward + backward)", None,
                      peak_source="MEASURED_PEAKS.json hbm_gbs (measured)" if peak_kind == "measured"
                      else "fallback 6.8 TB/s", algorithmic_bytes_per_launch=bytes_launch, avg_launch_ms=ls_ms,
                      tight_arc_fraction=tight_frac)

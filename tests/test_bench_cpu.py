@@ -163,3 +163,9 @@ def test_reference_arm_other_ranks_exit_quietly():
                    {"RANK": "1", "WORLD_SIZE": "2", "LOCAL_RANK": "1"})
     assert r.returncode == 0, r.stderr[-2000:]
     assert not [ln for ln in r.stdout.splitlines() if ln.startswith("{")]
+
+
+def test_kernel_name_is_what_ran():
+    assert bench.kernel_name({"levels": 128, "lockstep": 0, "given_back": 0}) == "lm_kernel"
+    assert bench.kernel_name({"levels": 0, "lockstep": 72, "given_back": 16}) == "ls_kernel"
+    assert bench.kernel_name({"levels": 600, "lockstep": 10, "given_back": 10}) == "lm_kernel"
