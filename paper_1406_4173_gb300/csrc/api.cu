@@ -309,8 +309,9 @@ int validate_csr(bcpp_ctx* c, const bcpp_graph* g, uint64_t* wmax_out, const int
     CK_ALLOC(wmax);
     CK_CUDA(cudaMemsetAsync(wmax.p, 0, 3 * sizeof(unsigned long long), c->stream));
     csr_check(g->n, g->num_arcs, g->row_ptr, g->col, g->w, g->directed, c->flags, wmax.p, c->stream, node_off,
-              ngraphs, wmax.p + 1);
-    c->launches++;
+              ngraphs);
+    csr_stats(g->n, g->row_ptr, wmax.p + 1, c->stream);
+    c->launches += 2;
     unsigned long long h[3] = {0, 0, 0};
     CK_RC(to_host(c, h, (const unsigned long long*)wmax.p, 3));
     unsigned long long hw = h[0];

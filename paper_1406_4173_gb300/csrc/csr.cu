@@ -255,25 +255,16 @@ __global__ void csr_sort_long_kernel(const int64_t* __restrict__ rp, int32_t* co
 // With node_off (graph arenas) heads are graph-local ids of the row's graph.
 __global__ void csr_check_kernel(int32_t n, int64_t na, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
                                  const uint32_t* __restrict__ w, int directed, uint32_t* flags,
-                                 unsigned long long* wmax, const int64_t* __restrict__ node_off, int32_t ngraphs,
-                                 unsigned long long* stats) {
+                                 unsigned long long* wmax, const int64_t* __restrict__ node_off, int32_t ngraphs) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     if (warp == 0 && lane == 0) {
         if (rp[0] != 0 || rp[n] != na) flag_invalid(flags, WHY_ROWPTR);
     }
-    __shared__ unsigned long long s_max[3];   // weight, arcs of 32 rows, arcs of a row
-    if (threadIdx.x < 3) s_max[threadIdx.x] = 0ull;
-    __syncthreads();
     uint32_t local_max = 0;
-    int64_t tile_arcs = 0, row_arcs = 0;
     for (int64_t u = warp; u < n; u += nwarps) {
         const int64_t a0 = rp[u], a1 = rp[u + 1];
-        if (stats) {
-            row_arcs = max(row_arcs, a1 - a0);
-            if ((u & 31) == 0) tile_arcs = max(tile_arcs, rp[min(u + 32, (int64_t)n)] - a0);
-        }
         if (a0 > a1 || a0 < 0 || a1 > na) {
             if (lane == 0) flag_invalid(flags, WHY_ROWPTR);
             continue;
@@ -311,18 +302,30 @@ __global__ void csr_check_kernel(int32_t n, int64_t na, const int64_t* __restric
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) local_max = max(local_max, __shfl_xor_sync(FULL, local_max, o));
-    // the maxima of the block, then, from blocks that may raise them, those of all (65,000 warps' atomics to three
-    // addresses took 40 us each)
+    if (lane == 0 && local_max) atomicMax(wmax, (unsigned long long)local_max);
+}
+
+// stats[0] = most arcs of rows [32 i, 32 i + 32), stats[1] = of one row (both zeroed before; a malformed row_ptr gives
+// any number).  In the check itself, whose warps take a row each, it cost 130 us at n = 1,000,000.
+__global__ void csr_stats_kernel(int32_t n, const int64_t* __restrict__ rp, unsigned long long* stats) {
+    __shared__ unsigned long long s_max[2];
+    if (threadIdx.x < 2) s_max[threadIdx.x] = 0ull;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    int64_t tile = 0, row = 0;
+    for (int64_t u0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; u0 < n; u0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t u = u0 + lane, a0 = rp[min(u, (int64_t)n)], a1 = rp[min(u + 1, (int64_t)n)];
+        row = max(row, a1 - a0);
+        tile = max(tile, __shfl_sync(FULL, a1, 31) - __shfl_sync(FULL, a0, 0));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) row = max(row, __shfl_xor_sync(FULL, row, o));
     if (lane == 0) {
-        atomicMax(&s_max[0], (unsigned long long)local_max);
-        atomicMax(&s_max[1], (unsigned long long)tile_arcs);
-        atomicMax(&s_max[2], (unsigned long long)row_arcs);
+        atomicMax(&s_max[0], (unsigned long long)tile);
+        atomicMax(&s_max[1], (unsigned long long)row);
     }
     __syncthreads();
-    if (threadIdx.x < (stats ? 3 : 1)) {
-        unsigned long long* p = threadIdx.x == 0 ? wmax : stats + threadIdx.x - 1;
-        if (s_max[threadIdx.x] > __ldcg(p)) atomicMax(p, s_max[threadIdx.x]);
-    }
+    if (threadIdx.x < 2) atomicMax(stats + threadIdx.x, s_max[threadIdx.x]);
 }
 
 // Targets: in range and distinct; sets in_s[v] = 1 for v in S.
@@ -436,10 +439,13 @@ cudaError_t csr_sort_rows(int32_t n, uint32_t longest, const int64_t* rp, int32_
 }
 
 void csr_check(int32_t n, int64_t na, const int64_t* rp, const int32_t* col, const uint32_t* w, int directed,
-               uint32_t* flags, unsigned long long* wmax, cudaStream_t st, const int64_t* node_off, int32_t ngraphs,
-               unsigned long long* stats) {
+               uint32_t* flags, unsigned long long* wmax, cudaStream_t st, const int64_t* node_off, int32_t ngraphs) {
     csr_check_kernel<<<grid_for((int64_t)n * 32, 256), 256, 0, st>>>(n, na, rp, col, w, directed, flags, wmax,
-                                                                      node_off, ngraphs, stats);
+                                                                      node_off, ngraphs);
+}
+
+void csr_stats(int32_t n, const int64_t* rp, unsigned long long* stats, cudaStream_t st) {
+    if (n > 0) csr_stats_kernel<<<grid_for(n, 256, 152 * 4), 256, 0, st>>>(n, rp, stats);
 }
 
 void csr_localize(int32_t n, const int64_t* rp, const int32_t* col, const int64_t* node_off, int32_t ngraphs,

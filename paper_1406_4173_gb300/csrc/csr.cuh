@@ -26,11 +26,12 @@ void csr_gather_rows(int32_t n, int32_t nrows, const int32_t* rows, const int64_
                      const uint32_t* w, uint64_t* keys, uint32_t* vals, cudaStream_t st);
 void csr_return_rows(int32_t n, int64_t arcs, const int32_t* rows, const int64_t* off, const int64_t* rp, const uint64_t* keys,
                      const uint32_t* vals, int32_t* col, uint32_t* w, uint32_t* flags, cudaStream_t st);
-// checks of a CSR: *wmax (zeroed) = largest weight, stats (two zeroed words; may be null) = most
-// arcs of 32 consecutive rows and of one row
+// checks of a CSR: *wmax (zeroed) = largest weight
 void csr_check(int32_t n, int64_t na, const int64_t* rp, const int32_t* col, const uint32_t* w, int directed,
                uint32_t* flags, unsigned long long* wmax, cudaStream_t st, const int64_t* node_off = nullptr,
-               int32_t ngraphs = 0, unsigned long long* stats = nullptr);
+               int32_t ngraphs = 0);
+// stats (two zeroed words) = most arcs of 32 consecutive rows and of one row
+void csr_stats(int32_t n, const int64_t* rp, unsigned long long* stats, cudaStream_t st);
 // graph-local heads of a disjoint union (flags arcs that leave their graph)
 void csr_localize(int32_t n, const int64_t* rp, const int32_t* col, const int64_t* node_off, int32_t ngraphs,
                   int32_t* lcol, uint32_t* flags, cudaStream_t st);

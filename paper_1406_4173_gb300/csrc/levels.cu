@@ -505,8 +505,9 @@ __device__ __noinline__ void mark_back(uint32_t* bdepth, int nitems, int most, u
     }
 }
 
-// A batch has a path count past 32 bits; more than `most` of them: the level is the last.
-__device__ __forceinline__ void note_wide(uint32_t* b, uint32_t* ctl, uint32_t* lvl, int most) {
+// A batch has a path count past 32 bits; more than `most` of them: the level is the last.  (Not inlined: n = 1,000,000,
+// 4,096 targets 135.9 -> 135.3 ms.)
+__device__ __noinline__ void note_wide(uint32_t* b, uint32_t* ctl, uint32_t* lvl, int most) {
     if (atomicExch(b + 1, 1u) == 0u && (int)(atomicAdd(ctl + CTL_WIDE, 1u) + 1u) > most) atomicOr(lvl, LVL_STOP);
 }
 
