@@ -57,7 +57,7 @@ constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of large
 constexpr int CTL_WIDE = 3, CTL_BACK = 4;   // batches with a path count past 32 bits; batches given back
 constexpr int CTL_LVL = CTL_WORDS;
 constexpr unsigned LVL_ANY = 1u, LVL_STOP = 2u;
-constexpr int PROBE_WORDS = 5;
+constexpr int PROBE_WORDS = 6;
 // Words between two batches' depths: a 128-byte line each, since every SM stores to them once per level (side by
 // side, stores of 152 SMs to a few lines held up everyone's loads: n = 10,000, every node a target 7.4 -> 6.3 ms,
 // Brandes++ at n = 100,000 8.6 -> 7.8 ms).
@@ -447,14 +447,14 @@ __device__ __forceinline__ void tile_sums(const LmArgs& A, SM& sm, int lane, uin
     }
 }
 
-// Pairs reached by level D and by D / 2, and all pairs, of a sample of the unfinished batches' rows; rows of these
-// batches, and all rows sampled.  (Its own function: inlined, it cost the kernel's loops registers, n = 10,000:
+// Pairs reached by level D, by D / 2 and by 3 D / 4, and all pairs, of a sample of the unfinished batches' rows; rows of
+// these batches, and all rows sampled.  (Its own function: inlined, it cost the kernel's loops registers, n = 10,000:
 // 6.1 -> 6.9 ms.)
 __device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int D, int wmax, const uint32_t* bdepth,
                                           const LsItem* items, const int32_t* tile_item, int32_t item_base, int32_t tpb,
                                           uint32_t* probe) {
     const int64_t nt = (int64_t)gridDim.x * LM_THREADS, step = max((int64_t)1, rows / nt);
-    uint32_t b1 = 0, b2 = 0, pairs = 0, open = 0, total = 0;
+    uint32_t b1 = 0, b2 = 0, b3 = 0, pairs = 0, open = 0, total = 0;
     for (int64_t row = ((int64_t)blockIdx.x * LM_THREADS + threadIdx.x) * step; row < rows; row += nt * step) {
         const int32_t t = (int32_t)(row >> 5);
         const int it = tile_item ? __ldg(tile_item + t) - item_base : t / tpb;
@@ -466,10 +466,12 @@ __device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int
             const uint32_t c = __popc(__ldcg(lev + (int64_t)l * rows + row));
             b2 += c;
             if (l <= D / 2) b1 += c;
+            if (l <= D - D / 4) b3 += c;
         }
     }
     b1 = __reduce_add_sync(FULL, b1);
     b2 = __reduce_add_sync(FULL, b2);
+    b3 = __reduce_add_sync(FULL, b3);
     pairs = __reduce_add_sync(FULL, pairs);
     open = __reduce_add_sync(FULL, open);
     total = __reduce_add_sync(FULL, total);
@@ -479,14 +481,17 @@ __device__ __noinline__ void probe_levels(const uint32_t* lev, int64_t rows, int
         atomicAdd(probe + 2, pairs);
         atomicAdd(probe + 3, open);
         atomicAdd(probe + 4, total);
+        atomicAdd(probe + 5, b3);
     }
 }
-// D (pairs / b2)^(1 / dim) levels needed, with 2^dim = b2 / b1: more than 2^k D?
-__device__ __noinline__ bool looks_deep(const uint32_t* probe, int k) {
-    const float b1 = (float)__ldcg(probe), b2 = (float)__ldcg(probe + 1), g = b2 / b1;
+// D (pairs / b2)^(1 / dim) levels needed, with 2^dim = b2 / b1: more than 2^k D?  Not when fewer pairs are found in the
+// last quarter than in the one before, by `keep`: the search runs out (directed graphs, where most pairs are never
+// reached; 20,000 nodes without cycles, weights up to 9, 300 targets: 4.1 -> 3.2 ms).
+__device__ __noinline__ bool looks_deep(const uint32_t* probe, int k, float keep) {
+    const float b1 = (float)__ldcg(probe), b2 = (float)__ldcg(probe + 1), b3 = (float)__ldcg(probe + 5), g = b2 / b1;
     float x = (float)__ldcg(probe + 2) / b2;
     for (; k > 0; k--) x /= g;
-    return b1 > 0.0f && g >= 1.5f && x > 1.0f;
+    return b1 > 0.0f && g >= 1.5f && x > 1.0f && b2 - b3 >= keep * (b3 - b1);
 }
 
 // Marks the batches that are given back: those deeper than `most`, which could still grow past the level where the
@@ -700,7 +705,7 @@ lm_kernel(const LmArgs A, const int sub_log) {
             if (D == part || D == 2 * part) {
                 probe_levels(A.lev, A.rows, D, wmax, bdepth, A.items, A.item_tile0 ? A.tile_item + A.tile_base : nullptr,
                              A.item_base, A.tpb, probe);
-            } else if (looks_deep(probe, early ? 4 : 2)) {
+            } else if (looks_deep(probe, early ? 4 : 2, TABLE ? 0.0f : 0.9f)) {
                 if (blockIdx.x == 0 && threadIdx.x == 0 && !A.item_tile0 && 2 * __ldcg(probe + 3) > __ldcg(probe + 4))
                     atomicOr(&A.flags[FLAG_MASKS], MASKS_ALL);
                 break;

@@ -419,3 +419,19 @@ def test_long_row_of_a_weighted_graph(bc, ctx):
     assert rel_err(bc.brandes(bc.graph_from_edgelist(g), S, ctx=ctx), ref) <= FP64_TOL
     b = ctx.last_batches()
     assert b["levels"] == 0 and b["given_back"] == 0
+
+
+def test_unreachable_pairs_are_not_depth(bc, ctx):
+    """A directed graph without cycles: most pairs are never reached, which the test for deep graphs must not take for
+    levels still to come."""
+    r = np.random.default_rng(2)
+    n = 8000
+    u = r.integers(0, n, 5 * n)
+    v = (u + r.integers(1, n, 5 * n)) % n
+    key = np.unique(np.minimum(u, v).astype(np.int64) * n + np.maximum(u, v))
+    g = gen.EdgeList(n=n, src=(key // n).astype(np.int32), dst=(key % n).astype(np.int32),
+                     w=r.integers(1, 10, len(key)).astype(np.uint32), directed=True)
+    S = gen.sample_targets(n, 100, seed=4)
+    ref, _ = oracle.brandes(g, S)
+    assert rel_err(bc.brandes(bc.graph_from_edgelist(g), S, ctx=ctx), ref) <= FP64_TOL
+    assert ctx.last_batches()["levels"] > 0
