@@ -23,13 +23,16 @@
 // 2 lanes per SM and cycle, are done for packed pairs only.
 //
 // Measured against the lockstep kernel (whole call, FP64): Chung-Lu n = 50,000, every node a target
-// 251 -> 120 ms; n = 1,000,000, 4,096 targets 709 -> 140 ms; directed, n = 100,000, weights 1 to 16,
-// 2,000 targets 141 -> 39 ms; 4,096 random graphs 427 -> 176 ms; n = 2,000, every node 1.76 -> 1.25 ms.
+// 251 -> 119 ms; n = 1,000,000, 4,096 targets 709 -> 135 ms; directed, n = 100,000, weights 1 to 16,
+// 2,000 targets 141 -> 34 ms; 4,096 random graphs 427 -> 177 ms; n = 2,000, every node 1.76 -> 0.77 ms.
 // Brandes_SK (Eq. 11 / Eq. 12: weights, multiplicities, 64-bit counts, and the distance rows that the
-// Centrality step reads) 51 -> 4.4 ms at n = 100,000 and 512 targets, 695 -> 135 ms at n = 1,000,000 and
+// Centrality step reads) 51 -> 4.1 ms at n = 100,000 and 512 targets, 695 -> 133 ms at n = 1,000,000 and
 // 2,048 targets.
-// Bound by the latency of its gathers (a profile at n = 10,000: instructions issued on 27% of the
-// cycles, FP64 pipe busy 33%) and, in the backward pass, by FP64 adds (pipe busy 63% of it).
+// Bound by the latency of its gathers (a profile at n = 10,000: instructions issued on 40% of the
+// cycles, FP64 pipe busy 38%) and, in the backward pass, by FP64 adds (pipe busy 63% of it).
+//
+// Giving back.  A batch that reaches a level past those provided for, or a path count of 2^32 in 32-bit rows, is marked
+// (LmArgs::back), left out of the backward pass and run by the lockstep kernel; the others finish.
 #include <algorithm>
 #include <type_traits>
 
