@@ -58,6 +58,7 @@ constexpr int LM_GATHERS = WEIGHTED ? 3 : 2;
 constexpr int LM_MAX_SUB = 3;      // units of 4 rows at least
 constexpr int LM_CAP = 256;        // arcs of one round of a tile (rows of larger degree go one by one)
 constexpr int CTL_WIDE = 3, CTL_BACK = 4;   // batches with a path count past 32 bits; batches given back
+constexpr int CTL_MOST = 5;                 // batches given back that take the others with them, less one
 constexpr int CTL_LVL = CTL_WORDS;
 constexpr unsigned LVL_ANY = 1u, LVL_STOP = 2u;
 constexpr int PROBE_WORDS = 6;
@@ -513,10 +514,10 @@ __device__ __noinline__ void mark_back(uint32_t* bdepth, int nitems, int most, u
     }
 }
 
-// A batch has a path count past 32 bits; more than `most` of them: the level is the last.  (Not inlined: n = 1,000,000,
+// A batch has a path count past 32 bits; more than ctl[CTL_MOST] of them: the level is the last.  (Not inlined: n = 1,000,000,
 // 4,096 targets 135.9 -> 135.3 ms.)
-__device__ __noinline__ void note_wide(uint32_t* b, uint32_t* ctl, uint32_t* lvl, int most) {
-    if (atomicExch(b + 1, 1u) == 0u && (int)(atomicAdd(ctl + CTL_WIDE, 1u) + 1u) > most) atomicOr(lvl, LVL_STOP);
+__device__ __noinline__ void note_wide(uint32_t* b, uint32_t* ctl, int D) {
+    if (atomicExch(b + 1, 1u) == 0u && atomicAdd(ctl + CTL_WIDE, 1u) + 1u > __ldcg(ctl + CTL_MOST)) atomicOr(ctl + CTL_LVL + D, LVL_STOP);
 }
 
 template <typename SG, typename DT, bool WEIGHTED, bool MULT, bool TABLE>
@@ -591,6 +592,7 @@ lm_kernel(const LmArgs A, const int sub_log) {
         }
     };
 
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl[CTL_MOST] = (uint32_t)(A.nitems / (A.few ? 3 : 2));
     // level 0: each batch's sources
     for (int t = wid; t < A.ntiles; t += nw) {
         const Tile x = tile_of(t);
@@ -670,7 +672,7 @@ lm_kernel(const LmArgs A, const int sub_log) {
                         A.ts[tab + (int64_t)r * nf + s] = acc;
                     }
                     if (drow) drow[r * 32 + s] = D;
-                    if (sizeof(SG) == 4 && (acc >> 32) != 0) note_wide(bdepth + x.it * DEPTH_STRIDE, A.ctl, lvl + D, A.nitems / (A.few ? 3 : 2));
+                    if (sizeof(SG) == 4 && (acc >> 32) != 0) note_wide(bdepth + x.it * DEPTH_STRIDE, A.ctl, D);
                 }
             };
             tile_sums<true, WEIGHTED, MULT, TABLE, SG, uint64_t>(
