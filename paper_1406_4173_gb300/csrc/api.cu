@@ -2869,24 +2869,24 @@ int csr_build_dev(bcpp_ctx* c, int32_t n, int64_t m, const int32_t* eu, const in
     }
     uint32_t* w = ew ? w_out : nullptr;
     const int64_t most = na / CSR_LONG_ROW + 1;   // rows above CSR_LONG_ROW, and one
-    DBuf<uint32_t> counts(c, (int64_t)n + 1), place(c, na), nlong(c, 1);
-    DBuf<CsrLong> info(c, 1);
+    const int64_t words = ((int64_t)n + 2) / 2 * 2;   // counts, then the long rows' figures and list length: zeroed together
+    DBuf<uint32_t> counts(c, words + sizeof(CsrLong) / 4 + 1), place(c, na);
     DBuf<int32_t> rows(c, most);
     DBuf<int64_t> len(c, most), stmp(c, scan_tmp_elems(std::max<int64_t>((int64_t)n + 1, most)));
-    CK_ALLOC(counts); CK_ALLOC(place); CK_ALLOC(nlong); CK_ALLOC(info); CK_ALLOC(rows); CK_ALLOC(len); CK_ALLOC(stmp);
-    CK_CUDA(cudaMemsetAsync(counts.p, 0, ((size_t)n + 1) * sizeof(uint32_t), c->stream));
-    CK_CUDA(cudaMemsetAsync(nlong.p, 0, sizeof(uint32_t), c->stream));
-    CK_CUDA(cudaMemsetAsync(info.p, 0, sizeof(CsrLong), c->stream));
-    csr_count(n, m, eu, ev, ew, directed, counts.p, place.p, info.p, rows.p, len.p, c->flags, c->stream);
+    CK_ALLOC(counts); CK_ALLOC(place); CK_ALLOC(rows); CK_ALLOC(len); CK_ALLOC(stmp);
+    CsrLong* info = reinterpret_cast<CsrLong*>(counts.p + words);
+    uint32_t* nlong = counts.p + words + sizeof(CsrLong) / 4;
+    CK_CUDA(cudaMemsetAsync(counts.p, 0, (size_t)counts.n * sizeof(uint32_t), c->stream));
+    csr_count(n, m, eu, ev, ew, directed, counts.p, place.p, info, rows.p, len.p, c->flags, c->stream);
     c->launches += 2;
     CsrLong h{};
-    CK_CUDA(cudaMemcpyAsync(&h, info.p, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    CK_CUDA(cudaMemcpyAsync(&h, info, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     CK_RC(sync_flags(c));
     if (c->hflags[FLAG_INVALID]) return BCPP_EINVAL;
     exclusive_scan<uint32_t>(counts.p, rp, (int64_t)n + 1, nullptr, stmp.p, c->stream, c->launches);
     csr_scatter(m, eu, ev, ew, directed, rp, place.p, col, w, c->stream);
     // (the counts are no longer needed: the list of long rows takes their place)
-    CK_CUDA(csr_sort_rows(n, h.longest, rp, col, w, reinterpret_cast<int32_t*>(counts.p), nlong.p, c->flags, c->stream));
+    CK_CUDA(csr_sort_rows(n, h.longest, rp, col, w, reinterpret_cast<int32_t*>(counts.p), nlong, c->flags, c->stream));
     c->launches += 3;
     if (h.rows) {
         place.free();

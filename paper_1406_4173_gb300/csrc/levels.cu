@@ -704,8 +704,8 @@ lm_kernel(const LmArgs A, const int sub_log) {
         // the wave.  (Binary tree of 131,071 nodes, weights up to 30, 512 sources: 92.7 -> 90.1 ms, 88.2 without the attempt.)
         // Balls that hardly grow any more belong to stragglers, not to a deep graph.
         const int part = A.lcap / 8;
-        if (A.probe && (D == part || D == part + 1 || D == 2 * part || D == 2 * part + 1)) {
-            const bool early = D <= part + 1;
+        const bool early = D <= part + 1;   // (small waves: the test costs about as much as it saves)
+        if (A.probe && (D == part || D == part + 1 || D == 2 * part || D == 2 * part + 1) && (!early || A.ntiles >= nw)) {
             uint32_t* probe = work + 2 * A.lcap + (early ? 0 : PROBE_WORDS);
             if (D == part || D == 2 * part) {
                 probe_levels(A.lev, A.rows, D, wmax, bdepth, A.items, A.item_tile0 ? A.tile_item + A.tile_base : nullptr,
